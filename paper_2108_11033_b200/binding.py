@@ -1,8 +1,10 @@
-"""Thin ctypes binding of libgrim.so: argument marshalling only.
+"""Thin binding of libgrim.so: argument marshalling only.
 
 Function names mirror the C ABI (include/grim.h).  Host arrays are NumPy arrays, device
-buffers are torch CUDA tensors (torch is used for device memory and streams only).  There
-is no fallback: if the shared library is missing, importing this module raises.
+buffers are torch CUDA tensors (torch is used for device memory and streams only).  Set-up and
+inspection calls go through ctypes; the calls that run once per product are native
+(csrc/grim_py.cpp), because their host time is a visible part of a small product.  There
+is no fallback: if a shared library is missing, importing this module raises.
 """
 from __future__ import annotations
 
@@ -10,6 +12,7 @@ import ctypes as C
 import os
 
 import numpy as np
+import torch  # noqa: F401  (loads the libraries that the native calls need)
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libgrim.so")
@@ -20,6 +23,11 @@ if not os.path.exists(LIB_PATH):
         "(there is no CPU or PyTorch fallback for the CUDA library)")
 
 lib = C.CDLL(LIB_PATH)
+
+# the per-product calls; documented, with their arguments, in csrc/grim_py.cpp and include/grim.h
+from . import _grim_py as _native  # noqa: E402
+from ._grim_py import (grim_bcr_conv2d, grim_bcr_spmm, grim_bcr_spmm_ex, grim_gru_seq, grim_gru_seq_static,  # noqa: E402, F401
+                       grim_gru_step, grim_maxpool2x2)
 
 GRIM_OK = 0
 GRIM_ERR_INVALID_ARG, GRIM_ERR_SHAPE, GRIM_ERR_DTYPE, GRIM_ERR_NOT_BCR = 1, 2, 3, 4
@@ -41,6 +49,9 @@ class GrimError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
         super().__init__(f"{where}: {status_string(status)} (status {status})")
+
+
+_native.set_error_class(GrimError)
 
 
 class grim_mat_t(C.Structure):
@@ -207,23 +218,12 @@ def grim_bcr_unpack_dense(h: int) -> np.ndarray:
 # ------------------------------------------------------------------------------------------ multiply
 
 
-def grim_bcr_spmm(h: int, X, Y, stream=None):
-    mx, my = _mat(X), _mat(Y)
-    _check(lib.grim_bcr_spmm(h, C.byref(mx), C.byref(my), _stream_ptr(stream)), "grim_bcr_spmm")
-
-
 def grim_bcr_reserve(h: int, max_ncols: int):
     _check(lib.grim_bcr_reserve(h, int(max_ncols)), "grim_bcr_reserve")
 
 
 def grim_bcr_status(h: int) -> int:
     return lib.grim_bcr_status(h)
-
-
-def grim_bcr_spmm_ex(h: int, X, Y, tile_n: int = 0, path: int = 0, stream=None):
-    mx, my = _mat(X), _mat(Y)
-    tune = grim_tune_t(tile_n, path)
-    _check(lib.grim_bcr_spmm_ex(h, C.byref(mx), C.byref(my), C.byref(tune), _stream_ptr(stream)), "grim_bcr_spmm_ex")
 
 
 def grim_bcr_tune(h: int, X, Y, reps: int = 5, stream=None):
@@ -233,22 +233,6 @@ def grim_bcr_tune(h: int, X, Y, reps: int = 5, stream=None):
     _check(lib.grim_bcr_tune(h, C.byref(mx), C.byref(my), reps, C.byref(best), C.byref(ms), _stream_ptr(stream)),
            "grim_bcr_tune")
     return dict(tile_n=best.tile_n, path=best.path, ms=ms.value)
-
-
-def grim_bcr_conv2d(h: int, x, out, ksize: int, stride: int = 1, pad: int = 0, bias=None, relu: bool = False,
-                    stream=None, kernel_flags: int = 0):
-    assert x.is_cuda and out.is_cuda and x.is_contiguous() and out.is_contiguous() and x.dim() == 4
-    d = grim_conv_desc_t(x.shape[0], x.shape[1], x.shape[2], x.shape[3], ksize, ksize, stride, pad,
-                         bias.data_ptr() if bias is not None else None, (GRIM_CONV_RELU if relu else 0) | kernel_flags,
-                         _torch_dtype_code(x), _torch_dtype_code(out))
-    _check(lib.grim_bcr_conv2d(h, C.byref(d), x.data_ptr(), out.data_ptr(), _stream_ptr(stream)), "grim_bcr_conv2d")
-
-
-def grim_maxpool2x2(x, out, stream=None):
-    assert x.is_cuda and out.is_cuda and x.is_contiguous() and out.is_contiguous()
-    n, c, hh, ww = x.shape
-    _check(lib.grim_maxpool2x2(x.data_ptr(), out.data_ptr(), n, c, hh, ww, _torch_dtype_code(x), _stream_ptr(stream)),
-           "grim_maxpool2x2")
 
 
 # ------------------------------------------------------------------------------------------ GRU
@@ -263,27 +247,6 @@ def grim_gru_create(W_ih, W_hh, b_ih, b_hh, max_T: int) -> int:
                              arr([k.ctypes.data for k in keep[L:]]), max_T, C.byref(g))
     _check(st, "grim_gru_create")
     return g.value
-
-
-def grim_gru_seq(g: int, x, y, h0=None, hT=None, stream=None):
-    assert x.is_cuda and y.is_cuda and x.is_contiguous() and y.is_contiguous()
-    _check(lib.grim_gru_seq(g, x.data_ptr(), x.shape[0], h0.data_ptr() if h0 is not None else None, y.data_ptr(),
-                            hT.data_ptr() if hT is not None else None, _stream_ptr(stream)), "grim_gru_seq")
-
-
-def grim_gru_seq_static(g: int, x, y, h0=None, hT=None, stream=None):
-    """grim_gru_seq for callers that may not allocate device memory: scratch comes from a fixed 8 MiB
-    array inside the library (shared by all calls; see include/grim.h for the size limit)."""
-    assert x.is_cuda and y.is_cuda and x.is_contiguous() and y.is_contiguous()
-    _check(lib.grim_gru_seq_static(g, x.data_ptr(), x.shape[0], h0.data_ptr() if h0 is not None else None,
-                                   y.data_ptr(), hT.data_ptr() if hT is not None else None, _stream_ptr(stream)),
-           "grim_gru_seq_static")
-
-
-def grim_gru_step(g: int, x, h, y=None, stream=None):
-    assert x.is_cuda and h.is_cuda and x.is_contiguous() and h.is_contiguous() and x.dim() == 2 and h.dim() == 3
-    _check(lib.grim_gru_step(g, x.data_ptr(), x.shape[0], h.data_ptr(), y.data_ptr() if y is not None else None,
-                             _stream_ptr(stream)), "grim_gru_step")
 
 
 def grim_gru_status(g: int) -> int:

@@ -1,9 +1,10 @@
-"""Builds libgrim.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libgrim.so (the C-ABI CUDA library, nvcc for sm_100a) and _grim_py.so (its calls on torch tensors, g++) in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -12,6 +13,8 @@ CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libgrim.so")
 SOURCES = ["grim_pack.cu", "grim_spmm.cu", "grim_stream.cu", "grim_ffma.cu", "grim_tc.cu", "grim_tc2.cu", "grim_api.cu", "grim_gru.cu", "grim_bcrc.cu", "grim_project.cu"]
+PY_SOURCE = os.path.join(CSRC, "grim_py.cpp")
+PY_LIB = os.path.join(PKG, "_grim_py.so")
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
 
@@ -61,7 +64,29 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    _build_py_module()
     return LIB
+
+
+def _build_py_module() -> str:
+    """The extension module: host code only, linked against libgrim.so beside it and the installed torch."""
+    header = os.path.join(ROOT, "include", "grim.h")
+    if not _newer(PY_LIB, [PY_SOURCE, header]):
+        return PY_LIB
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    tlib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"], "-isystem", "/usr/local/cuda/include"]
+    for d in include_paths():
+        cmd += ["-isystem", d]
+    cmd += [PY_SOURCE, "-o", PY_LIB, "-L", PKG, "-l:libgrim.so", "-L", tlib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+            "-Wl,-rpath,$ORIGIN", f"-Wl,-rpath,{tlib}"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        raise RuntimeError("building " + PY_LIB + " failed")
+    return PY_LIB
 
 
 if __name__ == "__main__":
