@@ -97,9 +97,13 @@ typedef struct {
                       pieces) with 1 / 2 groups (block height <= 8 / <= 4), or 17 / 18 / 20 = the 16-column tile
                       for N <= 16 (a lane owns one column) with 1 / 2 / 4 groups; plus 256 x the number of
                       thread blocks that share a tile's block columns (split multiply, 1 - 8);
+                      or 32 = the direct kernel (any N; one launch, everything read straight from L1 / L2: the
+                      default for small and middle-sized products and for right-hand sides whose rows are not
+                      16-byte aligned), 32 + 1, 2 or 4 = with that many columns per lane, then plus 256 x the
+                      number of warps that share a row band (1, 2, 4, 8, 16);
                       path 3: 1 = values staged in registers, 2 = values streamed through shared memory by bulk
                       asynchronous copies (persistent thread blocks), 0 = the streaming variant when it fits */
-  int32_t path;    /* 0 auto; 1 register-tiled CUDA-core kernel (N > 16); 2 tcgen05 tensor-core tiles (bf16
+  int32_t path;    /* 0 auto; 1 register-tiled CUDA-core kernel; 2 tcgen05 tensor-core tiles (bf16
                       handles only); 3 lane-per-column kernel (N <= 16, N = 1 is the matrix-vector product);
                       4 shared-memory slab kernel (any N; the fall-back for operands the others do not take);
                       5 paired tcgen05 kernel: two thread blocks multiply 256 rows x 512 columns together
@@ -243,6 +247,7 @@ grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, in
  * the request returns GRIM_ERR_UNSUPPORTED.  bf16 handles, 3x3 / stride 1 / pad 1 only. */
 #define GRIM_CONV_PAIRED 2u
 #define GRIM_CONV_SINGLE 4u
+#define GRIM_CONV_DIRECT 8u /* the direct CUDA-core kernel: any geometry with KH, KW <= 16, both data types */
 typedef struct {
   int64_t N, C, H, W;
   int32_t KH, KW, stride, pad;

@@ -56,6 +56,8 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
     if (!tc2_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc2(h, a, s);
   }
+  if (path == 1 && (a.tile_n & 32)) return launch_direct(h, a, s);
+  if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
   // 8 <= N <= 16, measured at 8192 x 8192 and 4096 x 4096: bf16 handles are fastest on the tensor-core tile (56 us
   // split over K against 102 us on the lane-per-column kernel), fp32 handles with blocks of 8 rows or more on the
   // CUDA-core kernel's 16-column tile (93 against 98 - 124 us); narrower right-hand sides stay on the lane-per-column
@@ -80,9 +82,8 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
   // (measured at 8192 x 8192, bf16: from N = 32 up the tensor-core tile is 2.6 times faster than the CUDA-core kernel,
   // which widens bf16 to fp32 on the way in; N <= 16 goes to the lane-per-column kernel above)
   if (path == 0 && tc_path_supported(h, a) && a.ncols > kSkinnyMaxN) return launch_spmm_tc(h, a, s);
-  if (ffma_path_supported(h, a)) return launch_ffma(h, a, s);
-  if (path == 1) return GRIM_ERR_UNSUPPORTED;
-  return launch_spmm(h, a, s);
+  if (path == 1) return ffma_path_supported(h, a) ? launch_ffma(h, a, s) : GRIM_ERR_UNSUPPORTED;
+  return launch_cuda_cores(h, a, s);
 }
 
 int dev_sms() {
@@ -124,6 +125,13 @@ __global__ void maxpool2x2_kernel(const T* __restrict__ in, T* __restrict__ out,
 
 }  // namespace
 
+namespace grim {
+grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
+  if (direct_preferred(h, a)) return launch_direct(h, a, s);
+  return ffma_path_supported(h, a) ? launch_ffma(h, a, s) : launch_spmm(h, a, s);
+}
+}  // namespace grim
+
 extern "C" grim_status_t grim_bcr_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, grim_stream_t stream) {
   return run_spmm(h, X, Y, nullptr, (cudaStream_t)stream);
 }
@@ -150,7 +158,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
   float best_t = -1.f;
   grim_tune_t cand_best{};
   // candidates: (path, tile_n); a candidate that cannot take the request is skipped
-  const int cand[][2] = {{1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
+  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
   for (const auto& cd : cand) {
     grim_tune_t c{};
     c.path = cd[0];
@@ -161,7 +169,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
     if (c.path == 1 && c.tile_n <= 4 && c.tile_n > (h->bh <= 4 ? 4 : (h->bh <= 8 ? 2 : 1))) continue;
     if (c.path == 1 && (c.tile_n == 8 || c.tile_n == 9) && (h->bh > (c.tile_n == 8 ? 8 : 4) || X->cols <= 128)) continue;
     // ... 17, 18, 20 = the narrow tile (at most 16 columns) with 1, 2, 4 bands per warp
-    if (c.path == 1 && c.tile_n >= 17 && (X->cols > 16 || c.tile_n - 16 > (h->bh <= 8 ? 4 : 2))) continue;
+    if (c.path == 1 && c.tile_n >= 17 && c.tile_n != 32 && (X->cols > 16 || c.tile_n - 16 > (h->bh <= 8 ? 4 : 2))) continue;
     if (c.path == 1 && c.tile_n < 17 && X->cols <= 16) continue;
     st = run_spmm(h, X, Y, &c, s);  // warm-up
     if (st == GRIM_ERR_UNSUPPORTED) { st = GRIM_OK; continue; }
@@ -225,7 +233,7 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   if (h->device < 0) return GRIM_ERR_INVALID_ARG;
   if (d->N <= 0 || d->C <= 0 || d->H <= 0 || d->W <= 0 || d->KH <= 0 || d->KW <= 0 || d->stride <= 0 || d->pad < 0)
     return GRIM_ERR_INVALID_ARG;
-  if (d->flags & ~(GRIM_CONV_RELU | GRIM_CONV_PAIRED | GRIM_CONV_SINGLE)) return GRIM_ERR_INVALID_ARG;
+  if (d->flags & ~(GRIM_CONV_RELU | GRIM_CONV_PAIRED | GRIM_CONV_SINGLE | GRIM_CONV_DIRECT)) return GRIM_ERR_INVALID_ARG;
   if (d->C * (int64_t)d->KH * d->KW != h->K) return GRIM_ERR_SHAPE;
   const int64_t OH = (d->H + 2 * d->pad - d->KH) / d->stride + 1;
   const int64_t OW = (d->W + 2 * d->pad - d->KW) / d->stride + 1;
@@ -239,7 +247,7 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   a.bias = d->bias_dev; a.relu = (d->flags & GRIM_CONV_RELU) ? 1 : 0;
   a.conv = 1; a.C = (int)d->C; a.H = (int)d->H; a.W = (int)d->W; a.KH = d->KH; a.KW = d->KW;
   a.stride = d->stride; a.pad = d->pad; a.OH = (int)OH; a.OW = (int)OW;
-  if (d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & (GRIM_CONV_PAIRED | GRIM_CONV_SINGLE))) {
+  if (d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & (GRIM_CONV_PAIRED | GRIM_CONV_SINGLE | GRIM_CONV_DIRECT))) {
     // 1 x 1 kernels: the expanded input IS the input - per image a plain Cout x C times C x (H*W) product on the
     // tensors as they lie in memory (row stride H*W), no gather at all; one launch per image
     const int64_t hw = d->H * d->W;
@@ -256,12 +264,12 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
           2 * ((h->tc_mtiles + 1) / 2) * ((hw + 511) / 512) * 3 >= 2 * (int64_t)sm_count(h->device))
         st = launch_spmm_tc2(h, m, (cudaStream_t)stream);
       else if (tc_path_supported(h, m) && hw >= 128) st = launch_spmm_tc(h, m, (cudaStream_t)stream);
-      else if (ffma_path_supported(h, m)) st = launch_ffma(h, m, (cudaStream_t)stream);
-      else st = launch_spmm(h, m, (cudaStream_t)stream);
+      else st = launch_cuda_cores(h, m, (cudaStream_t)stream);
       if (st != GRIM_OK) return st;
     }
     return GRIM_OK;
   }
+  if (d->flags & GRIM_CONV_DIRECT) return launch_direct(h, a, (cudaStream_t)stream);
   if (d->flags & GRIM_CONV_PAIRED) {
     if (!tc2_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc2(h, a, (cudaStream_t)stream);
@@ -272,8 +280,7 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
     return launch_spmm_tc2(h, a, (cudaStream_t)stream);
   if (tc_path_supported(h, a) && a.ncols >= 128) return launch_spmm_tc(h, a, (cudaStream_t)stream);
   if (d->flags & GRIM_CONV_SINGLE) return GRIM_ERR_UNSUPPORTED;
-  if (ffma_path_supported(h, a)) return launch_ffma(h, a, (cudaStream_t)stream);
-  return launch_spmm(h, a, (cudaStream_t)stream);
+  return launch_cuda_cores(h, a, (cudaStream_t)stream);
 }
 
 extern "C" grim_status_t grim_maxpool2x2(const void* in, void* out, int64_t N, int64_t C, int64_t H, int64_t W,

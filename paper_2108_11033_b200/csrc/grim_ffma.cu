@@ -638,6 +638,8 @@ size_t smem_need(const grim_bcr* h, int bpw, int esz, int sld = kTN + 4, int sta
 
 }  // namespace
 
+bool slab_rows_by_tma(const SpmmArgs& a) { return tma_eligible(a); }
+
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   if (h->device < 0 || !h->d_rc_stage || !h->d_status) return false;
   if (h->nbc > kJlistCap || h->rc_max_blob == 0 || h->rc_max_blob > 0xFFFF * 16u) return false;

@@ -932,7 +932,7 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
     a.y_prefilled = 1;  // every row of the buffer already holds b_ih (below): a split multiply adds onto it and
                         // needs neither its own clearing nor a bias pass; an unsplit one writes sum + bias as usual
     if (g->profile) profile_mark(g, 0, s);
-    const grim_status_t st = ffma_path_supported(wi, a) ? launch_ffma(wi, a, s) : launch_spmm(wi, a, s);
+    const grim_status_t st = launch_cuda_cores(wi, a, s);
     if (g->profile) profile_mark(g, 1, s);
     return st;
   };
@@ -1182,7 +1182,7 @@ extern "C" grim_status_t grim_gru_step(grim_gru_t g, const float* x, int64_t B, 
       a.x_sk = 1; a.x_sq = mats[t]->K; a.y_sr = 1; a.y_sq = 3 * H;
       a.x_dtype = GRIM_F32; a.y_dtype = GRIM_F32;
       a.bias = bias[t];
-      const grim_status_t st = ffma_path_supported(mats[t], a) ? launch_ffma(mats[t], a, s) : launch_spmm(mats[t], a, s);
+      const grim_status_t st = launch_cuda_cores(mats[t], a, s);
       if (st != GRIM_OK) return st;
     }
     const int64_t total = B * H;

@@ -72,6 +72,15 @@ struct RunDesc {
 // ---------------------------------------------------------------------------------------------
 constexpr int kRcBands = 16;
 constexpr int kRcChunk = 8;
+// Beside it, for the kernels that walk one band at a time, a table with what they need to know about a block before
+// they can ask for its weights and activations (one 16-byte load instead of stage entry -> header -> record):
+struct __align__(16) RcHead {
+  uint32_t rec16;    // record start in 16-byte units from the blob base
+  uint32_t rows_kc;  // kept rows (low half, bit mask) | kept columns << 16; 0: nothing kept
+  uint32_t cols[2];  // the first eight entries of cols
+};
+__host__ __device__ inline uint32_t rc_head_rows(uint32_t rows_kc) { return rows_kc & 0xFFFFu; }
+__host__ __device__ inline int rc_head_kc(uint32_t rows_kc) { return (int)(rows_kc >> 16); }
 struct RcStage {
   uint32_t off16;  // blob start in 16-byte units from the blob base
   uint32_t bytes;  // multiple of 16; 0 when no band of the group keeps anything in this block column
@@ -134,6 +143,8 @@ struct grim_bcr {
   // device
   int device = -1;
   grim::RcStage* d_rc_stage = nullptr;
+  grim::RcHead* d_rc_head = nullptr;
+  int64_t rc_chunks = 0;  // chunks of eight kept columns, summed over all blocks
   uint8_t* d_rc_blob = nullptr;
   // tensor-core layout
   int64_t tc_mtiles = 0, tc_ktiles = 0;
@@ -199,6 +210,13 @@ grim_status_t launch_stream(const grim_bcr* h, const void* X, int x_dtype, int64
 bool stream_path_supported(const grim_bcr* h, int64_t N);
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
+bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA
+// the CUDA-core kernel for a request: direct, slab or, for operands neither takes, the shared-memory slab fall-back
+grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
+// small and middle-sized products without a block-wide pipeline (also convolutions)
+grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
+bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a);
+bool direct_preferred(const grim_bcr* h, const SpmmArgs& a);  // over the other CUDA-core kernels, for this request
 grim_status_t launch_spmm_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool tc_path_supported(const grim_bcr* h, const SpmmArgs& a);
 // the paired (two thread blocks per tile pair) tensor-core kernel: matrices, bf16 handles

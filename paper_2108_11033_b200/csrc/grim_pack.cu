@@ -51,6 +51,7 @@ void free_device(grim_bcr* h) {
   cudaFree(h->d_run_ptr);
   cudaFree(h->d_runs);
   cudaFree(h->d_rc_stage);
+  cudaFree(h->d_rc_head);
   cudaFree(h->d_rc_blob);
   cudaFree(h->d_sl_colwords);
   cudaFree(h->d_sl_vals);
@@ -353,9 +354,11 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
     // ---- row-chunk layout for the register-tiled and tensor-core kernels
     std::vector<RcStage> rc_stage;
     std::vector<uint8_t> rc_blob;
+    std::vector<RcHead> rc_head;  // by schedule position and block column
     {
       h->rc_groups = (nbr + kRcBands - 1) / kRcBands;
       rc_stage.resize((size_t)(h->rc_groups * nbc));
+      rc_head.assign((size_t)(nbr * nbc), RcHead{0u, 0u, {0u, 0u}});
       rc_blob.reserve((size_t)nnz * 5 + (size_t)h->nonempty * 32 + 1024);
       uint32_t rc_max = 0;
       for (int64_t g = 0; g < h->rc_groups && st == GRIM_OK; ++g) {
@@ -392,6 +395,11 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
             for (int c = 0; c < 64; ++c)
               if ((hb.colmask >> c) & 1ull) cols[n++] = (uint8_t)c;
             for (int c = 0; c < nch * kRcChunk; ++c) rc_blob[rec + 8 + (size_t)c] = cols[c < kc ? c : 0];
+            RcHead& hd = rc_head[(size_t)(pos * nbc + j)];
+            hd.rec16 = (uint32_t)(rec / 16);
+            hd.rows_kc = hb.rowmask | ((uint32_t)kc << 16);
+            std::memcpy(hd.cols, &rc_blob[rec + 8], 8);
+            h->rc_chunks += nch;
             float* w = reinterpret_cast<float*>(&rc_blob[rec + idx_bytes]);
             const float* src = &h->vals[(size_t)hb.val_off];
             for (int c = 0; c < kc; ++c)
@@ -491,6 +499,7 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
       if (e == cudaSuccess && wide) e = upload(&h->d_blob, blob.data(), blob.size());
       if (e == cudaSuccess) e = upload(&h->d_band_order, h->band_order.data(), h->band_order.size() * 4);
       if (e == cudaSuccess && wide) e = upload(&h->d_rc_stage, rc_stage.data(), rc_stage.size() * sizeof(RcStage));
+      if (e == cudaSuccess && wide) e = upload(&h->d_rc_head, rc_head.data(), rc_head.size() * sizeof(RcHead));
       if (e == cudaSuccess && wide) e = upload(&h->d_rc_blob, rc_blob.data(), rc_blob.size());
       if (e == cudaSuccess && tc_shape && wide) {
         e = upload(&h->d_td_stage, td_stage.data(), td_stage.size() * sizeof(RcStage));

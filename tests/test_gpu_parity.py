@@ -195,6 +195,32 @@ def test_paired_tensor_core_kernel_explicit(B, case, y_bf16):
     check_spmm(B, W, mask, X, bh, bw, bf16=True, path=5, flags=1, y_bf16=y_bf16)
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("case", [(304, 520, 4, 16, 1, 1, 31), (300, 700, 8, 32, 1, 16, 33), (129, 333, 16, 64, 2, 16, 63),
+                                  (300, 520, 4, 16, 2, 4, 65), (260, 700, 16, 64, 4, 8, 131), (512, 768, 8, 32, 4, 2, 256),
+                                  (200, 300, 5, 20, 4, 1, 129), (7, 40, 3, 9, 2, 8, 5), (512, 2100, 8, 32, 2, 8, 130), (96, 96, 16, 16, 1, 2, 2)])
+def test_direct_kernel_explicit(B, case, bf16):
+    """Columns per lane x warps per band: widths around a tile's edge, vector and scalar loads of X, bands with nothing
+    kept, block sizes below the compiled row counts, more warps per band than block columns."""
+    M, K, bh, bw, nc, parts, N = case
+    W = gen.dense_weight(M, K, seed=171)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=3, dist="zipf", seed=172, empty_frac=0.3)
+    mask[:bh] = 0
+    X = gen.normal_f32((K, N), 1.0, 173, 0)
+    check_spmm(B, W, mask, X, bh, bw, bf16=bf16, path=1, tile_n=32 + nc + 256 * parts, y_bf16=bf16 and parts == 1)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("geom", [(3, 1, 1, 9, 13), (3, 2, 1, 15, 8), (5, 1, 2, 7, 7), (1, 2, 0, 9, 9), (16, 3, 5, 21, 19), (2, 1, 0, 6, 33)])
+def test_direct_kernel_convolution(B, geom, bf16):
+    ksize, stride, pad, hh, ww = geom
+    W = gen.dense_weight(40, 6 * ksize * ksize, seed=174)
+    mask = gen.bcr_mask(40, 6 * ksize * ksize, 8, 32, compression=3, dist="uniform", seed=175, empty_frac=0.2)
+    x = np.maximum(gen.normal_f32((3, 6, hh, ww), 1.0, 176, 0), 0.0)
+    L = dict(W=W, mask=mask, bias=gen.normal_f32((40,), 0.05, 177, 0), bh=8, bw=32)
+    check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=bf16, kernel_flags=B.GRIM_CONV_DIRECT)
+
+
 @pytest.mark.parametrize("split", [2, 5, 8])
 def test_split_multiply(B, split):
     """Few output tiles: several thread blocks share a tile's block columns and add their partial sums into a
