@@ -113,6 +113,14 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// True in one lane of a fully active warp.  Copies and multiplies take their operands from uniform registers: inside a
+// branch on elect.sync the compiler knows that one thread runs, inside one on the lane number it has to make sure of it
+// for every operand of every instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p = 0;
+  asm volatile("{\n.reg .b32 r;\n.reg .pred q;\nelect.sync r|q, 0xffffffff;\n@q mov.s32 %0, 1;\n}" : "+r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));

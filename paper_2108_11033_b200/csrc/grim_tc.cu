@@ -198,13 +198,13 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
   int fail_site = 0;
   if (warp == 0) {
     // ------------------------------------------------------------------ copies
-    if (lane == 0) {
+    if (elect_one()) {
       // the first records (the ring of records is deeper than the ring of tiles); later ones are requested by the
       // expansion warps as they free a record slot
       for (int rk = 0; rk < nr && rk < nkt; ++rk) request_records(rk, rk);
+      int slot = 0, round = 0;  // ring position; the ring has been gone through `round` times
       for (int kt = 0; kt < nkt && !CONV; ++kt) {  // the convolution builds its X tiles itself
-        const int slot = kt % ns;
-        if (kt >= ns && !mbar_wait(empty + slot, (unsigned)((kt / ns - 1) & 1), p.spin_limit, s_abort)) { failed = true, fail_site = 1; break; }
+        if (round > 0 && !mbar_wait(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
         uint8_t* st = stages + (size_t)slot * stage_bytes;
         // 64-column boxes that lie wholly past the last column are not requested (their part of the tile keeps
         // whatever it held; the accumulator columns computed from it are never stored)
@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
 #pragma unroll
         for (int i = 0; i < kTQ / 64; ++i)
           if (i < nbox) tma_load_2d(st + b_off + i * (64 * kTK * 2), &tmX, (int)q0 + 64 * i, (kbase + kt) * kTK, full + slot);
+        if (++slot == ns) { slot = 0; ++round; }
       }
     }
     if (CONV >= 2) {
@@ -221,12 +222,12 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ tensor core
-    if (lane == 0) {
+    if (elect_one()) {
+      int slot = 0;
+      unsigned par = 0;
       for (int kt = 0; kt < nkt; ++kt) {
-        const int slot = kt % ns;
-        const unsigned par = (unsigned)((kt / ns) & 1);
-        if ((!CONV && !mbar_wait(full + slot, par, p.spin_limit, s_abort)) || !mbar_wait(ready + slot, par, p.spin_limit, s_abort) ||
-            (CONV && !mbar_wait(built + slot, par, p.spin_limit, s_abort))) { failed = true, fail_site = 2; break; }
+        if ((!CONV && !mbar_wait(full + slot, par, p.spin_limit << 2, s_abort, 0)) || !mbar_wait(ready + slot, par, p.spin_limit << 2, s_abort, 0) ||
+            (CONV && !mbar_wait(built + slot, par, p.spin_limit << 2, s_abort, 0))) { failed = true, fail_site = 2; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a_addr = smem_u32(stages + (size_t)slot * stage_bytes);
         const uint32_t b_addr = a_addr + b_off;
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
           }
         }
         umma_commit(empty + slot);  // arrives when the multiplies above have read their operands
+        if (++slot == ns) { slot = 0; par ^= 1u; }
       }
       if (!failed) umma_commit(acc_done);
     }

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
         for (int rk = 0; rk < nr && rk < nkt; ++rk) request_record(rk, rk);
       __syncwarp();
       if (CONV >= 2 && !conv_copy_planes<CONV>(im, lane)) failed = true, fail_site = 1;
-    } else if (lane == 0) {
+    } else if (elect_one()) {
       for (int rk = 0; rk < nr && rk < nkt; ++rk) request_record(rk, rk);
       // 64-column boxes wholly past the last column are not requested (their part of the tile keeps whatever it
       // held; the accumulator columns computed from it are never stored)
@@ -222,20 +222,21 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
       constexpr int kPrefetch = 8;
       for (int kt = 0; kt < kPrefetch && kt < nkt; ++kt)
         for (int i = 0; i < nbox; ++i) tma_prefetch_2d(&tmX, (int)qb + 64 * i, kt * kK);
+      int slot = 0, round = 0;  // ring position; the ring has been gone through `round` times
       for (int kt = 0; kt < nkt; ++kt) {
-        const int slot = kt % ns;
         if (kt + kPrefetch < nkt)
           for (int i = 0; i < nbox; ++i) tma_prefetch_2d(&tmX, (int)qb + 64 * i, (kt + kPrefetch) * kK);
-        if (kt >= ns && !mbar_wait<true>(empty + slot, (unsigned)((kt / ns - 1) & 1), p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
+        if (round > 0 && !mbar_wait<true>(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
         uint8_t* bt = stages + (size_t)slot * kStageBytes + kABytes;
         if (rank == 0) mbar_arrive_expect_tx(ready + slot, pair_bytes);
 #pragma unroll
         for (int i = 0; i < kColsPerBlock / 64; ++i)
           if (i < nbox) tma_load_2d_pair(bt + i * (64 * kK * 2), &tmX, (int)qb + 64 * i, kt * kK, ready0 + (uint32_t)slot * 8u);
+        if (++slot == ns) { slot = 0; ++round; }
       }
     }
   } else if (warp == 1 || warp == kIssueWarp2) {
-    if (lane == 0 && rank == 0 && !((p.flags & 1) && warp != 1)) {
+    if (rank == 0 && !((p.flags & 1) && warp != 1) && elect_one()) {
       // ------------------------------------------------------------------ tensor core (even block)
       // Two issuing threads, one per accumulator.  Issuing is asynchronous but the queue is short, so a thread is
       // held while its multiplies wait their turn; its poll of the next stage's barrier (a few hundred cycles
@@ -245,12 +246,14 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
       // shared-memory round trip sits between the multiplies of consecutive stages.
       const int acc = warp == 1 ? 0 : 1;
       bool have = false;
+      int slot = 0;
+      unsigned par = 0;
       for (int kt = 0; kt < nkt; ++kt) {
-        const int slot = kt % ns;
-        const unsigned par = (unsigned)((kt / ns) & 1);
+        const int nslot = slot + 1 == ns ? 0 : slot + 1;
+        const unsigned npar = nslot ? par : par ^ 1u;
         if (!have && !mbar_wait<true>(ready + slot, par, p.spin_limit << 3, s_abort, 0)) { failed = true, fail_site = 2; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        have = kt + 1 < nkt && mbar_test_wait_cluster(ready + (kt + 1) % ns, (unsigned)(((kt + 1) / ns) & 1));
+        have = kt + 1 < nkt && mbar_test_wait_cluster(ready + nslot, npar);
         const uint32_t a_addr = smem_u32(stages + (size_t)slot * kStageBytes);
         const uint32_t b_addr = a_addr + kABytes;
         for (int ac = (p.flags & 1) ? 0 : acc; ac <= ((p.flags & 1) ? 1 : acc); ++ac) {
@@ -266,6 +269,8 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
         }
         umma2_commit_both(empty + slot);  // arrives in both blocks when this thread's multiplies have read their operands
         if (p.flags & 1) umma2_commit_both(empty + slot);
+        slot = nslot;
+        par = npar;
       }
       if (!failed) umma2_commit_both(acc_done);
       if (!failed && (p.flags & 1)) umma2_commit_both(acc_done);
