@@ -123,6 +123,34 @@ __global__ void maxpool2x2_kernel(const T* __restrict__ in, T* __restrict__ out,
   }
 }
 
+// The same with V outputs of a row per thread (the largest of 8, 4, 2 that divides the row and fills a 16-byte vector), two
+// vector loads.  The pass only moves memory; one 2-byte load and two 64-bit divisions per element kept it at 2.2 TB/s (64
+// channels, 224 x 224, 16 images, bf16: 59 us).
+template <typename T, int V>
+__global__ void __launch_bounds__(256) maxpool2x2_vec_kernel(const T* __restrict__ in, T* __restrict__ out, unsigned total, unsigned groups) {
+  struct __align__(sizeof(T) * 2 * V < 16 ? sizeof(T) * 2 * V : 16) In { T v[2 * V]; };
+  struct __align__(sizeof(T) * V < 16 ? sizeof(T) * V : 16) Out { T v[V]; };
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const unsigned i = blockIdx.x * 256u + threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (i >= total) return;
+  const unsigned line = i / groups, g = i - line * groups;  // output row (of all planes), piece of it
+  const unsigned W = groups * V * 2;
+  const T* p = in + (size_t)line * 2 * W + (size_t)g * 2 * V;
+  const In a = *reinterpret_cast<const In*>(p), b = *reinterpret_cast<const In*>(p + W);
+  Out o;
+#pragma unroll
+  for (int e = 0; e < V; ++e)
+    o.v[e] = (T)fmaxf(fmaxf((float)a.v[2 * e], (float)a.v[2 * e + 1]), fmaxf((float)b.v[2 * e], (float)b.v[2 * e + 1]));
+  *reinterpret_cast<Out*>(out + (size_t)line * groups * V + (size_t)g * V) = o;
+}
+template <typename T, int V>
+cudaError_t launch_maxpool(const void* in, void* out, int64_t planes, int64_t OH, int64_t OW, cudaStream_t s) {
+  const int64_t total = planes * OH * (OW / V);
+  return launch_pdl(maxpool2x2_vec_kernel<T, V>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, static_cast<const T*>(in),
+                    static_cast<T*>(out), (unsigned)total, (unsigned)(OW / V));
+}
+
 }  // namespace
 
 namespace grim {
@@ -288,7 +316,20 @@ extern "C" grim_status_t grim_maxpool2x2(const void* in, void* out, int64_t N, i
   if (!in || !out || N <= 0 || C <= 0 || H <= 0 || W <= 0) return GRIM_ERR_INVALID_ARG;
   if ((H & 1) || (W & 1)) return GRIM_ERR_SHAPE;
   if (dtype != GRIM_F32 && dtype != GRIM_BF16) return GRIM_ERR_DTYPE;
-  const int64_t total = N * C * (H / 2) * (W / 2);
+  const int64_t total = N * C * (H / 2) * (W / 2), planes = N * C, OH = H / 2, OW = W / 2;
+  // rows start at multiples of W, so pieces of V outputs are aligned when the tensors are
+  if ((OW & 1) == 0 && total < (int64_t(1) << 31) && reinterpret_cast<uintptr_t>(in) % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0) {
+    cudaStream_t st = (cudaStream_t)stream;
+    cudaError_t e;
+    if (dtype == GRIM_F32)
+      e = OW % 4 == 0 ? launch_maxpool<float, 4>(in, out, planes, OH, OW, st) : launch_maxpool<float, 2>(in, out, planes, OH, OW, st);
+    else
+      e = OW % 8 == 0 ? launch_maxpool<__nv_bfloat16, 8>(in, out, planes, OH, OW, st)
+                      : (OW % 4 == 0 ? launch_maxpool<__nv_bfloat16, 4>(in, out, planes, OH, OW, st) : launch_maxpool<__nv_bfloat16, 2>(in, out, planes, OH, OW, st));
+    count_launch();
+    if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+    return GRIM_OK;
+  }
   const int threads = 256;
   const int blocks = (int)std::min<int64_t>((total + threads - 1) / threads, (int64_t)dev_sms() * 16);
   cudaStream_t s = (cudaStream_t)stream;
