@@ -201,10 +201,10 @@ grim_status_t grim_bcr_unpack_dense(grim_bcr_t h, float* W_host, int64_t ldw);
 grim_status_t grim_bcr_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, grim_stream_t stream);
 
 /* Workspace of the split tensor-core multiply (Section 4.5: the tile plan depends on the problem; bf16 handles with
- * few output tiles and a long K - small batches of the deeper convolution layers - are split over K through an fp32
- * scratch of M x N floats).  Compute calls never allocate: grim_bcr_reserve allocates that scratch for right-hand
+ * few output tiles and a long K are split over K through an fp32 scratch) and of the tensor-core convolution (a
+ * channel-last copy of the input).  Compute calls never allocate: grim_bcr_reserve allocates that scratch for right-hand
  * sides of up to max_ncols columns (for a convolution: images x OH x OW), once, at set-up time; it synchronises the
- * device.  Without it (or beyond max_ncols) such multiplies simply run unsplit, slower.  max_ncols = 0 frees it.
+ * device.  Without it (or beyond max_ncols) such calls simply run on other kernels, slower.  max_ncols = 0 frees it.
  * More than 2^30 bytes -> GRIM_ERR_UNSUPPORTED. */
 grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols);
 
@@ -248,6 +248,8 @@ grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, in
 #define GRIM_CONV_PAIRED 2u
 #define GRIM_CONV_SINGLE 4u
 #define GRIM_CONV_DIRECT 8u /* the direct CUDA-core kernel: any geometry with KH, KW <= 16, both data types */
+#define GRIM_CONV_TENSOR 16u /* the tensor-core kernel on a channel-last copy of the input: bf16 handles, 3x3 and 5x5, any
+                                stride up to 8, needs grim_bcr_reserve; and any convolution with C * KH * KW <= 64 */
 typedef struct {
   int64_t N, C, H, W;
   int32_t KH, KW, stride, pad;

@@ -34,7 +34,7 @@ GRIM_ERR_INVALID_ARG, GRIM_ERR_SHAPE, GRIM_ERR_DTYPE, GRIM_ERR_NOT_BCR = 1, 2, 3
 GRIM_ERR_ALLOC, GRIM_ERR_CUDA, GRIM_ERR_UNSUPPORTED, GRIM_ERR_TIMEOUT = 5, 6, 7, 8
 GRIM_F32, GRIM_BF16 = 0, 1
 GRIM_PACK_REORDER, GRIM_PACK_HOST_ONLY, GRIM_PACK_NARROW_ONLY, GRIM_PACK_WIDE_ONLY = 1, 2, 4, 8
-GRIM_CONV_RELU, GRIM_CONV_PAIRED, GRIM_CONV_SINGLE, GRIM_CONV_DIRECT = 1, 2, 4, 8
+GRIM_CONV_RELU, GRIM_CONV_PAIRED, GRIM_CONV_SINGLE, GRIM_CONV_DIRECT, GRIM_CONV_TENSOR = 1, 2, 4, 8, 16
 
 EXPORTED = [
     "grim_bcr_pack", "grim_bcr_destroy", "grim_bcr_info", "grim_bcr_export", "grim_bcr_unpack_dense",

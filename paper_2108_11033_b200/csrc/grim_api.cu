@@ -242,8 +242,10 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
 extern "C" grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols) {
   if (!h || max_ncols < 0) return GRIM_ERR_INVALID_ARG;
   if (h->device < 0) return GRIM_ERR_INVALID_ARG;
-  const size_t need = (size_t)h->M * (size_t)max_ncols * 4;
-  if (need > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;  // the split multiply is only used for small outputs
+  const size_t acc = (size_t)h->M * (size_t)max_ncols * 4;
+  if (acc > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;
+  // the split multiply only takes outputs of at most half a tile per SM, which is less than 40 MiB
+  const size_t need = std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols));
   if (h->tc_acc_bytes >= need && need > 0) return GRIM_OK;
   if (cudaDeviceSynchronize() != cudaSuccess) return GRIM_ERR_CUDA;  // a launch in flight may still use the old scratch
   cudaFree(h->d_tc_acc);
@@ -261,7 +263,8 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   if (h->device < 0) return GRIM_ERR_INVALID_ARG;
   if (d->N <= 0 || d->C <= 0 || d->H <= 0 || d->W <= 0 || d->KH <= 0 || d->KW <= 0 || d->stride <= 0 || d->pad < 0)
     return GRIM_ERR_INVALID_ARG;
-  if (d->flags & ~(GRIM_CONV_RELU | GRIM_CONV_PAIRED | GRIM_CONV_SINGLE | GRIM_CONV_DIRECT)) return GRIM_ERR_INVALID_ARG;
+  constexpr uint32_t kKernelFlags = GRIM_CONV_PAIRED | GRIM_CONV_SINGLE | GRIM_CONV_DIRECT | GRIM_CONV_TENSOR;
+  if (d->flags & ~(GRIM_CONV_RELU | kKernelFlags)) return GRIM_ERR_INVALID_ARG;
   if (d->C * (int64_t)d->KH * d->KW != h->K) return GRIM_ERR_SHAPE;
   const int64_t OH = (d->H + 2 * d->pad - d->KH) / d->stride + 1;
   const int64_t OW = (d->W + 2 * d->pad - d->KW) / d->stride + 1;
@@ -275,7 +278,7 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   a.bias = d->bias_dev; a.relu = (d->flags & GRIM_CONV_RELU) ? 1 : 0;
   a.conv = 1; a.C = (int)d->C; a.H = (int)d->H; a.W = (int)d->W; a.KH = d->KH; a.KW = d->KW;
   a.stride = d->stride; a.pad = d->pad; a.OH = (int)OH; a.OW = (int)OW;
-  if (d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & (GRIM_CONV_PAIRED | GRIM_CONV_SINGLE | GRIM_CONV_DIRECT))) {
+  if (d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & kKernelFlags)) {
     // 1 x 1 kernels: the expanded input IS the input - per image a plain Cout x C times C x (H*W) product on the
     // tensors as they lie in memory (row stride H*W), no gather at all; one launch per image
     const int64_t hw = d->H * d->W;
@@ -302,7 +305,16 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
     if (!tc2_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc2(h, a, (cudaStream_t)stream);
   }
-  // bf16 handles: tensor cores; the paired kernel when its 256 x 512 tiles still give most SMs a thread block
+  if (d->flags & GRIM_CONV_TENSOR) return launch_conv_tc(h, a, (cudaStream_t)stream);
+  if (!(d->flags & GRIM_CONV_SINGLE) && conv_tc_supported(h, a)) {
+    // two launches and a pipeline to fill: below some 16 MFLOP the direct kernel is done earlier (96 -> 136 channels, 14 x 14,
+    // two images: 9.1 against 7.3 us; 64 -> 128, 56 x 56, stride 2, two images, 29 MFLOP: 8.1 against 15.2), except where
+    // the input needs no channel-last copy (3 -> 40 channels, 20 x 24: 5.7 against 9.2)
+    const bool small = 2.0 * (double)h->nnz * (double)a.ncols <= 1.6e7 && h->K > 64;
+    return small && direct_path_supported(h, a) ? launch_direct(h, a, (cudaStream_t)stream) : launch_conv_tc(h, a, (cudaStream_t)stream);
+  }
+  // without the workspace of grim_bcr_reserve: tensor-core kernels that build the expanded input tile by tile; the paired
+  // kernel when its 256 x 512 tiles still give most SMs a thread block
   if (!(d->flags & GRIM_CONV_SINGLE) && tc2_path_supported(h, a) && h->tc_mtiles >= 2 &&
       2 * ((h->tc_mtiles + 1) / 2) * ((a.ncols + 511) / 512) * 3 >= 2 * (int64_t)sm_count(h->device))
     return launch_spmm_tc2(h, a, (cudaStream_t)stream);

@@ -1,0 +1,700 @@
+// Tensor-core convolution for bf16 handles (Section 3.1: a convolution is a GEMM whose right-hand side is the expanded
+// input; Section 4.5: that matrix is never produced in memory).
+//
+//   out[pixel, channel] = sum over (tap, input channel) of in[pixel shifted by tap, input channel] * W[channel, tap, input channel]
+//
+// Two launches.  conv_nhwc_kernel turns the NCHW input channel-last in a scratch of the handle (one pass, channels padded
+// to a multiple of 8).  conv_tc_kernel then is a plain pipeline: TMA fetches the tile of input pixels of a tap straight
+// from the channel-last copy (im2col mode: the copy engine walks rows and images, applies stride and padding), TMA fetches
+// the tile of the expanded weights, one thread issues the multiplies, eight warps store the results.  Pixels are the rows
+// of the multiply, so a lane of the epilogue holds one pixel and a warp's store of one channel is contiguous in NCHW.
+// Convolutions whose whole K fits one tile of 64 (few input channels: the first layer of a network) skip the
+// channel-last copy: warps gather the tile of pixels from the NCHW input.
+//
+// The weights are expanded (zeros in place) once, when the matrix is packed: a convolution's matrix is small (4.7 MB for
+// 512 x 512 x 3 x 3) and read from L2 by every pixel tile, so expanding packed records per tile, as the matrix kernels
+// do, would only cost shared-memory bandwidth, which with the tensor core is what bounds the loop.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "grim_device.cuh"
+#include "grim_internal.h"
+
+namespace grim {
+namespace {
+
+using namespace ptx;
+
+// ------------------------------------------------------------------------------------------ NCHW -> channel-last
+// A thread block turns a 64-channel x 64-pixel tile around in shared memory.  Row pitch 65 elements: the eight lanes that
+// read eight channels of one pixel then fall into different banks (8 * 65 * 2 bytes = 4 banks apart).
+constexpr int kTrPitch = 65;
+__global__ void __launch_bounds__(256) conv_nhwc_kernel(const unsigned short* __restrict__ in, unsigned short* __restrict__ out, int C, int Cp,
+                                                        int hw, int vec) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __shared__ unsigned short t[64 * kTrPitch];
+  const int p0 = blockIdx.x * 64, c0 = blockIdx.y * 64;
+  const int64_t img = blockIdx.z;
+  in += img * C * hw;
+  out += img * hw * Cp;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (vec) {  // planes of a multiple of 8 pixels: 16-byte loads
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int v = threadIdx.x + i * 256, c = v >> 3, p = (v & 7) * 8;
+      uint4 u = make_uint4(0u, 0u, 0u, 0u);
+      if (c0 + c < C && p0 + p < hw) u = __ldg(reinterpret_cast<const uint4*>(in + (int64_t)(c0 + c) * hw + p0 + p));
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        t[c * kTrPitch + p + 2 * e] = (unsigned short)w[e];
+        t[c * kTrPitch + p + 2 * e + 1] = (unsigned short)(w[e] >> 16);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int v = threadIdx.x + i * 256, c = v >> 6, p = v & 63;
+      t[c * kTrPitch + p] = (c0 + c < C && p0 + p < hw) ? __ldg(in + (int64_t)(c0 + c) * hw + p0 + p) : (unsigned short)0;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int v = threadIdx.x + i * 256, p = v >> 3, c = (v & 7) * 8;
+    if (p0 + p >= hw || c0 + c >= Cp) continue;
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = t[(c + 2 * e) * kTrPitch + p] | ((uint32_t)t[(c + 2 * e + 1) * kTrPitch + p] << 16);
+    *reinterpret_cast<uint4*>(out + (int64_t)(p0 + p) * Cp + c0 + c) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// ------------------------------------------------------------------------------------------ the multiply
+constexpr int kPix = 128;          // pixels per thread block: the rows of its accumulator
+constexpr int kK = 64;             // k per stage
+constexpr int kABytes = kPix * kK * 2;
+constexpr int kMaxStages = 8;
+constexpr int kEpiWarps = 8;       // two per quarter of the tensor-memory lanes
+constexpr int kThreads = 96 + 32 * kEpiWarps;  // warp 0: pixel copies, 1: tensor core, 2: weight copies, then the epilogue
+constexpr int kGatherGroups = 2;   // gathering variant: groups of four warps that build tiles of pixels in turn
+constexpr int kGatherThreads = kThreads + 128 * kGatherGroups;
+constexpr int kHdrBytes = 2048;
+
+struct ConvParams {
+  unsigned* status;
+  int nkt, nstages, npt, nnt;        // K tiles, ring slots, pixel tiles, channel tiles
+  int n_tile, n_stride;              // output channels per tile; tensor-memory columns between the two accumulators
+  int g, cblocks, nsub;              // channels per copy of input pixels, copies per tap, taps * cblocks
+  int M, KH, KW, stride, pad, OH, OW;
+  int C, H, W, K;
+  int ksplit, kt_per;                // > 1: a cluster of ksplit blocks shares a tile, each multiplies kt_per K tiles
+  int64_t npix;                      // images * OH * OW
+  unsigned spin_limit;
+  const __nv_bfloat16* X;            // gathering variant: the NCHW input
+  const float* bias;
+  void* Y;
+  int y_bf16, relu;
+};
+
+__device__ __forceinline__ uint64_t k_major_desc(uint32_t saddr, int row_bytes) {
+  // K-major tile with rows of 128, 64 or 32 bytes in the swizzle of that width: eight rows are row_bytes * 8 apart
+  const uint64_t layout = row_bytes == 128 ? 2ull : (row_bytes == 64 ? 4ull : 6ull);
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)((row_bytes * 8) >> 4) << 32) | (1ull << 46) | (layout << 61);
+}
+
+template <int CG>
+__device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accumulate) {
+  if (CG == 1)
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+                 ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate) : "memory");
+  else
+    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+                 ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate) : "memory");
+}
+template <int CG>
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  if (CG == 1)
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+  else  // in both blocks of the pair
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
+}
+// Tile loads whose bytes are counted on a barrier given as a shared::cluster address (the even block's; no multicast).
+template <int CG>
+__device__ __forceinline__ void load_im2col(uint32_t dst, const void* map, int c, int w, int h, int n, unsigned short ow, unsigned short oh, uint32_t bar) {
+  if (CG == 1)
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(ow), "h"(oh) : "memory");
+  else
+    asm volatile("cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(ow), "h"(oh) : "memory");
+}
+template <int CG>
+__device__ __forceinline__ void load_rows(uint32_t dst, const void* map, int x, int y, uint32_t bar) {
+  if (CG == 1)
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+  else
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void put(float* y, float t) { *y = t; }
+__device__ __forceinline__ void put(__nv_bfloat16* y, float t) { *y = __float2bfloat16_rn(t); }
+// n channels of one pixel, planes of ohw elements
+template <typename T>
+__device__ __forceinline__ void store_channels(T* y, int64_t ohw, int n, const float (&t)[32]) {
+  if (n == 32) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i) put(y + i * ohw, t[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (i < n) put(y + i * ohw, t[i]);
+  }
+}
+
+// CG = 2: two thread blocks on neighbouring SMs share a tile of 256 pixels (128 each) and n_tile channels; each stages
+// its own pixels and half of the weight rows, the even one issues the multiplies for both.  That halves the weight bytes
+// an SM reads per flop.  CG = 1: one block, 128 pixels - smaller tiles for small outputs.
+// A thread block (pair) walks tiles blockIdx, blockIdx + grid, ...; two accumulators, so that storing a tile overlaps
+// the multiplies of the next.
+template <int CG, bool GATHER>
+__global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc_kernel(const __grid_constant__ CUtensorMap tm_in,
+                                                                                       const __grid_constant__ CUtensorMap tm_w, const ConvParams p) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);   // (even block) the tiles of a stage have landed, both blocks' bytes
+  uint64_t* empty = full + kMaxStages;                  // the multiplies of a stage are done
+  uint64_t* acc_full = empty + kMaxStages;              // [2] an accumulator is complete
+  uint64_t* acc_empty = acc_full + 2;                   // [2] (even block) it has been read by all epilogue warps
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + 384);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + 388);
+  int2* s_taps = reinterpret_cast<int2*>(smem + 1024);  // gathering variant: [k] (offset in the input, tap bits)
+  uint8_t* stages = smem + kHdrBytes;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
+  const int b_rows = p.n_tile / CG;
+  const uint32_t stage_bytes = (uint32_t)kABytes + (((uint32_t)b_rows * (kK * 2) + 1023u) & ~1023u);
+  const bool split = CG == 1 && !GATHER && p.ksplit > 1;
+  const uint32_t part = split ? cluster_ctarank() : 0u;  // this block's share of K
+  const int kt0 = split ? (int)part * p.kt_per : 0;
+  const int ns = p.nstages, nkt = split ? min(p.kt_per, p.nkt - kt0) : p.nkt;
+  const int per = split ? p.ksplit : CG;                 // blocks per tile
+  const int units = p.npt * p.nnt, u0 = (int)blockIdx.x / per, ustep = (int)gridDim.x / per;
+  const uint32_t tmem_cols = 2u * (uint32_t)p.n_stride;
+
+  if (tid == 32) {
+    if (!GATHER) asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_in) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_w) : "memory");
+  }
+  if (tid == 0) {
+    for (int s = 0; s < kMaxStages; ++s) {
+      // both copying threads of the even block announce the bytes of their loads; gathering: weights + four warps
+      mbar_init(full + s, GATHER ? 5 : 2);
+      mbar_init(empty + s, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(acc_full + i, 1);
+      mbar_init(acc_empty + i, kEpiWarps * CG);
+    }
+    *s_abort = 0;
+    fence_mbar_init();
+  }
+  if (GATHER && tid >= kThreads && tid < kThreads + kK) {
+    // k -> (channel, kh, kw); tap bits: kh in the low half, 16 + kw in the high half (none valid past the last k)
+    const int k = tid - kThreads, khw = p.KH * p.KW;
+    const int c = k / khw, rest = k - c * khw, kh = rest / p.KW, kw = rest - kh * p.KW;
+    s_taps[k] = k < p.K ? make_int2((c * p.H + kh) * p.W + kw, (int)((1u << kh) | (1u << (16 + kw)))) : make_int2(0, -1);
+  }
+  if (warp == 1) {
+    if (CG == 1) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(tmem_cols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (CG == 2) cluster_sync_all();  // both blocks' barriers exist before either signals the other
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *s_tmem;
+  // the channel-last copy of the input (the launch before) is complete and visible from here on
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  bool failed = false;
+  int fail_site = 0;
+  if (warp == 2) {
+    // ------------------------------------------------------------------ weight copies
+    // (a thread of their own: a copy costs the thread that issues it about 100 ns, and small tiles are done in less)
+    if (elect_one()) {
+      uint32_t full0 = smem_u32(full);  // the even block's barriers, as seen from this block
+      if (CG == 2) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(full0) : "r"(smem_u32(full)), "r"(0));
+      const uint32_t st0 = smem_u32(stages) + kABytes, b_bytes = (uint32_t)b_rows * (kK * 2);
+      // ring position: slot, and how often the ring has been gone through (a slot is refilled from the second round on)
+      int slot = 0, round = 0;
+      for (int u = u0; u < units && !failed; u += ustep) {
+        const int row0 = (u % p.nnt) * p.n_tile + (int)rank * b_rows;
+        for (int kt = 0; kt < nkt; ++kt) {
+          if (round > 0 && !mbar_wait<CG == 2>(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 5; break; }
+          if (rank == 0) mbar_arrive_expect_tx(full + slot, b_bytes * CG);
+          load_rows<CG>(st0 + (uint32_t)slot * stage_bytes, &tm_w, (kt0 + kt) * kK, row0, full0 + (uint32_t)slot * 8u);
+          if (++slot == ns) { slot = 0; ++round; }
+        }
+      }
+    }
+  } else if (warp == 0) {
+    // ------------------------------------------------------------------ pixel copies
+    if (!GATHER && elect_one()) {
+      uint32_t full0 = smem_u32(full);
+      if (CG == 2) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(full0) : "r"(smem_u32(full)), "r"(0));
+      const int ohw = p.OH * p.OW;
+      const int subs = kK / p.g;
+      const uint32_t st0 = smem_u32(stages), sub_bytes = (uint32_t)(kPix * p.g * 2);
+      int slot = 0, round = 0;
+      for (int u = u0; u < units && !failed; u += ustep) {
+        const int pt = u / p.nnt;
+        const int64_t px = ((int64_t)pt * CG + rank) * kPix;  // first pixel of this block
+        const int img = (int)(px / ohw);
+        const int rest = (int)(px - (int64_t)img * ohw);
+        const int oh = rest / p.OW, ow = rest - oh * p.OW;
+        const int w0 = ow * p.stride - p.pad, h0 = oh * p.stride - p.pad;
+        const int sub0 = kt0 * subs, tap0 = sub0 / p.cblocks;
+        int tap_h = tap0 / p.KW, tap_w = tap0 - tap_h * p.KW, cb = sub0 - tap0 * p.cblocks, left = p.nsub - sub0;
+        for (int kt = 0; kt < nkt; ++kt) {
+          if (round > 0 && !mbar_wait<CG == 2>(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
+          const uint32_t st = st0 + (uint32_t)slot * stage_bytes, bar = full0 + (uint32_t)slot * 8u;
+          const int nsub = left < subs ? left : subs;  // copies of input pixels in this stage
+          if (rank == 0) mbar_arrive_expect_tx(full + slot, sub_bytes * (uint32_t)nsub * CG);
+          for (int i = 0; i < nsub; ++i) {
+            load_im2col<CG>(st + (uint32_t)i * sub_bytes, &tm_in, cb * p.g, w0, h0, img, (unsigned short)tap_w, (unsigned short)tap_h, bar);
+            if (++cb == p.cblocks) {
+              cb = 0;
+              if (++tap_w == p.KW) { tap_w = 0; ++tap_h; }
+            }
+          }
+          left -= nsub;
+          if (++slot == ns) { slot = 0; ++round; }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ tensor core
+    if (rank == 0 && elect_one()) {
+      // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 pixels per block, N = n_tile channels
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n_tile >> 3) << 17) | ((uint32_t)((kPix * CG) >> 4) << 24);
+      const int row_bytes = p.g * 2, sub_shift = p.g == 64 ? 2 : (p.g == 32 ? 1 : 0);  // 16-wide k steps per copy: 4, 2, 1
+      const uint64_t ad0 = k_major_desc(smem_u32(stages), row_bytes), bd0 = k_major_desc(smem_u32(stages) + kABytes, 128);
+      uint32_t step[kK / 16];  // where the k steps of a stage start in the tile of pixels, in 16-byte units
+#pragma unroll
+      for (int s = 0; s < kK / 16; ++s) {
+        const int sub = s >> sub_shift, in_sub = s - (sub << sub_shift);
+        step[s] = (uint32_t)(sub * (kPix * row_bytes) + in_sub * 32) >> 4;
+      }
+      int slot = 0, tile = 0;
+      unsigned round = 0;
+      for (int u = u0; u < units && !failed; u += ustep, ++tile) {
+        const int acc = tile & 1;
+        if (tile >= 2 && !mbar_wait<CG == 2>(acc_empty + acc, (unsigned)((tile / 2 - 1) & 1), p.spin_limit << 2, s_abort, 0)) { failed = true, fail_site = 2; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem_base + (uint32_t)acc * (uint32_t)p.n_stride;
+        int left = GATHER ? (p.K + 15) >> 4 : (p.nsub << sub_shift) - kt0 * (kK / 16);  // k steps that exist
+        for (int kt = 0; kt < nkt; ++kt) {
+          if (!mbar_wait<CG == 2>(full + slot, round & 1u, p.spin_limit << 2, s_abort, 0)) { failed = true, fail_site = 3; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t off = ((uint32_t)slot * stage_bytes) >> 4;  // (the address field of a descriptor never carries: 227 KB < 2^18)
+          if (left >= kK / 16) {
+#pragma unroll
+            for (int s = 0; s < kK / 16; ++s) mma_bf16<CG>(d, ad0 + off + step[s], bd0 + off + 2u * s, idesc, (kt > 0 || s > 0) ? 1u : 0u);
+          } else {
+#pragma unroll
+            for (int s = 0; s < kK / 16; ++s)
+              if (s < left) mma_bf16<CG>(d, ad0 + off + step[s], bd0 + off + 2u * s, idesc, (kt > 0 || s > 0) ? 1u : 0u);
+          }
+          left -= kK / 16;
+          mma_commit<CG>(empty + slot);
+          if (++slot == ns) { slot = 0; ++round; }
+        }
+        if (!failed) mma_commit<CG>(acc_full + acc);
+      }
+    }
+  } else if (GATHER && warp >= 3 + kEpiWarps) {
+    // ------------------------------------------------------------------ gathering variant: a thread builds one pixel's row
+    const int grp = (warp - 3 - kEpiWarps) >> 2, bt = (tid - kThreads) & 127;
+    const int pieces = 2 * ((p.K + 15) >> 4);  // 16-byte pieces of a row that the multiplies read
+    const unsigned short* X = reinterpret_cast<const unsigned short*>(p.X);
+    const int64_t ohw = (int64_t)p.OH * p.OW;
+    int it = grp;
+    for (int u = u0 + grp * ustep; u < units; u += kGatherGroups * ustep, it += kGatherGroups) {
+      const int slot = it % ns;
+      if (it >= ns && !__all_sync(0xffffffffu, mbar_wait(empty + slot, (unsigned)((it / ns - 1) & 1), p.spin_limit, s_abort, 32))) { failed = true, fail_site = 6; break; }
+      const int64_t q = (int64_t)(u / p.nnt) * kPix + bt;
+      const bool ok = q < p.npix;
+      const int64_t img = ok ? q / ohw : 0;
+      const int pix = ok ? (int)(q - img * ohw) : 0;
+      const int oh = pix / p.OW, ow = pix - oh * p.OW;
+      const int h0 = oh * p.stride - p.pad, w0 = ow * p.stride - p.pad;
+      uint32_t in = 0;  // bit kh: row inside; bit 16 + kw: column inside
+      if (ok) {
+        for (int t = 0; t < p.KH; ++t) in |= (uint32_t)(h0 + t >= 0 && h0 + t < p.H) << t;
+        for (int t = 0; t < p.KW; ++t) in |= (uint32_t)(w0 + t >= 0 && w0 + t < p.W) << (16 + t);
+      }
+      const unsigned short* src = X + (img * p.C * p.H + h0) * p.W + w0;  // only dereferenced where a tap is inside
+      const uint32_t row = smem_u32(stages) + (uint32_t)slot * stage_bytes + (uint32_t)bt * 128u;
+      for (int pc = 0; pc < pieces; ++pc) {
+        uint32_t v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int2 t = s_taps[pc * 8 + e];
+          v[e] = 0u;
+          if ((in & (uint32_t)t.y) == (uint32_t)t.y) v[e] = __ldg(src + t.x);
+        }
+        sts128(row + (((uint32_t)pc ^ ((uint32_t)bt & 7u)) << 4), v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
+      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + slot);
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue: a lane holds one pixel
+    const int quarter = warp & 3;  // the tensor-memory lanes this warp may read
+    const int64_t ohw = (int64_t)p.OH * p.OW;
+    // the accumulator has been read by this warp: the multiplies of a later tile may overwrite it once all warps say so
+    auto release = [&](int acc) {
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        if (CG == 1 || rank == 0) mbar_arrive(acc_empty + acc);
+        else mbar_arrive_remote(acc_empty + acc, 0);
+      }
+    };
+    int tile = 0;
+    for (int u = u0; u < units; u += ustep, ++tile) {
+      const int acc = tile & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(acc_full + acc, (unsigned)((tile / 2) & 1), p.spin_limit << 2, s_abort, 64))) { failed = true, fail_site = 4; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (split) break;  // one tile per cluster; the shares meet below
+      const int pt = u / p.nnt, nt = u - pt * p.nnt;
+      const int64_t px = ((int64_t)pt * CG + rank) * kPix + quarter * 32 + lane;
+      const bool ok = px < p.npix;
+      const int64_t img = ok ? px / ohw : 0;
+      const int ch0 = nt * p.n_tile;
+      const int64_t base = (img * p.M + ch0) * ohw + (ok ? px - img * ohw : 0);
+      const int nch = p.M - ch0 < p.n_tile ? p.M - ch0 : p.n_tile;
+      // Two neighbouring pixels per store where planes have an even size (then pixels 2i and 2i + 1 share an image): lanes
+      // exchange halves so that even lanes hold both pixels of one channel and odd lanes of the next.
+      const bool pairs = p.y_bf16 && (ohw & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 3) == 0;
+      const int cb0 = ((warp - 3) >> 2) * 32;  // the two warps of a quarter take 32 channels in turn
+      for (int cb = cb0; cb < nch; cb += 64) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * p.n_stride + cb), v);
+        if (cb + 64 >= nch) release(acc);
+        const int n = nch - cb < 32 ? nch - cb : 32;
+        // lane i fetches the bias of channel i of this piece
+        const float bl = (p.bias && lane < n) ? __ldg(p.bias + ch0 + cb + lane) : 0.f;
+        float t[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          t[i] = __uint_as_float(v[i]) + __shfl_sync(0xffffffffu, bl, i);
+          if (p.relu) t[i] = fmaxf(t[i], 0.f);
+        }
+        if (pairs) {
+          uint32_t w[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float other = __shfl_xor_sync(0xffffffffu, (lane & 1) ? t[2 * i] : t[2 * i + 1], 1);
+            const __nv_bfloat162 h = (lane & 1) ? __floats2bfloat162_rn(other, t[2 * i + 1]) : __floats2bfloat162_rn(t[2 * i], other);
+            w[i] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+          if (ok) {
+            __nv_bfloat16* y = static_cast<__nv_bfloat16*>(p.Y) + base - (lane & 1) + (cb + (lane & 1)) * ohw;
+            if (n == 32) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) *reinterpret_cast<uint32_t*>(y + 2 * i * ohw) = w[i];
+            } else {
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                if (2 * i + (lane & 1) < n) *reinterpret_cast<uint32_t*>(y + 2 * i * ohw) = w[i];
+            }
+          }
+        } else if (ok) {
+          if (p.y_bf16) store_channels(static_cast<__nv_bfloat16*>(p.Y) + base + cb * ohw, ohw, n, t);
+          else store_channels(static_cast<float*>(p.Y) + base + cb * ohw, ohw, n, t);
+        }
+      }
+      if (cb0 >= nch) release(acc);  // nothing of this tile for this warp
+    }
+  }
+
+  if (__any_sync(0xffffffffu, failed)) {
+    *s_abort = 1;
+    if (fail_site) atomicOr(p.status, (unsigned)GRIM_ERR_TIMEOUT | (1u << (8 + fail_site)));
+  }
+  if (split) {
+    // Every block owns n_tile / ksplit of the tile's channels: each sends its sums to their owners' shared memory (the
+    // stages are free once all blocks have multiplied) and the owner adds them up.  [block][channel][pixel] floats.
+    __syncwarp();
+    cluster_sync_all();
+    const int nc = p.n_tile / p.ksplit;
+    const bool epi = warp >= 3;
+    if (epi) {
+      const int quarter = warp & 3;
+      const uint32_t dst = smem_u32(stages) + ((uint32_t)part * (uint32_t)nc * kPix + (uint32_t)(quarter * 32 + lane)) * 4u;
+      for (int cb = ((warp - 3) >> 2) * 32; cb < p.n_tile; cb += 64) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)cb, v);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const int owner = (cb + i) / nc, c = cb + i - owner * nc;
+          uint32_t at;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(dst + (uint32_t)c * (kPix * 4)), "r"(owner));
+          asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v[i]) : "memory");
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    if (epi) {
+      const float* sums = reinterpret_cast<const float*>(stages);
+      const int pt = u0 / p.nnt, nt = u0 - pt * p.nnt;
+      const int t = tid - 96, pl = t & (kPix - 1);
+      const int64_t px = (int64_t)pt * kPix + pl, ohw = (int64_t)p.OH * p.OW;
+      if (px < p.npix) {
+        const int64_t img = px / ohw, pix = px - img * ohw;
+        for (int c = t / kPix; c < nc; c += 32 * kEpiWarps / kPix) {
+          const int ch = nt * p.n_tile + (int)part * nc + c;
+          if (ch >= p.M) break;
+          float sum = 0.f;
+          for (int s = 0; s < p.ksplit; ++s) sum += sums[(s * nc + c) * kPix + pl];
+          if (p.bias) sum += __ldg(p.bias + ch);
+          if (p.relu) sum = fmaxf(sum, 0.f);
+          const int64_t off = (img * p.M + ch) * ohw + pix;
+          if (p.y_bf16) put(static_cast<__nv_bfloat16*>(p.Y) + off, sum);
+          else put(static_cast<float*>(p.Y) + off, sum);
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (*s_abort && tid == 0) {  // copies that were requested still land in this block's shared memory
+    for (int s = 0; s < ns; ++s)
+      for (unsigned i = 0; i < 4096u && !mbar_try_wait(full + s, 0) && !mbar_try_wait(full + s, 1); ++i) {}
+  }
+  if (CG == 2) cluster_sync_all();  // neither block leaves (or frees tensor memory) while the other may still use its memory
+  if (warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (CG == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------------------------------ host side
+// The driver's tensor-map encoders, looked up through the runtime so that the library does not link against the driver.
+template <typename F>
+F driver_entry(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  return reinterpret_cast<F>(p);
+}
+using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+using EncodeIm2colFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const int*,
+                                    const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn encode_tiled_fn() {
+  static const EncodeTiledFn fn = driver_entry<EncodeTiledFn>("cuTensorMapEncodeTiled");
+  return fn;
+}
+EncodeIm2colFn encode_im2col_fn() {
+  static const EncodeIm2colFn fn = driver_entry<EncodeIm2colFn>("cuTensorMapEncodeIm2col");
+  return fn;
+}
+
+bool gathers(const grim_bcr* h) { return h->conv[kConvGather].d_w != nullptr; }
+const ConvLayout* layout_for(const grim_bcr* h, const SpmmArgs& a) {
+  if (gathers(h)) return a.KH <= 16 && a.KW <= 16 ? &h->conv[kConvGather] : nullptr;
+  for (const ConvLayout& l : h->conv)
+    if (l.d_w && l.taps == a.KH * a.KW && (int64_t)a.C * l.taps == h->K) return &l;
+  return nullptr;
+}
+int64_t images_of(const SpmmArgs& a) { return a.ncols / ((int64_t)a.OH * a.OW); }
+int padded_channels(int C) { return (C + 7) / 8 * 8; }
+size_t nhwc_bytes(const SpmmArgs& a) { return (size_t)images_of(a) * a.H * a.W * padded_channels(a.C) * 2; }
+
+struct ConvPlan {
+  int cg, n_tile, nnt, npt, ksplit, kt_per, grid;
+};
+bool shape_plan(ConvPlan& pl, int nkt, int64_t npix, int64_t M, int sms) {
+  pl.nnt = (int)((M + pl.n_tile - 1) / pl.n_tile);
+  const int64_t npt = (npix + kPix * pl.cg - 1) / (kPix * pl.cg);
+  if (npt * pl.nnt > (int64_t(1) << 30)) return false;
+  pl.npt = (int)npt;
+  pl.kt_per = (nkt + pl.ksplit - 1) / pl.ksplit;
+  if (pl.ksplit > 1) {
+    // one tile per cluster, every block with something to multiply; the sums have to fit the stages
+    if (pl.cg != 1 || (pl.ksplit - 1) * pl.kt_per >= nkt || pl.n_tile % 32 || pl.n_tile % pl.ksplit) return false;
+    pl.grid = pl.npt * pl.nnt * pl.ksplit;
+    return pl.n_tile * kPix * 4 <= 128 * 1024;
+  }
+  pl.grid = (int)std::min<int64_t>(npt * pl.nnt, sms / pl.cg) * pl.cg;
+  return true;
+}
+// Tile shape: the candidate with the lowest estimated time, in ns.  A K tile costs the slowest of: the thread that issues a
+// copy (140), its bytes at the rate at which L2 feeds an SM's shared memory (120 per ns; 17 - 21 TB/s were measured over the
+// GPU), the multiplies (shared-memory reads of both operands at 128 bytes a cycle included).  A tile's store overlaps the next
+// tile's multiplies, the last one's does not; tiles are counted in whole waves.  The split over K trades a shorter loop for an
+// exchange of about 2 us and is only considered where one wave holds all parts.
+ConvPlan plan_for(int nkt, int64_t npix, int64_t M, int sms, bool gather) {
+  ConvPlan best{};
+  double best_t = -1.0;
+  for (int cg = gather ? 1 : 2; cg >= 1; --cg)
+    for (int n = 256; n >= 16 * cg; n -= 16 * cg)
+      for (int ks = 1; ks <= 8; ks *= 2) {
+        if (n > ((M + 31) / 32) * 32 || (ks > 1 && gather)) continue;
+        ConvPlan pl{cg, n, 0, 0, ks, 0, 0};
+        if (!shape_plan(pl, nkt, npix, M, sms)) continue;
+        const int64_t units = (int64_t)pl.npt * pl.nnt;
+        if (ks > 1 && units * ks > (ks == 8 ? 112 : sms - 8)) continue;
+        const double mma = cg == 1 ? 128.0 + n : std::max(128.0 + n / 2, 1.0 * n);  // cycles
+        const double kt = std::max(std::max(140.0, (kABytes + (double)n / cg * kK * 2) / 120.0), mma / 1.8);
+        const double epi = 250.0 + 6.0 * n;
+        const double waves = ks > 1 ? 1.0 : (double)((units + sms / cg - 1) / (sms / cg));
+        const double t = waves * std::max(pl.kt_per * kt, epi) + epi + (ks > 1 ? 2000.0 : 0.0) + (cg == 2 ? 1000.0 : 0.0);
+        if (best_t < 0.0 || t < best_t) { best_t = t; best = pl; }
+      }
+  return best;
+}
+
+}  // namespace
+
+// Channels per copy of input pixels for a convolution with `taps` kernel positions: as few K tiles as possible.
+ConvLayout conv_layout_shape(int64_t K, int taps) {
+  ConvLayout best;
+  const int64_t C = K / taps;
+  for (int g = 64; g >= 16; g /= 2) {
+    const int64_t cblocks = (C + g - 1) / g, nkt = (taps * cblocks * g + kK - 1) / kK;
+    if (best.taps == 0 || nkt < best.nkt) {
+      best.taps = taps; best.g = g; best.cblocks = (int)cblocks; best.nkt = (int)nkt;
+    }
+  }
+  return best;
+}
+
+size_t conv_scratch_bytes(const grim_bcr* h, int64_t max_ncols) {
+  size_t need = 0;
+  for (int i = 0; i < kConvGather && !gathers(h); ++i) {
+    const ConvLayout& l = h->conv[i];
+    if (!l.d_w) continue;
+    const size_t same = (size_t)max_ncols * padded_channels((int)(h->K / l.taps)) * 2;  // stride 1: as many input pixels as outputs
+    need = std::max(need, std::max(same, std::min(4 * same, (size_t)512 << 20)));       // stride 2: four times as many
+  }
+  return need;
+}
+
+bool conv_tc_supported(const grim_bcr* h, const SpmmArgs& a) {
+  if (h->device < 0 || !h->d_status || !a.conv || a.x_dtype != GRIM_BF16 || !layout_for(h, a)) return false;
+  if (a.ncols > (int64_t(1) << 31) - 512 || (int64_t)a.C * a.H * a.W >= (int64_t(1) << 31) || !encode_tiled_fn()) return false;
+  if (gathers(h)) return true;
+  if (a.KH != a.KW || a.stride > 8 || a.pad > 127 || a.H > 65535 || a.W > 65535 || images_of(a) > 65535 || (a.C + 63) / 64 > 65535) return false;
+  return h->d_tc_acc && h->tc_acc_bytes >= nhwc_bytes(a) && encode_im2col_fn();
+}
+
+grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
+  if (!conv_tc_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
+  const ConvLayout& l = *layout_for(h, a);
+  const bool gather = gathers(h);
+  const int Cp = padded_channels(a.C), hw = a.H * a.W;
+  const int64_t images = images_of(a);
+  const ConvPlan pl = plan_for(l.nkt, a.ncols, h->M, sm_count(h->device), gather);
+  if (pl.grid <= 0) return GRIM_ERR_UNSUPPORTED;
+
+  ConvParams p;
+  p.status = h->d_status;
+  p.nkt = l.nkt; p.npt = pl.npt; p.nnt = pl.nnt; p.n_tile = pl.n_tile; p.ksplit = pl.ksplit; p.kt_per = pl.kt_per;
+  p.n_stride = pl.n_tile <= 32 ? 32 : (pl.n_tile <= 64 ? 64 : (pl.n_tile <= 128 ? 128 : 256));
+  p.g = l.g; p.cblocks = l.cblocks; p.nsub = l.taps * l.cblocks;
+  p.M = (int)h->M; p.KH = a.KH; p.KW = a.KW; p.stride = a.stride; p.pad = a.pad; p.OH = a.OH; p.OW = a.OW;
+  p.C = a.C; p.H = a.H; p.W = a.W; p.K = (int)h->K;
+  p.npix = a.ncols; p.spin_limit = 1u << 20; p.X = static_cast<const __nv_bfloat16*>(a.X); p.bias = a.bias; p.Y = a.Y;
+  p.y_bf16 = a.y_dtype == GRIM_BF16; p.relu = a.relu;
+  const int b_rows = pl.n_tile / pl.cg;
+  const size_t stage = kABytes + (((size_t)b_rows * kK * 2 + 1023) & ~size_t(1023));
+  p.nstages = (int)std::min<size_t>(kMaxStages, (227 * 1024 - 1024 - kHdrBytes) / stage);
+  const size_t smem = 1024 + kHdrBytes + p.nstages * stage;
+
+  CUtensorMap tin, tw;
+  memset(&tin, 0, sizeof(tin));
+  memset(&tw, 0, sizeof(tw));
+  if (!gather) {
+    const cuuint64_t dims[4] = {(cuuint64_t)a.C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)images};
+    const cuuint64_t strides[3] = {(cuuint64_t)Cp * 2, (cuuint64_t)Cp * 2 * a.W, (cuuint64_t)Cp * 2 * hw};
+    const int lower[2] = {-a.pad, -a.pad}, upper[2] = {a.pad - (a.KW - 1), a.pad - (a.KH - 1)};
+    const cuuint32_t estr[4] = {1, (cuuint32_t)a.stride, (cuuint32_t)a.stride, 1};
+    const CUtensorMapSwizzle sw = l.g == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (l.g == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    if (encode_im2col_fn()(&tin, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, h->d_tc_acc, dims, strides, lower, upper, (cuuint32_t)l.g, kPix, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return GRIM_ERR_CUDA;
+  }
+  const cuuint64_t wdims[2] = {(cuuint64_t)l.nkt * kK, (cuuint64_t)h->M};
+  const cuuint64_t wstrides[1] = {(cuuint64_t)l.nkt * kK * 2};
+  const cuuint32_t wbox[2] = {(cuuint32_t)kK, (cuuint32_t)b_rows}, westr[2] = {1, 1};
+  if (encode_tiled_fn()(&tw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, l.d_w, wdims, wstrides, wbox, westr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return GRIM_ERR_CUDA;
+  cudaError_t e = cudaSuccess;
+  if (!gather) {
+    e = launch_pdl(conv_nhwc_kernel, dim3((unsigned)((hw + 63) / 64), (unsigned)((Cp + 63) / 64), (unsigned)images), dim3(256), 0, s,
+                   static_cast<const unsigned short*>(a.X), reinterpret_cast<unsigned short*>(h->d_tc_acc), a.C, Cp, hw,
+                   (hw % 8 == 0 && reinterpret_cast<uintptr_t>(a.X) % 16 == 0) ? 1 : 0);
+    count_launch();
+    if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+  }
+  auto kern = gather ? conv_tc_kernel<1, true> : (pl.cg == 2 ? conv_tc_kernel<2, false> : conv_tc_kernel<1, false>);
+  if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem) != cudaSuccess) return GRIM_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)pl.grid);
+  cfg.blockDim = dim3(gather ? kGatherThreads : kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)std::max(pl.cg, pl.ksplit);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pl.cg == 2 || pl.ksplit > 1 ? 2 : 1;
+  e = cudaLaunchKernelEx(&cfg, kern, tin, tw, p);
+  count_launch();
+  if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+  return GRIM_OK;
+}
+
+}  // namespace grim

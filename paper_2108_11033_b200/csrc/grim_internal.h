@@ -105,6 +105,22 @@ inline uint32_t td_offset(uint32_t row, uint32_t col) {
   return row * 128u + ((((col >> 3) ^ (row & 7u))) << 4) + (col & 7u) * 2u;
 }
 
+// ---------------------------------------------------------------------------------------------
+// Weights of the tensor-core convolution (bf16 handles whose K is a multiple of the kernel positions of a 3 x 3 or 5 x 5
+// convolution): expanded, rows in natural order, columns by (kernel position, input channel) instead of (input channel,
+// kernel position): g channels at a time, so that one copy of g channels of a tile of shifted input pixels meets them.
+//   column (tap * cblocks + c / g) * g + c % g, for input channel c
+// A K of at most 64 (any kernel size) is one tile and keeps its own column order.
+// ---------------------------------------------------------------------------------------------
+struct ConvLayout {
+  int taps = 0;            // kernel positions; 0: no such layout
+  int g = 0, cblocks = 0;  // channels per copy (64, 32 or 16), copies per kernel position
+  int nkt = 0;             // K tiles of 64; a row has nkt * 64 columns
+  uint16_t* d_w = nullptr;
+};
+constexpr int kConvGather = 2;   // index of the K <= 64 layout
+constexpr int kConvLayouts = 3;  // 3 x 3, 5 x 5, K <= 64
+
 struct HostBlock {
   uint64_t colmask = 0;
   uint32_t rowmask = 0;
@@ -142,6 +158,7 @@ struct grim_bcr {
   int64_t index_bytes_rc = 0;
   // device
   int device = -1;
+  void* d_arena = nullptr;  // the one allocation that holds every array below except the scratch
   grim::RcStage* d_rc_stage = nullptr;
   grim::RcHead* d_rc_head = nullptr;
   int64_t rc_chunks = 0;  // chunks of eight kept columns, summed over all blocks
@@ -152,7 +169,10 @@ struct grim_bcr {
   uint32_t td_max_rec = 0;
   grim::RcStage* d_td_stage = nullptr;
   uint8_t* d_td_blob = nullptr;
-  float* d_tc_acc = nullptr;  // fp32 scratch of the split tensor-core multiply (M x N); grim_bcr_reserve allocates it
+  grim::ConvLayout conv[grim::kConvLayouts];
+  // scratch that grim_bcr_reserve allocates: partial sums of the split tensor-core multiply (M x N fp32), or the
+  // channel-last copy of a convolution's input
+  float* d_tc_acc = nullptr;
   size_t tc_acc_bytes = 0;
   // answers of grim_bcr_tune, one per (log2 bucket of N, X dtype, Y dtype); path 0 = not tuned
   grim_tune_t tuned[32][2][2] = {};
@@ -222,6 +242,11 @@ bool tc_path_supported(const grim_bcr* h, const SpmmArgs& a);
 // the paired (two thread blocks per tile pair) tensor-core kernel: matrices, bf16 handles
 grim_status_t launch_spmm_tc2(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool tc2_path_supported(const grim_bcr* h, const SpmmArgs& a);
+// tensor-core convolution from a channel-last copy of the input (needs grim_bcr_reserve unless K <= 64)
+grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
+bool conv_tc_supported(const grim_bcr* h, const SpmmArgs& a);
+ConvLayout conv_layout_shape(int64_t K, int taps);
+size_t conv_scratch_bytes(const grim_bcr* h, int64_t max_ncols);
 void count_launch(int n = 1);
 // streaming multiprocessors of a device (read once per device through the runtime)
 int sm_count(int device);

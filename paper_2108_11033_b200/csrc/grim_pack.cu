@@ -29,39 +29,40 @@ inline uint16_t bf16_bits(float f) {
   return (uint16_t)(u >> 16);
 }
 
-template <typename T>
-cudaError_t upload(T** dst, const void* src, size_t bytes) {
-  *dst = nullptr;
-  size_t alloc = bytes ? bytes : 16;
-  cudaError_t e = cudaMalloc((void**)dst, alloc);
-  if (e != cudaSuccess) return e;
-  if (bytes) e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-  return e;
-}
+// Everything a handle keeps on the device lives in one allocation (an allocation per array cost more than packing a small
+// matrix): arrays are registered with their host source, then placed and copied together.
+class Arena {
+ public:
+  template <typename T>
+  void add(T** dst, const void* src, size_t bytes) {
+    items_.push_back({reinterpret_cast<void**>(dst), src, bytes, total_});
+    total_ += (std::max<size_t>(bytes, 16) + 255) / 256 * 256;
+  }
+  cudaError_t upload(void** base) {
+    cudaError_t e = cudaMalloc(base, total_);
+    if (e != cudaSuccess) { *base = nullptr; return e; }
+    uint8_t* d = static_cast<uint8_t*>(*base);
+    for (const Item& it : items_) *it.dst = d + it.off;
+    if (total_ <= ((size_t)4 << 20)) {  // small: one copy
+      std::vector<uint8_t> all(total_, 0);
+      for (const Item& it : items_)
+        if (it.bytes) std::memcpy(&all[it.off], it.src, it.bytes);
+      return cudaMemcpy(d, all.data(), total_, cudaMemcpyHostToDevice);
+    }
+    for (const Item& it : items_)
+      if (it.bytes && (e = cudaMemcpy(d + it.off, it.src, it.bytes, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    return cudaSuccess;
+  }
+
+ private:
+  struct Item { void** dst; const void* src; size_t bytes, off; };
+  std::vector<Item> items_;
+  size_t total_ = 0;
+};
 
 void free_device(grim_bcr* h) {
-  cudaFree(h->d_stage);
-  cudaFree(h->d_blob);
-  cudaFree(h->d_band_order);
-  cudaFree(h->d_gemv_band_ptr);
-  cudaFree(h->d_chunks);
-  cudaFree(h->d_colwords);
-  cudaFree(h->d_gemv_vals);
+  cudaFree(h->d_arena);
   cudaFree(h->d_tc_acc);
-  cudaFree(h->d_run_ptr);
-  cudaFree(h->d_runs);
-  cudaFree(h->d_rc_stage);
-  cudaFree(h->d_rc_head);
-  cudaFree(h->d_rc_blob);
-  cudaFree(h->d_sl_colwords);
-  cudaFree(h->d_sl_vals);
-  cudaFree(h->d_sl_run_ptr);
-  cudaFree(h->d_sl_runs);
-  cudaFree(h->d_sl_band_of);
-  cudaFree(h->d_sl_slice_of);
-  cudaFree(h->d_td_stage);
-  cudaFree(h->d_td_blob);
-  cudaFree(h->d_status);
 }
 
 int bands_per_group(int bh) { return bh <= 4 ? 32 : (bh <= 8 ? 16 : 8); }
@@ -490,39 +491,76 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
       h->index_bytes_tc = (int64_t)td_stage.size() * (int64_t)sizeof(RcStage) + (int64_t)td_blob.size() - (int64_t)nnz * 2 + nbr * 4;
     }
 
+    // ---- expanded weights of the tensor-core convolution (grim_internal.h), for matrices of a convolution layer's size
+    std::vector<uint16_t> conv_w[kConvLayouts];
+    if (vdt == GRIM_BF16 && !(flags & (GRIM_PACK_NARROW_ONLY | GRIM_PACK_HOST_ONLY))) {
+      const int taps[kConvLayouts] = {9, 25, 1};
+      for (int t = 0; t < kConvLayouts; ++t) {
+        const bool gather = t == kConvGather;
+        if (gather ? K > 64 : (K <= 64 || K % taps[t] != 0)) continue;
+        ConvLayout l = conv_layout_shape(K, taps[t]);
+        if (gather) l.g = 64, l.cblocks = 1, l.nkt = 1;
+        const size_t ld = (size_t)l.nkt * 64;
+        if ((size_t)M * ld * 2 > ((size_t)64 << 20)) continue;
+        std::vector<uint32_t> col((size_t)K);
+        for (int64_t k = 0; k < K; ++k) {
+          const int64_t c = k / taps[t], tap = k % taps[t];
+          col[(size_t)k] = gather ? (uint32_t)k : (uint32_t)((tap * l.cblocks + c / l.g) * l.g + c % l.g);
+        }
+        conv_w[t].assign((size_t)M * ld, 0);
+        for (int64_t i = 0; i < nbr; ++i)
+          for (int64_t j = 0; j < nbc; ++j) {
+            const HostBlock& hb = h->blocks[(size_t)(i * nbc + j)];
+            if (!(hb.kr && hb.kc)) continue;
+            size_t v = (size_t)hb.val_off;
+            for (uint32_t rm = hb.rowmask; rm; rm &= rm - 1) {
+              uint16_t* row = &conv_w[t][(size_t)(i * bh + __builtin_ctz(rm)) * ld];
+              for (uint64_t cm = hb.colmask; cm; cm &= cm - 1) row[col[(size_t)(j * bw + __builtin_ctzll(cm))]] = bf16_bits(h->vals[v++]);
+            }
+          }
+        h->conv[t] = l;
+      }
+    }
+
     // ---- upload
     if (!(flags & GRIM_PACK_HOST_ONLY)) {
       cudaError_t e = cudaGetDevice(&h->device);
       // a handle packed for one regime keeps only that regime's layouts in device memory
       const bool wide = !(flags & GRIM_PACK_NARROW_ONLY), narrow = !(flags & GRIM_PACK_WIDE_ONLY);
-      if (e == cudaSuccess && wide) e = upload(&h->d_stage, stage.data(), stage.size() * sizeof(StageEntry));
-      if (e == cudaSuccess && wide) e = upload(&h->d_blob, blob.data(), blob.size());
-      if (e == cudaSuccess) e = upload(&h->d_band_order, h->band_order.data(), h->band_order.size() * 4);
-      if (e == cudaSuccess && wide) e = upload(&h->d_rc_stage, rc_stage.data(), rc_stage.size() * sizeof(RcStage));
-      if (e == cudaSuccess && wide) e = upload(&h->d_rc_head, rc_head.data(), rc_head.size() * sizeof(RcHead));
-      if (e == cudaSuccess && wide) e = upload(&h->d_rc_blob, rc_blob.data(), rc_blob.size());
-      if (e == cudaSuccess && tc_shape && wide) {
-        e = upload(&h->d_td_stage, td_stage.data(), td_stage.size() * sizeof(RcStage));
-        if (e == cudaSuccess) e = upload(&h->d_td_blob, td_blob.data(), td_blob.size());
-      }
+      Arena ar;
       const unsigned zero = 0;
-      if (e == cudaSuccess) e = upload(&h->d_status, &zero, 4);
-      if (e == cudaSuccess && h->gemv_ok && narrow) {
-        e = upload(&h->d_gemv_band_ptr, nar.band_ptr.data(), nar.band_ptr.size() * 4);
-        if (e == cudaSuccess) e = upload(&h->d_chunks, nar.chunks.data(), nar.chunks.size() * sizeof(ChunkDesc));
-        if (e == cudaSuccess) e = upload(&h->d_colwords, nar.colwords.data(), nar.colwords.size() * 4);
-        if (e == cudaSuccess) e = upload((uint8_t**)&h->d_gemv_vals, nar.gvals.data(), nar.gvals.size());
-        if (e == cudaSuccess) e = upload(&h->d_run_ptr, nar.run_ptr.data(), nar.run_ptr.size() * 4);
-        if (e == cudaSuccess) e = upload(&h->d_runs, nar.runs.data(), nar.runs.size() * sizeof(RunDesc));
-        if (e == cudaSuccess && !sl.runs.empty()) {
-          e = upload(&h->d_sl_colwords, sl.colwords.data(), sl.colwords.size() * 4);
-          if (e == cudaSuccess) e = upload((uint8_t**)&h->d_sl_vals, sl.gvals.data(), sl.gvals.size());
-          if (e == cudaSuccess) e = upload(&h->d_sl_run_ptr, sl.run_ptr.data(), sl.run_ptr.size() * 4);
-          if (e == cudaSuccess) e = upload(&h->d_sl_runs, sl.runs.data(), sl.runs.size() * sizeof(RunDesc));
-          if (e == cudaSuccess) e = upload(&h->d_sl_band_of, sl_band_of.data(), sl_band_of.size() * 4);
-          if (e == cudaSuccess) e = upload(&h->d_sl_slice_of, sl_slice_of.data(), sl_slice_of.size() * 4);
+      ar.add(&h->d_status, &zero, 4);
+      ar.add(&h->d_band_order, h->band_order.data(), h->band_order.size() * 4);
+      if (wide) {
+        ar.add(&h->d_stage, stage.data(), stage.size() * sizeof(StageEntry));
+        ar.add(&h->d_blob, blob.data(), blob.size());
+        ar.add(&h->d_rc_stage, rc_stage.data(), rc_stage.size() * sizeof(RcStage));
+        ar.add(&h->d_rc_head, rc_head.data(), rc_head.size() * sizeof(RcHead));
+        ar.add(&h->d_rc_blob, rc_blob.data(), rc_blob.size());
+      }
+      if (tc_shape && wide) {
+        ar.add(&h->d_td_stage, td_stage.data(), td_stage.size() * sizeof(RcStage));
+        ar.add(&h->d_td_blob, td_blob.data(), td_blob.size());
+      }
+      for (int t = 0; t < kConvLayouts; ++t)
+        if (h->conv[t].taps) ar.add(&h->conv[t].d_w, conv_w[t].data(), conv_w[t].size() * 2);
+      if (h->gemv_ok && narrow) {
+        ar.add(&h->d_gemv_band_ptr, nar.band_ptr.data(), nar.band_ptr.size() * 4);
+        ar.add(&h->d_chunks, nar.chunks.data(), nar.chunks.size() * sizeof(ChunkDesc));
+        ar.add(&h->d_colwords, nar.colwords.data(), nar.colwords.size() * 4);
+        ar.add(&h->d_gemv_vals, nar.gvals.data(), nar.gvals.size());
+        ar.add(&h->d_run_ptr, nar.run_ptr.data(), nar.run_ptr.size() * 4);
+        ar.add(&h->d_runs, nar.runs.data(), nar.runs.size() * sizeof(RunDesc));
+        if (!sl.runs.empty()) {
+          ar.add(&h->d_sl_colwords, sl.colwords.data(), sl.colwords.size() * 4);
+          ar.add(&h->d_sl_vals, sl.gvals.data(), sl.gvals.size());
+          ar.add(&h->d_sl_run_ptr, sl.run_ptr.data(), sl.run_ptr.size() * 4);
+          ar.add(&h->d_sl_runs, sl.runs.data(), sl.runs.size() * sizeof(RunDesc));
+          ar.add(&h->d_sl_band_of, sl_band_of.data(), sl_band_of.size() * 4);
+          ar.add(&h->d_sl_slice_of, sl_slice_of.data(), sl_slice_of.size() * 4);
         }
       }
+      if (e == cudaSuccess) e = ar.upload(&h->d_arena);
       if (e != cudaSuccess) {
         st = (e == cudaErrorMemoryAllocation) ? GRIM_ERR_ALLOC : GRIM_ERR_CUDA;
         cudaGetLastError();

@@ -221,6 +221,34 @@ def test_direct_kernel_convolution(B, geom, bf16):
     check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=bf16, kernel_flags=B.GRIM_CONV_DIRECT)
 
 
+@pytest.mark.parametrize("out_bf16", [False, True])
+@pytest.mark.parametrize("geom", [
+    (1, 64, 64, 16, 16, 3, 1, 1), (2, 30, 72, 9, 13, 3, 1, 1), (2, 17, 48, 12, 10, 5, 2, 2), (1, 130, 300, 15, 17, 3, 2, 1),
+    (3, 96, 136, 14, 14, 3, 1, 0), (1, 512, 256, 7, 7, 3, 1, 1), (40, 40, 264, 30, 31, 3, 1, 1), (24, 64, 512, 28, 28, 3, 1, 1),
+    (2, 3, 40, 20, 24, 3, 1, 1), (3, 2, 70, 19, 23, 5, 2, 2), (1, 64, 24, 9, 9, 1, 2, 0), (1, 1, 16, 21, 13, 8, 3, 4)])
+def test_tensor_core_convolution(B, geom, out_bf16):
+    """Channel-last kernel: 16, 32 and 64 channels per copy, ragged channels, pixels and planes of odd size, several tiles per
+    thread block, pairs of blocks, K split over a cluster, stride and padding; and the gathering variant (K <= 64)."""
+    nb, cin, cout, hh, ww, ksize, stride, pad = geom
+    K = cin * ksize * ksize
+    W = gen.dense_weight(cout, K, seed=181)
+    mask = gen.bcr_mask(cout, K, 8, 32, compression=3, dist="uniform", seed=182, empty_frac=0.2)
+    mask[:8] = 0
+    x = np.maximum(gen.normal_f32((nb, cin, hh, ww), 1.0, 183, 0), 0.0)
+    L = dict(W=W, mask=mask, bias=gen.normal_f32((cout,), 0.05, 184, 0), bh=8, bw=32)
+    check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=True, out_bf16=out_bf16, kernel_flags=B.GRIM_CONV_TENSOR)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("hw", [(6, 10), (4, 8), (2, 24), (10, 16), (8, 32)])
+def test_maxpool_vector_widths(B, bf16, hw):
+    """Output rows of 5, 4, 12, 8 and 16 elements: scalar passes and vectors of 2, 4 and 8; exact."""
+    x = to_dev(gen.normal_f32((3, 5) + hw, 1.0, 185, 0), bf16)
+    out = torch.empty(3, 5, hw[0] // 2, hw[1] // 2, device="cuda", dtype=x.dtype)
+    B.grim_maxpool2x2(x, out)
+    assert torch.equal(out, torch.nn.functional.max_pool2d(x, 2))
+
+
 @pytest.mark.parametrize("split", [2, 5, 8])
 def test_split_multiply(B, split):
     """Few output tiles: several thread blocks share a tile's block columns and add their partial sums into a
