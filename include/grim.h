@@ -102,7 +102,9 @@ typedef struct {
                       16-byte aligned), 32 + 1, 2 or 4 = with that many columns per lane, then plus 256 x the
                       number of warps that share a row band (1, 2, 4, 8, 16);
                       path 3: 1 = values staged in registers, 2 = values streamed through shared memory by bulk
-                      asynchronous copies (persistent thread blocks), 0 = the streaming variant when it fits */
+                      asynchronous copies (persistent thread blocks), 0 = the streaming variant when it fits,
+                      4 = the gathering kernel (2 <= N <= 16), 8 / 16 / 32 / 64 = the same with 1 / 2 / 4 / 8 warps
+                      per row band */
   int32_t path;    /* 0 auto; 1 register-tiled CUDA-core kernel; 2 tcgen05 tensor-core tiles (bf16
                       handles only); 3 lane-per-column kernel (N <= 16, N = 1 is the matrix-vector product);
                       4 shared-memory slab kernel (any N; the fall-back for operands the others do not take);

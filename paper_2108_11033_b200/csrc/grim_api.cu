@@ -56,12 +56,16 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
     if (!tc2_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc2(h, a, s);
   }
+  if (path == 3 && a.tile_n >= 4) {
+    if (a.tile_n != 4 && a.tile_n != 8 && a.tile_n != 16 && a.tile_n != 32 && a.tile_n != 64) return GRIM_ERR_INVALID_ARG;
+    return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, a.tile_n == 4 ? 0 : a.tile_n / 8, s);
+  }
   if (path == 1 && (a.tile_n & 32)) return launch_direct(h, a, s);
   if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
-  // 8 <= N <= 16, measured at 8192 x 8192 and 4096 x 4096: bf16 handles are fastest on the tensor-core tile (56 us
-  // split over K against 102 us on the lane-per-column kernel), fp32 handles with blocks of 8 rows or more on the
-  // CUDA-core kernel's 16-column tile (93 against 98 - 124 us); narrower right-hand sides stay on the lane-per-column
-  // kernel
+  if (path == 0 && narrow_preferred(h, X->cols))
+    return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, 0, s);
+  // handles without the narrow layouts, and fp32 handles with 16-row blocks: the tensor-core tile, the 16-column tile of the
+  // slab kernel
   if (path == 0 && X->cols >= 8 && X->cols <= kSkinnyMaxN) {
     if (tc_path_supported(h, a) && h->tc_mtiles >= 8) return launch_spmm_tc(h, a, s);
     if (h->dtype == GRIM_F32 && h->bh >= 8 && ffma_path_supported(h, a)) return launch_ffma(h, a, s);
@@ -186,7 +190,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
   float best_t = -1.f;
   grim_tune_t cand_best{};
   // candidates: (path, tile_n); a candidate that cannot take the request is skipped
-  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
+  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {3, 4}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
   for (const auto& cd : cand) {
     grim_tune_t c{};
     c.path = cd[0];

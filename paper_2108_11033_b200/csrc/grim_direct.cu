@@ -134,13 +134,13 @@ bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
   // 86 -> 63, 32 images 1320 -> 1220; 64 channels, 112 x 112: 58 -> 26; 5 x 5 on 96 channels, 17 x 23: 416 -> 18).
   if (a.conv) return true;
   if (a.ncols <= kSkinnyMaxN) {
-    // Few columns leave most lanes idle, so the time goes with the number of chunks (about 2.5 us and 0.3 ns each):
-    // better than the other kernels' fixed cost up to some 17000 (2048^2, 8x32, N = 16: 12.5 -> 7.8; 4096^2: 21 -> 26).
-    // Widths that the lane-per-column kernel has to pad and cannot load in vectors are worth more (4096^2, N = 7: 41 -> 26).
+    // Few columns leave most lanes idle, so the time goes with the number of chunks (about 2.5 us and 0.3 ns each).  Against
+    // the gathering kernel, which has more to set up: up to some 5000 chunks (1024^2, 8 x 32, N = 7: 3.4 against 5.2; 512^2:
+    // 3.0 against 5.2), and where that one needs two passes up to 17000 (2048^2, 16 x 64, N = 16: 6.7 against 7.6).
     // (handles that hold only the wide regime's layouts refuse fewer than eight columns, as grim.h says)
-    if (h->dtype != GRIM_F32 || (a.ncols < 8 && (h->flags & GRIM_PACK_WIDE_ONLY))) return false;
-    const int64_t most = (a.ncols >= 5 && a.ncols < 8 && h->bh >= 8) ? 300000 : 17000;
-    return h->rc_chunks <= most && (a.ncols >= 5 || h->bh >= 8);
+    if (a.ncols < 8 && (h->flags & GRIM_PACK_WIDE_ONLY)) return false;
+    if (a.x_dtype == GRIM_BF16 && a.ncols >= 8) return !h->d_chunks && h->rc_chunks <= 5000;
+    return h->rc_chunks <= (h->bh > 8 && a.ncols > 8 ? 17000 : 5000) && a.ncols >= 5;
   }
   // The slab kernel needs rows of X that TMA can fetch; its other loaders are slow (N = 1023: 1477 -> 1213, N = 131 in
   // bf16: 328 -> 30), except that a slab row of 16-row bands is used often enough to pay for them in large products.

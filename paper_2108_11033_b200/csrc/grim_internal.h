@@ -50,7 +50,6 @@ struct ChunkDesc {
 // The streaming kernel moves the chunk layout in "runs": up to kRunChunks consecutive chunks of one band whose
 // values take at most kRunValueBytes (no single chunk is larger: 16 rows x 32 columns x 4 bytes is half of it).  Run r covers chunks [runs[r].c0, runs[r + 1].c0) and values [runs[r].v0, runs[r + 1].v0); the
 // table ends with a sentinel.  run_ptr[pos] .. run_ptr[pos + 1] are the runs of the band at schedule position pos.
-constexpr int kSliceRows = 1024;  // rows of X per K slice of the sliced copy (see grim_bcr::sl_*)
 constexpr int kRunChunks = 4;
 constexpr int kRunValueBytes = 4096;
 struct RunDesc {
@@ -187,17 +186,7 @@ struct grim_bcr {
   uint32_t* d_run_ptr = nullptr;
   grim::RunDesc* d_runs = nullptr;
   int64_t nruns = 0;
-  // K-sliced copy of the chunk layout for 2 <= N <= 16 (absent when K has a single slice): virtual band v = slice *
-  // nbr + schedule position; per virtual band its runs, its band and its slice
-  int sl_rows = 0;          // rows of X per slice (a multiple of bw)
-  int64_t sl_nslices = 0, sl_nruns = 0, index_bytes_sliced = 0;
-  uint32_t* d_sl_colwords = nullptr;
-  void* d_sl_vals = nullptr;
-  uint32_t* d_sl_run_ptr = nullptr;
-  grim::RunDesc* d_sl_runs = nullptr;
-  uint32_t* d_sl_band_of = nullptr;
-  uint32_t* d_sl_slice_of = nullptr;
-  // dense bf16 copy for the tensor-core path is decompressed on the fly; nothing stored here
+  void* d_xpad = nullptr;  // scratch of the gathering kernel: K rows of sixteen values
 };
 
 namespace grim {
@@ -228,6 +217,11 @@ grim_status_t launch_skinny(const grim_bcr* h, const void* X, int x_dtype, int64
 grim_status_t launch_stream(const grim_bcr* h, const void* X, int x_dtype, int64_t ldx, int64_t N, void* Y, int y_dtype,
                             int64_t ldy, cudaStream_t s);
 bool stream_path_supported(const grim_bcr* h, int64_t N);
+// 2 <= N <= 16, every warp gathering its columns' rows of X (parts: warps per band, 0 = chosen here)
+grim_status_t launch_narrow(const grim_bcr* h, const void* X, int x_dtype, int64_t ldx, int64_t N, void* Y, int y_dtype, int64_t ldy,
+                            int parts, cudaStream_t s);
+bool narrow_path_supported(const grim_bcr* h, int64_t N);
+bool narrow_preferred(const grim_bcr* h, int64_t N);
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA

@@ -34,9 +34,9 @@ inline uint16_t bf16_bits(float f) {
 class Arena {
  public:
   template <typename T>
-  void add(T** dst, const void* src, size_t bytes) {
+  void add(T** dst, const void* src, size_t bytes, size_t scratch = 0) {  // scratch: bytes behind them that are not copied
     items_.push_back({reinterpret_cast<void**>(dst), src, bytes, total_});
-    total_ += (std::max<size_t>(bytes, 16) + 255) / 256 * 256;
+    total_ += (std::max<size_t>(bytes + scratch, 16) + 255) / 256 * 256;
   }
   cudaError_t upload(void** base) {
     cudaError_t e = cudaMalloc(base, total_);
@@ -221,29 +221,25 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
                           nbr * 4;
 
     // ---- chunk layout for the N <= 16 kernels
-    // A "virtual band" is a band restricted to block columns [jlo, jhi): the whole band for the matrix-vector product,
-    // one K slice of it for 2 <= N <= 16 (see below).  build_narrow lays the chunks and runs of a list of virtual
-    // bands out, in list order.
-    struct VBand { int64_t pos, jlo, jhi; };
     struct Narrow {
-      std::vector<uint32_t> band_ptr;  // per virtual band: first chunk
+      std::vector<uint32_t> band_ptr;  // per band (schedule order): first chunk
       std::vector<ChunkDesc> chunks;
       std::vector<uint32_t> colwords;
       std::vector<uint8_t> gvals;
-      std::vector<uint32_t> run_ptr;   // per virtual band: first run
+      std::vector<uint32_t> run_ptr;   // per band: first run
       std::vector<RunDesc> runs;
     };
-    auto build_narrow = [&](const std::vector<VBand>& vb, Narrow& o) {
-      const int64_t nv = (int64_t)vb.size();
+    auto build_narrow = [&](Narrow& o) {
+      const int64_t nv = nbr;
       o.band_ptr.assign((size_t)nv + 1, 0);
       o.gvals.reserve((size_t)nnz * vsz);
       std::vector<int64_t> order;
       uint64_t gv_elems = 0;
       for (int64_t v = 0; v < nv; ++v) {
-        const int64_t i = h->band_order[(size_t)vb[(size_t)v].pos];
+        const int64_t i = h->band_order[(size_t)v];
         o.band_ptr[(size_t)v] = (uint32_t)o.chunks.size();
         order.clear();
-        for (int64_t j = vb[(size_t)v].jlo; j < vb[(size_t)v].jhi; ++j)
+        for (int64_t j = 0; j < nbc; ++j)
           if (h->blocks[(size_t)(i * nbc + j)].kr && h->blocks[(size_t)(i * nbc + j)].kc) order.push_back(j);
         std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
           return h->blocks[(size_t)(i * nbc + a)].kr > h->blocks[(size_t)(i * nbc + b)].kr;
@@ -315,13 +311,10 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
       o.run_ptr[(size_t)nv] = (uint32_t)o.runs.size();
       o.runs.push_back(RunDesc{(uint32_t)o.chunks.size(), (uint32_t)gv_elems});
     };
-    Narrow nar, sl;  // whole bands; K slices
-    std::vector<uint32_t> sl_band_of, sl_slice_of;  // sliced copy: band and slice of every virtual band
+    Narrow nar;
     h->gemv_ok = K <= 65536;
     if (h->gemv_ok) {
-      std::vector<VBand> vb;
-      for (int64_t pos = 0; pos < nbr; ++pos) vb.push_back(VBand{pos, 0, nbc});
-      build_narrow(vb, nar);
+      build_narrow(nar);
       h->nruns = (int64_t)nar.runs.size() - 1;
       h->nchunks = (int64_t)nar.chunks.size();
       h->h_gemv_band_ptr = nar.band_ptr;
@@ -330,26 +323,6 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
       // what the streaming kernel reads besides the values: column words, the run table, the band tables
       h->index_bytes_gemv = (int64_t)nar.colwords.size() * 4 + (int64_t)nar.runs.size() * (int64_t)sizeof(RunDesc) +
                             (nbr + 1) * 4 + nbr * 4;
-      // K slices for 2 <= N <= 16: a thread block stages the slice's rows of X in shared memory once and multiplies the
-      // slice's part of many bands from there (Section 4.4: a needed input row is loaded once), instead of gathering
-      // them from L2 for every band.  A second copy of the values in slice-major order; only built when K has more
-      // than one slice (otherwise the whole-band layout is its own single slice).
-      const int64_t spb = std::max<int64_t>(1, kSliceRows / bw);  // block columns per slice
-      h->sl_rows = (int)(spb * bw);
-      h->sl_nslices = (nbc + spb - 1) / spb;
-      if (h->sl_nslices > 1 && !(flags & GRIM_PACK_WIDE_ONLY)) {
-        std::vector<VBand> vs;
-        for (int64_t sidx = 0; sidx < h->sl_nslices; ++sidx)
-          for (int64_t pos = 0; pos < nbr; ++pos) {
-            vs.push_back(VBand{pos, sidx * spb, std::min<int64_t>((sidx + 1) * spb, nbc)});
-            sl_band_of.push_back(h->band_order[(size_t)pos]);
-            sl_slice_of.push_back((uint32_t)sidx);
-          }
-        build_narrow(vs, sl);
-        h->sl_nruns = (int64_t)sl.runs.size() - 1;
-        h->index_bytes_sliced = (int64_t)sl.colwords.size() * 4 + (int64_t)sl.runs.size() * (int64_t)sizeof(RunDesc) +
-                                ((int64_t)vs.size() + 1) * 4 + (int64_t)vs.size() * 8;
-      }
     }
 
     // ---- row-chunk layout for the register-tiled and tensor-core kernels
@@ -551,14 +524,7 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
         ar.add(&h->d_gemv_vals, nar.gvals.data(), nar.gvals.size());
         ar.add(&h->d_run_ptr, nar.run_ptr.data(), nar.run_ptr.size() * 4);
         ar.add(&h->d_runs, nar.runs.data(), nar.runs.size() * sizeof(RunDesc));
-        if (!sl.runs.empty()) {
-          ar.add(&h->d_sl_colwords, sl.colwords.data(), sl.colwords.size() * 4);
-          ar.add(&h->d_sl_vals, sl.gvals.data(), sl.gvals.size());
-          ar.add(&h->d_sl_run_ptr, sl.run_ptr.data(), sl.run_ptr.size() * 4);
-          ar.add(&h->d_sl_runs, sl.runs.data(), sl.runs.size() * sizeof(RunDesc));
-          ar.add(&h->d_sl_band_of, sl_band_of.data(), sl_band_of.size() * 4);
-          ar.add(&h->d_sl_slice_of, sl_slice_of.data(), sl_slice_of.size() * 4);
-        }
+        ar.add(&h->d_xpad, nullptr, 0, (size_t)K * 16 * vsz);
       }
       if (e == cudaSuccess) e = ar.upload(&h->d_arena);
       if (e != cudaSuccess) {

@@ -249,6 +249,21 @@ def test_maxpool_vector_widths(B, bf16, hw):
     assert torch.equal(out, torch.nn.functional.max_pool2d(x, 2))
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("parts", [1, 2, 4, 8])
+@pytest.mark.parametrize("case", [(300, 700, 8, 32, 2), (304, 520, 4, 16, 3), (129, 1333, 16, 64, 4), (300, 520, 4, 16, 7), (512, 2100, 8, 32, 8),
+                                  (260, 700, 16, 64, 9), (200, 300, 5, 20, 12), (7, 40, 3, 9, 15), (520, 1040, 8, 32, 16), (264, 512, 4, 16, 16)])
+def test_gathering_kernel(B, case, parts, bf16):
+    """One to several passes over the columns, rows of X with and without aligned pieces, bands with fewer chunks than warps
+    or none, short last chunks, block heights below the compiled ones."""
+    M, K, bh, bw, N = case
+    W = gen.dense_weight(M, K, seed=191)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=4, dist="zipf", seed=192, empty_frac=0.3)
+    mask[:bh] = 0
+    X = gen.normal_f32((K, N), 1.0, 193, 0)
+    check_spmm(B, W, mask, X, bh, bw, bf16=bf16, path=3, tile_n=8 * parts, y_bf16=bf16 and parts == 2)
+
+
 @pytest.mark.parametrize("split", [2, 5, 8])
 def test_split_multiply(B, split):
     """Few output tiles: several thread blocks share a tile's block columns and add their partial sums into a
