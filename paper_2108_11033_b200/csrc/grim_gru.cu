@@ -21,6 +21,7 @@
 
 #include "grim_device.cuh"
 #include "grim_internal.h"
+#include "grim_rowwalk.cuh"
 
 namespace cg = cooperative_groups;
 using namespace grim;
@@ -35,13 +36,16 @@ struct ModeCfg {
 };
 }  // namespace
 
+namespace { struct GruParams; }
+
 struct grim_gru {
   int L = 0;
   int64_t H = 0, max_T = 0;
   int bh = 0;
   std::vector<const grim_bcr*> Wih, Whh;
   std::vector<float*> d_bih, d_bhh;
-  std::vector<uint32_t*> d_pos_of_band;
+  std::vector<uint32_t*> d_pos_of_band;     // schedule position of every band of W_hh
+  std::vector<uint32_t*> d_pos_of_band_ih;  // ... of W_ih
   std::vector<float*> d_img_val;      // per layer: register image of the register-resident kernel (may be empty)
   std::vector<uint32_t*> d_img_col;
   std::vector<float*> d_gi_saved;  // grim_gru_seq_static parks d_gi here while it points the pass at the static array
@@ -61,7 +65,7 @@ struct grim_gru {
   unsigned* d_sync = nullptr;  // [0..L): barrier counters, [L]: status word
   ModeCfg grid, cluster;       // launch shapes of the shared-memory kernels
   ModeCfg regc;                // launch shape of the register-resident cluster kernel
-  int reg_ni = 0, reg_s = 0;   // its compiled (items per warp, slots per item) variant
+  void (*reg_kern)(const GruParams) = nullptr;  // its compiled variant
   int device = -1;
   cudaStream_t last_stream = nullptr;
   int dbg_skip_cta = -1;
@@ -131,6 +135,24 @@ __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
 }
 
 __device__ __forceinline__ float sigmoidf_(float v) { return 1.f / (1.f + expf(-v)); }
+
+// tanh without a branch: the recurrent step waits for it, and lanes on both sides of a threshold would take both paths in
+// turn.  Below 0.5 the Taylor series about 0 (eight terms, remainder below 1e-8 of the result), above it
+// 1 - 2 / (1 + e^(2|x|)).  Within 2.1 units in the last place.
+__device__ __forceinline__ float tanh_both(float x) {
+  const float ax = fabsf(x), x2 = x * x;
+  float p = 6404582.f / 10854718875.f;
+  p = fmaf(p, x2, -929569.f / 638512875.f);
+  p = fmaf(p, x2, 21844.f / 6081075.f);
+  p = fmaf(p, x2, -1382.f / 155925.f);
+  p = fmaf(p, x2, 62.f / 2835.f);
+  p = fmaf(p, x2, -17.f / 315.f);
+  p = fmaf(p, x2, 2.f / 15.f);
+  p = fmaf(p, x2, -1.f / 3.f);
+  const float small = fmaf(x * x2, p, x);
+  const float big = fmaf(__frcp_rn(1.f + expf(2.f * ax)), -2.f, 1.f);
+  return ax < 0.5f ? small : copysignf(big, x);
+}
 
 // Per-CTA view of its bands' chunks: either the global arrays or copies in shared memory.
 struct BandView {
@@ -368,17 +390,17 @@ __global__ void __launch_bounds__(1024, 1) gru_cluster_kernel(const GruParams p)
 // ---------------------------------------------------------------------------------------------
 // cluster version with W_hh in registers.  Every warp keeps its share of the bands in registers for the whole
 // sequence, and the new state travels by asynchronous shared-memory stores counted on mbarriers instead of through a
-// cluster barrier (whose release / acquire pair was the largest stall of a step): a band is cut in two halves (work items), an
-// item's kept columns are dealt to S slots x 32 lanes, and a lane holds per slot the column index and
+// cluster barrier (whose release / acquire pair was the largest stall of a step): a band is cut into ks parts (work items),
+// an item's kept columns are dealt to S slots x 32 lanes, and a lane holds per slot the column index and
 // the column's BH values expanded to row positions (zeros where the row is not kept).  A time step then
-// costs one shared-memory gather of h and BH FMAs per slot - no index decoding, no predicates.
-// NI = items per warp.  Shapes that need more slots than the compiled menu use the other kernels.
+// costs one shared-memory gather of h and BH / 2 packed FMAs (two rows each) per slot - no index decoding, no predicates.
+// NI = items per warp, THREADS = the most threads a variant is launched with.  What bounds a step is a chain of latencies
+// (gather, sums, reduction, gates, exchange), in which the issue of a scheduler's warps is the largest part that the shape
+// decides: the variant with the fewest issued instructions per step is taken.  Shapes that need more slots than the compiled
+// menu use the other kernels.  No variant's weights may spill: reloading them every step cost more than any schedule gains.
 // ---------------------------------------------------------------------------------------------
-constexpr int kRegThreads = 512;
-constexpr int kRegWarps = kRegThreads / 32;
-
-template <int BH, int NI, int S>
-__global__ void __launch_bounds__(kRegThreads, 1) gru_cluster_reg_kernel(const GruParams p) {
+template <int BH, int NI, int S, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruParams p) {
   extern __shared__ __align__(16) float smem_f[];
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -387,44 +409,59 @@ __global__ void __launch_bounds__(kRegThreads, 1) gru_cluster_reg_kernel(const G
   const int nb = 3 * p.tpc;
   const int U = p.tpc * p.bh;
   const int H = p.H;
-  const int nbands_gate = H / p.bh;
-  float* hs = smem_f;                         // [2][H]
-  float* hnew = hs + 2 * H;                   // [U]
-  float* partial = hnew + ((U + 3) & ~3);     // [nb][2][BH]
+  const int ks = p.ks;
+  float* hs = smem_f;                          // [2][H]
+  float* partial = hs + 2 * H;                 // [2][nb][ks][BH]: steps alternate, so that a warp that is ahead overwrites nothing
+  const int part_len = nb * ks * BH;
 
   // ---- one-time: this thread's share of W_hh (built on the host when the handle was created): coalesced loads
-  float val[NI][S][BH];
-  uint32_t col[NI][S];
+  unsigned long long val[NI][S][BH / 2];  // pairs of neighbouring rows
+  uint32_t col[NI][(S + 1) / 2];          // columns of two slots
   {
-    const float* iv = p.img_val + (size_t)rank * NI * S * BH * kRegThreads + tid;
-    const uint32_t* ic = p.img_col + (size_t)rank * NI * S * kRegThreads + tid;
+    const float2* iv = reinterpret_cast<const float2*>(p.img_val) + (size_t)rank * NI * S * (BH / 2) * THREADS + tid;
+    const uint32_t* ic = p.img_col + (size_t)rank * NI * ((S + 1) / 2) * THREADS + tid;
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
+    for (int i = 0; i < NI; ++i) {
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        col[i][s] = __ldg(ic + (size_t)(i * S + s) * kRegThreads);
+      for (int s = 0; s < (S + 1) / 2; ++s) col[i][s] = __ldg(ic + (size_t)(i * ((S + 1) / 2) + s) * THREADS);
 #pragma unroll
-        for (int r = 0; r < BH; ++r) val[i][s][r] = __ldg(iv + (size_t)((i * S + s) * BH + r) * kRegThreads);
-      }
+      for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int r = 0; r < BH / 2; ++r) {
+          const float2 v = __ldg(iv + (size_t)((i * S + s) * (BH / 2) + r) * THREADS);
+          val[i][s][r] = walk_pair(v.x, v.y);
+        }
+    }
   }
 
-  const bool gate_live = tid < U;
-  const int g_tri = tid / p.bh, g_r = tid % p.bh;
-  const int unit = rank * U + tid;
+  // The gates of the CTA's U hidden units are worked out by several groups of warps at once, each of which sends the new
+  // values to its share of the cluster (sixteen stores one after the other by the same warp were 300 cycles of the step).
+  const int wg = (U + 31) / 32, groups = min(min((int)(blockDim.x >> 5) / wg, 4), CS), group = warp / wg;
+  const int gu = (warp - group * wg) * 32 + lane;
+  const int g_tri = gu / p.bh, g_r = gu % p.bh;
+  const int unit = rank * U + gu;
+  const bool gate_live = group < groups && gu < U && unit < H;  // (the last CTAs may own fewer groups of units, or none)
+  const int dst0 = CS * group / groups, dst1 = CS * (group + 1) / groups;
+  const bool stores = group == groups - 1;
   float bq[3] = {0.f, 0.f, 0.f};
   float gi[3] = {0.f, 0.f, 0.f};
-  if (gate_live)
+  float h_own = 0.f;  // the unit's state
+  if (gate_live) {
     for (int g = 0; g < 3; ++g) {
       bq[g] = p.b_hh[g * H + unit];
       gi[g] = __ldg(p.gi + g * H + unit);
     }
-  for (int i = tid; i < H; i += kRegThreads) hs[i] = p.h0 ? p.h0[i] : 0.f;
-  // The state exchange: the thread that owns a hidden unit sends its new value into the next-step buffer of every
-  // CTA of the cluster with asynchronous stores that count their bytes on the receiver's mbarrier; a CTA starts a
-  // step when the H values of that step have been counted.  No cluster-wide barrier and no fence per step: a
-  // buffer is written again only after every CTA has received the whole state computed from it, i.e. after every
-  // warp of the cluster is done reading it.
-  uint64_t* hbar = reinterpret_cast<uint64_t*>(partial + nb * 2 * BH);  // [2], 8-byte aligned (all counts are even)
+    h_own = p.h0 ? p.h0[unit] : 0.f;
+  }
+  for (int i = tid; i < H; i += (int)blockDim.x) hs[i] = p.h0 ? p.h0[i] : 0.f;
+  // The state exchange: the threads that own a hidden unit send its new value into the next-step buffer of every
+  // CTA of the cluster with asynchronous stores that count their bytes on the receiver's mbarrier; a warp starts a
+  // step when the H values of that step have been counted.  No cluster-wide barrier and no fence per step: values of a
+  // step leave a CTA only after all its warps have read the state before it (the block barrier below), and a buffer is
+  // written again only by CTAs that have received such values from everybody.
+  uint64_t* hbar = reinterpret_cast<uint64_t*>(partial + 2 * part_len);  // [2], 8-byte aligned (all counts are even)
+  volatile int* s_failed = reinterpret_cast<volatile int*>(hbar + 2);
+  if (tid == 0) *s_failed = 0;
   if (tid == 0) {
     gru_mbar_init(hbar, 1);
     gru_mbar_init(hbar + 1, 1);
@@ -432,11 +469,11 @@ __global__ void __launch_bounds__(kRegThreads, 1) gru_cluster_reg_kernel(const G
   }
   cluster.sync();
   const uint32_t hs_local = (uint32_t)__cvta_generic_to_shared(hs), bar_local = (uint32_t)__cvta_generic_to_shared(hbar);
-  bool failed = false;
 
   for (int t = 0; t < p.T; ++t) {
     const int cur = t & 1, nxt = cur ^ 1;
     const float* hcur = hs + cur * H;
+    float* part_t = partial + cur * part_len;
     // this step's outputs arrive on the next buffer's barrier: announce the byte count (fast CTAs may already be
     // sending, which drives the count negative; the pending arrival keeps the phase open until it is announced)
     if (tid == 0 && t + 1 < p.T) gru_mbar_arrive_expect_tx(hbar + nxt, (unsigned)H * 4u);
@@ -447,51 +484,69 @@ __global__ void __launch_bounds__(kRegThreads, 1) gru_cluster_reg_kernel(const G
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const int item = warp * NI + i;
-      float acc[BH];
+      unsigned long long sum[BH / 2];
 #pragma unroll
-      for (int r = 0; r < BH; ++r) acc[r] = 0.f;
+      for (int r = 0; r < BH / 2; ++r) sum[r] = 0ull;
 #pragma unroll
       for (int s = 0; s < S; ++s) {
-        const float xv = hcur[col[i][s]];
+        const float xv = hcur[(s & 1) ? col[i][s / 2] >> 16 : col[i][s / 2] & 0xFFFFu];
+        const unsigned long long x2 = walk_pair(xv, xv);
 #pragma unroll
-        for (int r = 0; r < BH; ++r) acc[r] = fmaf(val[i][s][r], xv, acc[r]);
+        for (int r = 0; r < BH / 2; ++r) walk_ffma2(sum[r], val[i][s][r], x2);
+      }
+      float acc[BH];
+#pragma unroll
+      for (int r = 0; r < BH / 2; ++r) {
+        acc[2 * r] = __uint_as_float((unsigned)sum[r]);
+        acc[2 * r + 1] = __uint_as_float((unsigned)(sum[r] >> 32));
       }
       warp_reduce_rows<BH>(acc, lane);
-      if (item < nb * 2) partial[item * BH + warp_row<BH>(lane)] = acc[0];
+      if (item < nb * ks) part_t[item * BH + warp_row<BH>(lane)] = acc[0];
     }
     __syncthreads();
-    float hnew_val = 0.f;
     if (gate_live) {
-      // the thread that owns a hidden unit computes it; below it is sent straight to the next-step buffer of every CTA
-      const float hn = gru_gate(partial, bq, gi, g_tri, g_r, 2, BH, hcur[unit]);
-      hnew_val = hn;
-      p.out[(int64_t)t * H + unit] = hn;
-      if (p.outT) p.outT[(int64_t)unit * p.ldT + t] = hn;
-      if (t == p.T - 1 && p.hT) p.hT[unit] = hn;
-    }
-    if (gate_live && t + 1 < p.T) {
-      // one 4-byte store per destination (pooling four neighbours' values into 16-byte stores was slower: the
-      // shuffles lengthen the chain more than the fewer messages save)
-      const uint32_t dst_local = hs_local + (uint32_t)(nxt * H + unit) * 4u, bar_nxt = bar_local + (uint32_t)nxt * 8u;
+      float q[3];
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        const float* part = part_t + (g_tri * 3 + g) * ks * BH + g_r;
+        q[g] = bq[g] + part[0];
+        for (int k = 1; k < ks; ++k) q[g] += part[k * BH];
+      }
+      const float rg = __frcp_rn(1.f + expf(-(gi[0] + q[0]))), zg = __frcp_rn(1.f + expf(-(gi[1] + q[1])));
+      const float ng = tanh_both(gi[2] + rg * q[2]);
+      h_own = (1.f - zg) * ng + zg * h_own;
+      if (t + 1 < p.T) {
+        // one 4-byte store per destination (pooling four neighbours' values into 16-byte stores was slower: the
+        // shuffles lengthen the chain more than the fewer messages save)
+        const uint32_t dst_local = hs_local + (uint32_t)(nxt * H + unit) * 4u, bar_nxt = bar_local + (uint32_t)nxt * 8u;
 #pragma unroll 4
-      for (int dst = 0; dst < CS; ++dst) gru_st_async_f32(dst_local, bar_nxt, (uint32_t)dst, hnew_val);
+        for (int dst = dst0; dst < dst1; ++dst) gru_st_async_f32(dst_local, bar_nxt, (uint32_t)dst, h_own);
+      }
+      if (stores) {  // after the exchange has left: nobody waits for these
+        p.out[(int64_t)t * H + unit] = h_own;
+        if (p.outT) p.outT[(int64_t)unit * p.ldT + t] = h_own;
+        if (t == p.T - 1 && p.hT) p.hT[unit] = h_own;
+      }
     }
 #pragma unroll
     for (int g = 0; g < 3; ++g) gi[g] = gi_next[g];
-    if (t + 1 < p.T && warp == 0) {
-      // the next step's state: bounded wait on the local barrier (its (t / 2)-th use).  One thread polls for the
-      // whole block; the others sleep in the block barrier below (many pollers slow the arrival of the stores down)
+    if (t + 1 < p.T) {
+      // the next step's state: bounded wait on the local barrier (its (t / 2)-th use), one thread of every warp.  When it
+      // runs out the block goes through its remaining steps without waiting: the results are invalid and reported.
       const unsigned parity = (unsigned)((t >> 1) & 1);
-      bool ok = false;
-      if (lane == 0)
-        for (unsigned it = 0; it < p.spin_limit && !ok; ++it) ok = gru_mbar_try_wait(hbar + nxt, parity);
-      __syncwarp();
-      if (!__shfl_sync(0xffffffffu, ok, 0)) {
-        failed = true;
-        if (lane == 0) atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
+      if (lane == 0 && !*s_failed) {
+        bool ok = false;
+        for (unsigned it = 0; it < p.spin_limit && !ok; ++it) {
+          ok = gru_mbar_try_wait(hbar + nxt, parity);
+          if (!ok && (it & 63u) == 63u && *s_failed) break;
+        }
+        if (!ok && !*s_failed) {
+          *s_failed = 1;
+          atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
+        }
       }
+      __syncwarp();
     }
-    if (__syncthreads_or(failed ? 1 : 0)) break;  // the state of the next step is there (or a wait ran out)
   }
   cluster.sync();  // no CTA leaves while another may still address its shared memory
 }
@@ -566,29 +621,41 @@ cudaError_t launch_cluster(Kern kern, const ModeCfg& m, const GruParams& p, cuda
   return e;
 }
 
-// The compiled variants of the register-resident kernel: (BH, items per warp, slots per item).
+// The compiled variants of the register-resident kernel.
 using GruKernel = void (*)(const GruParams);
-GruKernel reg_kernel(int BH, int ni, int s) {
-  if (BH != 8) return nullptr;
-  if (ni == 1 && s == 2) return gru_cluster_reg_kernel<8, 1, 2>;
-  if (ni == 1 && s == 4) return gru_cluster_reg_kernel<8, 1, 4>;
-  if (ni == 3 && s == 3) return gru_cluster_reg_kernel<8, 3, 3>;
-  if (ni == 3 && s == 4) return gru_cluster_reg_kernel<8, 3, 4>;
-  return nullptr;
-}
+struct RegVariant {
+  int BH, ni, s, threads;
+  GruKernel kern;
+};
+const RegVariant kRegVariants[] = {
+    {8, 1, 2, 512, gru_cluster_reg_kernel<8, 1, 2, 512>},
+    {8, 1, 4, 768, gru_cluster_reg_kernel<8, 1, 4, 768>},
+    {8, 2, 6, 384, gru_cluster_reg_kernel<8, 2, 6, 384>},
+    {8, 3, 8, 256, gru_cluster_reg_kernel<8, 3, 8, 256>},
+    {4, 1, 2, 768, gru_cluster_reg_kernel<4, 1, 2, 768>},
+    {4, 1, 4, 768, gru_cluster_reg_kernel<4, 1, 4, 768>},
+    {4, 2, 4, 384, gru_cluster_reg_kernel<4, 2, 4, 384>},
+    {4, 4, 4, 384, gru_cluster_reg_kernel<4, 4, 4, 384>},
+    {4, 4, 6, 384, gru_cluster_reg_kernel<4, 4, 6, 384>},
+    {4, 4, 7, 384, gru_cluster_reg_kernel<4, 4, 7, 384>},
+    {4, 6, 8, 256, gru_cluster_reg_kernel<4, 6, 8, 256>},
+    {16, 1, 2, 512, gru_cluster_reg_kernel<16, 1, 2, 512>},
+    {16, 1, 4, 512, gru_cluster_reg_kernel<16, 1, 4, 512>},
+    {16, 1, 6, 384, gru_cluster_reg_kernel<16, 1, 6, 384>},
+    {16, 1, 8, 384, gru_cluster_reg_kernel<16, 1, 8, 384>}};
 GruKernel smem_cluster_kernel(int BH) {
   return BH == 4 ? gru_cluster_kernel<4> : (BH == 8 ? gru_cluster_kernel<8> : gru_cluster_kernel<16>);
 }
 
-// Largest number of kept columns in half a band, over all bands of all layers.
-int max_half_band_columns(const grim_gru* g) {
+// Largest number of kept columns in a band, over all bands of all layers.
+int max_band_columns(const grim_gru* g) {
   uint32_t mx = 0;
   for (const grim_bcr* wh : g->Whh)
     for (int64_t pos = 0; pos < wh->nbr; ++pos) {
       uint32_t n = 0;
       for (uint32_t k = wh->h_gemv_band_ptr[(size_t)pos]; k < wh->h_gemv_band_ptr[(size_t)pos + 1]; ++k)
         n += wh->h_chunks[k].ncols_kr & 0xFFFFu;
-      mx = std::max(mx, (n + 1) / 2);
+      mx = std::max(mx, n);
     }
   return (int)mx;
 }
@@ -624,6 +691,7 @@ void destroy(grim_gru* g) {
   for (float* p : g->d_bih) cudaFree(p);
   for (float* p : g->d_bhh) cudaFree(p);
   for (uint32_t* p : g->d_pos_of_band) cudaFree(p);
+  for (uint32_t* p : g->d_pos_of_band_ih) cudaFree(p);
   for (float* p : g->d_img_val) cudaFree(p);
   for (uint32_t* p : g->d_img_col) cudaFree(p);
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
@@ -704,14 +772,19 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
       g->Whh.push_back(wh);
       std::vector<uint32_t> pos_of_band((size_t)wh->nbr);
       for (size_t p = 0; p < pos_of_band.size(); ++p) pos_of_band[wh->band_order[p]] = (uint32_t)p;
+      const grim_bcr* wi = W_ih[l];
+      std::vector<uint32_t> pos_ih((size_t)wi->nbr);
+      for (size_t p = 0; p < pos_ih.size(); ++p) pos_ih[wi->band_order[p]] = (uint32_t)p;
       float *db1 = nullptr, *db2 = nullptr;
-      uint32_t* dp = nullptr;
+      uint32_t *dp = nullptr, *dpi = nullptr;
       cudaError_t e = cudaMalloc((void**)&db1, (size_t)3 * H * 4);
       if (e == cudaSuccess) { g->d_bih.push_back(db1); e = cudaMalloc((void**)&db2, (size_t)3 * H * 4); }
       if (e == cudaSuccess) { g->d_bhh.push_back(db2); e = cudaMalloc((void**)&dp, pos_of_band.size() * 4); }
+      if (e == cudaSuccess) { g->d_pos_of_band.push_back(dp); e = cudaMalloc((void**)&dpi, pos_ih.size() * 4); }
       if (e == cudaSuccess) {
-        g->d_pos_of_band.push_back(dp);
-        e = cudaMemcpy(db1, b_ih[l], (size_t)3 * H * 4, cudaMemcpyHostToDevice);
+        g->d_pos_of_band_ih.push_back(dpi);
+        e = cudaMemcpy(dpi, pos_ih.data(), pos_ih.size() * 4, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(db1, b_ih[l], (size_t)3 * H * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(db2, b_hh[l], (size_t)3 * H * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(dp, pos_of_band.data(), pos_of_band.size() * 4, cudaMemcpyHostToDevice);
       }
@@ -779,30 +852,35 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
         g->cluster.ok = cluster_fits(smem_cluster_kernel(BHc), g->cluster);
         if (!g->cluster.ok) g->cluster = ModeCfg{};
       }
-      // ---- register-resident cluster shape: 16 warps, two work items per band
-      const int slots_needed = (max_half_band_columns(g) + 31) / 32;
-      for (int cs = 16; cs >= 1 && !g->regc.ok; cs >>= 1) {
-        if (ntri % cs) continue;
-        ModeCfg t;
-        t.tpc = ntri / cs;
-        const int nb = 3 * t.tpc;
-        if (t.tpc * bh > kRegThreads) continue;
-        const int ni_needed = (nb * 2 + kRegWarps - 1) / kRegWarps;
-        const int menu[4][2] = {{1, 2}, {1, 4}, {3, 3}, {3, 4}};
-        for (const auto& v : menu) {
-          if (v[0] < ni_needed || v[1] < slots_needed || !reg_kernel(BHc, v[0], v[1])) continue;
-          t.ctas = cs; t.ks = 2; t.threads = kRegThreads; t.resident = 1;
-          t.smem = ((((size_t)2 * H + (size_t)((t.tpc * bh + 3) & ~3) + (size_t)nb * 2 * BHc) * 4 + 15) & ~size_t(15)) + 16;  // + the two state barriers
-          if (t.smem > kSmemLimit || !cluster_fits(reg_kernel(BHc, v[0], v[1]), t)) continue;
-          t.ok = true;
-          g->regc = t; g->reg_ni = v[0]; g->reg_s = v[1];
-          break;
-        }
+      // ---- register-resident cluster shape
+      const int max_cols = max_band_columns(g);
+      const RegVariant* rv = nullptr;
+      for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
+        const int tpc = (ntri + cs - 1) / cs, nb = 3 * tpc;
+        double best = -1.0;
+        ModeCfg shape;
+        for (const RegVariant& v : kRegVariants)
+          for (int ks = 1; ks <= 8; ks *= 2) {
+            const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
+            if (v.BH != BHc || 32 * v.s * ks < max_cols + ks - 1 || std::max(32 * warps, (tpc * bh + 31) / 32 * 32) > v.threads) continue;
+            // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
+            // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
+            const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
+            if (best >= 0.0 && cost >= best) continue;
+            ModeCfg t;
+            t.ctas = cs; t.ks = ks; t.tpc = tpc; t.resident = 1;
+            t.threads = std::max(32 * warps, std::max((tpc * bh + 31) / 32 * 32, 128));
+            t.smem = ((((size_t)2 * H + (size_t)2 * nb * ks * BHc) * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
+            if (t.smem > kSmemLimit || !cluster_fits(v.kern, t)) continue;
+            best = cost; shape = t; rv = &v;
+          }
+        if (best >= 0.0) { shape.ok = true; g->regc = shape; g->reg_kern = rv->kern; }
       }
       if (g->regc.ok) {
-        // register image: for every thread of every CTA the columns it owns (global index + values at row positions)
-        const int NI = g->reg_ni, S = g->reg_s, tpc = g->regc.tpc, cs = g->regc.ctas, nbb = 3 * tpc;
-        const size_t nval = (size_t)cs * NI * S * BHc * kRegThreads, ncol = (size_t)cs * NI * S * kRegThreads;
+        // register image: for every thread of every CTA the columns it owns (global index + values at row positions); threads
+        // are numbered with the variant's stride
+        const int NI = rv->ni, S = rv->s, S2 = (S + 1) / 2, TH = rv->threads, ks = g->regc.ks, tpc = g->regc.tpc, cs = g->regc.ctas, nbb = 3 * tpc;
+        const size_t nval = (size_t)cs * NI * S * BHc * TH, ncol = (size_t)cs * NI * S2 * TH;
         std::vector<float> iv(nval);
         std::vector<uint32_t> ic(ncol);
         struct ColRec { uint32_t col; float v[16]; };
@@ -813,6 +891,7 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
           std::fill(ic.begin(), ic.end(), 0u);
           for (int rank = 0; rank < cs; ++rank)
             for (int lb = 0; lb < nbb; ++lb) {
+              if (rank * tpc + lb / 3 >= ntri) continue;
               const int64_t band = (int64_t)(lb % 3) * ntri + (int64_t)rank * tpc + lb / 3;
               cols.clear();
               for (int64_t j = 0; j < wh->nbc; ++j) {
@@ -832,18 +911,25 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
                   ++bidx;
                 }
               }
-              const size_t n = cols.size(), mid = (n + 1) / 2;
-              for (int half = 0; half < 2; ++half) {
-                const int item = lb * 2 + half, warp = item / NI, i = item % NI;
-                const size_t c0 = half ? mid : 0, c1 = half ? n : mid;
-                for (size_t ci = c0; ci < c1; ++ci) {
-                  const size_t k = ci - c0;
-                  const int sl = (int)(k / 32), lane = (int)(k % 32);
-                  if (sl >= S || warp >= kRegWarps) { st = GRIM_ERR_UNSUPPORTED; break; }
-                  const int tid = warp * 32 + lane;
-                  ic[((size_t)(rank * NI + i) * S + sl) * kRegThreads + tid] = cols[ci].col;
+              const size_t n = cols.size();
+              for (int part = 0; part < ks; ++part) {
+                const int item = lb * ks + part, warp = item / NI, i = item % NI;
+                const size_t c0 = n * part / ks, c1 = n * (part + 1) / ks;
+                // dealt so that the 32 columns of a slot fall into different shared-memory banks as far as they go (any 32 of
+                // a thousand meet three or four to a bank): one from every bank's pile in turn, the longest piles first
+                std::vector<size_t> pile[32], deal;
+                for (size_t ci = c0; ci < c1; ++ci) pile[cols[ci].col % 32].push_back(ci);
+                std::stable_sort(pile, pile + 32, [](const std::vector<size_t>& x, const std::vector<size_t>& y) { return x.size() > y.size(); });
+                for (size_t r = 0; deal.size() < c1 - c0; ++r)
+                  for (const auto& pl : pile)
+                    if (pl.size() > r) deal.push_back(pl[r]);
+                for (size_t k = 0; k < deal.size(); ++k) {
+                  const size_t ci = deal[k];
+                  const int sl = (int)(k / 32), tid = warp * 32 + (int)(k % 32);
+                  if (sl >= S || tid >= TH) { st = GRIM_ERR_UNSUPPORTED; break; }
+                  ic[((size_t)(rank * NI + i) * S2 + sl / 2) * TH + tid] |= cols[ci].col << (16 * (sl & 1));
                   for (int r = 0; r < BHc; ++r)
-                    iv[(((size_t)(rank * NI + i) * S + sl) * BHc + r) * kRegThreads + tid] = cols[ci].v[r];
+                    iv[((((size_t)(rank * NI + i) * S + sl) * (BHc / 2) + r / 2) * TH + tid) * 2 + (r & 1)] = cols[ci].v[r];
                 }
               }
             }
@@ -957,7 +1043,7 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
     if (g->profile) profile_mark(g, 2, s);
     cudaError_t e;
     if (use_reg) {
-      e = launch_cluster(reg_kernel(BHc, g->reg_ni, g->reg_s), m, p, s);
+      e = launch_cluster(g->reg_kern, m, p, s);
     } else if (use_cluster) {
       e = launch_cluster(smem_cluster_kernel(BHc), m, p, s);
     } else {
@@ -1137,11 +1223,158 @@ extern "C" grim_status_t grim_gru_seq_static(grim_gru_t g, const float* x, int64
 }
 
 // -------------------------------------------------------------------------------------------------------------
-// One time step for a batch of sequences (Section 6.3 times the GRU at sequence length 1 and batch 32): per layer two
-// sparse multiplies with the batch as right-hand side (W_ih x and W_hh h, each with its bias in the epilogue) and one
-// fused gate kernel.
+// One time step for a batch of sequences (Section 6.3 times the GRU at sequence length 1 and batch 32): one launch turns
+// the input and the layers' states feature-major, then one launch per layer multiplies both matrices and applies the gates.
+// A thread block owns bh hidden units and 32 sequences; its 24 warps share the six bands (r, z, n of W_ih and of W_hh) that
+// produce them (grim_rowwalk.cuh), their sums meet in shared memory.  (Two multiplies on batch-major operands, whose gathers
+// do not coalesce, two bias passes, two clears and a gate kernel per layer took 80 us for two layers of 1024 and a batch of 32.)
+// Matrices of different block heights, or without the wide layouts, take that older way, below.
 // -------------------------------------------------------------------------------------------------------------
 namespace {
+struct StepParams {
+  RowWalk w[2];               // W_ih, W_hh
+  const uint32_t* pos[2];     // schedule position of every band
+  const float* bias[2];
+  SpmmArgs a[2];              // feature-major operands
+  float* h;                   // B x H, updated in place
+  float* hT;                  // null, or H x B: the new state, feature-major (input of the next layer)
+  float* y;                   // null, or B x H
+  int64_t B;
+  int H, bh, part[2];         // warps per band
+};
+constexpr int kStepWarps = 24, kStepLd = 36;
+template <int BH>
+constexpr size_t step_smem() { return (size_t)kStepWarps * (kWalkBufFloats + BH * kStepLd) * 4; }
+
+template <int BH>
+__global__ void __launch_bounds__(kStepWarps * 32, 1) gru_step_kernel(const StepParams p) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  extern __shared__ __align__(16) float ssm[];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int m = warp < 3 * p.part[0] ? 0 : 1, local = m ? warp - 3 * p.part[0] : warp;
+  const int gate = local / p.part[m], part = local - gate * p.part[m];
+  const int tri = blockIdx.x, ntri = p.H / p.bh;
+  const int64_t b0 = (int64_t)blockIdx.y * 32;
+  float* sums = ssm + kStepWarps * kWalkBufFloats;  // [warp][row][sequence]
+  float acc1[BH];
+  unsigned long long acc2[1][1];
+#pragma unroll
+  for (int r = 0; r < BH; ++r) acc1[r] = 0.f;
+  WalkCols<1, 1> wc;
+  walk_setup<1, 1, float, 0>(p.a[m], b0, lane, wc);
+  const int pos = (int)__ldg(p.pos[m] + gate * ntri + tri);
+  row_walk<BH, 1, 1, float, 0>(p.w[m], p.a[m], pos, part, p.part[m], wc, ssm + warp * kWalkBufFloats, lane, acc1, acc2,
+                               [] { asm volatile("griddepcontrol.wait;" ::: "memory"); });
+#pragma unroll
+  for (int r = 0; r < BH; ++r) sums[(warp * BH + r) * kStepLd + lane] = acc1[r];
+  __syncthreads();
+  for (int i = tid; i < p.bh * 32; i += kStepWarps * 32) {
+    const int r = i % p.bh, bl = i / p.bh, unit = tri * p.bh + r;  // neighbouring threads: neighbouring units of a sequence
+    const int64_t b = b0 + bl;
+    if (b >= p.B) continue;
+    float v[2][3];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        float t = __ldg(p.bias[k] + g * p.H + unit);
+        const int w0 = k * 3 * p.part[0] + g * p.part[k];
+        for (int s = 0; s < p.part[k]; ++s) t += sums[((w0 + s) * BH + r) * kStepLd + bl];
+        v[k][g] = t;
+      }
+    const int64_t at = b * p.H + unit;
+    const float rg = sigmoidf_(v[0][0] + v[1][0]), zg = sigmoidf_(v[0][1] + v[1][1]);
+    const float n = tanhf(v[0][2] + rg * v[1][2]);
+    const float hn = (1.f - zg) * n + zg * p.h[at];
+    p.h[at] = hn;
+    if (p.y) p.y[at] = hn;
+    if (p.hT) p.hT[(int64_t)unit * p.B + b] = hn;
+  }
+}
+
+// Turns matrices of B rows feature-major: z = 0 the input (K0 columns), z > 0 the state of layer z - 1 (H columns).
+constexpr int kStepMaxLayers = 16;
+struct TransposeArgs {
+  const float* in[kStepMaxLayers + 1];
+  float* out[kStepMaxLayers + 1];
+  int cols[kStepMaxLayers + 1];
+};
+__global__ void __launch_bounds__(256) transpose_states_kernel(const __grid_constant__ TransposeArgs t, int B) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __shared__ float tile[32][33];
+  const int k0 = blockIdx.x * 32, b0 = blockIdx.y * 32, K = t.cols[blockIdx.z];
+  const float* in = t.in[blockIdx.z];
+  float* out = t.out[blockIdx.z];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (k0 >= K) return;
+#pragma unroll
+  for (int i = 0; i < 32; i += 8)
+    if (b0 + y + i < B && k0 + x < K) tile[y + i][x] = in[(int64_t)(b0 + y + i) * K + k0 + x];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 32; i += 8)
+    if (k0 + y + i < K && b0 + x < B) out[(int64_t)(k0 + y + i) * B + b0 + x] = tile[x][y + i];
+}
+
+template <int BH>
+cudaError_t launch_step(const StepParams& p, cudaStream_t s) {
+  auto kern = gru_step_kernel<BH>;
+  constexpr size_t smem = step_smem<BH>();
+  const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3((unsigned)(p.H / p.bh), (unsigned)((p.B + 31) / 32)), dim3(kStepWarps * 32), smem, s, p);
+}
+
+bool fused_step_supported(const grim_gru* g, int64_t B) {
+  if (g->L > kStepMaxLayers || B > 65535 * 32) return false;
+  for (int l = 0; l < g->L; ++l)
+    if (!g->Wih[(size_t)l]->d_rc_head || !g->Whh[(size_t)l]->d_rc_head || g->Wih[(size_t)l]->bh != g->bh) return false;
+  return true;
+}
+
+grim_status_t fused_step(grim_gru* g, const float* x, int64_t B, float* h, float* y, cudaStream_t s) {
+  const int64_t H = g->H;
+  TransposeArgs t = {};
+  int widest = (int)g->Wih[0]->K;
+  t.in[0] = x; t.out[0] = g->d_xT; t.cols[0] = widest;
+  for (int l = 0; l < g->L; ++l) {
+    t.in[l + 1] = h + (int64_t)l * B * H;
+    t.out[l + 1] = g->d_gi[(size_t)l];  // H x B; the new state follows it (a layer's scratch holds at least 6 * H * B floats)
+    t.cols[l + 1] = (int)H;
+  }
+  widest = std::max(widest, (int)H);
+  cudaError_t e = launch_pdl(transpose_states_kernel, dim3((unsigned)((widest + 31) / 32), (unsigned)((B + 31) / 32), (unsigned)(g->L + 1)),
+                             dim3(256), 0, s, t, (int)B);
+  count_launch();
+  for (int l = 0; l < g->L && e == cudaSuccess; ++l) {
+    const grim_bcr* w[2] = {g->Wih[(size_t)l], g->Whh[(size_t)l]};
+    StepParams p;
+    for (int m = 0; m < 2; ++m) {
+      p.w[m].head = w[m]->d_rc_head; p.w[m].blob = w[m]->d_rc_blob; p.w[m].nbc = (int)w[m]->nbc; p.w[m].bw = w[m]->bw;
+      p.a[m].ncols = B; p.a[m].x_sk = B; p.a[m].x_sq = 1; p.a[m].x_dtype = GRIM_F32;
+    }
+    p.a[0].X = l == 0 ? g->d_xT : g->d_gi[(size_t)l - 1] + H * B;
+    p.a[1].X = g->d_gi[(size_t)l];
+    p.pos[0] = g->d_pos_of_band_ih[(size_t)l]; p.pos[1] = g->d_pos_of_band[(size_t)l];
+    p.bias[0] = g->d_bih[(size_t)l]; p.bias[1] = g->d_bhh[(size_t)l];
+    p.h = h + (int64_t)l * B * H;
+    p.hT = l + 1 < g->L ? g->d_gi[(size_t)l] + H * B : nullptr;
+    p.y = l + 1 == g->L ? y : nullptr;
+    p.B = B; p.H = (int)H; p.bh = g->bh;
+    // the eight warps of a gate are dealt to the two matrices by their block columns
+    const double share = (double)w[0]->nbc / (double)(w[0]->nbc + w[1]->nbc);
+    p.part[0] = std::min(7, std::max(1, (int)(8 * share + 0.5)));
+    p.part[1] = 8 - p.part[0];
+    e = g->bh <= 4 ? launch_step<4>(p, s) : (g->bh <= 8 ? launch_step<8>(p, s) : launch_step<16>(p, s));
+    count_launch();
+  }
+  if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+  g->last_stream = s;
+  return GRIM_OK;
+}
+
 // h'[b, u] = (1 - z) * n + z * h[b, u] with r, z, n from the two pre-activation buffers (batch-major, 3H per row);
 // the state is updated in place and copied to y when given.
 __global__ void gru_gate_kernel(const float* __restrict__ gi, const float* __restrict__ gh, float* __restrict__ h,
@@ -1165,6 +1398,7 @@ extern "C" grim_status_t grim_gru_step(grim_gru_t g, const float* x, int64_t B, 
   if (!g || !x || !h || B <= 0) return GRIM_ERR_INVALID_ARG;
   if (2 * B > g->max_T) return GRIM_ERR_SHAPE;  // both pre-activation buffers of a layer live in its T x 3H scratch
   cudaStream_t s = (cudaStream_t)stream;
+  if (fused_step_supported(g, B)) return fused_step(g, x, B, h, y, s);
   const int64_t H = g->H;
   const float* in = x;
   for (int l = 0; l < g->L; ++l) {

@@ -697,6 +697,35 @@ def test_gru_four_layers_and_odd_hidden_size(B):
     assert e.value.status == B.GRIM_ERR_UNSUPPORTED
 
 
+@pytest.mark.parametrize("cfg", [(20, 592, 1, 9, 8, 32, 10), (16, 1024, 1, 6, 4, 16, 10), (16, 1024, 1, 6, 16, 64, 10), (16, 1024, 2, 70, 16, 64, 16),
+                                 (30, 240, 2, 66, 16, 64, 8), (12, 272, 3, 67, 4, 16, 8), (9, 512, 1, 5, 4, 16, 8), (9, 1024, 1, 4, 8, 32, 8),
+                                 (9, 1024, 1, 4, 16, 64, 8), (5, 20, 1, 3, 5, 16, 2), (7, 16, 2, 4, 16, 16, 2)])
+def test_gru_block_shapes_and_hidden_sizes(B, cfg):
+    """All block heights, unit groups that do not divide by the cluster, more columns per band than the register variants take."""
+    in_f, H, L, T, bh, bw, rate = cfg
+    check_gru(B, gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=201), h0=gen.normal_f32((L, H), 0.5, 202, 0))
+
+
+@pytest.mark.parametrize("cfg", [(37, 128, 2, 33, 4, 16), (20, 96, 1, 31, 16, 32), (64, 160, 3, 64, 16, 64), (9, 60, 2, 2, 5, 16), (500, 64, 2, 7, 8, 32)])
+def test_gru_batched_step_block_shapes(B, cfg):
+    """Batches around a tile of 32 sequences, block heights, inputs wider and narrower than the state."""
+    in_f, H, L, batch, bh, bw = cfg
+    m = gen.gru_model(in_f, H, L, 2, bh=bh, bw=bw, compression=3, seed=203)
+    g, handles = build_gru(B, m, 2 * batch)
+    try:
+        x, h0 = gen.normal_f32((batch, in_f), 1.0, 204, 0), gen.normal_f32((L, batch, H), 0.5, 205, 0)
+        h, y = to_dev(h0), torch.empty(batch, H, device="cuda")
+        B.grim_gru_step(g, to_dev(x), h, y)
+        assert B.grim_gru_status(g) == B.GRIM_OK
+        for b in range(batch):
+            yb, hb = orc.gru_seq(m["layers"], x[b:b + 1], h0=h0[:, b])
+            assert rel_fro(y[b].cpu().numpy(), yb[0]) <= F32_TOL and rel_fro(h[:, b].cpu().numpy(), hb) <= F32_TOL
+    finally:
+        B.grim_gru_destroy(g)
+        for hd in handles:
+            B.grim_bcr_destroy(hd)
+
+
 @pytest.mark.parametrize("grid_kernel", [False, True])
 def test_config2_gru_full(B, grid_kernel):
     check_gru(B, gen.gru_model(), grid_kernel=grid_kernel)
