@@ -481,27 +481,33 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
     float gi_next[3] = {0.f, 0.f, 0.f};
     if (gate_live && t + 1 < p.T)
       for (int g = 0; g < 3; ++g) gi_next[g] = __ldg(p.gi + (int64_t)(t + 1) * 3 * H + g * H + unit);
+    // RI items are multiplied and then reduced together (their exchanges overlap)
+    constexpr int RI = NI * BH == 16 || NI * BH == 32 ? NI : 1;
 #pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      const int item = warp * NI + i;
-      unsigned long long sum[BH / 2];
+    for (int i0 = 0; i0 < NI; i0 += RI) {
+      float acc[RI * BH];
 #pragma unroll
-      for (int r = 0; r < BH / 2; ++r) sum[r] = 0ull;
+      for (int i = 0; i < RI; ++i) {
+        unsigned long long sum[BH / 2];
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        const float xv = hcur[(s & 1) ? col[i][s / 2] >> 16 : col[i][s / 2] & 0xFFFFu];
-        const unsigned long long x2 = walk_pair(xv, xv);
+        for (int r = 0; r < BH / 2; ++r) sum[r] = 0ull;
 #pragma unroll
-        for (int r = 0; r < BH / 2; ++r) walk_ffma2(sum[r], val[i][s][r], x2);
+        for (int s = 0; s < S; ++s) {
+          const uint32_t cw = col[i0 + i][s / 2];
+          const float xv = hcur[(s & 1) ? cw >> 16 : cw & 0xFFFFu];
+          const unsigned long long x2 = walk_pair(xv, xv);
+#pragma unroll
+          for (int r = 0; r < BH / 2; ++r) walk_ffma2(sum[r], val[i0 + i][s][r], x2);
+        }
+#pragma unroll
+        for (int r = 0; r < BH / 2; ++r) {
+          acc[i * BH + 2 * r] = __uint_as_float((unsigned)sum[r]);
+          acc[i * BH + 2 * r + 1] = __uint_as_float((unsigned)(sum[r] >> 32));
+        }
       }
-      float acc[BH];
-#pragma unroll
-      for (int r = 0; r < BH / 2; ++r) {
-        acc[2 * r] = __uint_as_float((unsigned)sum[r]);
-        acc[2 * r + 1] = __uint_as_float((unsigned)(sum[r] >> 32));
-      }
-      warp_reduce_rows<BH>(acc, lane);
-      if (item < nb * ks) part_t[item * BH + warp_row<BH>(lane)] = acc[0];
+      warp_reduce_rows<RI * BH>(acc, lane);
+      const int at = (warp * NI + i0) * BH + warp_row<RI * BH>(lane);
+      if (at < part_len) part_t[at] = acc[0];
     }
     __syncthreads();
     if (gate_live) {
@@ -977,8 +983,9 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
   // state from that buffer while layer l + 2 may already be writing it: such stacks run one layer after the other.
   if (g->pipeline && L > 1 && L <= 3 && (use_reg || use_cluster))
     chunks = g->want_chunks > 0 ? (int)std::min<int64_t>(g->want_chunks, T)
-                                : (int)std::max<int64_t>(1, std::min<int64_t>(3, T / 64));
+                                : (int)std::max<int64_t>(1, std::min<int64_t>(5, T / 40));
   const int64_t clen = ((T + chunks - 1) / chunks + 3) / 4 * 4;  // a multiple of 4: chunk starts stay 16-byte aligned
+  chunks = (int)((T + clen - 1) / clen);  // the rounding may have left the last chunks empty: their events would never be recorded
   const int64_t ldT = (T + 3) / 4 * 4;
   const bool tin = g->transposed_inputs && g->d_xT != nullptr;
   auto stream_of = [&](int l) { return (chunks > 1 && l > 0) ? g->lstream[(size_t)l - 1] : s0; };
