@@ -78,16 +78,21 @@ constexpr int kPix = 128;          // pixels per thread block: the rows of its a
 constexpr int kK = 64;             // k per stage
 constexpr int kABytes = kPix * kK * 2;
 constexpr int kMaxStages = 8;
-constexpr int kEpiWarps = 8;       // two per quarter of the tensor-memory lanes
-constexpr int kThreads = 96 + 32 * kEpiWarps;  // warp 0: pixel copies, 1: tensor core, 2: weight copies, then the epilogue
+constexpr int kEpiWarps = 8;       // of an epilogue group: two per quarter of the tensor-memory lanes
+constexpr int kEpiGroups = 2;      // they take tiles in turn: with few K tiles to a tile, storing it takes as long as multiplying it
+constexpr int kEpi0 = 4;           // warps 0 and 3: pixel copies, 1: tensor core, 2: weight copies, from kEpi0 on the epilogue
+constexpr int kThreads = 32 * (kEpi0 + kEpiWarps * kEpiGroups);
 constexpr int kGatherGroups = 2;   // gathering variant: groups of four warps that build tiles of pixels in turn
 constexpr int kGatherThreads = kThreads + 128 * kGatherGroups;
-constexpr int kHdrBytes = 2048;
+constexpr int kHdrBytes = 4096;
+constexpr int kBiasCap = 512;      // output channels whose biases are kept in shared memory
 
 struct ConvParams {
   unsigned* status;
   int nkt, nstages, npt, nnt;        // K tiles, ring slots, pixel tiles, channel tiles
-  int n_tile, n_stride;              // output channels per tile; tensor-memory columns between the two accumulators
+  int n_tile, n_stride, nacc;        // output channels per tile; tensor-memory columns between accumulators; 2 or 4 of them
+  int resident;                      // the weights of all K tiles stay in shared memory (one tile of output channels)
+  int c_end;                         // a multiple of g past the last channel
   int g, cblocks, nsub;              // channels per copy of input pixels, copies per tap, taps * cblocks
   int M, KH, KW, stride, pad, OH, OW;
   int C, H, W, K;
@@ -176,7 +181,8 @@ __device__ __forceinline__ void store_channels(T* y, int64_t ohw, int n, const f
 // an SM reads per flop.  CG = 1: one block, 128 pixels - smaller tiles for small outputs.
 // A thread block (pair) walks tiles blockIdx, blockIdx + grid, ...; two accumulators, so that storing a tile overlaps
 // the multiplies of the next.
-template <int CG, bool GATHER>
+// GATHER: the tiles of pixels are gathered from the NCHW input (K <= 64).  KPS: K tiles per stage.
+template <int CG, bool GATHER, int KPS>
 __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc_kernel(const __grid_constant__ CUtensorMap tm_in,
                                                                                        const __grid_constant__ CUtensorMap tm_w, const ConvParams p) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -184,24 +190,32 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);   // (even block) the tiles of a stage have landed, both blocks' bytes
   uint64_t* empty = full + kMaxStages;                  // the multiplies of a stage are done
-  uint64_t* acc_full = empty + kMaxStages;              // [2] an accumulator is complete
-  uint64_t* acc_empty = acc_full + 2;                   // [2] (even block) it has been read by all epilogue warps
+  uint64_t* acc_full = empty + kMaxStages;              // [nacc] an accumulator is complete
+  uint64_t* acc_empty = acc_full + 4;                   // [nacc] (even block) it has been read by all warps of its group
+  uint64_t* w_full = acc_empty + 4;                     // resident weights have landed (even block: both blocks' bytes)
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + 384);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + 388);
   int2* s_taps = reinterpret_cast<int2*>(smem + 1024);  // gathering variant: [k] (offset in the input, tap bits)
-  uint8_t* stages = smem + kHdrBytes;
+  float* s_bias = reinterpret_cast<float*>(smem + 2048);
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
   const int b_rows = p.n_tile / CG;
-  const uint32_t stage_bytes = (uint32_t)kABytes + (((uint32_t)b_rows * (kK * 2) + 1023u) & ~1023u);
+  const uint32_t b_tile = ((uint32_t)b_rows * (kK * 2) + 1023u) & ~1023u;
+  const bool resident = p.resident != 0;
+  uint8_t* wbase = smem + kHdrBytes;  // resident weights
+  const int wtiles = (p.nkt + KPS - 1) / KPS * KPS;
+  uint8_t* stages = wbase + (resident ? (uint32_t)wtiles * b_tile : 0u);
+  const uint32_t kt_bytes = (uint32_t)kABytes + (resident ? 0u : b_tile);
+  const uint32_t stage_bytes = kt_bytes * (uint32_t)KPS;
   const bool split = CG == 1 && !GATHER && p.ksplit > 1;
   const uint32_t part = split ? cluster_ctarank() : 0u;  // this block's share of K
   const int kt0 = split ? (int)part * p.kt_per : 0;
   const int ns = p.nstages, nkt = split ? min(p.kt_per, p.nkt - kt0) : p.nkt;
   const int per = split ? p.ksplit : CG;                 // blocks per tile
   const int units = p.npt * p.nnt, u0 = (int)blockIdx.x / per, ustep = (int)gridDim.x / per;
-  const uint32_t tmem_cols = 2u * (uint32_t)p.n_stride;
+  const uint32_t tmem_cols = (uint32_t)(p.nacc * p.n_stride);
+  const int stages_per_tile = (nkt + KPS - 1) / KPS;
 
   if (tid == 32) {
     if (!GATHER) asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_in) : "memory");
@@ -209,17 +223,20 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
   }
   if (tid == 0) {
     for (int s = 0; s < kMaxStages; ++s) {
-      // both copying threads of the even block announce the bytes of their loads; gathering: weights + four warps
-      mbar_init(full + s, GATHER ? 5 : 2);
+      // the copying threads of the even block announce the bytes of their loads; gathering: four warps arrive
+      mbar_init(full + s, (GATHER ? 4 : 1) + (resident ? 0 : 1));
       mbar_init(empty + s, 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 4; ++i) {
       mbar_init(acc_full + i, 1);
       mbar_init(acc_empty + i, kEpiWarps * CG);
     }
+    mbar_init(w_full, 1);
     *s_abort = 0;
     fence_mbar_init();
   }
+  if (p.bias && p.M <= kBiasCap)
+    for (int i = tid; i < kBiasCap; i += (int)blockDim.x) s_bias[i] = i < p.M ? __ldg(p.bias + i) : 0.f;
   if (GATHER && tid >= kThreads && tid < kThreads + kK) {
     // k -> (channel, kh, kw); tap bits: kh in the low half, 16 + kw in the high half (none valid past the last k)
     const int k = tid - kThreads, khw = p.KH * p.KW;
@@ -252,51 +269,75 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
       uint32_t full0 = smem_u32(full);  // the even block's barriers, as seen from this block
       if (CG == 2) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(full0) : "r"(smem_u32(full)), "r"(0));
       const uint32_t st0 = smem_u32(stages) + kABytes, b_bytes = (uint32_t)b_rows * (kK * 2);
-      // ring position: slot, and how often the ring has been gone through (a slot is refilled from the second round on)
-      int slot = 0, round = 0;
-      for (int u = u0; u < units && !failed; u += ustep) {
+      if (resident) {
+        uint32_t wf = smem_u32(w_full);
+        if (CG == 2) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(wf) : "r"(smem_u32(w_full)), "r"(0));
+        if (rank == 0) mbar_arrive_expect_tx(w_full, b_bytes * (uint32_t)(wtiles * CG));  // (tiles past the last are zeros)
+        for (int kt = 0; kt < wtiles; ++kt) load_rows<CG>(smem_u32(wbase) + (uint32_t)kt * b_tile, &tm_w, kt * kK, (int)rank * b_rows, wf);
+      }
+      // ring position: slot, and the parity of its last emptying (a fresh barrier counts as emptied one round before)
+      int slot = 0;
+      unsigned par = 1;
+      for (int u = u0; u < units && !failed && !resident; u += ustep) {
         const int row0 = (u % p.nnt) * p.n_tile + (int)rank * b_rows;
-        for (int kt = 0; kt < nkt; ++kt) {
-          if (round > 0 && !mbar_wait<CG == 2>(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 5; break; }
-          if (rank == 0) mbar_arrive_expect_tx(full + slot, b_bytes * CG);
-          load_rows<CG>(st0 + (uint32_t)slot * stage_bytes, &tm_w, (kt0 + kt) * kK, row0, full0 + (uint32_t)slot * 8u);
-          if (++slot == ns) { slot = 0; ++round; }
+        for (int stg = 0; stg < stages_per_tile; ++stg) {
+          if (!mbar_wait_tight<CG == 2>(empty + slot, par, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 5; break; }
+          if (rank == 0) mbar_arrive_expect_tx(full + slot, b_bytes * (uint32_t)(KPS * CG));
+#pragma unroll
+          for (int j = 0; j < KPS; ++j)
+            load_rows<CG>(st0 + (uint32_t)slot * stage_bytes + (uint32_t)j * kt_bytes, &tm_w, (kt0 + stg * KPS + j) * kK, row0, full0 + (uint32_t)slot * 8u);
+          slot = slot + 1 == ns ? 0 : slot + 1;
+          par ^= slot == 0 ? 1u : 0u;
         }
       }
     }
-  } else if (warp == 0) {
-    // ------------------------------------------------------------------ pixel copies
+  } else if (warp == 0 || warp == 3) {
+    // ------------------------------------------------------------------ pixel copies: two threads take stages in turn
     if (!GATHER && elect_one()) {
       uint32_t full0 = smem_u32(full);
       if (CG == 2) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(full0) : "r"(smem_u32(full)), "r"(0));
       const int ohw = p.OH * p.OW;
       const int subs = kK / p.g;
       const uint32_t st0 = smem_u32(stages), sub_bytes = (uint32_t)(kPix * p.g * 2);
-      int slot = 0, round = 0;
+      const int cut = KPS * subs;    // copies per stage
+      int slot = warp == 0 ? 0 : 1, skip = slot;  // this thread's first stage, and how many of the next tile's come before it
+      unsigned par = 1;
       for (int u = u0; u < units && !failed; u += ustep) {
-        const int pt = u / p.nnt;
-        const int64_t px = ((int64_t)pt * CG + rank) * kPix;  // first pixel of this block
-        const int img = (int)(px / ohw);
-        const int rest = (int)(px - (int64_t)img * ohw);
+        const int px = ((u / p.nnt) * CG + (int)rank) * kPix;  // first pixel of this block
+        const int img = px / ohw, rest = px - img * ohw;
         const int oh = rest / p.OW, ow = rest - oh * p.OW;
         const int w0 = ow * p.stride - p.pad, h0 = oh * p.stride - p.pad;
-        const int sub0 = kt0 * subs, tap0 = sub0 / p.cblocks;
-        int tap_h = tap0 / p.KW, tap_w = tap0 - tap_h * p.KW, cb = sub0 - tap0 * p.cblocks, left = p.nsub - sub0;
-        for (int kt = 0; kt < nkt; ++kt) {
-          if (round > 0 && !mbar_wait<CG == 2>(empty + slot, (unsigned)(round - 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
+        const int sub = kt0 * subs + skip * cut, tap = sub / p.cblocks;
+        int cb = sub - tap * p.cblocks, tap_h = tap / p.KW, tap_w = tap - tap_h * p.KW;
+        auto advance = [&]() {  // the next copy's channels and kernel position
+          const bool wc = cb + 1 == p.cblocks;
+          cb = wc ? 0 : cb + 1;
+          tap_w += wc ? 1 : 0;
+          const bool ww = tap_w == p.KW;
+          tap_w = ww ? 0 : tap_w;
+          tap_h += ww ? 1 : 0;
+        };
+        int stg = skip;
+        for (; stg < stages_per_tile; stg += 2) {
+          if (!mbar_wait_tight<CG == 2>(empty + slot, par, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
           const uint32_t st = st0 + (uint32_t)slot * stage_bytes, bar = full0 + (uint32_t)slot * 8u;
-          const int nsub = left < subs ? left : subs;  // copies of input pixels in this stage
-          if (rank == 0) mbar_arrive_expect_tx(full + slot, sub_bytes * (uint32_t)nsub * CG);
-          for (int i = 0; i < nsub; ++i) {
-            load_im2col<CG>(st + (uint32_t)i * sub_bytes, &tm_in, cb * p.g, w0, h0, img, (unsigned short)tap_w, (unsigned short)tap_h, bar);
-            if (++cb == p.cblocks) {
-              cb = 0;
-              if (++tap_w == p.KW) { tap_w = 0; ++tap_h; }
+          if (rank == 0) mbar_arrive_expect_tx(full + slot, sub_bytes * (uint32_t)(cut * CG));
+#pragma unroll
+          for (int j = 0; j < KPS; ++j)
+            for (int i = 0; i < subs; ++i) {
+              // a stage is always filled: copies past the last kernel position take channels that do not exist (zeros)
+              const bool past = tap_h >= p.KH;
+              load_im2col<CG>(st + (uint32_t)j * kt_bytes + (uint32_t)i * sub_bytes, &tm_in, past ? p.c_end : cb * p.g, w0, h0, img,
+                              (unsigned short)(past ? 0 : tap_w), (unsigned short)(past ? 0 : tap_h), bar);
+              advance();
             }
-          }
-          left -= nsub;
-          if (++slot == ns) { slot = 0; ++round; }
+          for (int i = 0; i < cut; ++i) advance();
+          slot += 2;
+          const bool wrap = slot >= ns;
+          slot -= wrap ? ns : 0;
+          par ^= wrap ? 1u : 0u;
         }
+        skip = stg - stages_per_tile;
       }
     }
   } else if (warp == 1) {
@@ -305,70 +346,78 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
       // fp32 accumulate, bf16 x bf16, both operands K-major, M = 128 pixels per block, N = n_tile channels
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.n_tile >> 3) << 17) | ((uint32_t)((kPix * CG) >> 4) << 24);
       const int row_bytes = p.g * 2, sub_shift = p.g == 64 ? 2 : (p.g == 32 ? 1 : 0);  // 16-wide k steps per copy: 4, 2, 1
-      const uint64_t ad0 = k_major_desc(smem_u32(stages), row_bytes), bd0 = k_major_desc(smem_u32(stages) + kABytes, 128);
-      uint32_t step[kK / 16];  // where the k steps of a stage start in the tile of pixels, in 16-byte units
+      const uint64_t ad0 = k_major_desc(smem_u32(stages), row_bytes), bd0 = k_major_desc(resident ? smem_u32(wbase) : smem_u32(stages) + kABytes, 128);
+      uint32_t step[kK / 16];  // where the k steps of a K tile start in the tile of pixels, in 16-byte units
 #pragma unroll
       for (int s = 0; s < kK / 16; ++s) {
         const int sub = s >> sub_shift, in_sub = s - (sub << sub_shift);
         step[s] = (uint32_t)(sub * (kPix * row_bytes) + in_sub * 32) >> 4;
       }
       int slot = 0, tile = 0;
-      unsigned round = 0;
+      unsigned par = 0;
+      if (resident && !mbar_wait<CG == 2>(w_full, 0, p.spin_limit << 2, s_abort, 0)) failed = true, fail_site = 7;
+      const uint32_t stage16 = stage_bytes >> 4, kt16 = kt_bytes >> 4;
+      const uint32_t bstep = resident ? b_tile >> 4 : kt16;  // resident weights have places of their own
+      const unsigned limit = p.spin_limit << 2;
+      const int nacc = p.nacc, n_stride = p.n_stride;
       for (int u = u0; u < units && !failed; u += ustep, ++tile) {
-        const int acc = tile & 1;
-        if (tile >= 2 && !mbar_wait<CG == 2>(acc_empty + acc, (unsigned)((tile / 2 - 1) & 1), p.spin_limit << 2, s_abort, 0)) { failed = true, fail_site = 2; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem_base + (uint32_t)acc * (uint32_t)p.n_stride;
-        int left = GATHER ? (p.K + 15) >> 4 : (p.nsub << sub_shift) - kt0 * (kK / 16);  // k steps that exist
-        for (int kt = 0; kt < nkt; ++kt) {
-          if (!mbar_wait<CG == 2>(full + slot, round & 1u, p.spin_limit << 2, s_abort, 0)) { failed = true, fail_site = 3; break; }
+        const int acc = tile & (nacc - 1), use = tile / nacc;
+        if (!mbar_wait_tight<CG == 2>(acc_empty + acc, (unsigned)(use + 1) & 1u, limit, s_abort)) { failed = true, fail_site = 2; break; }
+        const uint32_t d = tmem_base + (uint32_t)(acc * n_stride);
+        uint32_t more = 0u, wk = 0u;
+        for (int stg = 0; stg < stages_per_tile; ++stg) {
+          if (!mbar_wait_tight<CG == 2>(full + slot, par, limit, s_abort)) { failed = true, fail_site = 3; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t off = ((uint32_t)slot * stage_bytes) >> 4;  // (the address field of a descriptor never carries: 227 KB < 2^18)
-          if (left >= kK / 16) {
+          const uint32_t off = (uint32_t)slot * stage16;  // (the address field of a descriptor never carries: 227 KB < 2^18)
+          const uint32_t boff = resident ? wk : off;
 #pragma unroll
-            for (int s = 0; s < kK / 16; ++s) mma_bf16<CG>(d, ad0 + off + step[s], bd0 + off + 2u * s, idesc, (kt > 0 || s > 0) ? 1u : 0u);
-          } else {
+          for (int j = 0; j < KPS; ++j)
 #pragma unroll
-            for (int s = 0; s < kK / 16; ++s)
-              if (s < left) mma_bf16<CG>(d, ad0 + off + step[s], bd0 + off + 2u * s, idesc, (kt > 0 || s > 0) ? 1u : 0u);
-          }
-          left -= kK / 16;
+            for (int s = 0; s < (GATHER ? 4 : kK / 16); ++s)
+              mma_bf16<CG>(d, ad0 + (off + (uint32_t)j * kt16 + step[s]), bd0 + (boff + (uint32_t)j * bstep + 2u * s), idesc, j + s > 0 ? 1u : more);
           mma_commit<CG>(empty + slot);
-          if (++slot == ns) { slot = 0; ++round; }
+          more = 1u;
+          wk += KPS * bstep;
+          slot = slot + 1 == ns ? 0 : slot + 1;
+          par ^= slot == 0 ? 1u : 0u;
         }
         if (!failed) mma_commit<CG>(acc_full + acc);
       }
     }
-  } else if (GATHER && warp >= 3 + kEpiWarps) {
+  } else if (GATHER && warp >= kEpi0 + kEpiWarps * kEpiGroups) {
     // ------------------------------------------------------------------ gathering variant: a thread builds one pixel's row
-    const int grp = (warp - 3 - kEpiWarps) >> 2, bt = (tid - kThreads) & 127;
-    const int pieces = 2 * ((p.K + 15) >> 4);  // 16-byte pieces of a row that the multiplies read
+    const int grp = (warp - kEpi0 - kEpiWarps * kEpiGroups) >> 2, bt = (tid - kThreads) & 127;
+    const int pieces = (p.K + 7) >> 3;  // 16-byte pieces of a row that hold something
     const unsigned short* X = reinterpret_cast<const unsigned short*>(p.X);
-    const int64_t ohw = (int64_t)p.OH * p.OW;
+    const int ohw = p.OH * p.OW;
     int it = grp;
     for (int u = u0 + grp * ustep; u < units; u += kGatherGroups * ustep, it += kGatherGroups) {
       const int slot = it % ns;
       if (it >= ns && !__all_sync(0xffffffffu, mbar_wait(empty + slot, (unsigned)((it / ns - 1) & 1), p.spin_limit, s_abort, 32))) { failed = true, fail_site = 6; break; }
-      const int64_t q = (int64_t)(u / p.nnt) * kPix + bt;
-      const bool ok = q < p.npix;
-      const int64_t img = ok ? q / ohw : 0;
-      const int pix = ok ? (int)(q - img * ohw) : 0;
+      const int q = (u / p.nnt) * kPix + bt;
+      const bool ok = q < (int)p.npix;
+      const int img = ok ? q / ohw : 0, pix = ok ? q - img * ohw : 0;
       const int oh = pix / p.OW, ow = pix - oh * p.OW;
       const int h0 = oh * p.stride - p.pad, w0 = ow * p.stride - p.pad;
       uint32_t in = 0;  // bit kh: row inside; bit 16 + kw: column inside
-      if (ok) {
-        for (int t = 0; t < p.KH; ++t) in |= (uint32_t)(h0 + t >= 0 && h0 + t < p.H) << t;
-        for (int t = 0; t < p.KW; ++t) in |= (uint32_t)(w0 + t >= 0 && w0 + t < p.W) << (16 + t);
-      }
-      const unsigned short* src = X + (img * p.C * p.H + h0) * p.W + w0;  // only dereferenced where a tap is inside
+      for (int t = 0; t < p.KH; ++t) in |= (uint32_t)(ok && h0 + t >= 0 && h0 + t < p.H) << t;
+      for (int t = 0; t < p.KW; ++t) in |= (uint32_t)(w0 + t >= 0 && w0 + t < p.W) << (16 + t);
+      const int64_t base = ((int64_t)img * p.C * p.H + h0) * p.W + w0;
       const uint32_t row = smem_u32(stages) + (uint32_t)slot * stage_bytes + (uint32_t)bt * 128u;
-      for (int pc = 0; pc < pieces; ++pc) {
+#pragma unroll 2
+      for (int pc = 0; pc < 8; ++pc) {
         uint32_t v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int2 t = s_taps[pc * 8 + e];
-          v[e] = 0u;
-          if ((in & (uint32_t)t.y) == (uint32_t)t.y) v[e] = __ldg(src + t.x);
+        for (int e = 0; e < 8; ++e) v[e] = 0u;
+        if (pc < pieces) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            // (selected, not skipped: a branch per element costs more than the load)
+            const int2 t = s_taps[pc * 8 + e];
+            const bool inside = (in & (uint32_t)t.y) == (uint32_t)t.y;
+            const uint32_t x = __ldg(X + (inside ? base + t.x : 0));
+            v[e] = inside ? x : 0u;
+          }
         }
         sts128(row + (((uint32_t)pc ^ ((uint32_t)bt & 7u)) << 4), v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
       }
@@ -389,10 +438,11 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
         else mbar_arrive_remote(acc_empty + acc, 0);
       }
     };
-    int tile = 0;
-    for (int u = u0; u < units; u += ustep, ++tile) {
-      const int acc = tile & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(acc_full + acc, (unsigned)((tile / 2) & 1), p.spin_limit << 2, s_abort, 64))) { failed = true, fail_site = 4; break; }
+    const int egrp = (warp - kEpi0) / kEpiWarps, ewarp = (warp - kEpi0) % kEpiWarps;
+    int tile = egrp;
+    for (int u = u0 + egrp * ustep; u < units; u += kEpiGroups * ustep, tile += kEpiGroups) {
+      const int acc = tile & (p.nacc - 1);
+      if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(acc_full + acc, (unsigned)(tile / p.nacc) & 1u, p.spin_limit << 2, s_abort, 32))) { failed = true, fail_site = 4; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (split) break;  // one tile per cluster; the shares meet below
       const int pt = u / p.nnt, nt = u - pt * p.nnt;
@@ -405,42 +455,60 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
       // Two neighbouring pixels per store where planes have an even size (then pixels 2i and 2i + 1 share an image): lanes
       // exchange halves so that even lanes hold both pixels of one channel and odd lanes of the next.
       const bool pairs = p.y_bf16 && (ohw & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 3) == 0;
-      const int cb0 = ((warp - 3) >> 2) * 32;  // the two warps of a quarter take 32 channels in turn
+      const int cb0 = (ewarp >> 2) * 32;  // the two warps of a quarter take 32 channels in turn
       for (int cb = cb0; cb < nch; cb += 64) {
         uint32_t v[32];
         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * p.n_stride + cb), v);
         if (cb + 64 >= nch) release(acc);
         const int n = nch - cb < 32 ? nch - cb : 32;
-        // lane i fetches the bias of channel i of this piece
-        const float bl = (p.bias && lane < n) ? __ldg(p.bias + ch0 + cb + lane) : 0.f;
         float t[32];
+        if (p.bias && p.M <= kBiasCap) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          t[i] = __uint_as_float(v[i]) + __shfl_sync(0xffffffffu, bl, i);
-          if (p.relu) t[i] = fmaxf(t[i], 0.f);
+          for (int i = 0; i < 32; i += 4) {
+            // (ranges of channels start at multiples of 16; what is read past the last one is not stored)
+            const float4 bv = *reinterpret_cast<const float4*>(s_bias + ((ch0 + cb + i) & (kBiasCap - 1)));
+            t[i] = __uint_as_float(v[i]) + bv.x;
+            t[i + 1] = __uint_as_float(v[i + 1]) + bv.y;
+            t[i + 2] = __uint_as_float(v[i + 2]) + bv.z;
+            t[i + 3] = __uint_as_float(v[i + 3]) + bv.w;
+          }
+        } else if (p.bias) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) t[i] = __uint_as_float(v[i]) + (i < n ? __ldg(p.bias + ch0 + cb + i) : 0.f);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) t[i] = __uint_as_float(v[i]);
         }
         if (pairs) {
+          // rounded channel by channel pair, activation on pairs, then one exchange and one byte permutation per pair
+          const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;
           uint32_t w[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            const float other = __shfl_xor_sync(0xffffffffu, (lane & 1) ? t[2 * i] : t[2 * i + 1], 1);
-            const __nv_bfloat162 h = (lane & 1) ? __floats2bfloat162_rn(other, t[2 * i + 1]) : __floats2bfloat162_rn(t[2 * i], other);
-            w[i] = *reinterpret_cast<const uint32_t*>(&h);
+            __nv_bfloat162 h = __floats2bfloat162_rn(t[2 * i], t[2 * i + 1]);
+            if (p.relu) h = __hmax2(h, __floats2bfloat162_rn(0.f, 0.f));
+            const uint32_t own = *reinterpret_cast<const uint32_t*>(&h);
+            w[i] = __byte_perm(own, __shfl_xor_sync(0xffffffffu, own, 1), sel);
           }
           if (ok) {
             __nv_bfloat16* y = static_cast<__nv_bfloat16*>(p.Y) + base - (lane & 1) + (cb + (lane & 1)) * ohw;
             if (n == 32) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) *reinterpret_cast<uint32_t*>(y + 2 * i * ohw) = w[i];
+              for (int i = 0; i < 16; ++i, y += 2 * ohw) *reinterpret_cast<uint32_t*>(y) = w[i];
             } else {
 #pragma unroll
-              for (int i = 0; i < 16; ++i)
-                if (2 * i + (lane & 1) < n) *reinterpret_cast<uint32_t*>(y + 2 * i * ohw) = w[i];
+              for (int i = 0; i < 16; ++i, y += 2 * ohw)
+                if (2 * i + (lane & 1) < n) *reinterpret_cast<uint32_t*>(y) = w[i];
             }
           }
-        } else if (ok) {
-          if (p.y_bf16) store_channels(static_cast<__nv_bfloat16*>(p.Y) + base + cb * ohw, ohw, n, t);
-          else store_channels(static_cast<float*>(p.Y) + base + cb * ohw, ohw, n, t);
+        } else {
+          if (p.relu)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) t[i] = fmaxf(t[i], 0.f);
+          if (ok) {
+            if (p.y_bf16) store_channels(static_cast<__nv_bfloat16*>(p.Y) + base + cb * ohw, ohw, n, t);
+            else store_channels(static_cast<float*>(p.Y) + base + cb * ohw, ohw, n, t);
+          }
         }
       }
       if (cb0 >= nch) release(acc);  // nothing of this tile for this warp
@@ -457,11 +525,11 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
     __syncwarp();
     cluster_sync_all();
     const int nc = p.n_tile / p.ksplit;
-    const bool epi = warp >= 3;
+    const bool epi = warp >= kEpi0 && warp < kEpi0 + kEpiWarps;
     if (epi) {
       const int quarter = warp & 3;
       const uint32_t dst = smem_u32(stages) + ((uint32_t)part * (uint32_t)nc * kPix + (uint32_t)(quarter * 32 + lane)) * 4u;
-      for (int cb = ((warp - 3) >> 2) * 32; cb < p.n_tile; cb += 64) {
+      for (int cb = ((warp - kEpi0) >> 2) * 32; cb < p.n_tile; cb += 64) {
         uint32_t v[32];
         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)cb, v);
 #pragma unroll
@@ -478,7 +546,7 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
     if (epi) {
       const float* sums = reinterpret_cast<const float*>(stages);
       const int pt = u0 / p.nnt, nt = u0 - pt * p.nnt;
-      const int t = tid - 96, pl = t & (kPix - 1);
+      const int t = tid - 32 * kEpi0, pl = t & (kPix - 1);
       const int64_t px = (int64_t)pt * kPix + pl, ohw = (int64_t)p.OH * p.OW;
       if (px < p.npix) {
         const int64_t img = px / ohw, pix = px - img * ohw;
@@ -556,6 +624,7 @@ bool shape_plan(ConvPlan& pl, int nkt, int64_t npix, int64_t M, int sms) {
   if (npt * pl.nnt > (int64_t(1) << 30)) return false;
   pl.npt = (int)npt;
   pl.kt_per = (nkt + pl.ksplit - 1) / pl.ksplit;
+  if (pl.ksplit > 1) pl.kt_per = (pl.kt_per + 1) / 2 * 2;  // whole stages
   if (pl.ksplit > 1) {
     // one tile per cluster, every block with something to multiply; the sums have to fit the stages
     if (pl.cg != 1 || (pl.ksplit - 1) * pl.kt_per >= nkt || pl.n_tile % 32 || pl.n_tile % pl.ksplit) return false;
@@ -637,16 +706,25 @@ grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
   ConvParams p;
   p.status = h->d_status;
   p.nkt = l.nkt; p.npt = pl.npt; p.nnt = pl.nnt; p.n_tile = pl.n_tile; p.ksplit = pl.ksplit; p.kt_per = pl.kt_per;
+  p.nacc = pl.n_tile <= 128 ? 4 : 2;
   p.n_stride = pl.n_tile <= 32 ? 32 : (pl.n_tile <= 64 ? 64 : (pl.n_tile <= 128 ? 128 : 256));
   p.g = l.g; p.cblocks = l.cblocks; p.nsub = l.taps * l.cblocks;
   p.M = (int)h->M; p.KH = a.KH; p.KW = a.KW; p.stride = a.stride; p.pad = a.pad; p.OH = a.OH; p.OW = a.OW;
+  p.c_end = (a.C + l.g - 1) / l.g * l.g;
   p.C = a.C; p.H = a.H; p.W = a.W; p.K = (int)h->K;
   p.npix = a.ncols; p.spin_limit = 1u << 20; p.X = static_cast<const __nv_bfloat16*>(a.X); p.bias = a.bias; p.Y = a.Y;
   p.y_bf16 = a.y_dtype == GRIM_BF16; p.relu = a.relu;
   const int b_rows = pl.n_tile / pl.cg;
-  const size_t stage = kABytes + (((size_t)b_rows * kK * 2 + 1023) & ~size_t(1023));
-  p.nstages = (int)std::min<size_t>(kMaxStages, (227 * 1024 - 1024 - kHdrBytes) / stage);
-  const size_t smem = 1024 + kHdrBytes + p.nstages * stage;
+  // Handing a stage over costs the threads on both sides more than the multiplies of a K tile of up to 128 channels take: two
+  // K tiles then share a stage.
+  const int kps = !gather && pl.n_tile <= 128 && pl.kt_per > 1 ? 2 : 1;
+  const size_t b_tile = ((size_t)b_rows * kK * 2 + 1023) & ~size_t(1023);
+  // a single tile of output channels with a short K: its weights are loaded once per thread block, not once per pixel tile
+  const size_t weights = b_tile * ((l.nkt + kps - 1) / kps * kps);
+  p.resident = pl.nnt == 1 && pl.ksplit == 1 && weights <= 80 * 1024;
+  const size_t fixed = 1024 + kHdrBytes + (p.resident ? weights : 0), stage = (kABytes + (p.resident ? 0 : b_tile)) * kps;
+  p.nstages = (int)std::min<size_t>(kMaxStages, (227 * 1024 - fixed) / stage);
+  const size_t smem = fixed + p.nstages * stage;
 
   CUtensorMap tin, tw;
   memset(&tin, 0, sizeof(tin));
@@ -675,7 +753,9 @@ grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
     count_launch();
     if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
   }
-  auto kern = gather ? conv_tc_kernel<1, true> : (pl.cg == 2 ? conv_tc_kernel<2, false> : conv_tc_kernel<1, false>);
+  auto kern = gather ? conv_tc_kernel<1, true, 1>
+                     : (kps == 2 ? (pl.cg == 2 ? conv_tc_kernel<2, false, 2> : conv_tc_kernel<1, false, 2>)
+                                 : (pl.cg == 2 ? conv_tc_kernel<2, false, 1> : conv_tc_kernel<1, false, 1>));
   if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem) != cudaSuccess) return GRIM_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)pl.grid);

@@ -95,6 +95,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsign
   }
   return false;
 }
+// The same for the loops of single issuing threads: no branch but the one that is not taken when the phase is complete.  A
+// branch costs such a thread some 50 cycles, and its loop is what a pipeline of small tiles waits for.
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait_tight(uint64_t* bar, unsigned parity, unsigned limit, const volatile int* abort_flag,
+                                                unsigned sleep_ns = 0) {
+  if (__builtin_expect(CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity), 1)) return true;
+  return mbar_wait<CLUSTER>(bar, parity, limit, abort_flag, sleep_ns);
+}
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
