@@ -79,11 +79,14 @@ constexpr int kK = 64;             // k per stage
 constexpr int kABytes = kPix * kK * 2;
 constexpr int kMaxStages = 8;
 constexpr int kEpiWarps = 8;       // of an epilogue group: two per quarter of the tensor-memory lanes
-constexpr int kEpiGroups = 2;      // they take tiles in turn: with few K tiles to a tile, storing it takes as long as multiplying it
+// Epilogue groups take tiles in turn: with few K tiles to a tile, storing it takes as long as multiplying it.  (Gathering, the
+// warps are needed to build tiles.)
+__host__ __device__ constexpr int epi_groups(bool gather) { return gather ? 1 : 2; }
 constexpr int kEpi0 = 4;           // warps 0 and 3: pixel copies, 1: tensor core, 2: weight copies, from kEpi0 on the epilogue
-constexpr int kThreads = 32 * (kEpi0 + kEpiWarps * kEpiGroups);
-constexpr int kGatherGroups = 2;   // gathering variant: groups of four warps that build tiles of pixels in turn
-constexpr int kGatherThreads = kThreads + 128 * kGatherGroups;
+constexpr int kThreads = 32 * (kEpi0 + kEpiWarps * epi_groups(false));
+constexpr int kGatherGroups = 4;   // gathering variant: groups of four warps that build tiles of pixels in turn
+constexpr int kGather0 = kEpi0 + kEpiWarps * epi_groups(true);  // their first warp
+constexpr int kGatherThreads = 32 * kGather0 + 128 * kGatherGroups;
 constexpr int kHdrBytes = 4096;
 constexpr int kBiasCap = 512;      // output channels whose biases are kept in shared memory
 
@@ -237,9 +240,9 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
   }
   if (p.bias && p.M <= kBiasCap)
     for (int i = tid; i < kBiasCap; i += (int)blockDim.x) s_bias[i] = i < p.M ? __ldg(p.bias + i) : 0.f;
-  if (GATHER && tid >= kThreads && tid < kThreads + kK) {
+  if (GATHER && tid >= 32 * kGather0 && tid < 32 * kGather0 + kK) {
     // k -> (channel, kh, kw); tap bits: kh in the low half, 16 + kw in the high half (none valid past the last k)
-    const int k = tid - kThreads, khw = p.KH * p.KW;
+    const int k = tid - 32 * kGather0, khw = p.KH * p.KW;
     const int c = k / khw, rest = k - c * khw, kh = rest / p.KW, kw = rest - kh * p.KW;
     s_taps[k] = k < p.K ? make_int2((c * p.H + kh) * p.W + kw, (int)((1u << kh) | (1u << (16 + kw)))) : make_int2(0, -1);
   }
@@ -384,9 +387,9 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
         if (!failed) mma_commit<CG>(acc_full + acc);
       }
     }
-  } else if (GATHER && warp >= kEpi0 + kEpiWarps * kEpiGroups) {
+  } else if (GATHER && warp >= kGather0) {
     // ------------------------------------------------------------------ gathering variant: a thread builds one pixel's row
-    const int grp = (warp - kEpi0 - kEpiWarps * kEpiGroups) >> 2, bt = (tid - kThreads) & 127;
+    const int grp = (warp - kGather0) >> 2, bt = (tid - 32 * kGather0) & 127;
     const int pieces = (p.K + 7) >> 3;  // 16-byte pieces of a row that hold something
     const unsigned short* X = reinterpret_cast<const unsigned short*>(p.X);
     const int ohw = p.OH * p.OW;
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
     };
     const int egrp = (warp - kEpi0) / kEpiWarps, ewarp = (warp - kEpi0) % kEpiWarps;
     int tile = egrp;
-    for (int u = u0 + egrp * ustep; u < units; u += kEpiGroups * ustep, tile += kEpiGroups) {
+    for (int u = u0 + egrp * ustep; u < units; u += epi_groups(GATHER) * ustep, tile += epi_groups(GATHER)) {
       const int acc = tile & (p.nacc - 1);
       if (!__all_sync(0xffffffffu, mbar_wait<CG == 2>(acc_full + acc, (unsigned)(tile / p.nacc) & 1u, p.spin_limit << 2, s_abort, 32))) { failed = true, fail_site = 4; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
