@@ -15,8 +15,8 @@
 // not of FMA units.  With two pieces per lane the slab addresses, the weight loads and the row tests of a block are
 // shared by twice the FMAs (measured 17 % faster than one piece; two bands per warp buy nothing).  Accumulator
 // registers are indexed statically: the rows of the band are walked in order with one warp-uniform test of the
-// block's row mask each.  Grids that would leave most SMs idle are split over block columns (partial sums added
-// into a zeroed Y).
+// block's row mask each.  Tiles that would leave SMs idle in the last round are shared by the blocks of a cluster, each
+// multiplying a part of the block columns; the sums meet over distributed shared memory.
 //
 // Narrow tile (N <= 16): a lane owns one output column and the two halves of a warp split the kept columns of a
 // chunk; the stages are small, so the ring is deeper (8 slots, 6 in flight) and two thread blocks share an SM.
@@ -43,6 +43,7 @@ constexpr int kAhead = 2;         // stages requested ahead of the one being mul
 constexpr int kNarrowStages = 8;
 constexpr int kNarrowAhead = 6;
 constexpr int kMaxRing = 8;
+constexpr int kMaxSplit = 8;     // blocks of a cluster that share a tile
 constexpr int kJlistCap = 2048;   // block columns per matrix the stage list can hold
 constexpr int kHdrBytes = (192 + kMaxRing * 16 + kJlistCap * 2 + 127) / 128 * 128;  // barriers, flags, per-slot blob sizes, stage list
 
@@ -57,7 +58,10 @@ struct FParams {
   uint32_t blob_stride, slab_bytes;
   unsigned spin_limit;
   int slab_ld;  // floats between slab rows: kTN, or kTN + 4 when the gather writes down the columns (X stored q-major)
-  int ksplit;  // > 1: blockIdx.z takes a share of the block columns and adds its partial sums into a zeroed Y
+  int qtiles;  // tiles across the output columns; tile t covers columns tile t % qtiles and band groups t / qtiles
+  int tile0;   // the launch's first tile
+  int split;   // > 1: the blocks of a cluster share a tile, each multiplies a part of the block columns
+  int first_of_two, second_of_two;  // this multiply is two launches: whole tiles, then the split ones
   SpmmArgs a;
 };
 
@@ -133,8 +137,8 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
   uint64_t* empty = full + kMaxRing;
   // the launch that follows in the stream may start as SMs free up: it waits (griddepcontrol.wait) before it reads or
-  // writes anything this launch touches
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // writes anything this launch touches.  (Two launches for one multiply: below)
+  if (!p.first_of_two) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + 128);
   int* s_nst = reinterpret_cast<int*>(smem + 132);
   uint32_t* s_meta = reinterpret_cast<uint32_t*>(smem + 192);               // [ring slot][4] blob bytes per band group
@@ -148,8 +152,11 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   // in every lane: branches on the band's header and row mask then need no divergence handling
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const SpmmArgs& a = p.a;
-  const int64_t q0 = (int64_t)blockIdx.x * TN;
-  const int g0 = blockIdx.y * BPW;
+  const int split = p.split;
+  const int part = split > 1 ? (int)cluster_ctarank() : 0;
+  const int tile = p.tile0 + (int)blockIdx.x / split;
+  const int64_t q0 = (int64_t)(tile % p.qtiles) * TN;
+  const int g0 = tile / p.qtiles * BPW;
 
   if (warp == 0) {
     int n = 0;
@@ -176,10 +183,14 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   __syncthreads();
   // (programmatic dependent launch) whatever earlier launches in the stream wrote - X, a cleared scratch or Y - is
   // complete and visible from here on; up to here only the packed matrix and this block's own shared memory were touched
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Two launches for one multiply: the first lets the second start only after its own wait, so whatever both read is
+  // there when the second starts; that one waits for the first at its end instead, which keeps its blocks at work while
+  // the first one's last blocks finish, and still makes its completion mean that both are done.
+  if (!p.second_of_two) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.first_of_two) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // with a split over block columns this thread block multiplies only its share of the stage list
   const int nst_all = *s_nst;
-  const int n_lo = (int)((int64_t)blockIdx.z * nst_all / p.ksplit), n_hi = (int)((int64_t)(blockIdx.z + 1) * nst_all / p.ksplit);
+  const int n_lo = (int)((int64_t)part * nst_all / split), n_hi = (int)((int64_t)(part + 1) * nst_all / split);
   const int nst = n_hi - n_lo;
   jlist += n_lo;
 
@@ -322,14 +333,12 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
       if (s_meta[slot * 4 + b] == 0) continue;
       const uint8_t* blob = base + p.slab_bytes + b * p.blob_stride;
       const uint32_t hdr = __shfl_sync(0xffffffffu, reinterpret_cast<const uint32_t*>(blob)[warp], 0);
-      const int kr = (hdr >> 16) & 0xFF, nch = hdr >> 24;
+      const int kr = (hdr >> 16) & 0xFF, nhalf4 = hdr >> 24, nch = (nhalf4 + 1) >> 1;
       if (kr == 0) continue;
       const uint8_t* rec = blob + (hdr & 0xFFFFu) * 16;
       const unsigned rm = __shfl_sync(0xffffffffu, *reinterpret_cast<const unsigned*>(rec), 0);  // kept rows of this block
       const uint8_t* cols = rec + 8;
       const float4* wp = reinterpret_cast<const float4*>(rec + ((8 + nch * kRcChunk + 15) & ~15));
-      // The slab rows of KS kept columns are held in registers at a time: all eight of a chunk for one piece per
-      // lane, four when a lane owns two pieces (the registers go to the accumulators instead).
       if constexpr (NARROW) {
         const float4* wq0 = wp + nhalf;
         for (int ch = 0; ch < nch; ++ch) {
@@ -354,44 +363,61 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
         }
         continue;
       }
+      // The slab rows of KS kept columns are held in registers at a time: all eight of a chunk for one piece per lane, four
+      // when a lane owns two pieces (the registers go to the accumulators instead; the second half of a last chunk is then
+      // skipped where it is all padding).
       constexpr int KS = kRcChunk / (NARROW ? 1 : CW);
-      for (int ch = 0; ch < nch; ++ch) {
-        const uint2 cc = *reinterpret_cast<const uint2*>(cols + ch * kRcChunk);
+      auto multiply = [&](uint32_t c0, uint32_t c1, const float4* wq) {
+        const uint32_t cc[2] = {c0, c1};
+        // the next row's weights are requested while a row is multiplied, except in the variant that has no registers left
+        // (8192 x 8192, 16 x 64, N = 1024: 602 -> 567 us; 8 x 32 with two pieces 727 -> 752)
+        constexpr bool AHEAD = !(BH == 8 && CW == 2);
+        float4 wn[KS / 4];
+        if (AHEAD) {
 #pragma unroll
-        for (int hs = 0; hs < kRcChunk / KS; ++hs) {
-          ulonglong2 x[KS][NARROW ? 1 : CW];
+          for (int g = 0; g < KS / 4; ++g) wn[g] = wq[g];
+        }
+        ulonglong2 x[KS][NARROW ? 1 : CW];
 #pragma unroll
-          for (int e = 0; e < KS; ++e) {
-            const int idx = hs * KS + e;
-            const unsigned col = ((idx < 4 ? cc.x : cc.y) >> (8 * (idx & 3))) & 0xFFu;
+        for (int e = 0; e < KS; ++e)
 #pragma unroll
-            for (int c = 0; c < CW; ++c) x[e][c] = ld_x4(slab + c * kTN, col, lane4, sld);
-          }
-          // one test per row of the band; a kept row owns the next eight weights of the chunk
-          const float4* wq = wp;
+          for (int c = 0; c < CW; ++c) x[e][c] = ld_x4(slab + c * kTN, (cc[e / 4] >> (8 * (e & 3))) & 0xFFu, lane4, sld);
+        // one test per row of the band; a kept row owns the next eight weights of the chunk
 #pragma unroll
-          for (int r = 0; r < BH; ++r) {
-            if ((rm >> r) & 1u) {
+        for (int r = 0; r < BH; ++r) {
+          if ((rm >> r) & 1u) {
+            float4 wc[KS / 4];
 #pragma unroll
-              for (int g = 0; g < KS / 4; ++g) {
-                const float4 w = wq[KS == kRcChunk ? g : hs];
-                const float wv[4] = {w.x, w.y, w.z, w.w};
+            for (int g = 0; g < KS / 4; ++g) wc[g] = AHEAD ? wn[g] : wq[g];
+            wq += 2;
+            if (AHEAD) {  // (past the last row it stays inside the ring and its slack)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const unsigned long long w2 = dup2(wv[j]);
+              for (int g = 0; g < KS / 4; ++g) wn[g] = wq[g];
+            }
 #pragma unroll
-                  for (int c = 0; c < CW; ++c) {
-                    ffma2(acc[b][r][2 * c], w2, x[4 * g + j][c].x);
-                    ffma2(acc[b][r][2 * c + 1], w2, x[4 * g + j][c].y);
-                  }
+            for (int g = 0; g < KS / 4; ++g) {
+              const float wv[4] = {wc[g].x, wc[g].y, wc[g].z, wc[g].w};
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const unsigned long long w2 = dup2(wv[j]);
+#pragma unroll
+                for (int c = 0; c < CW; ++c) {
+                  ffma2(acc[b][r][2 * c], w2, x[4 * g + j][c].x);
+                  ffma2(acc[b][r][2 * c + 1], w2, x[4 * g + j][c].y);
                 }
               }
-              wq += 2;
             }
           }
         }
+      };
+      for (int ch = 0; ch < (KS == kRcChunk ? nch : nhalf4 >> 1); ++ch) {
+        const uint2 cc = *reinterpret_cast<const uint2*>(cols);
+        multiply(cc.x, cc.y, wp);
+        if (KS < kRcChunk) multiply(cc.y, 0, wp + 1);
+        cols += kRcChunk;
         wp += 2 * kr;
       }
+      if (KS < kRcChunk && (nhalf4 & 1)) multiply(*reinterpret_cast<const uint32_t*>(cols), 0, wp);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(empty + slot);
@@ -403,15 +429,119 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
     if (lane == 0) atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
   }
   __syncthreads();
+  if (p.second_of_two) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (*s_abort) {
     if (tid == 0)
       for (int s = 0; s < NS; ++s)
         for (unsigned i = 0; i < 4096u && !mbar_try_wait(full + s, 0) && !mbar_try_wait(full + s, 1); ++i) {}
+    __syncwarp();
+    if (split > 1) { cluster_sync_all(); cluster_sync_all(); }  // (the others' sums; they are of no use now)
     return;
   }
 
   // ---- epilogue: bias, activation, store every row of the band (rows kept by no block are +0)
   const int64_t ohw = (int64_t)a.OH * a.OW;
+  // four neighbouring columns of a row
+  auto store4 = [&](int64_t row, int64_t q, float (&t)[4]) {
+    const float bias = a.bias ? __ldg(a.bias + row) : 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      t[e] += bias;
+      if (a.relu) t[e] = fmaxf(t[e], 0.f);
+    }
+    int64_t off0;
+    bool contiguous;
+    if (a.conv) {
+      const int64_t img = q / ohw;
+      const int64_t pix = q - img * ohw;
+      off0 = (img * p.M + row) * ohw + pix;
+      contiguous = (pix + 3 < ohw) && (q + 3 < a.ncols);
+    } else {
+      off0 = row * a.y_sr + q * a.y_sq;
+      contiguous = a.y_sq == 1 && (q + 3 < a.ncols);
+    }
+    if (a.y_dtype == GRIM_F32) {
+      float* y = static_cast<float*>(a.Y);
+      if (contiguous && ((reinterpret_cast<uintptr_t>(y + off0) & 15) == 0)) {
+        *reinterpret_cast<float4*>(y + off0) = make_float4(t[0], t[1], t[2], t[3]);
+        return;
+      }
+    } else {
+      __nv_bfloat16* y = static_cast<__nv_bfloat16*>(a.Y);
+      if (contiguous && ((reinterpret_cast<uintptr_t>(y + off0) & 7) == 0)) {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(t[0], t[1]);
+        __nv_bfloat162 hi = __floats2bfloat162_rn(t[2], t[3]);
+        uint2 u;
+        u.x = *reinterpret_cast<unsigned*>(&lo);
+        u.y = *reinterpret_cast<unsigned*>(&hi);
+        *reinterpret_cast<uint2*>(y + off0) = u;
+        return;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (q + e >= a.ncols) break;
+      int64_t off;
+      if (a.conv) {
+        const int64_t img = (q + e) / ohw;
+        const int64_t pix = (q + e) - img * ohw;
+        off = (img * p.M + row) * ohw + pix;
+      } else {
+        off = row * a.y_sr + (q + e) * a.y_sq;
+      }
+      if (a.y_dtype == GRIM_F32) static_cast<float*>(a.Y)[off] = t[e];
+      else static_cast<__nv_bfloat16*>(a.Y)[off] = __float2bfloat16_rn(t[e]);
+    }
+  };
+  if (split > 1) {
+    // The parts' sums meet over distributed shared memory: every block leaves its own as lines of TN columns, one per
+    // output row of the tile, in what was the ring, and then adds up and stores every split-th line.
+    float* sums = reinterpret_cast<float*>(slots);
+#pragma unroll
+    for (int b = 0; b < BPW; ++b)
+#pragma unroll
+      for (int r = 0; r < BH; ++r) {
+        float* line = sums + ((b * kFWarps + warp) * BH + r) * TN;
+        if constexpr (NARROW) {
+          float t = nacc[b][r];
+          t += __shfl_xor_sync(0xffffffffu, t, 16);
+          if (nhalf == 0) line[nq] = t;
+        } else {
+#pragma unroll
+          for (int cp = 0; cp < CW; ++cp)
+            *reinterpret_cast<ulonglong2*>(line + cp * kTN + lane4) = make_ulonglong2(acc[b][r][2 * cp], acc[b][r][2 * cp + 1]);
+        }
+      }
+    cluster_sync_all();
+    constexpr int kPieces = TN / 4;                           // 16-byte pieces of a line
+    constexpr int kAtOnce = kPieces > 32 ? 1 : 32 / kPieces;  // lines of a warp's pass
+    for (int l0 = (part * kFWarps + warp) * kAtOnce; l0 < BPW * kFWarps * BH; l0 += split * kFWarps * kAtOnce) {
+      const int line = l0 + (kPieces > 32 ? 0 : lane / kPieces);
+      const int pos = g0 * kRcBands + line / BH;
+      if (pos >= p.nbr) continue;
+      const int r = line % BH;
+      const int64_t row = (int64_t)p.band_order[pos] * p.bh + r;
+      if (r >= p.bh || row >= p.M) continue;
+#pragma unroll
+      for (int cp = 0; cp < (kPieces > 32 ? kPieces / 32 : 1); ++cp) {
+        const int piece = cp * 32 + lane % kPieces;
+        const uint32_t at = smem_u32(sums + line * TN + piece * 4);
+        float4 v[kMaxSplit];
+#pragma unroll
+        for (int s = 0; s < kMaxSplit; ++s)  // requested together: one at a time they cost 0.2 us each
+          if (s < split) v[s] = ld_cluster128(at, s);
+        float t[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+        for (int s = 1; s < kMaxSplit; ++s)
+          if (s < split) { t[0] += v[s].x; t[1] += v[s].y; t[2] += v[s].z; t[3] += v[s].w; }
+        const int64_t q = q0 + piece * 4;
+        if (q < a.ncols) store4(row, q, t);
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();  // no block leaves while another may still read its sums
+    return;
+  }
   if constexpr (NARROW) {
     const int64_t q = q0 + nq;
     int64_t qbase = 0;  // offset of column q in row 0 of the output
@@ -436,10 +566,6 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
         const int64_t row = (int64_t)band * p.bh + r;
         if (r >= p.bh || row >= p.M || nhalf != 0 || q >= a.ncols) continue;
         const int64_t off = row * rstride + qbase;
-        if (p.ksplit > 1) {
-          if (t != 0.f) atomicAdd(static_cast<float*>(a.Y) + off, t);
-          continue;
-        }
         t += a.bias ? __ldg(a.bias + row) : 0.f;
         if (a.relu) t = fmaxf(t, 0.f);
         if (a.y_dtype == GRIM_F32) static_cast<float*>(a.Y)[off] = t;
@@ -448,90 +574,24 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
     }
   } else {
 #pragma unroll
-  for (int cp = 0; cp < CW; ++cp) {
-  const int64_t q = q0 + cp * kTN + lane4;
-  if (q >= a.ncols) continue;
+    for (int cp = 0; cp < CW; ++cp) {
+      const int64_t q = q0 + cp * kTN + lane4;
+      if (q >= a.ncols) continue;
 #pragma unroll
-  for (int b = 0; b < BPW; ++b) {
-    const int pos = (g0 + b) * kRcBands + warp;
-    if (pos >= p.nbr) continue;
-    const int band = p.band_order[pos];
+      for (int b = 0; b < BPW; ++b) {
+        const int pos = (g0 + b) * kRcBands + warp;
+        if (pos >= p.nbr) continue;
+        const int band = p.band_order[pos];
 #pragma unroll
-    for (int r = 0; r < BH; ++r) {
-      const int64_t row = (int64_t)band * p.bh + r;
-      if (r >= p.bh || row >= p.M) continue;
-      const float2 t01 = unpack2(acc[b][r][2 * cp]), t23 = unpack2(acc[b][r][2 * cp + 1]);
-      float t[4] = {t01.x, t01.y, t23.x, t23.y};
-      if (p.ksplit > 1) {
-        // partial sums of one share of the block columns: added into Y (fp32, zeroed before the launch);
-        // bias and activation follow in a separate pass
-        float* y = static_cast<float*>(a.Y);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (q + e >= a.ncols) break;
-          int64_t off;
-          if (a.conv) {
-            const int64_t img = (q + e) / ohw;
-            off = (img * p.M + row) * ohw + ((q + e) - img * ohw);
-          } else {
-            off = row * a.y_sr + (q + e) * a.y_sq;
-          }
-          if (t[e] != 0.f) atomicAdd(y + off, t[e]);
+        for (int r = 0; r < BH; ++r) {
+          const int64_t row = (int64_t)band * p.bh + r;
+          if (r >= p.bh || row >= p.M) continue;
+          const float2 t01 = unpack2(acc[b][r][2 * cp]), t23 = unpack2(acc[b][r][2 * cp + 1]);
+          float t[4] = {t01.x, t01.y, t23.x, t23.y};
+          store4(row, q, t);
         }
-        continue;
-      }
-      const float bias = a.bias ? __ldg(a.bias + row) : 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        t[e] += bias;
-        if (a.relu) t[e] = fmaxf(t[e], 0.f);
-      }
-      int64_t off0;
-      bool contiguous;
-      if (a.conv) {
-        const int64_t img = q / ohw;
-        const int64_t pix = q - img * ohw;
-        off0 = (img * p.M + row) * ohw + pix;
-        contiguous = (pix + 3 < ohw) && (q + 3 < a.ncols);
-      } else {
-        off0 = row * a.y_sr + q * a.y_sq;
-        contiguous = a.y_sq == 1 && (q + 3 < a.ncols);
-      }
-      if (a.y_dtype == GRIM_F32) {
-        float* y = static_cast<float*>(a.Y);
-        if (contiguous && ((reinterpret_cast<uintptr_t>(y + off0) & 15) == 0)) {
-          *reinterpret_cast<float4*>(y + off0) = make_float4(t[0], t[1], t[2], t[3]);
-          continue;
-        }
-      } else {
-        __nv_bfloat16* y = static_cast<__nv_bfloat16*>(a.Y);
-        if (contiguous && ((reinterpret_cast<uintptr_t>(y + off0) & 7) == 0)) {
-          __nv_bfloat162 lo = __floats2bfloat162_rn(t[0], t[1]);
-          __nv_bfloat162 hi = __floats2bfloat162_rn(t[2], t[3]);
-          uint2 u;
-          u.x = *reinterpret_cast<unsigned*>(&lo);
-          u.y = *reinterpret_cast<unsigned*>(&hi);
-          *reinterpret_cast<uint2*>(y + off0) = u;
-          continue;
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (q + e >= a.ncols) break;
-        int64_t off;
-        if (a.conv) {
-          const int64_t img = (q + e) / ohw;
-          const int64_t pix = (q + e) - img * ohw;
-          off = (img * p.M + row) * ohw + pix;
-        } else {
-          off = row * a.y_sr + (q + e) * a.y_sq;
-        }
-        if (a.y_dtype == GRIM_F32) static_cast<float*>(a.Y)[off] = t[e];
-        else static_cast<__nv_bfloat16*>(a.Y)[off] = __float2bfloat16_rn(t[e]);
       }
     }
-  }
-  }  // pieces
   }
 }
 
@@ -554,43 +614,10 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// Second pass of a split multiply: Y = act(Y + bias) in place.
-__global__ void bcr_finalize_kernel(const SpmmArgs a, int M) {
-  const int64_t total = (int64_t)M * a.ncols;
-  const int64_t ohw = (int64_t)a.OH * a.OW;
-  float* y = static_cast<float*>(a.Y);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t off, row;
-    if (a.conv) {  // i runs over the NCHW output
-      off = i;
-      row = (i / ohw) % M;
-    } else if (a.y_sq == 1) {
-      row = i / a.ncols;
-      off = row * a.y_sr + (i - row * a.ncols);
-    } else {
-      const int64_t q = i / M;
-      row = i - q * M;
-      off = row * a.y_sr + q * a.y_sq;
-    }
-    float v = y[off] + (a.bias ? __ldg(a.bias + row) : 0.f);
-    if (a.relu) v = fmaxf(v, 0.f);
-    y[off] = v;
-  }
-}
-
 bool tma_eligible(const SpmmArgs& a) {
   if (a.conv || a.x_sq != 1) return false;
   const int esz = a.x_dtype == GRIM_F32 ? 4 : 2;
   return (reinterpret_cast<uintptr_t>(a.X) % 16 == 0) && ((a.x_sk * esz) % 16 == 0) && a.ncols < (int64_t(1) << 31);
-}
-
-// Zeroes the M x ncols region of Y that a split multiply accumulates into.
-cudaError_t zero_output(const SpmmArgs& a, int64_t M, cudaStream_t s) {
-  float* y = static_cast<float*>(a.Y);
-  if (a.conv) return cudaMemsetAsync(y, 0, (size_t)M * a.ncols * 4, s);
-  if (a.y_sq == 1) return cudaMemset2DAsync(y, (size_t)a.y_sr * 4, 0, (size_t)a.ncols * 4, (size_t)M, s);
-  if (a.y_sr == 1) return cudaMemset2DAsync(y, (size_t)a.y_sq * 4, 0, (size_t)M * 4, (size_t)a.ncols, s);
-  return cudaErrorInvalidValue;
 }
 
 template <int BH, int BPW, int CW, typename XT, int MODE>
@@ -598,7 +625,21 @@ cudaError_t launch_variant(const CUtensorMap& tm, const FParams& p, size_t smem,
   auto kern = bcr_ffma_kernel<BH, BPW, CW, XT, MODE>;
   cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, grid, dim3(kFThreads), smem, s, tm, p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kFThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)p.split;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.split > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, tm, p);
 }
 
 // The accumulators of a lane take BH * BPW * CW * 4 registers: at most 64.
@@ -633,7 +674,7 @@ int slab_ld_for(const SpmmArgs& a, bool tma, int cw) { return (!tma && !a.conv &
 size_t slab_bytes_for(const grim_bcr* h, int sld, int esz) { return ((size_t)h->bw * sld * esz + 127) & ~size_t(127); }
 size_t smem_need(const grim_bcr* h, int bpw, int esz, int sld = kTN + 4, int stages = kStages) {
   const size_t blob_stride = ((size_t)h->rc_max_blob + 127) & ~size_t(127);
-  return kHdrBytes + (size_t)stages * (slab_bytes_for(h, sld, esz) + bpw * blob_stride);
+  return kHdrBytes + 128 /* slack: weights are read one row ahead */ + (size_t)stages * (slab_bytes_for(h, sld, esz) + bpw * blob_stride);
 }
 
 }  // namespace
@@ -683,19 +724,25 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
   }
   if (!fits(bpw, cw)) return GRIM_ERR_UNSUPPORTED;
   const int64_t qtiles = (a.ncols + tile_cols(cw) - 1) / tile_cols(cw);
-  const int64_t gy = (h->rc_groups + bpw - 1) / bpw;
-  if (gy > 65535) return GRIM_ERR_UNSUPPORTED;
-  // too few tiles for the GPU: split the block columns over several thread blocks (fp32 output only)
-  int ksplit = 1;
-  const bool split_ok = a.y_dtype == GRIM_F32 && (a.conv || a.y_sq == 1 || a.y_sr == 1);
-  if (split_ok && qtiles * gy * 2 <= sms) {
-    ksplit = (int)std::min<int64_t>(std::min<int64_t>(8, sms / (qtiles * gy)), std::max<int64_t>(1, h->nbc / 4));
-    if (ksplit < 1) ksplit = 1;
+  const int64_t gy = (h->rc_groups + bpw - 1) / bpw, tiles = qtiles * gy;
+  if (tiles > (int64_t(1) << 27)) return GRIM_ERR_UNSUPPORTED;
+  // Whole rounds of one tile per SM are launched as they are; the tiles of the last round, which would leave SMs idle, are
+  // split over the block columns, each shared by a cluster.  The part that takes the least time is chosen, in stages: a
+  // split costs about four more (the meeting of the sums).
+  const int64_t slots = cw ? sms : 2 * sms;  // narrow tiles are light: two thread blocks share an SM
+  int64_t tail = tiles % slots;
+  int split = 1;
+  if (tail) {
+    int64_t best = h->nbc;
+    for (int c = 2; c <= kMaxSplit && h->nbc >= 4 * c; c *= 2) {
+      // clusters that run at once: they do not straddle the GPU's partitions (of 148 SMs 74 x 2, 33 x 4, 15 x 8)
+      const int64_t at_once = std::max<int64_t>(1, (c == 2 ? sms / 2 : (c == 4 ? sms * 33 / 148 : sms * 15 / 148)) * (slots / sms));
+      const int64_t cost = (tail + at_once - 1) / at_once * ((h->nbc + c - 1) / c + 4);
+      if (cost < best) { best = cost; split = c; }
+    }
   }
-  // narrow tiles are light (two thread blocks share an SM): as many parts as still run in one wave
-  if (cw == 0 && split_ok && qtiles * gy < 2 * sms)
-    ksplit = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(8, 2 * sms / (qtiles * gy)), h->nbc / 4));
-  if (a.tile_n >= 256) ksplit = split_ok ? std::max(1, std::min(8, a.tile_n / 256)) : 1;  // test / tuning override
+  if (a.tile_n >= 256) { split = std::max(1, std::min(kMaxSplit, a.tile_n / 256)); tail = tiles; }  // test / tuning override
+  if (split == 1) tail = 0;
 
   FParams p;
   p.stage = h->d_rc_stage; p.blob = h->d_rc_blob; p.band_order = h->d_band_order; p.status = h->d_status;
@@ -705,7 +752,7 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
   p.slab_ld = slab_ld_for(a, tma, cw);
   p.slab_bytes = (uint32_t)slab_bytes_for(h, p.slab_ld, esz);
   p.spin_limit = 1u << 20;
-  p.ksplit = ksplit;
+  p.qtiles = (int)qtiles;
   p.a = a;
 
   CUtensorMap tm;
@@ -723,27 +770,29 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
                                               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return GRIM_ERR_CUDA;
   }
-  const size_t smem = smem_need(h, bpw, esz, p.slab_ld, cw ? kStages : kNarrowStages);
-  dim3 grid((unsigned)qtiles, (unsigned)gy, (unsigned)ksplit);
-  cudaError_t e = cudaSuccess;
-  if (ksplit > 1 && !(a.y_prefilled && !a.relu)) {
-    e = zero_output(a, h->M, s);
-    if (e != cudaSuccess) return GRIM_ERR_CUDA;
-  }
-  if (tma) {
-    e = esz == 4 ? launch_bh<float, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s)
-                 : launch_bh<__nv_bfloat16, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s);
-  } else {
-    e = launch_bh<float, kModeGather>(BHc, bpw, cw, tm, p, smem, grid, s);
-  }
-  count_launch();
-  if (e == cudaSuccess && ksplit > 1 && (a.bias || a.relu) && !(a.y_prefilled && !a.relu)) {
-    const int64_t total = h->M * a.ncols;
-    bcr_finalize_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, (int64_t)sm_count(h->device) * 8), 256, 0, s>>>(a, (int)h->M);
+  const size_t ring = smem_need(h, bpw, esz, p.slab_ld, cw ? kStages : kNarrowStages);
+  // whole tiles, then the split ones
+  const int64_t first = tiles - tail;
+  for (int half = 0; half < 2; ++half) {
+    const int64_t n = half ? tail : first;
+    if (!n) continue;
+    p.tile0 = half ? (int)first : 0;
+    p.split = half ? split : 1;
+    p.first_of_two = !half && tail;
+    p.second_of_two = half && first;
+    const size_t smem = half ? std::max(ring, kHdrBytes + (size_t)bpw * kFWarps * BHc * tile_cols(cw) * 4) : ring;
+    const dim3 grid((unsigned)(n * p.split));
+    cudaError_t e;
+    if (tma) {
+      e = esz == 4 ? launch_bh<float, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s)
+                   : launch_bh<__nv_bfloat16, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s);
+    } else {
+      e = launch_bh<float, kModeGather>(BHc, bpw, cw, tm, p, smem, grid, s);
+    }
     count_launch();
-    e = cudaGetLastError();
+    if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
   }
-  return e == cudaSuccess ? GRIM_OK : GRIM_ERR_CUDA;
+  return GRIM_OK;
 }
 
 }  // namespace grim

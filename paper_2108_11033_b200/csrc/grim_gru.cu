@@ -719,12 +719,6 @@ constexpr size_t kSmemLimit = 200 * 1024;
 }  // namespace
 
 namespace {
-// out[t, :] = bias for t < T (n = row length, a multiple of 4).
-__global__ void fill_rows_kernel(float* __restrict__ out, const float* __restrict__ bias, int64_t T, int64_t n) {
-  const int64_t total4 = T * n / 4, n4 = n / 4;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total4; i += (int64_t)gridDim.x * blockDim.x)
-    reinterpret_cast<float4*>(out)[i] = __ldg(reinterpret_cast<const float4*>(bias) + i % n4);
-}
 // out[k * ld + t] = in[t * K + k]: the caller's T x K input, feature-major.
 __global__ void transpose_input_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t T, int64_t K, int64_t ld) {
   __shared__ float tile[32][33];
@@ -995,18 +989,6 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
       if (cudaStreamWaitEvent(g->lstream[(size_t)l - 1], g->ev_fork, 0) != cudaSuccess) return GRIM_ERR_CUDA;
   }
   if (g->profile) g->ev_used = 0;
-  // every row of a pre-activation buffer starts as b_ih: the projections may add partial sums onto it
-  auto prefill = [&](int l, cudaStream_t s) {
-    const int64_t total = T * 3 * H;
-    fill_rows_kernel<<<(unsigned)std::min<int64_t>((total / 4 + 255) / 256, (int64_t)sm_count(g->device) * 8), 256, 0, s>>>(g->d_gi[(size_t)l], g->d_bih[(size_t)l], T, 3 * H);
-    count_launch();
-    return cudaGetLastError() == cudaSuccess;
-  };
-  for (int l = 0; l < L; ++l) {
-    if (l > 0 && g->d_gi[(size_t)l] == g->d_gi[0]) break;  // one shared buffer: filled per layer, below
-    if (!prefill(l, stream_of(l))) return GRIM_ERR_CUDA;
-  }
-
   auto launch_projection = [&](int l, const float* seq_in, int64_t t0, int64_t n, cudaStream_t s) -> grim_status_t {
     const grim_bcr* wi = g->Wih[(size_t)l];
     // gi[t, :] = W_ih x_t + b_ih for the n steps from t0 (X given q-major as n x in, output n x 3H)
@@ -1022,8 +1004,6 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
     }
     a.x_dtype = GRIM_F32; a.y_dtype = GRIM_F32;
     a.bias = g->d_bih[(size_t)l];
-    a.y_prefilled = 1;  // every row of the buffer already holds b_ih (below): a split multiply adds onto it and
-                        // needs neither its own clearing nor a bias pass; an unsplit one writes sum + bias as usual
     if (g->profile) profile_mark(g, 0, s);
     const grim_status_t st = launch_cuda_cores(wi, a, s);
     if (g->profile) profile_mark(g, 1, s);
@@ -1074,8 +1054,6 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
       const float* seq_in = l == 0 ? x : g->d_seq[(l - 1) & 1];
       float* seq_out = (l == L - 1) ? y : g->d_seq[l & 1];
       grim_status_t st = GRIM_OK;
-      if (l > 0 && c == 0 && g->d_gi[(size_t)l] == g->d_gi[0] && !prefill(l, s))
-        return GRIM_ERR_CUDA;  // layers share one buffer (allocation-free variant): fill it again for this layer
       if (l == 0) {
         if (c == 0) {  // the first layer's input is all there: one launch (after turning it feature-major)
           if (tin) {

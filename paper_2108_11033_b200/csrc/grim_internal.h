@@ -61,10 +61,10 @@ struct RunDesc {
 // Device layout for the register-tiled N > 16 kernel and the tensor-core kernel ("row-chunk"
 // layout).  Bands in schedule order are cut into groups of kRcBands; for group g and block column
 // j one contiguous blob:
-//   u32 hdr[kRcBands]     per band slot: record offset in 16-byte units | kr << 16 | nch << 24
+//   u32 hdr[kRcBands]     per band slot: record offset in 16-byte units | kr << 16 | ceil(kc / 4) << 24
 //   per band with kr > 0, 16-byte aligned:
 //     u32 rowmask, u32 kc bit r of rowmask set: block-local row r kept (kept rows are numbered a = 0.. ascending)
-//     u8  cols[nch * 8]   block-local kept columns, padded to a multiple of 8 by repeating the
+//     u8  cols[nch * 8]   (nch = ceil(kc / 8)) block-local kept columns, padded to a multiple of 8 by repeating the
 //                         first kept column (its padded weights are 0); then padding to 16 bytes
 //     f32 w[nch][kr][8]   w[c][a][e] = weight of kept row a and column cols[c * 8 + e]
 // Values are always fp32 here (bf16 handles store the rounded values widened to fp32).
@@ -205,8 +205,6 @@ struct SpmmArgs {
   int conv = 0;
   int C = 0, H = 0, W = 0, KH = 0, KW = 0, stride = 1, pad = 0, OH = 0, OW = 0;
   int tile_n = 0;  // 0 = default
-  int y_prefilled = 0;  // Y already holds the bias in every column: a split multiply adds onto it (no clearing, no
-                        // bias pass; not with relu); an unsplit multiply ignores the flag
 };
 
 grim_status_t launch_spmm(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);

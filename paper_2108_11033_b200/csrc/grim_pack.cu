@@ -358,7 +358,7 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
             if (!(hb.kr && hb.kc)) continue;
             const int kr = hb.kr, kc = hb.kc, nch = (kc + kRcChunk - 1) / kRcChunk;
             const size_t rec = rc_blob.size();
-            const uint32_t hdr = (uint32_t)((rec - start) / 16) | ((uint32_t)kr << 16) | ((uint32_t)nch << 24);
+            const uint32_t hdr = (uint32_t)((rec - start) / 16) | ((uint32_t)kr << 16) | ((uint32_t)((kc + 3) / 4) << 24);
             std::memcpy(&rc_blob[start + (size_t)b * 4], &hdr, 4);
             const size_t idx_bytes = ((size_t)8 + (size_t)nch * kRcChunk + 15) / 16 * 16;
             rc_blob.resize(rec + idx_bytes + (size_t)nch * kr * kRcChunk * 4, 0);

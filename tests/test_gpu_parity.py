@@ -276,6 +276,17 @@ def test_split_multiply(B, split):
     check_spmm(B, W, mask, X, bh, bw, path=1, tile_n=1 + 256 * split)
 
 
+@pytest.mark.parametrize("case", [(2600, 330, 1100, 4, 16, 9), (5000, 400, 520, 8, 32, 8), (4800, 300, 1000, 16, 64, 1), (2500, 520, 260, 16, 32, 1)])
+def test_slab_kernel_whole_and_split_tiles(B, case):
+    """More tiles than SMs with few left over for the last round: whole tiles first, the rest shared by clusters in a second
+    launch that starts before the first has ended.  Blocks whose last chunk is half padding or all of it in use."""
+    M, K, N, bh, bw, tile = case
+    W = gen.dense_weight(M, K, seed=87)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=6, dist="zipf", seed=88, empty_frac=0.2)
+    X = gen.normal_f32((K, N), 1.0, 89, 0)
+    check_spmm(B, W, mask, X, bh, bw, path=1, tile_n=tile)
+
+
 def test_conv_split_with_bias_and_relu(B):
     """A layer with few output pixels and many input channels takes the split path (separate bias / ReLU pass)."""
     L = gen.conv_layer(1, 96, 48, 9, ksize=3, bh=8, bw=32, compression=4, seed=86)
