@@ -61,7 +61,7 @@ struct FParams {
   int qtiles;  // tiles across the output columns; tile t covers columns tile t % qtiles and band groups t / qtiles
   int tile0;   // the launch's first tile
   int split;   // > 1: the blocks of a cluster share a tile, each multiplies a part of the block columns
-  int first_of_two, second_of_two;  // this multiply is two launches: whole tiles, then the split ones
+  int followed, follows;  // this multiply is several launches: whole tiles, then split ones
   SpmmArgs a;
 };
 
@@ -137,8 +137,8 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
   uint64_t* empty = full + kMaxRing;
   // the launch that follows in the stream may start as SMs free up: it waits (griddepcontrol.wait) before it reads or
-  // writes anything this launch touches.  (Two launches for one multiply: below)
-  if (!p.first_of_two) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // writes anything this launch touches.  (Several launches for one multiply: below)
+  if (!p.followed || p.follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + 128);
   int* s_nst = reinterpret_cast<int*>(smem + 132);
   uint32_t* s_meta = reinterpret_cast<uint32_t*>(smem + 192);               // [ring slot][4] blob bytes per band group
@@ -183,11 +183,11 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   __syncthreads();
   // (programmatic dependent launch) whatever earlier launches in the stream wrote - X, a cleared scratch or Y - is
   // complete and visible from here on; up to here only the packed matrix and this block's own shared memory were touched
-  // Two launches for one multiply: the first lets the second start only after its own wait, so whatever both read is
-  // there when the second starts; that one waits for the first at its end instead, which keeps its blocks at work while
-  // the first one's last blocks finish, and still makes its completion mean that both are done.
-  if (!p.second_of_two) asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (p.first_of_two) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Several launches for one multiply: the first lets the next start only after its own wait, so whatever all read is there
+  // when the others start; each of those waits for the one before it at its end instead, which keeps its blocks at work
+  // while that one's last blocks finish, and still makes the last one's completion mean that all are done.
+  if (!p.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.followed && !p.follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // with a split over block columns this thread block multiplies only its share of the stage list
   const int nst_all = *s_nst;
   const int n_lo = (int)((int64_t)part * nst_all / split), n_hi = (int)((int64_t)(part + 1) * nst_all / split);
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
     if (lane == 0) atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
   }
   __syncthreads();
-  if (p.second_of_two) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (*s_abort) {
     if (tid == 0)
       for (int s = 0; s < NS; ++s)
@@ -727,22 +727,43 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
   const int64_t gy = (h->rc_groups + bpw - 1) / bpw, tiles = qtiles * gy;
   if (tiles > (int64_t(1) << 27)) return GRIM_ERR_UNSUPPORTED;
   // Whole rounds of one tile per SM are launched as they are; the tiles of the last round, which would leave SMs idle, are
-  // split over the block columns, each shared by a cluster.  The part that takes the least time is chosen, in stages: a
-  // split costs about four more (the meeting of the sums).
+  // shared by clusters that split the block columns.  Of the ways to do that - one cluster size for all, or pairs for as
+  // many as run at once and another size for the rest - the one that takes the least time is chosen, in stages: a split
+  // costs about four more (the meeting of the sums).
   const int64_t slots = cw ? sms : 2 * sms;  // narrow tiles are light: two thread blocks share an SM
-  int64_t tail = tiles % slots;
-  int split = 1;
-  if (tail) {
-    int64_t best = h->nbc;
-    for (int c = 2; c <= kMaxSplit && h->nbc >= 4 * c; c *= 2) {
-      // clusters that run at once: they do not straddle the GPU's partitions (of 148 SMs 74 x 2, 33 x 4, 15 x 8)
-      const int64_t at_once = std::max<int64_t>(1, (c == 2 ? sms / 2 : (c == 4 ? sms * 33 / 148 : sms * 15 / 148)) * (slots / sms));
-      const int64_t cost = (tail + at_once - 1) / at_once * ((h->nbc + c - 1) / c + 4);
-      if (cost < best) { best = cost; split = c; }
+  struct Segment { int64_t n; int split; } seg[3];
+  int nseg = 0;
+  if (a.tile_n >= 256) {  // test / tuning override
+    seg[nseg++] = {tiles, std::max(1, std::min(kMaxSplit, a.tile_n / 256))};
+  } else {
+    const int64_t tail = tiles % slots;
+    // clusters that run at once: they do not straddle the GPU's partitions (of 148 SMs 74 x 2, 45 x 3, 33 x 4, 15 x 8)
+    auto at_once = [&](int c) {
+      return std::max<int64_t>(1, (c == 1 ? sms : (c == 2 ? sms / 2 : (c == 3 ? sms * 45 / 148 : (c == 4 ? sms * 33 / 148 : sms * 15 / 148)))) * (slots / sms));
+    };
+    int best_c = 1;
+    auto best = [&](int64_t n) {  // stages that n tiles take, and the cluster size for it
+      int64_t least = INT64_MAX;
+      for (int c : {1, 2, 3, 4, 8}) {
+        if (c > 1 && h->nbc < 4 * c) break;
+        const int64_t cost = (n + at_once(c) - 1) / at_once(c) * ((h->nbc + c - 1) / c + (c > 1 ? 4 : 0));
+        if (cost < least) { least = cost; best_c = c; }
+      }
+      return n ? least : 0;
+    };
+    int64_t pairs = 0;
+    const int64_t alone = best(tail);
+    int c = best_c;
+    if (tail > at_once(2) && h->nbc >= 8) {
+      const int64_t both = (h->nbc + 1) / 2 + 4 + best(tail - at_once(2));
+      if (both < alone) { pairs = at_once(2); c = best_c; }
     }
+    if (c == 1) pairs = 0;
+    const int64_t whole = c == 1 ? tiles : tiles - tail;
+    if (whole) seg[nseg++] = {whole, 1};
+    if (pairs) seg[nseg++] = {pairs, 2};
+    if (tiles - whole - pairs) seg[nseg++] = {tiles - whole - pairs, c};
   }
-  if (a.tile_n >= 256) { split = std::max(1, std::min(kMaxSplit, a.tile_n / 256)); tail = tiles; }  // test / tuning override
-  if (split == 1) tail = 0;
 
   FParams p;
   p.stage = h->d_rc_stage; p.blob = h->d_rc_blob; p.band_order = h->d_band_order; p.status = h->d_status;
@@ -771,17 +792,13 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
     if (r != CUDA_SUCCESS) return GRIM_ERR_CUDA;
   }
   const size_t ring = smem_need(h, bpw, esz, p.slab_ld, cw ? kStages : kNarrowStages);
-  // whole tiles, then the split ones
-  const int64_t first = tiles - tail;
-  for (int half = 0; half < 2; ++half) {
-    const int64_t n = half ? tail : first;
-    if (!n) continue;
-    p.tile0 = half ? (int)first : 0;
-    p.split = half ? split : 1;
-    p.first_of_two = !half && tail;
-    p.second_of_two = half && first;
-    const size_t smem = half ? std::max(ring, kHdrBytes + (size_t)bpw * kFWarps * BHc * tile_cols(cw) * 4) : ring;
-    const dim3 grid((unsigned)(n * p.split));
+  p.tile0 = 0;
+  for (int k = 0; k < nseg; ++k) {
+    p.split = seg[k].split;
+    p.follows = k > 0;
+    p.followed = k + 1 < nseg;
+    const size_t smem = p.split > 1 ? std::max(ring, kHdrBytes + (size_t)bpw * kFWarps * BHc * tile_cols(cw) * 4) : ring;
+    const dim3 grid((unsigned)(seg[k].n * p.split));
     cudaError_t e;
     if (tma) {
       e = esz == 4 ? launch_bh<float, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s)
@@ -791,6 +808,7 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
     }
     count_launch();
     if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+    p.tile0 += (int)seg[k].n;
   }
   return GRIM_OK;
 }
