@@ -145,9 +145,13 @@ bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
   // The slab kernel needs rows of X that TMA can fetch; its other loaders are slow (N = 1023: 1477 -> 1213, N = 131 in
   // bf16: 328 -> 30), except that a slab row of 16-row bands is used often enough to pay for them in large products.
   if (!slab_rows_by_tma(a)) return a.x_dtype == GRIM_BF16 || h->bh <= 8 || flops <= 1e9;
-  // Otherwise: up to about half a GFLOP the slab kernel's pipeline is all start-up (1024^2, N = 128: 16.5 -> 6.1;
-  // 2048^2, N = 128: 20.6 -> 12.6; 4096^2, N = 128: 39.6 -> 39.5); beyond, re-reading X from L2 for every band costs more.
-  return flops <= 5e8;
+  // Otherwise: whichever is estimated to be done first.  The direct kernel's time goes with the chunks and 128-column tiles
+  // (0.33, 0.5 and 1.0 ns each for 4, 8 and 16 rows, less for up to 64 columns), the slab kernel's with the stages it takes one after the other.
+  // (1024^2, N = 128: 6.4 against 11; 2048^2, 4 x 16, N = 256: 44 against 26; 8 x 32: 23 against 22; 4096 x 1024, N = 256:
+  // 26 against 21; 1024 x 4096: 22 against 33.)
+  const bool few = a.ncols <= 64;
+  const double per_chunk = h->bh <= 4 ? (few ? 0.29e-3 : 0.33e-3) : (h->bh <= 8 ? (few ? 0.44e-3 : 0.5e-3) : (few ? 0.6e-3 : 1.0e-3));
+  return 4.0 + per_chunk * (double)h->rc_chunks * (double)((a.ncols + 127) / 128) <= slab_time(h, a);
 }
 
 grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {

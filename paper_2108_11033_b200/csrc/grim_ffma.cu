@@ -677,20 +677,15 @@ size_t smem_need(const grim_bcr* h, int bpw, int esz, int sld = kTN + 4, int sta
   return kHdrBytes + 128 /* slack: weights are read one row ahead */ + (size_t)stages * (slab_bytes_for(h, sld, esz) + bpw * blob_stride);
 }
 
-}  // namespace
-
-bool slab_rows_by_tma(const SpmmArgs& a) { return tma_eligible(a); }
-
-bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a) {
-  if (h->device < 0 || !h->d_rc_stage || !h->d_status) return false;
-  if (h->nbc > kJlistCap || h->rc_max_blob == 0 || h->rc_max_blob > 0xFFFF * 16u) return false;
-  if (a.ncols <= 0 || a.ncols > (int64_t(1) << 31) - 2 * kTN) return false;
-  const bool tma = tma_eligible(a);
-  return smem_need(h, 1, (tma && a.x_dtype == GRIM_BF16) ? 2 : 4) <= kSmemBudget;
-}
-
-grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
-  if (!ffma_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
+struct Segment { int64_t n; int split; };
+struct SlabPlan {
+  int bpw = 1, cw = 1;
+  int64_t qtiles = 0, tiles = 0;
+  Segment seg[3];  // tiles of each launch and the blocks that share one
+  int nseg = 0;
+  int64_t stages = 0;  // stages one after the other
+};
+bool plan_slab(const grim_bcr* h, const SpmmArgs& a, SlabPlan& pl) {
   const bool tma = tma_eligible(a);
   const int esz = (tma && a.x_dtype == GRIM_BF16) ? 2 : 4;  // bytes per slab element (the gather loader widens bf16)
   const int BHc = h->bh <= 4 ? 4 : (h->bh <= 8 ? 8 : 16);
@@ -722,19 +717,18 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
       while (bpw > 1 && (!fits(bpw, 1) || tiles_of(bpw, 1) < sms)) bpw >>= 1;
     }
   }
-  if (!fits(bpw, cw)) return GRIM_ERR_UNSUPPORTED;
+  if (!fits(bpw, cw)) return false;
   const int64_t qtiles = (a.ncols + tile_cols(cw) - 1) / tile_cols(cw);
   const int64_t gy = (h->rc_groups + bpw - 1) / bpw, tiles = qtiles * gy;
-  if (tiles > (int64_t(1) << 27)) return GRIM_ERR_UNSUPPORTED;
+  if (tiles > (int64_t(1) << 27)) return false;
   // Whole rounds of one tile per SM are launched as they are; the tiles of the last round, which would leave SMs idle, are
   // shared by clusters that split the block columns.  Of the ways to do that - one cluster size for all, or pairs for as
   // many as run at once and another size for the rest - the one that takes the least time is chosen, in stages: a split
   // costs about four more (the meeting of the sums).
   const int64_t slots = cw ? sms : 2 * sms;  // narrow tiles are light: two thread blocks share an SM
-  struct Segment { int64_t n; int split; } seg[3];
-  int nseg = 0;
   if (a.tile_n >= 256) {  // test / tuning override
-    seg[nseg++] = {tiles, std::max(1, std::min(kMaxSplit, a.tile_n / 256))};
+    pl.seg[pl.nseg++] = {tiles, std::max(1, std::min(kMaxSplit, a.tile_n / 256))};
+    pl.stages = tiles * h->nbc / slots;
   } else {
     const int64_t tail = tiles % slots;
     // clusters that run at once: they do not straddle the GPU's partitions (of 148 SMs 74 x 2, 45 x 3, 33 x 4, 15 x 8)
@@ -743,27 +737,59 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
     };
     int best_c = 1;
     auto best = [&](int64_t n) {  // stages that n tiles take, and the cluster size for it
-      int64_t least = INT64_MAX;
+      int64_t t = INT64_MAX;
       for (int c : {1, 2, 3, 4, 8}) {
         if (c > 1 && h->nbc < 4 * c) break;
         const int64_t cost = (n + at_once(c) - 1) / at_once(c) * ((h->nbc + c - 1) / c + (c > 1 ? 4 : 0));
-        if (cost < least) { least = cost; best_c = c; }
+        if (cost < t) { t = cost; best_c = c; }
       }
-      return n ? least : 0;
+      return n ? t : 0;
     };
-    int64_t pairs = 0;
-    const int64_t alone = best(tail);
+    int64_t pairs = 0, least = best(tail);
     int c = best_c;
     if (tail > at_once(2) && h->nbc >= 8) {
       const int64_t both = (h->nbc + 1) / 2 + 4 + best(tail - at_once(2));
-      if (both < alone) { pairs = at_once(2); c = best_c; }
+      if (both < least && best_c > 1) { pairs = at_once(2); c = best_c; least = both; }
     }
-    if (c == 1) pairs = 0;
     const int64_t whole = c == 1 ? tiles : tiles - tail;
-    if (whole) seg[nseg++] = {whole, 1};
-    if (pairs) seg[nseg++] = {pairs, 2};
-    if (tiles - whole - pairs) seg[nseg++] = {tiles - whole - pairs, c};
+    pl.stages = tiles / slots * h->nbc + least;
+    if (whole) pl.seg[pl.nseg++] = {whole, 1};
+    if (pairs) pl.seg[pl.nseg++] = {pairs, 2};
+    if (tiles - whole - pairs) pl.seg[pl.nseg++] = {tiles - whole - pairs, c};
   }
+  pl.bpw = bpw; pl.cw = cw; pl.qtiles = qtiles; pl.tiles = tiles;
+  return true;
+}
+
+}  // namespace
+
+bool slab_rows_by_tma(const SpmmArgs& a) { return tma_eligible(a); }
+
+// Microseconds: about five to start, and per stage what the slower of copying and multiplying takes.
+double slab_time(const grim_bcr* h, const SpmmArgs& a) {
+  SlabPlan pl;
+  if (!ffma_path_supported(h, a) || !plan_slab(h, a, pl)) return 1e30;
+  const double per_stage = (double)h->nnz / ((double)h->rc_groups * (double)h->nbc) * pl.bpw * tile_cols(pl.cw);
+  return 5.0 + (double)pl.stages * std::max(pl.cw == 2 ? 0.53 : 0.66, 0.35 + 7.8e-6 * per_stage);
+}
+
+bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a) {
+  if (h->device < 0 || !h->d_rc_stage || !h->d_status) return false;
+  if (h->nbc > kJlistCap || h->rc_max_blob == 0 || h->rc_max_blob > 0xFFFF * 16u) return false;
+  if (a.ncols <= 0 || a.ncols > (int64_t(1) << 31) - 2 * kTN) return false;
+  const bool tma = tma_eligible(a);
+  return smem_need(h, 1, (tma && a.x_dtype == GRIM_BF16) ? 2 : 4) <= kSmemBudget;
+}
+
+grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
+  if (!ffma_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
+  const bool tma = tma_eligible(a);
+  const int esz = (tma && a.x_dtype == GRIM_BF16) ? 2 : 4;  // bytes per slab element (the gather loader widens bf16)
+  const int BHc = h->bh <= 4 ? 4 : (h->bh <= 8 ? 8 : 16);
+  const int sms = sm_count(h->device);
+  SlabPlan pl;
+  if (!plan_slab(h, a, pl)) return GRIM_ERR_UNSUPPORTED;
+  const int bpw = pl.bpw, cw = pl.cw;
 
   FParams p;
   p.stage = h->d_rc_stage; p.blob = h->d_rc_blob; p.band_order = h->d_band_order; p.status = h->d_status;
@@ -773,7 +799,7 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
   p.slab_ld = slab_ld_for(a, tma, cw);
   p.slab_bytes = (uint32_t)slab_bytes_for(h, p.slab_ld, esz);
   p.spin_limit = 1u << 20;
-  p.qtiles = (int)qtiles;
+  p.qtiles = (int)pl.qtiles;
   p.a = a;
 
   CUtensorMap tm;
@@ -793,12 +819,12 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
   }
   const size_t ring = smem_need(h, bpw, esz, p.slab_ld, cw ? kStages : kNarrowStages);
   p.tile0 = 0;
-  for (int k = 0; k < nseg; ++k) {
-    p.split = seg[k].split;
+  for (int k = 0; k < pl.nseg; ++k) {
+    p.split = pl.seg[k].split;
     p.follows = k > 0;
-    p.followed = k + 1 < nseg;
+    p.followed = k + 1 < pl.nseg;
     const size_t smem = p.split > 1 ? std::max(ring, kHdrBytes + (size_t)bpw * kFWarps * BHc * tile_cols(cw) * 4) : ring;
-    const dim3 grid((unsigned)(seg[k].n * p.split));
+    const dim3 grid((unsigned)(pl.seg[k].n * p.split));
     cudaError_t e;
     if (tma) {
       e = esz == 4 ? launch_bh<float, kModeTma>(BHc, bpw, cw, tm, p, smem, grid, s)
@@ -808,7 +834,7 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) 
     }
     count_launch();
     if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
-    p.tile0 += (int)seg[k].n;
+    p.tile0 += (int)pl.seg[k].n;
   }
   return GRIM_OK;
 }

@@ -223,6 +223,7 @@ bool narrow_preferred(const grim_bcr* h, int64_t N);
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA
+double slab_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
 // the CUDA-core kernel for a request: direct, slab or, for operands neither takes, the shared-memory slab fall-back
 grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 // small and middle-sized products without a block-wide pipeline (also convolutions)
