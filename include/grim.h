@@ -206,7 +206,8 @@ grim_status_t grim_bcr_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, gr
  * few output tiles and a long K are split over K through an fp32 scratch) and of the tensor-core convolution (a
  * channel-last copy of the input).  Compute calls never allocate: grim_bcr_reserve allocates that scratch for right-hand
  * sides of up to max_ncols columns (for a convolution: images x OH x OW), once, at set-up time; it synchronises the
- * device.  Without it (or beyond max_ncols) such calls simply run on other kernels, slower.  max_ncols = 0 frees it.
+ * device.  Without it (or beyond max_ncols) such calls simply run on other kernels, slower.  A bf16 right-hand side whose rows are not
+ * multiples of 16 bytes is copied to rows that are (up to 64 MiB).  max_ncols = 0 frees it.
  * More than 2^30 bytes -> GRIM_ERR_UNSUPPORTED. */
 grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols);
 

@@ -78,7 +78,17 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
     return launch_skinny(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, s);
   }
   if (path == 4) return launch_spmm(h, a, s);
-  // bf16 handles, wide right-hand sides: tensor cores.  The paired kernel when its 256 x 512 tiles still give most
+  // bf16 handles, wide right-hand sides: tensor cores, except for small products, which the direct kernel has done before the
+  // tensor-core kernels' start-up of some 14 us is over (1024^2, 8 x 32, N = 128: 15.3 -> 7.0 us).  Rows that TMA cannot fetch are
+  // copied to aligned ones first where grim_bcr_reserve has made room (3000^2, N = 333: 112 -> 33).
+  if (path == 0 && a.x_dtype == GRIM_BF16 && a.ncols > kSkinnyMaxN) {
+    if (direct_path_supported(h, a) && direct_time(h, a) <= 12.0) return launch_direct(h, a, s);
+    if (!tc_path_supported(h, a) && x_copy_possible(h, a)) {
+      const grim_status_t cs = launch_x_copy(h, a, s);
+      if (cs != GRIM_OK) return cs;
+    }
+  }
+  // The paired kernel when its 256 x 512 tiles still give most
   // SMs a thread block (measured: with fewer, the single-block kernel's smaller tiles win).
   if (path == 0 && tc2_path_supported(h, a) && a.ncols >= 256 && h->tc_mtiles >= 2 &&
       2 * ((h->tc_mtiles + 1) / 2) * ((a.ncols + 511) / 512) * 3 >= 2 * (int64_t)sm_count(h->device))
@@ -246,18 +256,20 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
 extern "C" grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols) {
   if (!h || max_ncols < 0) return GRIM_ERR_INVALID_ARG;
   if (h->device < 0) return GRIM_ERR_INVALID_ARG;
-  const size_t acc = (size_t)h->M * (size_t)max_ncols * 4;
-  if (acc > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;
+  if ((size_t)h->M * (size_t)max_ncols * 4 > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;
+  const size_t acc = (size_t)h->M * (size_t)((max_ncols + 3) / 4 * 4) * 4;
   // the split multiply only takes outputs of at most half a tile per SM, which is less than 40 MiB
-  const size_t need = std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols));
-  if (h->tc_acc_bytes >= need && need > 0) return GRIM_OK;
+  const size_t need = (std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols)) + 255) / 256 * 256;
+  const size_t copy = x_copy_size(h, max_ncols);
+  if (h->tc_acc_bytes >= need && h->x_copy_bytes >= copy && need > 0) return GRIM_OK;
   if (cudaDeviceSynchronize() != cudaSuccess) return GRIM_ERR_CUDA;  // a launch in flight may still use the old scratch
   cudaFree(h->d_tc_acc);
   h->d_tc_acc = nullptr;
-  h->tc_acc_bytes = 0;
+  h->tc_acc_bytes = h->x_copy_bytes = 0;
   if (need == 0) return GRIM_OK;
-  if (cudaMalloc((void**)&h->d_tc_acc, need) != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_ALLOC; }
+  if (cudaMalloc((void**)&h->d_tc_acc, need + copy) != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_ALLOC; }
   h->tc_acc_bytes = need;
+  h->x_copy_bytes = copy;
   return GRIM_OK;
 }
 

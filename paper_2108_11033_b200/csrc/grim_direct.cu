@@ -125,6 +125,12 @@ bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   return true;
 }
 
+double direct_time(const grim_bcr* h, const SpmmArgs& a) {
+  const bool few = a.ncols <= 64;
+  const double per_chunk = h->bh <= 4 ? (few ? 0.29e-3 : 0.33e-3) : (h->bh <= 8 ? (few ? 0.44e-3 : 0.5e-3) : (few ? 0.6e-3 : 1.0e-3));
+  return 4.0 + per_chunk * (double)h->rc_chunks * (double)((a.ncols + 127) / 128);
+}
+
 // Where the direct kernel is the faster of the CUDA-core kernels (measured on square matrices of 512 to 8192, pruning rate
 // 8, the three block shapes; times in us, slab kernel -> direct kernel).
 bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
@@ -149,9 +155,7 @@ bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
   // (0.33, 0.5 and 1.0 ns each for 4, 8 and 16 rows, less for up to 64 columns), the slab kernel's with the stages it takes one after the other.
   // (1024^2, N = 128: 6.4 against 11; 2048^2, 4 x 16, N = 256: 44 against 26; 8 x 32: 23 against 22; 4096 x 1024, N = 256:
   // 26 against 21; 1024 x 4096: 22 against 33.)
-  const bool few = a.ncols <= 64;
-  const double per_chunk = h->bh <= 4 ? (few ? 0.29e-3 : 0.33e-3) : (h->bh <= 8 ? (few ? 0.44e-3 : 0.5e-3) : (few ? 0.6e-3 : 1.0e-3));
-  return 4.0 + per_chunk * (double)h->rc_chunks * (double)((a.ncols + 127) / 128) <= slab_time(h, a);
+  return direct_time(h, a) <= slab_time(h, a);
 }
 
 grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {

@@ -173,6 +173,8 @@ struct grim_bcr {
   // channel-last copy of a convolution's input
   float* d_tc_acc = nullptr;
   size_t tc_acc_bytes = 0;
+  // ... and, behind it, an aligned copy of a bf16 right-hand side whose rows TMA cannot fetch as they lie
+  size_t x_copy_bytes = 0;
   // answers of grim_bcr_tune, one per (log2 bucket of N, X dtype, Y dtype); path 0 = not tuned
   grim_tune_t tuned[32][2][2] = {};
   unsigned* d_status = nullptr;  // error word written by kernels whose bounded waits ran out
@@ -223,6 +225,11 @@ bool narrow_preferred(const grim_bcr* h, int64_t N);
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA
+double direct_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us (plain products)
+// bf16 handles: a copy of X with aligned rows for the tensor-core kernels, where the scratch for it is there
+size_t x_copy_size(const grim_bcr* h, int64_t ncols);
+bool x_copy_possible(const grim_bcr* h, const SpmmArgs& a);
+grim_status_t launch_x_copy(const grim_bcr* h, SpmmArgs& a, cudaStream_t s);  // a.X and a.x_sk become the copy's
 double slab_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
 // the CUDA-core kernel for a request: direct, slab or, for operands neither takes, the shared-memory slab fall-back
 grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);

@@ -62,7 +62,8 @@ struct TcParams {
   int seg_off, seg_len;  // staged convolution: elements in front of the tile's first pixel / per channel segment
   int nseg;              // staged convolution: slots of the ring of staged planes
   int ksplit, kt_per;    // > 1: blockIdx.z takes kt_per K tiles and adds its partial sums into the fp32 scratch `acc`
-  float* acc;            // [M][ncols] when ksplit > 1
+  float* acc;            // [M][acc_ld] when ksplit > 1
+  int64_t acc_ld;        // ncols rounded up to four
   uint32_t seg_bytes;    // bytes of one such slot
   SpmmArgs a;
 };
@@ -290,6 +291,8 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
       const int trow = quarter * 32 + lane;         // row of the tile held by this thread's lane
       const int r = trow & (BH - 1);
       const int cb0 = ((warp - 2) >> 2) * (kTQ / 64), cb1 = cb0 + kTQ / 64;  // warps 2-5: columns 0-127, warps 6-9: 128-255
+      const int esz = a.y_dtype == GRIM_F32 ? 4 : 2;
+      const bool rows_aligned = (a.y_sr * esz) % 16 == 0 && reinterpret_cast<uintptr_t>(a.Y) % 16 == 0;
       for (int m = 0; m < p.mt; ++m) {
       const int pos = pos0 + m * p.slots_per_tile + (trow >> p.bh_shift);
       int64_t row = -1;
@@ -300,21 +303,42 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
         uint32_t v[32];
         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(m * (int)kTmemCols + cb * 32), v);
         const int64_t q = q0 + cb * 32;
-        if (!row_ok || q >= a.ncols) continue;
+        if (q >= a.ncols) continue;
+        if (!CONV && p.ksplit == 1 && !(rows_aligned && q + 31 < a.ncols)) {
+          // rows that 16-byte stores cannot fill: through shared memory (all multiplies are done with it), so that a store
+          // writes neighbouring columns of one row and not one column of 32 rows (3000^2, N = 333: 44 -> 33 us)
+          float* stg = reinterpret_cast<float*>(stages) + (warp - 2) * (33 * 32);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float t = __uint_as_float(v[i]) + bias;
+            stg[lane * 33 + i] = a.relu ? fmaxf(t, 0.f) : t;
+          }
+          __syncwarp();
+          const bool col_ok = q + lane < a.ncols;
+#pragma unroll 8
+          for (int i = 0; i < 32; ++i) {
+            const int rr = __shfl_sync(0xffffffffu, row_ok ? (int)row : -1, i);
+            const float t = stg[i * 33 + lane];
+            if (rr < 0 || !col_ok) continue;
+            const int64_t o = (int64_t)rr * a.y_sr + q + lane;
+            if (a.y_dtype == GRIM_F32) static_cast<float*>(a.Y)[o] = t;
+            else static_cast<__nv_bfloat16*>(a.Y)[o] = __float2bfloat16_rn(t);
+          }
+          __syncwarp();
+          continue;
+        }
+        if (!row_ok) continue;
         if (p.ksplit > 1) {
           // split multiply: partial sums go to the zeroed fp32 scratch; bias, activation and the output layout are
           // applied by a pass over the scratch when all parts are in
-          float* dst = p.acc + row * a.ncols + q;
-          if (q + 31 < a.ncols && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-            // eight 16-byte reductions instead of thirty-two 4-byte ones
+          float* dst = p.acc + row * p.acc_ld + q;
+          // 16-byte reductions (rows of the scratch are multiples of four; columns past the last one add zeros)
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+          for (int i = 0; i < 8; ++i)
+            if (q + 4 * i < p.acc_ld)
               asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + 4 * i), "f"(__uint_as_float(v[4 * i])),
                            "f"(__uint_as_float(v[4 * i + 1])), "f"(__uint_as_float(v[4 * i + 2])), "f"(__uint_as_float(v[4 * i + 3]))
                            : "memory");
-          } else {
-            for (int i = 0; i < 32 && q + i < a.ncols; ++i) atomicAdd(dst + i, __uint_as_float(v[i]));
-          }
           continue;
         }
         float t[32];
@@ -382,12 +406,12 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
 }
 
 // Second pass of a split multiply: scratch + bias -> activation -> Y in its layout and type.
-__global__ void tc_finalize_kernel(const float* __restrict__ acc, int64_t ncols, int M, const float* __restrict__ bias, int relu,
+__global__ void tc_finalize_kernel(const float* __restrict__ acc, int64_t acc_ld, int64_t ncols, int M, const float* __restrict__ bias, int relu,
                                    void* Y, int y_dtype, int64_t y_sr, int conv, int64_t ohw) {
   const int64_t total = (int64_t)M * ncols;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t row = i / ncols, q = i - row * ncols;
-    float v = acc[i] + (bias ? __ldg(bias + row) : 0.f);
+    float v = acc[row * acc_ld + q] + (bias ? __ldg(bias + row) : 0.f);
     if (relu) v = fmaxf(v, 0.f);
     int64_t off = row * y_sr + q;
     if (conv) {
@@ -458,6 +482,69 @@ bool tc_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   return encode_tiled_fn() != nullptr;
 }
 
+namespace {
+// dst[k][0 .. ld) = the N columns of row k of src, whose rows start at any even address: a thread puts eight elements together
+// from 4-byte words (shifted by half a word where the row starts inside one).  Bound by its launch: 3000 x 333 takes 3 us.
+__global__ void __launch_bounds__(256) align_rows_kernel(const unsigned short* __restrict__ src, int64_t src_ld, unsigned short* __restrict__ dst,
+                                                         int ld, int n, int64_t rows) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int per_row = ld / 8;
+  const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const int64_t k = i / per_row;
+  if (k >= rows) return;
+  const int c = (int)(i - k * per_row) * 8;
+  const unsigned short* in = src + k * src_ld + c;
+  uint4 out;
+  if (c + 8 <= n) {
+    const bool odd = (reinterpret_cast<uintptr_t>(in) & 2) != 0;  // then one element before the eight and one behind them are
+    unsigned w[5];                                                // read with the words; the one behind only if it exists
+    const unsigned* words = reinterpret_cast<const unsigned*>(reinterpret_cast<uintptr_t>(in) & ~uintptr_t(3));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = __ldg(words + j);
+    w[4] = odd ? (unsigned)__ldg(in + 7) : 0u;
+    const int sh = odd ? 16 : 0;
+    out.x = __funnelshift_r(w[0], w[1], sh); out.y = __funnelshift_r(w[1], w[2], sh);
+    out.z = __funnelshift_r(w[2], w[3], sh); out.w = __funnelshift_r(w[3], w[4], sh);
+  } else {
+    unsigned v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = c + e < n ? (unsigned)__ldg(in + e) : 0u;
+    out = make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
+  }
+  *reinterpret_cast<uint4*>(dst + k * ld + c) = out;
+}
+constexpr size_t kMaxCopy = (size_t)64 << 20;
+}  // namespace
+
+size_t x_copy_size(const grim_bcr* h, int64_t ncols) {
+  if (h->dtype != GRIM_BF16 || ncols <= kSkinnyMaxN) return 0;
+  const size_t n = (size_t)h->K * (size_t)((ncols + 7) / 8 * 8) * 2;
+  return n <= kMaxCopy ? n : 0;
+}
+
+bool x_copy_possible(const grim_bcr* h, const SpmmArgs& a) {
+  if (a.conv || a.x_dtype != GRIM_BF16 || a.x_sq != 1 || a.ncols > (1 << 30)) return false;
+  const size_t n = x_copy_size(h, a.ncols);
+  if (n == 0 || n > h->x_copy_bytes) return false;
+  SpmmArgs b = a;
+  b.X = reinterpret_cast<uint8_t*>(h->d_tc_acc) + h->tc_acc_bytes;
+  b.x_sk = (a.ncols + 7) / 8 * 8;
+  return tc_path_supported(h, b);
+}
+
+grim_status_t launch_x_copy(const grim_bcr* h, SpmmArgs& a, cudaStream_t s) {
+  unsigned short* dst = reinterpret_cast<unsigned short*>(reinterpret_cast<uint8_t*>(h->d_tc_acc) + h->tc_acc_bytes);
+  const int64_t ld = (a.ncols + 7) / 8 * 8, n = h->K * (ld / 8);
+  const cudaError_t e = launch_pdl(align_rows_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, static_cast<const unsigned short*>(a.X),
+                                   a.x_sk, dst, (int)ld, (int)a.ncols, h->K);
+  count_launch();
+  if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+  a.X = dst;
+  a.x_sk = ld;
+  return GRIM_OK;
+}
+
 grim_status_t launch_spmm_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
   if (!tc_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
   TcParams p;
@@ -502,7 +589,8 @@ grim_status_t launch_spmm_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
     // the reductions into it and the second pass cost more than the shorter K loop saves)
     int want = (int)std::min<int64_t>(16, sms / std::max<int64_t>(blocks, 1));
     want = std::min(want, p.nkt / 4);  // at least four K tiles per part
-    const size_t need = (size_t)h->M * (size_t)a.ncols * 4;
+    p.acc_ld = (a.ncols + 3) / 4 * 4;
+    const size_t need = (size_t)h->M * (size_t)p.acc_ld * 4;
     if (want >= 2 && p.nkt >= 16 && blocks * 2 <= sms && need <= ((size_t)1 << 30)) {
       // the scratch is reserved ahead of time (grim_bcr_reserve); without it, or when it is too small, the multiply runs unsplit
       if (h->d_tc_acc && h->tc_acc_bytes >= need) {
@@ -518,7 +606,7 @@ grim_status_t launch_spmm_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
     if (p.ksplit <= 1) return GRIM_OK;
     const int64_t total = (int64_t)h->M * a.ncols;
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sm_count(h->device) * 8);
-    tc_finalize_kernel<<<blocks, 256, 0, s>>>(p.acc, a.ncols, (int)h->M, a.bias, a.relu, a.Y, a.y_dtype, a.y_sr, a.conv,
+    tc_finalize_kernel<<<blocks, 256, 0, s>>>(p.acc, p.acc_ld, a.ncols, (int)h->M, a.bias, a.relu, a.Y, a.y_dtype, a.y_sr, a.conv,
                                               (int64_t)a.OH * a.OW);
     count_launch();
     return cudaGetLastError() == cudaSuccess ? GRIM_OK : GRIM_ERR_CUDA;

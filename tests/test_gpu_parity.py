@@ -287,6 +287,32 @@ def test_slab_kernel_whole_and_split_tiles(B, case):
     check_spmm(B, W, mask, X, bh, bw, path=1, tile_n=tile)
 
 
+@pytest.mark.parametrize("case", [(300, 5000, 24, 33, 1), (1100, 1300, 257, 257, 0), (700, 900, 40, 41, 3), (520, 1203, 1024, 1025, 2), (264, 6000, 17, 19, 0)])
+@pytest.mark.parametrize("y_bf16", [False, True])
+def test_tensor_core_rows_made_aligned(B, case, y_bf16):
+    """bf16 right-hand sides whose rows TMA cannot fetch: copied to aligned rows (odd and even widths, rows that start inside a
+    word, the last element of the buffer), outputs whose rows are not aligned either, with and without a split over K."""
+    M, K, N, ld, off = case
+    bh, bw = 8, 32
+    W = gen.dense_weight(M, K, seed=301)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=2, dist="uniform", seed=302, empty_frac=0.1)
+    X = gen.bf16_representable(gen.normal_f32((K, N), 1.0, 303, 0))
+    flat = torch.full((off + (K - 1) * ld + N,), float("nan"), device="cuda", dtype=torch.bfloat16)
+    Xd = torch.as_strided(flat, (K, N), (ld, 1), off)
+    Xd.copy_(to_dev(X, True))
+    h = B.grim_bcr_pack(W, mask, bh, bw, B.GRIM_BF16, 0)
+    try:
+        B.grim_bcr_reserve(h, N)
+        Yd = torch.full((M, N), float("nan"), device="cuda", dtype=torch.bfloat16 if y_bf16 else torch.float32)
+        B.grim_bcr_spmm(h, Xd, Yd)
+        ref = (gen.bf16_representable(W) * mask).astype(np.float64) @ X.astype(np.float64)
+        # bf16 products are exact in fp32; sums of a few thousand terms lose about sqrt(K) ulps, a bf16 result 2^-9
+        assert rel_fro(Yd.float().cpu().numpy(), ref) <= (3e-3 if y_bf16 else 1e-5)
+        assert B.grim_bcr_status(h) == 0
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 def test_conv_split_with_bias_and_relu(B):
     """A layer with few output pixels and many input channels takes the split path (separate bias / ReLU pass)."""
     L = gen.conv_layer(1, 96, 48, 9, ksize=3, bh=8, bw=32, compression=4, seed=86)
