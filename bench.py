@@ -316,8 +316,9 @@ class SpmmWorkload:
             # operands that are streamed from HBM every step (the rotating sets) are tuned with a cold L2 as well
             self.tuned = B.grim_bcr_tune(h, x, y, reps=-5 if self.rotating else 5)
         torch.cuda.synchronize()
-        names = {1: "bcr_ffma_kernel", 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
-                 3: "bcr_skinny_kernel" if self.tuned["tile_n"] == 1 else "bcr_stream_kernel"}
+        tile = self.tuned["tile_n"]
+        names = {1: "bcr_direct_kernel" if tile & 32 else "bcr_ffma_kernel", 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
+                 3: "bcr_narrow_kernel" if tile >= 4 else ("bcr_skinny_kernel" if tile == 1 else "bcr_stream_kernel")}
         self.kernel = names.get(self.tuned["path"], self.kernel)
         self.peak_kind = "tensor" if self.tuned["path"] in (2, 5) else "alu"
         if self.peak_kind == "tensor":
@@ -452,7 +453,7 @@ class ConvWorkload:
         self.min_bytes = float(i.value_bytes + min_index_bytes(i) + self.x.numel() * esz + self.y.numel() * esz)
         self.h2d = self.x_host.numel() * esz
         self.d2h = self.y_host.numel() * esz
-        self.kernel = "bcr_tc_kernel (implicit im2col)" if self.bf16 else "bcr_ffma_kernel (implicit im2col)"
+        self.kernel = "conv_tc_kernel (implicit im2col)" if self.bf16 else "bcr_direct_kernel (implicit im2col)"
         self.peak_kind = "tensor" if self.bf16 else "alu"
         self._ev = (torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
         self.sets = [(self.h, self.x, self.y)]
@@ -522,7 +523,7 @@ class VggWorkload:
         self.flops = sum(2.0 * int(L["mask"].sum()) * batch * L["hw"] * L["hw"] for L in self.net["layers"])
         self.peak_kind = "tensor"
         self.dense_elems = sum(int(L["mask"].size) for L in self.net["layers"])
-        self.kernel = "bcr_tc_kernel (implicit im2col, per layer)"
+        self.kernel = "conv_tc_kernel (implicit im2col, per layer)"
 
     def setup(self, B, torch):
         self.B, self.torch = B, torch

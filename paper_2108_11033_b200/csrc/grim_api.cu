@@ -48,6 +48,13 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
   if (path == 0 && tune && tune->tile_n >= 16) path = 4;  // a column-tile width only means something to the slab kernel
   SpmmArgs a = mat_args(X, Y);
   a.tile_n = tune ? tune->tile_n : 0;
+  auto align = [&]() {  // tensor cores, rows that TMA cannot fetch: copied to aligned ones where grim_bcr_reserve has made room
+    return a.ncols > kSkinnyMaxN && !tc_path_supported(h, a) && x_copy_possible(h, a) ? launch_x_copy(h, a, s) : GRIM_OK;
+  };
+  if (path == 2 || path == 5) {
+    st = align();
+    if (st != GRIM_OK) return st;
+  }
   if (path == 2) {
     if (!tc_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc(h, a, s);
@@ -80,13 +87,11 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
   if (path == 4) return launch_spmm(h, a, s);
   // bf16 handles, wide right-hand sides: tensor cores, except for small products, which the direct kernel has done before the
   // tensor-core kernels' start-up of some 14 us is over (1024^2, 8 x 32, N = 128: 15.3 -> 7.0 us).  Rows that TMA cannot fetch are
-  // copied to aligned ones first where grim_bcr_reserve has made room (3000^2, N = 333: 112 -> 33).
+  // copied first (3000^2, N = 333: 112 -> 33).
   if (path == 0 && a.x_dtype == GRIM_BF16 && a.ncols > kSkinnyMaxN) {
     if (direct_path_supported(h, a) && direct_time(h, a) <= 12.0) return launch_direct(h, a, s);
-    if (!tc_path_supported(h, a) && x_copy_possible(h, a)) {
-      const grim_status_t cs = launch_x_copy(h, a, s);
-      if (cs != GRIM_OK) return cs;
-    }
+    st = align();
+    if (st != GRIM_OK) return st;
   }
   // The paired kernel when its 256 x 512 tiles still give most
   // SMs a thread block (measured: with fewer, the single-block kernel's smaller tiles win).
@@ -294,10 +299,19 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   a.bias = d->bias_dev; a.relu = (d->flags & GRIM_CONV_RELU) ? 1 : 0;
   a.conv = 1; a.C = (int)d->C; a.H = (int)d->H; a.W = (int)d->W; a.KH = d->KH; a.KW = d->KW;
   a.stride = d->stride; a.pad = d->pad; a.OH = (int)OH; a.OW = (int)OW;
-  if (d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & kKernelFlags)) {
+  const bool one = d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & kKernelFlags);
+  const int64_t hw = d->H * d->W;
+  // 1 x 1 kernels on several images: a launch per image costs 6 us and more each, so all images go through one convolution -
+  // the gathering tensor-core kernel's where it can, the direct kernel's up to the image size from which a product per image
+  // is large enough (bf16: 32 images, 64 channels, 56 x 56: 187 -> 16 us; 512 channels, 7 x 7, 8 images: 25 -> 12;
+  // 28 x 28, 128 -> 512, 16 images: 118 -> 81 .. 122)
+  if (one && d->N > 1) {
+    if (conv_tc_supported(h, a)) return launch_conv_tc(h, a, (cudaStream_t)stream);
+    if (direct_path_supported(h, a) && (hw <= 1024 || (h->dtype == GRIM_F32 && hw <= 4096 && (h->bh > 4 || d->N >= 16)))) return launch_direct(h, a, (cudaStream_t)stream);
+  }
+  if (one) {
     // 1 x 1 kernels: the expanded input IS the input - per image a plain Cout x C times C x (H*W) product on the
     // tensors as they lie in memory (row stride H*W), no gather at all; one launch per image
-    const int64_t hw = d->H * d->W;
     const size_t in_esz = d->in_dtype == GRIM_BF16 ? 2 : 4, out_esz = d->out_dtype == GRIM_BF16 ? 2 : 4;
     for (int64_t n = 0; n < d->N; ++n) {
       SpmmArgs m;
