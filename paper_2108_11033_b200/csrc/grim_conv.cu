@@ -238,8 +238,6 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
     *s_abort = 0;
     fence_mbar_init();
   }
-  if (p.bias && p.M <= kBiasCap)
-    for (int i = tid; i < kBiasCap; i += (int)blockDim.x) s_bias[i] = i < p.M ? __ldg(p.bias + i) : 0.f;
   if (GATHER && tid >= 32 * kGather0 && tid < 32 * kGather0 + kK) {
     // k -> (channel, kh, kw); tap bits: kh in the low half, 16 + kw in the high half (none valid past the last k)
     const int k = tid - 32 * kGather0, khw = p.KH * p.KW;
@@ -260,7 +258,8 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
   if (CG == 2) cluster_sync_all();  // both blocks' barriers exist before either signals the other
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *s_tmem;
-  // the channel-last copy of the input (the launch before) is complete and visible from here on
+  // whatever earlier launches in the stream wrote - the channel-last copy of the input, the input, the biases - is complete and
+  // visible from here on; up to here only the packed matrix and this block's own shared memory were touched
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   bool failed = false;
@@ -432,6 +431,11 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
     // ------------------------------------------------------------------ epilogue: a lane holds one pixel
     const int quarter = warp & 3;  // the tensor-memory lanes this warp may read
     const int64_t ohw = (int64_t)p.OH * p.OW;
+    if (p.bias && p.M <= kBiasCap) {
+      constexpr int kEpiThreads = 32 * kEpiWarps * epi_groups(GATHER);
+      for (int i = tid - 32 * kEpi0; i < kBiasCap; i += kEpiThreads) s_bias[i] = i < p.M ? __ldg(p.bias + i) : 0.f;
+      named_barrier(1, kEpiThreads);
+    }
     // the accumulator has been read by this warp: the multiplies of a later tile may overwrite it once all warps say so
     auto release = [&](int acc) {
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -239,6 +239,34 @@ def test_tensor_core_convolution(B, geom, out_bf16):
     check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=True, out_bf16=out_bf16, kernel_flags=B.GRIM_CONV_TENSOR)
 
 
+@pytest.mark.parametrize("cin", [3, 16])
+def test_convolution_bias_from_the_call_before(B, cin):
+    """The biases are the result of a product issued just before on the same stream (few long bands: it runs long after its
+    launch has let the next one start); with and without the channel-last launch in between.  Bit for bit what the
+    convolution gives when the product has long been done."""
+    cout, Kb = 40, 60000
+    hb = B.grim_bcr_pack(gen.dense_weight(cout, Kb, seed=188), gen.bcr_mask(cout, Kb, 8, 32, compression=2, dist="uniform", seed=189), 8, 32, B.GRIM_F32, 0)
+    K = cin * 9
+    h = B.grim_bcr_pack(gen.dense_weight(cout, K, seed=190), gen.bcr_mask(cout, K, 8, 32, compression=3, dist="uniform", seed=191), 8, 32, B.GRIM_BF16, 0)
+    try:
+        xb = to_dev(gen.normal_f32((Kb, 1), 1.0, 192, 0))
+        x = to_dev(gen.normal_f32((2, cin, 20, 24), 1.0, 193, 0), True)
+        B.grim_bcr_reserve(h, 2 * 20 * 24)
+        bias, out, want = torch.empty(cout, 1, device="cuda"), torch.empty(2, cout, 20, 24, device="cuda"), torch.empty(2, cout, 20, 24, device="cuda")
+        B.grim_bcr_spmm(hb, xb, bias)
+        torch.cuda.synchronize()
+        B.grim_bcr_conv2d(h, x, want, 3, 1, 1, bias=bias, kernel_flags=B.GRIM_CONV_TENSOR)
+        for _ in range(20):
+            bias.fill_(1e6)
+            torch.cuda.synchronize()
+            B.grim_bcr_spmm(hb, xb, bias)
+            B.grim_bcr_conv2d(h, x, out, 3, 1, 1, bias=bias, kernel_flags=B.GRIM_CONV_TENSOR)
+            assert torch.equal(out, want)
+    finally:
+        B.grim_bcr_destroy(h)
+        B.grim_bcr_destroy(hb)
+
+
 @pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("hw", [(6, 10), (4, 8), (2, 24), (10, 16), (8, 32)])
 def test_maxpool_vector_widths(B, bf16, hw):
