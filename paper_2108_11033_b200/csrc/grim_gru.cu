@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
   const int gu = (warp - group * wg) * 32 + lane;
   const int g_tri = gu / p.bh, g_r = gu % p.bh;
   const int unit = rank * U + gu;
-  const bool gate_live = group < groups && gu < U && unit < H;  // (the last CTAs may own fewer groups of units, or none)
+  const bool gate_live = group < groups && gu < U && unit < H;  // (the last CTA may own fewer groups of units)
   const int dst0 = CS * group / groups, dst1 = CS * (group + 1) / groups;
   const bool stores = group == groups - 1;
   float bq[3] = {0.f, 0.f, 0.f};
@@ -460,7 +460,8 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
   // CTA of the cluster with asynchronous stores that count their bytes on the receiver's mbarrier; a warp starts a
   // step when the H values of that step have been counted.  No cluster-wide barrier and no fence per step: values of a
   // step leave a CTA only after all its warps have read the state before it (the block barrier below), and a buffer is
-  // written again only by CTAs that have received such values from everybody.
+  // written again only by CTAs that have received such values from everybody - so every CTA has to own units and send: one
+  // that does not could fall two steps behind and find the bytes of two states in one phase of its barrier.
   uint64_t* hbar = reinterpret_cast<uint64_t*>(partial + 2 * part_len);  // [2], 8-byte aligned (all counts are even)
   volatile int* s_failed = reinterpret_cast<volatile int*>(hbar + 2);
   if (tid == 0) *s_failed = 0;
@@ -860,7 +861,8 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
       const int max_cols = max_band_columns(g);
       const RegVariant* rv = nullptr;
       for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
-        const int tpc = (ntri + cs - 1) / cs, nb = 3 * tpc;
+        // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
+        const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc;
         double best = -1.0;
         ModeCfg shape;
         for (const RegVariant& v : kRegVariants)
@@ -872,7 +874,7 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
             const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
             if (best >= 0.0 && cost >= best) continue;
             ModeCfg t;
-            t.ctas = cs; t.ks = ks; t.tpc = tpc; t.resident = 1;
+            t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
             t.threads = std::max(32 * warps, std::max((tpc * bh + 31) / 32 * 32, 128));
             t.smem = ((((size_t)2 * H + (size_t)2 * nb * ks * BHc) * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
             if (t.smem > kSmemLimit || !cluster_fits(v.kern, t)) continue;

@@ -771,6 +771,16 @@ def test_gru_block_shapes_and_hidden_sizes(B, cfg):
     check_gru(B, gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=201), h0=gen.normal_f32((L, H), 0.5, 202, 0))
 
 
+@pytest.mark.parametrize("cfg", [(8, 136, 1, 60, 8, 32), (8, 528, 2, 90, 16, 64), (8, 592, 1, 60, 8, 32), (8, 260, 2, 100, 4, 16), (8, 392, 1, 61, 8, 32)])
+def test_gru_unit_groups_for_fewer_blocks_than_the_largest_cluster(B, cfg):
+    """17, 33, 74, 65 and 49 groups of units: dealt evenly to sixteen thread blocks they would leave seven, five, one, three
+    and three of them without any.  Many steps, repeated: nothing times out and the results are right."""
+    in_f, H, L, T, bh, bw = cfg
+    m = gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=8, seed=206)
+    for _ in range(3):
+        check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 207, 0))
+
+
 @pytest.mark.parametrize("cfg", [(37, 128, 2, 33, 4, 16), (20, 96, 1, 31, 16, 32), (64, 160, 3, 64, 16, 64), (9, 60, 2, 2, 5, 16), (500, 64, 2, 7, 8, 32)])
 def test_gru_batched_step_block_shapes(B, cfg):
     """Batches around a tile of 32 sequences, block heights, inputs wider and narrower than the state."""
