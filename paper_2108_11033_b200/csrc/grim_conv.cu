@@ -573,10 +573,7 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (*s_abort && tid == 0) {  // copies that were requested still land in this block's shared memory
-    for (int s = 0; s < ns; ++s)
-      for (unsigned i = 0; i < 4096u && !mbar_try_wait(full + s, 0) && !mbar_try_wait(full + s, 1); ++i) {}
-  }
+  if (*s_abort) let_copies_land();
   if (CG == 2) cluster_sync_all();  // neither block leaves (or frees tensor memory) while the other may still use its memory
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -103,6 +103,12 @@ __device__ __forceinline__ bool mbar_wait_tight(uint64_t* bar, unsigned parity, 
   if (__builtin_expect(CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity), 1)) return true;
   return mbar_wait<CLUSTER>(bar, parity, limit, abort_flag, sleep_ns);
 }
+// After a wait has run out: copies that were requested, and multiplies that read them, may still be on their way, and which is
+// not known any more (the phase of a barrier that nobody follows up says nothing).  The block stays for a time in which any
+// of them is done, some hundred times the latency of a copy, before it gives its memory back.
+__device__ __forceinline__ void let_copies_land() {
+  for (int i = 0; i < 200; ++i) __nanosleep(1000);
+}
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");

@@ -424,16 +424,14 @@ __global__ void __launch_bounds__(kFThreads, CW == 0 ? 2 : 1) bcr_ffma_kernel(co
   }
 
   if (failed) {
-    // a bounded wait ran out: tell every warp, record it, let copies that were requested land, leave
+    // a bounded wait ran out: tell every warp, record it, leave
     *s_abort = 1;
     if (lane == 0) atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
   }
   __syncthreads();
   if (p.follows) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (*s_abort) {
-    if (tid == 0)
-      for (int s = 0; s < NS; ++s)
-        for (unsigned i = 0; i < 4096u && !mbar_try_wait(full + s, 0) && !mbar_try_wait(full + s, 1); ++i) {}
+    let_copies_land();
     __syncwarp();
     if (split > 1) { cluster_sync_all(); cluster_sync_all(); }  // (the others' sums; they are of no use now)
     return;

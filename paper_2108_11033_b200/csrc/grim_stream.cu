@@ -360,9 +360,8 @@ __global__ void __launch_bounds__(NW * 32, 1) bcr_stream_kernel(const StreamPara
     __syncthreads();
   }
   if (failed) {
-    // copies that were requested still land in this block's shared memory: give them a bounded time to finish
-    for (int s = 0; s < nslots; ++s)
-      for (unsigned i = 0; i < 4096u && !mbar_try_wait(my_full + s, 0) && !mbar_try_wait(my_full + s, 1); ++i) {}
+    // copies that were requested still land in this block's shared memory
+    ptx::let_copies_land();
   }
 }
 

@@ -390,6 +390,7 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (*s_abort) let_copies_land();
   cluster_sync_all();  // neither block leaves (or frees tensor memory) while the other may still use its memory
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
