@@ -193,6 +193,10 @@ grim_status_t grim_bcr_unpack_dense(grim_bcr_t h, float* W_host, int64_t ldw);
  * the handle's value dtype; Y->dtype is GRIM_F32, or GRIM_BF16 for bf16 handles (rounded once,
  * after fp32 accumulation).  Y is fully overwritten (all M rows, beta = 0): rows kept by no
  * block are written as +0.  N = 1 selects the matrix-vector kernel.  X and Y must not overlap.
+ * Infinities and NaN in X: with at most 16 columns (and no explicit kernel choice, and a handle with the narrow layouts) they
+ * reach the rows whose weight at their position is kept, and no others.  Beyond that, results are defined for finite X: the
+ * tensor-core kernels (bf16 handles, products and convolutions) multiply pruned positions by zero, so that such a value makes
+ * NaN of its whole output column, and the CUDA-core kernels may turn an infinity into NaN in the rows that keep it.
  * Shape mismatch -> GRIM_ERR_SHAPE, dtype mismatch -> GRIM_ERR_DTYPE, both before any launch.
  * Asynchronous on `stream`; never allocates.  A handle is used on one stream at a time.  The kernels are launched
  * with programmatic stream serialization: their set-up may overlap the end of the launch before them on the stream,

@@ -56,7 +56,8 @@ __global__ void __launch_bounds__(NC == 4 ? 256 : 512, NC == 4 ? 2 : 1) bcr_dire
   if (pos < p.nbr) {
     WalkCols<NC, XV> wc;
     walk_setup<NC, XV, XT, CONV>(a, q0, lane, wc);
-    row_walk<BH, NC, XV, XT, CONV>(p.w, a, pos, part, p.parts, wc, wbuf, lane, acc1, acc2, wait_stream);
+    // (one column per lane: the few columns that the lane-per-column kernels, which touch nothing but kept weights, took before)
+    row_walk<BH, NC, XV, XT, CONV, NC == 1>(p.w, a, pos, part, p.parts, wc, wbuf, lane, acc1, acc2, wait_stream);
   } else {
     wait_stream();
   }

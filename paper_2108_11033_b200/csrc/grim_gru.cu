@@ -1267,7 +1267,7 @@ __global__ void __launch_bounds__(kStepWarps * 32, 1) gru_step_kernel(const Step
   WalkCols<1, 1> wc;
   walk_setup<1, 1, float, 0>(p.a[m], b0, lane, wc);
   const int pos = (int)__ldg(p.pos[m] + gate * ntri + tri);
-  row_walk<BH, 1, 1, float, 0>(p.w[m], p.a[m], pos, part, p.part[m], wc, ssm + warp * kWalkBufFloats, lane, acc1, acc2,
+  row_walk<BH, 1, 1, float, 0, false>(p.w[m], p.a[m], pos, part, p.part[m], wc, ssm + warp * kWalkBufFloats, lane, acc1, acc2,
                                [] { asm volatile("griddepcontrol.wait;" ::: "memory"); });
 #pragma unroll
   for (int r = 0; r < BH; ++r) sums[(warp * BH + r) * kStepLd + lane] = acc1[r];

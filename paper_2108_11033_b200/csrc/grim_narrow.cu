@@ -68,8 +68,33 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// A warp's sums, product by kept product: what the tensor core's cannot be used for when activations are not finite, because it
+// multiplies the rows of a band that do not keep a column by zero.  Lane l works out outputs l, l + 32, ...
+template <int BH, int NQ>
+__device__ __noinline__ void kept_products(const NParams& p, int pos, int part, int q0, int lane, float* mine) {
+  const unsigned short* vals = reinterpret_cast<const unsigned short*>(p.vals);
+  const unsigned short* X = static_cast<const unsigned short*>(p.X);
+  const int c0 = pos < p.nbr ? (int)__ldg(p.band_ptr + pos) + part : 0, c1 = pos < p.nbr ? (int)__ldg(p.band_ptr + pos + 1) : 0;
+  for (int i = lane; i < BH * NQ; i += 32) {
+    const int r = i / NQ, q = q0 + i % NQ;
+    float t = 0.f;
+    for (int c = c0; c < c1 && q < p.N; c += p.parts) {
+      const ChunkDesc d = p.chunks[c];
+      const uint32_t ncols = d.ncols_kr & 0xFFFFu;
+      for (uint32_t j = 0; j < ncols; ++j) {
+        const uint32_t w = __ldg(p.colwords + (size_t)c * 32 + j), rm = w >> 16;
+        if (!((rm >> r) & 1u)) continue;
+        const uint32_t v = vals[d.val_off + (uint32_t)__popc(rm & ((1u << r) - 1u)) * ncols + j];
+        const uint32_t x = X[(int64_t)(w & 0xFFFFu) * p.ldx + q];
+        t = fmaf(__uint_as_float(v << 16), __uint_as_float(x << 16), t);
+      }
+    }
+    mine[i] = t;
+  }
+}
+
 template <int BH, int NQ, typename VT>
-__global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 4 ? 1 : 2) bcr_narrow_kernel(const NParams p) {
+__global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 4 ? 1 : 2) bcr_narrow_kernel(const __grid_constant__ NParams p) {
   using S = Stage<BH, NQ, VT>;
   constexpr bool MMA = sizeof(VT) == 2;
   constexpr int D = S::kDepth;
@@ -235,6 +260,16 @@ __global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 
         const int m = (lane >> 2) + 8 * (i >> 1), n = 2 * (lane & 3) + (i & 1) + 8 * t;
         if (m < NQ && n < BH) mine[n * NQ + m] = frag[t][i];
       }
+    // an infinity or a NaN among the activations has reached every row of the band: those sums are not finite
+    bool finite = true;
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) finite = finite && fabsf(frag[t][i]) <= 3.4028234e38f;
+    if (!__all_sync(0xffffffffu, finite)) {
+      __syncwarp();
+      kept_products<BH, NQ>(p, pos, part, q0, lane, mine);
+    }
   }
   __syncthreads();
   for (int i = tid; i < bpc * BH * NQ; i += kNWarps * 32) {

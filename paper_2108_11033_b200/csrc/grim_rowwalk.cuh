@@ -74,11 +74,13 @@ __device__ __forceinline__ void walk_setup(const SpmmArgs& a, int64_t q0, int la
 
 // Accumulates block columns part, part + parts, ... of the band at schedule position pos into acc (pairs of the lane's
 // outputs; NC = 1 uses acc1).  wbuf: this warp's kWalkBufFloats floats.  before_x() runs once, after the first records
-// have been requested and before X is first read.
+// have been requested and before X is first read.  SKIP: padding columns of a chunk are not read and count as zero; otherwise
+// they read the block's first kept column again and meet zero weights, which makes a NaN of an infinity there.  (For every
+// product it would cost 3 to 4 % of the wider ones and of the GRU step.)
 //
 // One chunk is in flight ahead of the one that is multiplied.  (Two were measured: no gain, the copies between register
 // sets cost what the latency gave - these kernels issue instructions most of the time.)
-template <int BH, int NC, int XV, typename XT, int CONV, typename BeforeX>
+template <int BH, int NC, int XV, typename XT, int CONV, bool SKIP, typename BeforeX>
 __device__ __forceinline__ void row_walk(const RowWalk& w, const SpmmArgs& a, int pos, int part, int parts, const WalkCols<NC, XV>& wc,
                                          float* wbuf, int lane, float (&acc1)[NC == 1 ? BH : 1],
                                          unsigned long long (&acc2)[NC == 1 ? 1 : BH][NC == 1 ? 1 : NC / 2], BeforeX before_x) {
@@ -131,7 +133,8 @@ __device__ __forceinline__ void row_walk(const RowWalk& w, const SpmmArgs& a, in
   auto fetch_x = [&]() {
     int koff = 0;
     unsigned tap = 0;
-    const bool half = kc - ch * kRcChunk <= 4;  // nothing in the second half of the chunk
+    const int live = kc - ch * kRcChunk;  // columns of the chunk from here on are padding
+    const bool half = live <= 4;          // nothing in the second half of the chunk
     if (CONV) {
       // lanes 0 .. 7 take the chunk's columns apart into (channel, kh, kw)
       const int k = k0 + (int)(((lane & 4 ? c1 : c0) >> (8 * (lane & 3))) & 0xFFu);
@@ -150,11 +153,16 @@ __device__ __forceinline__ void row_walk(const RowWalk& w, const SpmmArgs& a, in
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
           float v = 0.f;
-          if ((wc.valid[c] & t) == t) v = to_f32(static_cast<const XT*>(wc.ptr[c / XV])[off]);
+          if ((!SKIP || e < live) && (wc.valid[c] & t) == t) v = to_f32(static_cast<const XT*>(wc.ptr[c / XV])[off]);
           x[e][c] = v;
         }
       } else {
         const uint32_t k = (uint32_t)k0 + (((e < 4 ? c0 : c1) >> (8 * (e & 3))) & 0xFFu);
+        if (SKIP && e >= live) {  // (uniform)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) x[e][c] = 0.f;
+          continue;
+        }
 #pragma unroll
         for (int v = 0; v < NC / XV; ++v) {
           const XT* src = reinterpret_cast<const XT*>(static_cast<const uint8_t*>(wc.ptr[v]) + (uint64_t)k * ldb);

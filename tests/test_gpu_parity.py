@@ -292,6 +292,42 @@ def test_gathering_kernel(B, case, parts, bf16):
     check_spmm(B, W, mask, X, bh, bw, bf16=bf16, path=3, tile_n=8 * parts, y_bf16=bf16 and parts == 2)
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("case", [(300, 700, 8, 32, 1), (300, 700, 8, 32, 3), (300, 700, 8, 32, 5), (304, 520, 4, 16, 7), (260, 700, 16, 64, 2), (260, 700, 16, 64, 6),
+                                  (129, 1333, 16, 64, 12), (520, 1040, 8, 32, 16), (304, 520, 4, 16, 16), (264, 700, 8, 32, 11), (2048, 2048, 8, 32, 6), (200, 300, 5, 20, 8)])
+def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
+    """At most sixteen columns: infinities and a NaN in X meet the rows whose weight at their column is kept, and no other."""
+    M, K, bh, bw, N = case
+    W = gen.dense_weight(M, K, seed=311)
+    W[np.abs(W) < 1e-3] = 0.01  # (a kept weight of zero would make a NaN of an infinity)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=4, dist="zipf", seed=312, empty_frac=0.2)
+    mask[:bh] = 0
+    X = gen.normal_f32((K, N), 1.0, 313, 0)
+    X = gen.bf16_representable(X) if bf16 else X
+    used = np.flatnonzero(mask.any(axis=0))
+    X[used[3], 0], X[used[len(used) // 2], N // 2], X[used[-1], N - 1] = np.inf, -np.inf, np.nan
+    Wd = gen.bf16_representable(W) if bf16 else W
+    h = B.grim_bcr_pack(W, mask, bh, bw, B.GRIM_BF16 if bf16 else B.GRIM_F32, 0)
+    try:
+        Yd = torch.full((M, N), 7.0, device="cuda")
+        B.grim_bcr_spmm(h, to_dev(X, bf16), Yd)
+        got = Yd.cpu().numpy()
+    finally:
+        B.grim_bcr_destroy(h)
+    fin = np.isfinite(X)
+    want = (Wd * mask).astype(np.float64) @ np.where(fin, X, 0.0).astype(np.float64)
+    for k, q in zip(*np.nonzero(~fin)):
+        rows = mask[:, k] != 0
+        with np.errstate(invalid="ignore"):
+            want[rows, q] += Wd[rows, k].astype(np.float64) * X[k, q]
+    bad = ~np.isfinite(want)
+    assert bad.any() and not bad.all()
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
+    # finite results as ever: bf16 products are exact in fp32, sums of some hundred terms lose about sqrt(K) ulps of their terms
+    scale = np.linalg.norm(Wd * mask, axis=1)[:, None] * np.linalg.norm(np.where(fin, X, 0.0), axis=0)[None, :]
+    assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
+
+
 @pytest.mark.parametrize("split", [2, 5, 8])
 def test_split_multiply(B, split):
     """Few output tiles: several thread blocks share a tile's block columns and add their partial sums into a
