@@ -121,6 +121,7 @@ cudaError_t launch_rows(const DParams& p, int nc, int xv, dim3 grid, cudaStream_
 bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   if (h->device < 0 || !h->d_rc_head) return false;
   if (a.ncols <= 0 || a.ncols > (int64_t(1) << 31) - 256) return false;
+  if ((h->nbr + kDWarps - 1) / kDWarps > 65535) return false;  // bands are dealt to the grid's second dimension
   if (!a.conv && a.x_sk * (a.x_dtype == GRIM_F32 ? 4 : 2) >= (int64_t(1) << 32)) return false;
   if (a.conv && (a.KH > 16 || a.KW > 16 || (int64_t)a.C * a.H * a.W >= (int64_t(1) << 31))) return false;
   return true;

@@ -211,6 +211,24 @@ def test_direct_kernel_explicit(B, case, bf16):
 
 
 @pytest.mark.parametrize("bf16", [False, True])
+def test_more_bands_than_the_direct_kernel_takes(B, bf16):
+    """Half a million rows in blocks of one row, rows of X that TMA cannot fetch: the other CUDA-core kernels take them."""
+    M, K, N = 524288 + 24, 32, 17
+    W = gen.normal_f32((M, K), 1.0, 178, 0)
+    mask = (gen.normal_f32((M, K), 1.0, 179, 0) > 0.7).astype(np.uint8)
+    X = gen.normal_f32((K, N), 1.0, 180, 0)
+    if bf16:
+        W, X = gen.bf16_representable(W), gen.bf16_representable(X)
+    h = B.grim_bcr_pack(W, mask, 1, 32, B.GRIM_BF16 if bf16 else B.GRIM_F32, 0)
+    try:
+        Y = torch.full((M, N), float("nan"), device="cuda")
+        B.grim_bcr_spmm(h, to_dev(X, bf16), Y)
+        assert rel_fro(Y.cpu().numpy(), (W * mask).astype(np.float64) @ X.astype(np.float64)) <= F32_TOL
+    finally:
+        B.grim_bcr_destroy(h)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("geom", [(3, 1, 1, 9, 13), (3, 2, 1, 15, 8), (5, 1, 2, 7, 7), (1, 2, 0, 9, 9), (16, 3, 5, 21, 19), (2, 1, 0, 6, 33)])
 def test_direct_kernel_convolution(B, geom, bf16):
     ksize, stride, pad, hh, ww = geom
