@@ -36,13 +36,9 @@ grim_tune_t* tuned_slot(grim_bcr_t h, const grim_mat_t* X, const grim_mat_t* Y) 
   return &h->tuned[b][X->dtype == GRIM_BF16 ? 1 : 0][Y->dtype == GRIM_BF16 ? 1 : 0];
 }
 
-grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const grim_tune_t* tune, cudaStream_t s) {
-  grim_status_t st = check_mats(h, X, Y);
-  if (st != GRIM_OK) return st;
-  if (!tune) {  // no explicit choice: an earlier grim_bcr_tune for this kind of request decides
-    const grim_tune_t* t = tuned_slot(h, X, Y);
-    if (t->path != 0) tune = t;
-  }
+// The product by the given choice of kernel (null: by the library's rules); operands already checked.
+grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const grim_tune_t* tune, cudaStream_t s) {
+  grim_status_t st = GRIM_OK;
   int path = tune ? tune->path : 0;
   if (path < 0 || path > 5) return GRIM_ERR_INVALID_ARG;
   if (path == 0 && tune && tune->tile_n >= 16) path = 4;  // a column-tile width only means something to the slab kernel
@@ -103,6 +99,20 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
   if (path == 0 && tc_path_supported(h, a) && a.ncols > kSkinnyMaxN) return launch_spmm_tc(h, a, s);
   if (path == 1) return ffma_path_supported(h, a) ? launch_ffma(h, a, s) : GRIM_ERR_UNSUPPORTED;
   return launch_cuda_cores(h, a, s);
+}
+
+grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const grim_tune_t* tune, cudaStream_t s) {
+  grim_status_t st = check_mats(h, X, Y);
+  if (st != GRIM_OK) return st;
+  if (tune) return run_choice(h, X, Y, tune, s);
+  // no explicit choice: an earlier grim_bcr_tune for this kind of request decides, unless its kernel cannot take these operands
+  // (it was found with others, whose alignment or strides may differ)
+  const grim_tune_t* t = tuned_slot(h, X, Y);
+  if (t->path != 0) {
+    st = run_choice(h, X, Y, t, s);
+    if (st != GRIM_ERR_UNSUPPORTED) return st;
+  }
+  return run_choice(h, X, Y, nullptr, s);
 }
 
 int dev_sms() {

@@ -346,6 +346,26 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+def test_tuned_choice_that_cannot_take_the_operands(B):
+    """Tuned on aligned rows (a tensor-core kernel wins); a product of the same kind whose rows start at odd elements, with no
+    workspace to copy them to, runs all the same."""
+    M, K, N = 2048, 2048, 512
+    W, mask = gen.dense_weight(M, K, seed=321), gen.bcr_mask(M, K, 8, 32, compression=4, dist="uniform", seed=322)
+    X = gen.bf16_representable(gen.normal_f32((K, N), 1.0, 323, 0))
+    h = B.grim_bcr_pack(W, mask, 8, 32, B.GRIM_BF16, 0)
+    try:
+        Y = torch.empty(M, N, device="cuda")
+        Xa = to_dev(X, True)
+        assert B.grim_bcr_tune(h, Xa, Y)["path"] in (2, 5)
+        Xu = torch.empty(K, N + 1, device="cuda", dtype=torch.bfloat16)[:, 1:]
+        Xu.copy_(Xa)
+        Y.fill_(float("nan"))
+        B.grim_bcr_spmm(h, Xu, Y)
+        assert rel_fro(Y.cpu().numpy(), (gen.bf16_representable(W) * mask).astype(np.float64) @ X.astype(np.float64)) <= F32_TOL
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 @pytest.mark.parametrize("split", [2, 5, 8])
 def test_split_multiply(B, split):
     """Few output tiles: several thread blocks share a tile's block columns and add their partial sums into a
