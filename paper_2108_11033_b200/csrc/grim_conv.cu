@@ -685,6 +685,7 @@ size_t conv_scratch_bytes(const grim_bcr* h, int64_t max_ncols) {
     const ConvLayout& l = h->conv[i];
     if (!l.d_w) continue;
     const size_t same = (size_t)max_ncols * padded_channels((int)(h->K / l.taps)) * 2;  // stride 1: as many input pixels as outputs
+    if (same > ((size_t)1 << 30)) continue;  // beyond what grim_bcr_reserve allocates: such calls run on other kernels
     need = std::max(need, std::max(same, std::min(4 * same, (size_t)512 << 20)));       // stride 2: four times as many
   }
   return need;

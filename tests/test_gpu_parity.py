@@ -346,6 +346,22 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+def test_reserve_stays_within_its_limit(B):
+    """Few output channels, many input channels: M x max_ncols is within the limit, the channel-last copy would be 8 GiB."""
+    K = 512 * 9
+    h = B.grim_bcr_pack(gen.dense_weight(32, K, seed=324), gen.bcr_mask(32, K, 8, 32, compression=8, dist="uniform", seed=325), 8, 32, B.GRIM_BF16, 0)
+    try:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        B.grim_bcr_reserve(h, (1 << 30) // (32 * 4))
+        assert free - torch.cuda.mem_get_info()[0] <= (1 << 30) + (64 << 20)
+        with pytest.raises(B.GrimError) as e:
+            B.grim_bcr_reserve(h, (1 << 30) // (32 * 4) + 1)
+        assert e.value.status == B.GRIM_ERR_UNSUPPORTED
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 def test_tuned_choice_that_cannot_take_the_operands(B):
     """Tuned on aligned rows (a tensor-core kernel wins); a product of the same kind whose rows start at odd elements, with no
     workspace to copy them to, runs all the same."""
