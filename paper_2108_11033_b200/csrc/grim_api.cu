@@ -274,9 +274,10 @@ extern "C" grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols) {
   if ((size_t)h->M * (size_t)max_ncols * 4 > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;
   const size_t acc = (size_t)h->M * (size_t)((max_ncols + 3) / 4 * 4) * 4;
   // the split multiply only takes outputs of at most half a tile per SM, which is less than 40 MiB
-  const size_t need = (std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols)) + 255) / 256 * 256;
-  const size_t copy = x_copy_size(h, max_ncols);
+  size_t need = (std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols)) + 255) / 256 * 256;
+  size_t copy = x_copy_area(h, max_ncols);
   if (h->tc_acc_bytes >= need && h->x_copy_bytes >= copy && need > 0) return GRIM_OK;
+  if (need > 0) need = std::max(need, h->tc_acc_bytes), copy = std::max(copy, h->x_copy_bytes);  // neither part shrinks
   if (cudaDeviceSynchronize() != cudaSuccess) return GRIM_ERR_CUDA;  // a launch in flight may still use the old scratch
   cudaFree(h->d_tc_acc);
   h->d_tc_acc = nullptr;

@@ -228,6 +228,7 @@ bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab 
 double direct_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us (plain products)
 // bf16 handles: a copy of X with aligned rows for the tensor-core kernels, where the scratch for it is there
 size_t x_copy_size(const grim_bcr* h, int64_t ncols);
+size_t x_copy_area(const grim_bcr* h, int64_t max_ncols);  // what is reserved for copies of up to max_ncols columns
 bool x_copy_possible(const grim_bcr* h, const SpmmArgs& a);
 grim_status_t launch_x_copy(const grim_bcr* h, SpmmArgs& a, cudaStream_t s);  // a.X and a.x_sk become the copy's
 double slab_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us

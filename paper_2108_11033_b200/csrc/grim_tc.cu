@@ -520,9 +520,9 @@ constexpr size_t kMaxCopy = (size_t)64 << 20;
 
 size_t x_copy_size(const grim_bcr* h, int64_t ncols) {
   if (h->dtype != GRIM_BF16 || ncols <= kSkinnyMaxN) return 0;
-  const size_t n = (size_t)h->K * (size_t)((ncols + 7) / 8 * 8) * 2;
-  return n <= kMaxCopy ? n : 0;
+  return (size_t)h->K * (size_t)((ncols + 7) / 8 * 8) * 2;
 }
+size_t x_copy_area(const grim_bcr* h, int64_t max_ncols) { return std::min(x_copy_size(h, max_ncols), kMaxCopy); }
 
 bool x_copy_possible(const grim_bcr* h, const SpmmArgs& a) {
   if (a.conv || a.x_dtype != GRIM_BF16 || a.x_sq != 1 || a.ncols > (1 << 30)) return false;

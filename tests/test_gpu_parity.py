@@ -346,6 +346,26 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+def test_reserve_of_more_columns_keeps_what_fewer_had(B):
+    """An area for rows made aligned and one for the channel-last copy, whatever was reserved before or after: K x 7840 columns
+    are more than the former may hold, 333 columns are not."""
+    K = 512 * 9
+    h = B.grim_bcr_pack(gen.dense_weight(128, K, seed=326), gen.bcr_mask(128, K, 8, 32, compression=8, dist="uniform", seed=327), 8, 32, B.GRIM_BF16, 0)
+    try:
+        X, Y = torch.zeros(K, 333, device="cuda", dtype=torch.bfloat16), torch.empty(128, 333, device="cuda")
+        x, y = torch.zeros(10, 512, 28, 28, device="cuda", dtype=torch.bfloat16), torch.empty(10, 128, 28, 28, device="cuda")
+        for ncols in ((7840,), (333, 7840), (7840, 333), (7840, 16)):
+            B.grim_bcr_reserve(h, 0)
+            for n in ncols:
+                B.grim_bcr_reserve(h, n)
+            B.grim_bcr_spmm_ex(h, X, Y, path=2)  # (refused where the rows cannot be copied)
+            B.grim_bcr_conv2d(h, x, y, 3, 1, 1, kernel_flags=B.GRIM_CONV_TENSOR)
+        torch.cuda.synchronize()
+        assert B.grim_bcr_status(h) == 0 and not Y.any() and not y.any()
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 def test_reserve_stays_within_its_limit(B):
     """Few output channels, many input channels: M x max_ncols is within the limit, the channel-last copy would be 8 GiB."""
     K = 512 * 9
