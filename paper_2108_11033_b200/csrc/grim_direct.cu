@@ -145,8 +145,11 @@ bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
     // Few columns leave most lanes idle, so the time goes with the number of chunks (about 2.5 us and 0.3 ns each).  Against
     // the gathering kernel, which has more to set up: up to some 5000 chunks (1024^2, 8 x 32, N = 7: 3.4 against 5.2; 512^2:
     // 3.0 against 5.2), and where that one needs two passes up to 17000 (2048^2, 16 x 64, N = 16: 6.7 against 7.6).
-    // (handles that hold only the wide regime's layouts refuse fewer than eight columns, as grim.h says)
-    if (a.ncols < 8 && (h->flags & GRIM_PACK_WIDE_ONLY)) return false;
+    // Handles that hold only the wide regime's layouts go on refusing what grim.h says they refuse: they only take these widths
+    // from eight columns on, and where the tensor-core tile or the slab kernel's narrow tile is there for them.
+    if ((h->flags & GRIM_PACK_WIDE_ONLY) && h->gemv_ok &&
+        (a.ncols < 8 || !(h->dtype == GRIM_F32 ? h->bh >= 8 && ffma_path_supported(h, a) : tc_path_supported(h, a) && h->tc_mtiles >= 8)))
+      return false;
     if (a.x_dtype == GRIM_BF16 && a.ncols >= 8) return !h->d_chunks && h->rc_chunks <= 5000;
     return h->rc_chunks <= (h->bh > 8 && a.ncols > 8 ? 17000 : 5000) && a.ncols >= 5;
   }

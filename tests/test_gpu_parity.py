@@ -346,6 +346,25 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+@pytest.mark.parametrize("case", [(300, 4, 16, False, 7, False), (300, 4, 16, False, 12, False), (300, 8, 32, False, 7, False), (300, 8, 32, False, 12, True),
+                                  (300, 8, 32, True, 12, False), (1100, 8, 32, True, 16, True), (300, 8, 32, True, 17, True)])
+def test_wide_handles_refuse_few_columns(B, case):
+    """Handles with only the wide layouts: the widths, block heights and sizes that they refuse, and those that they take."""
+    M, bh, bw, bf16, N, takes = case
+    h = B.grim_bcr_pack(gen.dense_weight(M, 400, seed=328), gen.bcr_mask(M, 400, bh, bw, compression=8, dist="uniform", seed=329), bh, bw,
+                        B.GRIM_BF16 if bf16 else B.GRIM_F32, B.GRIM_PACK_WIDE_ONLY)
+    try:
+        X, Y = torch.zeros(400, N, device="cuda", dtype=torch.bfloat16 if bf16 else torch.float32), torch.empty(M, N, device="cuda")
+        if takes:
+            B.grim_bcr_spmm(h, X, Y)
+        else:
+            with pytest.raises(B.GrimError) as e:
+                B.grim_bcr_spmm(h, X, Y)
+            assert e.value.status == B.GRIM_ERR_UNSUPPORTED
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 def test_reserve_of_more_columns_keeps_what_fewer_had(B):
     """An area for rows made aligned and one for the channel-last copy, whatever was reserved before or after: K x 7840 columns
     are more than the former may hold, 333 columns are not."""
