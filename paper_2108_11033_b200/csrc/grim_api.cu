@@ -59,11 +59,11 @@ grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const
     if (!tc2_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
     return launch_spmm_tc2(h, a, s);
   }
-  if (path == 3 && a.tile_n >= 4) {
-    if (a.tile_n != 4 && a.tile_n != 8 && a.tile_n != 16 && a.tile_n != 32 && a.tile_n != 64) return GRIM_ERR_INVALID_ARG;
+  // (other values under paths 1 and 3 mean the default, as they did before these kernels had numbers)
+  if (path == 3 && a.ncols > 1 && (a.tile_n == 4 || a.tile_n == 8 || a.tile_n == 16 || a.tile_n == 32 || a.tile_n == 64)) {
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, a.tile_n == 4 ? 0 : a.tile_n / 8, s);
   }
-  if (path == 1 && (a.tile_n & 32)) return launch_direct(h, a, s);
+  if (path == 1 && direct_choice(a.tile_n)) return launch_direct(h, a, s);
   if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
   if (path == 0 && narrow_preferred(h, X->cols))
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, 0, s);
@@ -220,7 +220,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
     grim_tune_t c{};
     c.path = cd[0];
     c.tile_n = cd[1];
-    if (c.path == 3 && X->cols > kSkinnyMaxN) continue;
+    if (c.path == 3 && (X->cols > kSkinnyMaxN || (c.tile_n == 4 && X->cols == 1))) continue;
     if (c.path == 4 && c.tile_n > 16 && c.tile_n / 2 >= X->cols) continue;  // idle lanes only
     // CUDA-core kernel: 1, 2, 4 = bands per warp; 8, 9 = two 128-column pieces per lane with one or two bands per warp
     if (c.path == 1 && c.tile_n <= 4 && c.tile_n > (h->bh <= 4 ? 4 : (h->bh <= 8 ? 2 : 1))) continue;

@@ -118,6 +118,13 @@ cudaError_t launch_rows(const DParams& p, int nc, int xv, dim3 grid, cudaStream_
 
 }  // namespace
 
+// 32, or 32 + columns per lane + 256 * warps per band
+bool direct_choice(int tile_n) {
+  if (tile_n == 32) return true;
+  const int nc = tile_n % 256 - 32, parts = tile_n / 256;
+  return tile_n > 0 && (nc == 1 || nc == 2 || nc == 4) && (parts == 1 || parts == 2 || parts == 4 || parts == 8 || (parts == 16 && nc < 4));
+}
+
 bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   if (h->device < 0 || !h->d_rc_head) return false;
   if (a.ncols <= 0 || a.ncols > (int64_t(1) << 31) - 256) return false;
@@ -172,10 +179,8 @@ grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s
   const int BHc = h->bh <= 4 ? 4 : (h->bh <= 8 ? 8 : 16);
   const int sms = sm_count(h->device);
   int nc, parts;
-  if (a.tile_n > 32) {  // explicit choice: 32 + columns per lane + 256 * warps per band
+  if (a.tile_n > 32 && direct_choice(a.tile_n)) {
     nc = a.tile_n % 32; parts = a.tile_n / 256;
-    if ((nc != 1 && nc != 2 && nc != 4) || (parts != 1 && parts != 2 && parts != 4 && parts != 8 && !(parts == 16 && nc < 4))) return GRIM_ERR_INVALID_ARG;
-    if (a.conv && nc == 1) nc = 2;
   } else {
     auto warps = [&](int n) { return ((a.ncols + 32 * n - 1) / (32 * n)) * h->nbr; };
     nc = a.ncols <= 32 && !a.conv ? 1 : 2;

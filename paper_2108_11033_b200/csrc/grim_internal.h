@@ -237,6 +237,7 @@ grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream
 // small and middle-sized products without a block-wide pipeline (also convolutions)
 grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a);
+bool direct_choice(int tile_n);  // grim_tune_t::tile_n asks for this kernel (path 1)
 bool direct_preferred(const grim_bcr* h, const SpmmArgs& a);  // over the other CUDA-core kernels, for this request
 grim_status_t launch_spmm_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool tc_path_supported(const grim_bcr* h, const SpmmArgs& a);

@@ -346,6 +346,14 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+@pytest.mark.parametrize("choice", [(1, 544, 40), (1, 33, 40), (1, 96, 40), (1, 128, 40), (1, 1056, 40), (3, 4, 1), (3, 8, 1), (3, 5, 7), (3, 12, 7), (3, 128, 7)])
+def test_tile_values_without_a_meaning_run_the_default(B, choice):
+    """Values of tile_n that name no tile of the path, or one for other widths."""
+    path, tile_n, N = choice
+    W, mask = gen.dense_weight(200, 520, seed=331), gen.bcr_mask(200, 520, 8, 32, compression=4, dist="uniform", seed=332)
+    check_spmm(B, W, mask, gen.normal_f32((520, N), 1.0, 333, 0), 8, 32, path=path, tile_n=tile_n)
+
+
 @pytest.mark.parametrize("case", [(300, 4, 16, False, 7, False), (300, 4, 16, False, 12, False), (300, 8, 32, False, 7, False), (300, 8, 32, False, 12, True),
                                   (300, 8, 32, True, 12, False), (1100, 8, 32, True, 16, True), (300, 8, 32, True, 17, True)])
 def test_wide_handles_refuse_few_columns(B, case):
