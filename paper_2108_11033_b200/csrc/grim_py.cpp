@@ -53,9 +53,12 @@ bool parse(const char* fn, const char* const* names, int n, int required, PyObje
   return true;
 }
 
+// The integer that grim_bcr_pack and grim_gru_create return, None, or a ctypes.c_void_p.
 bool to_handle(PyObject* o, void** out) {
-  if (o == Py_None) { *out = nullptr; return true; }
-  *out = PyLong_AsVoidPtr(o);
+  PyObject* value = !PyLong_Check(o) && o != Py_None && PyObject_HasAttrString(o, "value") ? PyObject_GetAttrString(o, "value") : nullptr;
+  if (value) o = value;
+  *out = o == Py_None ? nullptr : PyLong_AsVoidPtr(o);
+  Py_XDECREF(value);
   return !(*out == nullptr && PyErr_Occurred());
 }
 
@@ -120,7 +123,7 @@ bool to_opt_ptr(const char* fn, PyObject* o, void** out) {
   return true;
 }
 
-// None: torch's current stream; an object with a cuda_stream attribute; or the stream's address.
+// None: torch's current stream; an object with a cuda_stream attribute; or the stream's address, as anything int() takes.
 bool to_stream(PyObject* o, grim_stream_t* out) {
   if (!o || o == Py_None) {
     *out = (grim_stream_t)c10::cuda::getCurrentCUDAStream().stream();
@@ -130,10 +133,10 @@ bool to_stream(PyObject* o, grim_stream_t* out) {
   if (PyLong_Check(o)) {
     p = PyLong_AsVoidPtr(o);
   } else {
-    PyObject* attr = PyObject_GetAttrString(o, "cuda_stream");
-    if (!attr) return false;
-    p = PyLong_AsVoidPtr(attr);
-    Py_DECREF(attr);
+    PyObject* number = PyObject_HasAttrString(o, "cuda_stream") ? PyObject_GetAttrString(o, "cuda_stream") : PyNumber_Long(o);
+    if (!number) return false;
+    p = PyLong_AsVoidPtr(number);
+    Py_DECREF(number);
   }
   if (!p && PyErr_Occurred()) return false;
   *out = (grim_stream_t)p;

@@ -346,6 +346,27 @@ def test_non_finite_activations_reach_only_rows_that_keep_them(B, case, bf16):
     assert np.all(np.abs(got[~bad] - want[~bad]) <= 1e-5 * scale[~bad])
 
 
+def test_handles_and_streams_in_other_forms(B):
+    """A handle as a ctypes pointer; a stream as a torch stream, its address, or a number that is not a Python int."""
+    import ctypes
+    W, mask = gen.dense_weight(64, 96, seed=334), gen.bcr_mask(64, 96, 8, 32, compression=4, dist="uniform", seed=335)
+    X = gen.normal_f32((96, 24), 1.0, 336, 0)
+    h = B.grim_bcr_pack(W, mask, 8, 32, B.GRIM_F32, 0)
+    try:
+        want, Xd, s = (W * mask).astype(np.float64) @ X.astype(np.float64), to_dev(X), torch.cuda.Stream()
+        for handle, stream in ((ctypes.c_void_p(h), None), (h, s), (h, s.cuda_stream), (h, np.int64(s.cuda_stream))):
+            Y = torch.empty(64, 24, device="cuda")
+            torch.cuda.synchronize()
+            B.grim_bcr_spmm(handle, Xd, Y, stream)
+            torch.cuda.synchronize()
+            assert rel_fro(Y.cpu().numpy(), want) <= F32_TOL
+        for handle, stream in ((2.5, None), ("h", None), (h, "s")):
+            with pytest.raises((TypeError, ValueError)):
+                B.grim_bcr_spmm(handle, Xd, Y, stream)
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 @pytest.mark.parametrize("choice", [(1, 544, 40), (1, 33, 40), (1, 96, 40), (1, 128, 40), (1, 1056, 40), (3, 4, 1), (3, 8, 1), (3, 5, 7), (3, 12, 7), (3, 128, 7)])
 def test_tile_values_without_a_meaning_run_the_default(B, choice):
     """Values of tile_n that name no tile of the path, or one for other widths."""
