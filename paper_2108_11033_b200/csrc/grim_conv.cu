@@ -6,8 +6,9 @@
 // Two launches.  conv_nhwc_kernel turns the NCHW input channel-last in a scratch of the handle (one pass, channels padded
 // to a multiple of 8).  conv_tc_kernel then is a plain pipeline: TMA fetches the tile of input pixels of a tap straight
 // from the channel-last copy (im2col mode: the copy engine walks rows and images, applies stride and padding), TMA fetches
-// the tile of the expanded weights, one thread issues the multiplies, eight warps store the results.  Pixels are the rows
-// of the multiply, so a lane of the epilogue holds one pixel and a warp's store of one channel is contiguous in NCHW.
+// the tile of the expanded weights, one thread issues the multiplies, sixteen warps store the results (eight where others
+// gather).  Pixels are the rows of the multiply, so a lane of the epilogue holds one pixel and a warp's store of one channel
+// is contiguous in NCHW.
 // Convolutions whose whole K fits one tile of 64 (few input channels: the first layer of a network) skip the
 // channel-last copy: warps gather the tile of pixels from the NCHW input.
 //
@@ -96,7 +97,7 @@ struct ConvParams {
   int n_tile, n_stride, nacc;        // output channels per tile; tensor-memory columns between accumulators; 2 or 4 of them
   int resident;                      // the weights of all K tiles stay in shared memory (one tile of output channels)
   int c_end;                         // a multiple of g past the last channel
-  int g, cblocks, nsub;              // channels per copy of input pixels, copies per tap, taps * cblocks
+  int g, cblocks;                    // channels per copy of input pixels, copies per tap
   int M, KH, KW, stride, pad, OH, OW;
   int C, H, W, K;
   int ksplit, kt_per;                // > 1: a cluster of ksplit blocks shares a tile, each multiplies kt_per K tiles
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
 #pragma unroll
           for (int j = 0; j < KPS; ++j)
 #pragma unroll
-            for (int s = 0; s < (GATHER ? 4 : kK / 16); ++s)
+            for (int s = 0; s < kK / 16; ++s)
               mma_bf16<CG>(d, ad0 + (off + (uint32_t)j * kt16 + step[s]), bd0 + (boff + (uint32_t)j * bstep + 2u * s), idesc, j + s > 0 ? 1u : more);
           mma_commit<CG>(empty + slot);
           more = 1u;
@@ -713,7 +714,7 @@ grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
   p.nkt = l.nkt; p.npt = pl.npt; p.nnt = pl.nnt; p.n_tile = pl.n_tile; p.ksplit = pl.ksplit; p.kt_per = pl.kt_per;
   p.nacc = pl.n_tile <= 128 ? 4 : 2;
   p.n_stride = pl.n_tile <= 32 ? 32 : (pl.n_tile <= 64 ? 64 : (pl.n_tile <= 128 ? 128 : 256));
-  p.g = l.g; p.cblocks = l.cblocks; p.nsub = l.taps * l.cblocks;
+  p.g = l.g; p.cblocks = l.cblocks;
   p.M = (int)h->M; p.KH = a.KH; p.KW = a.KW; p.stride = a.stride; p.pad = a.pad; p.OH = a.OH; p.OW = a.OW;
   p.c_end = (a.C + l.g - 1) / l.g * l.g;
   p.C = a.C; p.H = a.H; p.W = a.W; p.K = (int)h->K;
