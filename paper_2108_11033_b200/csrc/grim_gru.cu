@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <new>
+#include <numeric>
 
 #include "grim_device.cuh"
 #include "grim_internal.h"
@@ -399,7 +400,8 @@ __global__ void __launch_bounds__(1024, 1) gru_cluster_kernel(const GruParams p)
 // NI = items per warp, THREADS = the most threads a variant is launched with.  What bounds a step is a chain of latencies
 // (gather, sums, reduction, gates, exchange), in which the issue of a scheduler's warps is the largest part that the shape
 // decides: the variant with the fewest issued instructions per step is taken.  Shapes that need more slots than the compiled
-// menu use the other kernels.  No variant's weights may spill: reloading them every step cost more than any schedule gains.
+// menu use the other kernels.  The menu's sizes are what registers hold: reloading weights every step costs more than any
+// schedule gains.  (Three of the widest spill a little: <16, 1, 8, 384> 88 bytes a thread, <4, 4, 7, 384> 36, <4, 6, 8, 256> 8.)
 // ---------------------------------------------------------------------------------------------
 template <int BH, int NI, int S, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruParams p) {
@@ -871,8 +873,8 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
       for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
         // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
         const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc;
-        double best = -1.0;
-        ModeCfg shape;
+        struct Candidate { double cost; const RegVariant* v; ModeCfg shape; };
+        std::vector<Candidate> cands;
         for (const RegVariant& v : kRegVariants)
           for (int ks = 1; ks <= 8; ks *= 2) {
             const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
@@ -880,15 +882,19 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
             // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
             // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
             const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
-            if (best >= 0.0 && cost >= best) continue;
             ModeCfg t;
             t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
             t.threads = std::max(32 * warps, std::max((tpc * bh + 31) / 32 * 32, 128));
             t.smem = ((((size_t)2 * H + (size_t)2 * nb * ks * BHc) * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
-            if (t.smem > kSmemLimit || !cluster_fits(v.kern, t)) continue;
-            best = cost; shape = t; rv = &v;
+            if (t.smem <= kSmemLimit) cands.push_back({cost, &v, t});
           }
-        if (best >= 0.0) { shape.ok = true; g->regc = shape; g->reg_kern = rv->kern; }
+        // (asked in the order of their costs: the question costs more than all else here)
+        std::stable_sort(cands.begin(), cands.end(), [](const Candidate& x, const Candidate& y) { return x.cost < y.cost; });
+        for (const Candidate& c : cands)
+          if (cluster_fits(c.v->kern, c.shape)) {
+            rv = c.v; g->regc = c.shape; g->regc.ok = true; g->reg_kern = rv->kern;
+            break;
+          }
       }
       if (g->regc.ok) {
         // register image: for every thread of every CTA the columns it owns (global index + values at row positions); threads
@@ -897,8 +903,9 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
         const size_t nval = (size_t)cs * NI * S * BHc * TH, ncol = (size_t)cs * NI * S2 * TH;
         std::vector<float> iv(nval);
         std::vector<uint32_t> ic(ncol);
-        struct ColRec { uint32_t col; float v[16]; };
-        std::vector<ColRec> cols;
+        struct ColRec { uint32_t col, rowmask, kc; const float* v; };  // kept row a (of rowmask) has v[a * kc]
+        std::vector<ColRec> cols, dealt;
+        std::vector<size_t> before;  // columns dealt before each round
         for (int l = 0; l < layers && st == GRIM_OK; ++l) {
           const grim_bcr* wh = W_hh[l];
           std::fill(iv.begin(), iv.end(), 0.f);
@@ -914,14 +921,7 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
                 int bidx = 0;
                 for (int c = 0; c < wh->bw; ++c) {
                   if (!((hb.colmask >> c) & 1ull)) continue;
-                  ColRec cr;
-                  cr.col = (uint32_t)(j * wh->bw + c);
-                  int a = 0;
-                  for (int r = 0; r < 16; ++r) {
-                    cr.v[r] = 0.f;
-                    if ((hb.rowmask >> r) & 1u) cr.v[r] = wh->vals[(size_t)hb.val_off + (size_t)(a++) * hb.kc + (size_t)bidx];
-                  }
-                  cols.push_back(cr);
+                  cols.push_back({(uint32_t)(j * wh->bw + c), hb.rowmask, hb.kc, &wh->vals[(size_t)hb.val_off + (size_t)bidx]});
                   ++bidx;
                 }
               }
@@ -931,19 +931,34 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
                 const size_t c0 = n * part / ks, c1 = n * (part + 1) / ks;
                 // dealt so that the 32 columns of a slot fall into different shared-memory banks as far as they go (any 32 of
                 // a thousand meet three or four to a bank): one from every bank's pile in turn, the longest piles first
-                std::vector<size_t> pile[32], deal;
-                for (size_t ci = c0; ci < c1; ++ci) pile[cols[ci].col % 32].push_back(ci);
-                std::stable_sort(pile, pile + 32, [](const std::vector<size_t>& x, const std::vector<size_t>& y) { return x.size() > y.size(); });
-                for (size_t r = 0; deal.size() < c1 - c0; ++r)
-                  for (const auto& pl : pile)
-                    if (pl.size() > r) deal.push_back(pl[r]);
-                for (size_t k = 0; k < deal.size(); ++k) {
-                  const size_t ci = deal[k];
+                size_t size[32] = {}, place[32];
+                int bank[32];
+                for (size_t ci = c0; ci < c1; ++ci) ++size[cols[ci].col % 32];
+                std::iota(bank, bank + 32, 0);
+                std::stable_sort(bank, bank + 32, [&](int x, int y) { return size[x] > size[y]; });
+                // column number r of a pile comes after those of earlier rounds and, in its round, of longer piles
+                dealt.resize(c1 - c0);
+                size_t taken[32] = {};
+                for (int b = 0; b < 32; ++b) place[bank[b]] = (size_t)b;
+                const size_t rounds = size[bank[0]];
+                before.assign(rounds + 1, 0);
+                for (int b = 0; b < 32; ++b)
+                  for (size_t r = 0; r < size[b]; ++r) ++before[r + 1];
+                for (size_t r = 0; r < rounds; ++r) before[r + 1] += before[r];
+                for (size_t ci = c0; ci < c1; ++ci) {
+                  const int b = (int)(cols[ci].col % 32);
+                  dealt[before[taken[b]++] + place[b]] = cols[ci];
+                }
+                for (size_t k = 0; k < dealt.size(); ++k) {
+                  const ColRec& cr = dealt[k];
                   const int sl = (int)(k / 32), tid = warp * 32 + (int)(k % 32);
                   if (sl >= S || tid >= TH) { st = GRIM_ERR_UNSUPPORTED; break; }
-                  ic[((size_t)(rank * NI + i) * S2 + sl / 2) * TH + tid] |= cols[ci].col << (16 * (sl & 1));
-                  for (int r = 0; r < BHc; ++r)
-                    iv[((((size_t)(rank * NI + i) * S + sl) * (BHc / 2) + r / 2) * TH + tid) * 2 + (r & 1)] = cols[ci].v[r];
+                  ic[((size_t)(rank * NI + i) * S2 + sl / 2) * TH + tid] |= cr.col << (16 * (sl & 1));
+                  const float* v = cr.v;
+                  for (uint32_t rm = cr.rowmask; rm; rm &= rm - 1, v += cr.kc) {
+                    const int r = __builtin_ctz(rm);
+                    iv[((((size_t)(rank * NI + i) * S + sl) * (BHc / 2) + r / 2) * TH + tid) * 2 + (r & 1)] = *v;
+                  }
                 }
               }
             }
