@@ -929,6 +929,35 @@ def test_gru_block_shapes_and_hidden_sizes(B, cfg):
     check_gru(B, gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=201), h0=gen.normal_f32((L, H), 0.5, 202, 0))
 
 
+def test_recurrent_kernel_tanh(B):
+    """One step from a zero state on a zero input, update gate shut by its bias: the new state is tanh of the third gate's
+    bias, element by element.  The kernel states 2.1 units in the last place against tanh itself; magnitudes from where tanh(x)
+    is x to where it is 1, dense around the place where the two formulas meet."""
+    H = 1024
+    m = gen.gru_model(16, H, 1, 1, bh=8, bw=32, compression=10, seed=209)
+    lay = m["layers"][0]
+    ih, hh = (B.grim_bcr_pack(lay[w], lay[k], 8, 32, B.GRIM_F32, 0) for w, k in (("W_ih", "mask_ih"), ("W_hh", "mask_hh")))
+    rng = np.random.default_rng(210)
+    points = [np.geomspace(1e-30, 20.0, H), np.linspace(0.45, 0.55, H), np.linspace(0.0, 0.6, H), np.linspace(0.5, 10.0, H)]
+    points += [rng.uniform(0.3, 3.0, H) for _ in range(4)]
+    try:
+        x, y = torch.zeros(1, 16, device="cuda"), torch.empty(1, H, device="cuda")
+        worst = 0.0
+        for v in points:
+            v = (v * rng.choice([-1.0, 1.0], H)).astype(np.float32)
+            b_ih = np.concatenate([np.zeros(H), np.full(H, -200.0), v]).astype(np.float32)
+            g = B.grim_gru_create([ih], [hh], [b_ih], [np.zeros(3 * H, np.float32)], 1)
+            B.grim_gru_seq(g, x, y)
+            assert B.grim_gru_status(g) == B.GRIM_OK
+            want = np.tanh(v.astype(np.float64))
+            worst = max(worst, float(np.max(np.abs(y[0].cpu().numpy() - want) / np.spacing(np.abs(want).astype(np.float32)))))
+            B.grim_gru_destroy(g)
+        assert worst <= 2.1, worst
+    finally:
+        B.grim_bcr_destroy(ih)
+        B.grim_bcr_destroy(hh)
+
+
 @pytest.mark.parametrize("cfg", [(8, 136, 1, 60, 8, 32), (8, 528, 2, 90, 16, 64), (8, 592, 1, 60, 8, 32), (8, 260, 2, 100, 4, 16), (8, 392, 1, 61, 8, 32)])
 def test_gru_unit_groups_for_fewer_blocks_than_the_largest_cluster(B, cfg):
     """17, 33, 74, 65 and 49 groups of units: dealt evenly to sixteen thread blocks they would leave seven, five, one, three
