@@ -723,20 +723,23 @@ bool plan_slab(const grim_bcr* h, const SpmmArgs& a, SlabPlan& pl) {
   // shared by clusters that split the block columns.  Of the ways to do that - one cluster size for all, or pairs for as
   // many as run at once and another size for the rest - the one that takes the least time is chosen, in stages: a split
   // costs about four more (the meeting of the sums).
-  const int64_t slots = cw ? sms : 2 * sms;  // narrow tiles are light: two thread blocks share an SM
+  // (narrow tiles are light: two thread blocks share an SM where their rings fit)
+  const int per_sm = cw == 0 && 2 * (smem_need(h, bpw, esz, slab_ld_for(a, tma, cw), kNarrowStages) + 1024) <= 228 * 1024 ? 2 : 1;
+  const int64_t slots = (int64_t)per_sm * sms;
   if (a.tile_n >= 256) {  // test / tuning override
     pl.seg[pl.nseg++] = {tiles, std::max(1, std::min(kMaxSplit, a.tile_n / 256))};
     pl.stages = tiles * h->nbc / slots;
   } else {
     const int64_t tail = tiles % slots;
-    // clusters that run at once: they do not straddle the GPU's partitions (of 148 SMs 74 x 2, 45 x 3, 33 x 4, 15 x 8)
-    auto at_once = [&](int c) {
-      return std::max<int64_t>(1, (c == 1 ? sms : (c == 2 ? sms / 2 : (c == 3 ? sms * 45 / 148 : (c == 4 ? sms * 33 / 148 : sms * 15 / 148)))) * (slots / sms));
-    };
+    // clusters that run at once: they do not straddle the GPU's partitions (what the runtime reports for 148 SMs).  Sizes five and
+    // six matter where a few dozen tiles would need two rounds of larger clusters (2217 x 6212, N = 32: 65.5 with four, 47 with
+    // six, 71 with eight); seven fits no better than eight.
+    static const int kAtOnce[2][9] = {{0, 148, 74, 45, 33, 26, 22, 15, 15}, {0, 296, 148, 93, 71, 56, 45, 37, 33}};
+    auto at_once = [&](int c) { return std::max<int64_t>(1, (int64_t)sms * kAtOnce[per_sm - 1][c] / 148); };
     int best_c = 1;
     auto best = [&](int64_t n) {  // stages that n tiles take, and the cluster size for it
       int64_t t = INT64_MAX;
-      for (int c : {1, 2, 3, 4, 8}) {
+      for (int c : {1, 2, 3, 4, 5, 6, 8}) {
         if (c > 1 && h->nbc < 4 * c) break;
         const int64_t cost = (n + at_once(c) - 1) / at_once(c) * ((h->nbc + c - 1) / c + (c > 1 ? 4 : 0));
         if (cost < t) { t = cost; best_c = c; }
@@ -763,12 +766,16 @@ bool plan_slab(const grim_bcr* h, const SpmmArgs& a, SlabPlan& pl) {
 
 bool slab_rows_by_tma(const SpmmArgs& a) { return tma_eligible(a); }
 
-// Microseconds: about five to start, and per stage what the slower of copying and multiplying takes.
+// Microseconds: about five to start, and per stage what the slower of copying and multiplying takes; gathering a slab element by
+// element (0.33 ns each) overlaps with little (4096^2, N = 131: 8 x 32 2.9 us a stage, 16 x 64 3.6, 4 x 16 1.6).  Narrow tiles: one.
 double slab_time(const grim_bcr* h, const SpmmArgs& a) {
   SlabPlan pl;
   if (!ffma_path_supported(h, a) || !plan_slab(h, a, pl)) return 1e30;
-  const double per_stage = (double)h->nnz / ((double)h->rc_groups * (double)h->nbc) * pl.bpw * tile_cols(pl.cw);
-  return 5.0 + (double)pl.stages * std::max(pl.cw == 2 ? 0.53 : 0.66, 0.35 + 7.8e-6 * per_stage);
+  const double products = (double)h->nnz / ((double)h->rc_groups * (double)h->nbc) * pl.bpw * tile_cols(pl.cw);
+  const double multiply = 0.35 + 7.8e-6 * products;
+  double stage = std::max(pl.cw == 2 ? 0.53 : (pl.cw == 1 ? 0.66 : 1.05), multiply);
+  if (!tma_eligible(a)) stage = std::max(stage, 0.2 + 0.33e-3 * h->bw * tile_cols(pl.cw) + 0.1 * multiply);
+  return 5.0 + (double)pl.stages * stage;
 }
 
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a) {

@@ -473,6 +473,15 @@ def test_slab_kernel_whole_and_split_tiles(B, case):
     check_spmm(B, W, mask, X, bh, bw, path=1, tile_n=tile)
 
 
+@pytest.mark.parametrize("case", [(2300, 1030, 32, 8, 32), (2840, 1030, 30, 8, 32), (5630, 1025, 60, 16, 64), (2300, 1030, 12, 8, 32), (1000, 2050, 300, 4, 16)])
+def test_slab_kernel_few_tiles(B, case):
+    """Eighteen to thirty tiles, which clusters of five and six blocks share where the next size would take two rounds."""
+    M, K, N, bh, bw = case
+    W = gen.dense_weight(M, K, seed=85)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=8, dist="uniform", seed=84, empty_frac=0.2)
+    check_spmm(B, W, mask, gen.normal_f32((K, N), 1.0, 83, 0), bh, bw, path=1, tile_n=17 if N <= 16 else 0)
+
+
 @pytest.mark.parametrize("case", [(300, 5000, 24, 33, 1), (1100, 1300, 257, 257, 0), (700, 900, 40, 41, 3), (520, 1203, 1024, 1025, 2), (264, 6000, 17, 19, 0)])
 @pytest.mark.parametrize("y_bf16", [False, True])
 def test_tensor_core_rows_made_aligned(B, case, y_bf16):
