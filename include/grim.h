@@ -66,7 +66,9 @@ typedef struct {
 #define GRIM_PACK_HOST_ONLY 2u /* build host-side data only (no CUDA call); compute calls then fail */
 /* A handle normally uploads one private device layout per kernel regime (3 - 4 x the compact size in device memory).
  * A handle that will only see narrow right-hand sides (N <= 16, GRU matrices) or only wide ones can say so and keep
- * just that regime's layouts; a multiply outside the regime then returns GRIM_ERR_UNSUPPORTED. */
+ * just that regime's layouts; a multiply outside the regime then returns GRIM_ERR_UNSUPPORTED.  bf16 handles with the wide
+ * layouts whose K is a multiple of 9 or 25, or at most 64, also hold the weights expanded for tensor-core convolutions: about
+ * M x K x 2 bytes for each that applies, none where that is more than 64 MiB. */
 #define GRIM_PACK_NARROW_ONLY 4u
 #define GRIM_PACK_WIDE_ONLY 8u
 
@@ -212,10 +214,10 @@ grim_status_t grim_bcr_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, gr
  * sides of up to max_ncols columns (for a convolution: images x OH x OW), once, at set-up time; it synchronises the
  * device.  Without it (or beyond max_ncols) such calls simply run on other kernels, slower.  A bf16 right-hand side whose rows are not
  * multiples of 16 bytes is copied to rows that are (up to 64 MiB).  max_ncols = 0 frees it.
- * M x max_ncols x 4 of more than 2^30 bytes -> GRIM_ERR_UNSUPPORTED.  What is allocated: the larger of the partial sums (M x
- * max_ncols x 4 bytes, at most 40 MiB) and, for bf16 handles whose K is C x 9 or C x 25, the channel-last copy (max_ncols x C x 2
- * bytes, four times that up to 512 MiB so that stride 2 fits; none where max_ncols x C x 2 is more than 2^30); then the
- * aligned rows (K x max_ncols x 2, at most 64 MiB). */
+ * M x max_ncols x 4 of more than 2^30 bytes -> GRIM_ERR_UNSUPPORTED.  What is allocated: the partial sums (M x max_ncols x 4 bytes,
+ * at most 40 MiB) and, bf16 handles, the aligned rows (K x max_ncols x 2, at most 64 MiB), or, for bf16 handles whose K is C x 9
+ * or C x 25, the channel-last copy if that is more (max_ncols x C x 2 bytes, four times that up to 512 MiB so that stride 2 fits;
+ * none where max_ncols x C x 2 is more than 2^30). */
 grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols);
 
 /* The multiply kernels bound every device-side wait (on a shared-memory barrier that an asynchronous copy

@@ -272,20 +272,26 @@ extern "C" grim_status_t grim_bcr_reserve(grim_bcr_t h, int64_t max_ncols) {
   if (!h || max_ncols < 0) return GRIM_ERR_INVALID_ARG;
   if (h->device < 0) return GRIM_ERR_INVALID_ARG;
   if ((size_t)h->M * (size_t)max_ncols * 4 > ((size_t)1 << 30)) return GRIM_ERR_UNSUPPORTED;
-  const size_t acc = (size_t)h->M * (size_t)((max_ncols + 3) / 4 * 4) * 4;
-  // the split multiply only takes outputs of at most half a tile per SM, which is less than 40 MiB
-  size_t need = (std::max(std::min(acc, (size_t)40 << 20), conv_scratch_bytes(h, max_ncols)) + 255) / 256 * 256;
-  size_t copy = x_copy_area(h, max_ncols);
-  if (h->tc_acc_bytes >= need && h->x_copy_bytes >= copy && need > 0) return GRIM_OK;
-  if (need > 0) need = std::max(need, h->tc_acc_bytes), copy = std::max(copy, h->x_copy_bytes);  // neither part shrinks
+  // partial sums (the split multiply only takes outputs of at most half a tile per SM, which is less than 40 MiB) and behind them the
+  // aligned rows; the channel-last copy of a convolution, which needs neither, may take all of it.  No part shrinks.
+  auto up = [](size_t n) { return (n + 255) / 256 * 256; };
+  size_t acc = up(std::min((size_t)h->M * (size_t)((max_ncols + 3) / 4 * 4) * 4, (size_t)40 << 20));
+  size_t copy = x_copy_area(h, max_ncols), all = std::max(up(conv_scratch_bytes(h, max_ncols)), acc + copy);
+  if (acc > 0) {
+    if (h->tc_acc_bytes >= acc && h->x_copy_bytes >= copy && h->scratch_bytes >= all) return GRIM_OK;
+    acc = std::max(acc, h->tc_acc_bytes);
+    copy = std::max(copy, h->x_copy_bytes);
+    all = std::max(std::max(all, h->scratch_bytes), acc + copy);
+  }
   if (cudaDeviceSynchronize() != cudaSuccess) return GRIM_ERR_CUDA;  // a launch in flight may still use the old scratch
   cudaFree(h->d_tc_acc);
   h->d_tc_acc = nullptr;
-  h->tc_acc_bytes = h->x_copy_bytes = 0;
-  if (need == 0) return GRIM_OK;
-  if (cudaMalloc((void**)&h->d_tc_acc, need + copy) != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_ALLOC; }
-  h->tc_acc_bytes = need;
+  h->tc_acc_bytes = h->x_copy_bytes = h->scratch_bytes = 0;
+  if (acc == 0) return GRIM_OK;
+  if (cudaMalloc((void**)&h->d_tc_acc, all) != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_ALLOC; }
+  h->tc_acc_bytes = acc;
   h->x_copy_bytes = copy;
+  h->scratch_bytes = all;
   return GRIM_OK;
 }
 

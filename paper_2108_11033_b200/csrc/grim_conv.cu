@@ -697,7 +697,7 @@ bool conv_tc_supported(const grim_bcr* h, const SpmmArgs& a) {
   if (a.ncols > (int64_t(1) << 31) - 512 || (int64_t)a.C * a.H * a.W >= (int64_t(1) << 31) || !encode_tiled_fn()) return false;
   if (gathers(h)) return true;
   if (a.KH != a.KW || a.stride > 8 || a.pad > 127 || a.H > 65535 || a.W > 65535 || images_of(a) > 65535 || (a.C + 63) / 64 > 65535) return false;
-  return h->d_tc_acc && h->tc_acc_bytes >= nhwc_bytes(a) && encode_im2col_fn();
+  return h->d_tc_acc && h->scratch_bytes >= nhwc_bytes(a) && encode_im2col_fn();
 }
 
 grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {

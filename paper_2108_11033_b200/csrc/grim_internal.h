@@ -169,12 +169,11 @@ struct grim_bcr {
   grim::RcStage* d_td_stage = nullptr;
   uint8_t* d_td_blob = nullptr;
   grim::ConvLayout conv[grim::kConvLayouts];
-  // scratch that grim_bcr_reserve allocates: partial sums of the split tensor-core multiply (M x N fp32), or the
-  // channel-last copy of a convolution's input
+  // scratch that grim_bcr_reserve allocates, scratch_bytes in all: the channel-last copy of a convolution's input, or partial sums
+  // of the split tensor-core multiply (M x N fp32, tc_acc_bytes) and behind them an aligned copy of a bf16 right-hand side whose
+  // rows TMA cannot fetch as they lie (x_copy_bytes)
   float* d_tc_acc = nullptr;
-  size_t tc_acc_bytes = 0;
-  // ... and, behind it, an aligned copy of a bf16 right-hand side whose rows TMA cannot fetch as they lie
-  size_t x_copy_bytes = 0;
+  size_t scratch_bytes = 0, tc_acc_bytes = 0, x_copy_bytes = 0;
   // answers of grim_bcr_tune, one per (log2 bucket of N, X dtype, Y dtype); path 0 = not tuned
   grim_tune_t tuned[32][2][2] = {};
   unsigned* d_status = nullptr;  // error word written by kernels whose bounded waits ran out
