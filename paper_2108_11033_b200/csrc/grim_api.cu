@@ -65,7 +65,7 @@ grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const
   }
   if (path == 1 && direct_choice(a.tile_n)) return launch_direct(h, a, s);
   if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
-  if (path == 0 && narrow_preferred(h, X->cols))
+  if (path == 0 && narrow_preferred(h, a))
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, 0, s);
   // handles without the narrow layouts, and fp32 handles with 16-row blocks: the tensor-core tile, the 16-column tile of the
   // slab kernel
@@ -81,11 +81,13 @@ grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const
     return launch_skinny(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, s);
   }
   if (path == 4) return launch_spmm(h, a, s);
-  // bf16 handles, wide right-hand sides: tensor cores, except for small products, which the direct kernel has done before the
-  // tensor-core kernels' start-up of some 14 us is over (1024^2, 8 x 32, N = 128: 15.3 -> 7.0 us).  Rows that TMA cannot fetch are
-  // copied first (3000^2, N = 333: 112 -> 33).
+  // bf16 handles, wide right-hand sides: tensor cores, except for small products, which the direct kernel is estimated to have done
+  // earlier (tensor cores against direct: 1024^2, 8 x 32, N = 128: 15.3 - 7.0; 6400 x 256, N = 96: 6.8 - 13.1; 728 x 448, N = 512: 10.7 -
+  // 14.1; 1018 x 3008, 16 x 64, N = 64: 14.5 - 17.8).  A tensor-core product of little work takes about 5 us and 0.65 per K tile, up to
+  // 16 (a long K is split), and where rows that TMA cannot fetch are copied first (3000^2, N = 333: 112 -> 33) 5 more.
   if (path == 0 && a.x_dtype == GRIM_BF16 && a.ncols > kSkinnyMaxN) {
-    if (direct_path_supported(h, a) && direct_time(h, a) <= 12.0) return launch_direct(h, a, s);
+    const double tc_time = std::min(5.0 + 0.65 * (double)h->tc_ktiles, 16.0) + (tc_path_supported(h, a) ? 0.0 : 5.0);
+    if (direct_path_supported(h, a) && direct_time(h, a) <= tc_time) return launch_direct(h, a, s);
     st = align();
     if (st != GRIM_OK) return st;
   }

@@ -134,40 +134,71 @@ bool direct_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   return true;
 }
 
+namespace {
+// Columns per lane and warps per band: enough warps to hide latency (some 16 per SM), four columns where that does not leave too
+// much of the last tile unused.
+struct Shape { int nc, parts; };
+Shape shape_for(const grim_bcr* h, const SpmmArgs& a) {
+  const int sms = sm_count(h->device);
+  auto warps = [&](int n) { return ((a.ncols + 32 * n - 1) / (32 * n)) * h->nbr; };
+  Shape s{a.ncols <= 32 && !a.conv ? 1 : 2, 1};
+  if (a.ncols > 64 && warps(4) >= sms && 4 * ((a.ncols + 127) / 128) * 4 <= 5 * 2 * ((a.ncols + 63) / 64)) s.nc = 4;
+  while (s.parts < (s.nc == 4 ? 8 : 16) && warps(s.nc) * s.parts * 2 <= (int64_t)sms * 16 && h->nbc >= 2 * s.parts) s.parts *= 2;
+  return s;
+}
+}  // namespace
+
+// What a warp does one after the other (its chunks), what all warps issue (chunks and bands times tiles).  Fitted to 400 products and
+// 340 convolutions of 100 .. 8192 rows, 200 .. 8192 columns of W, N of 2 to 1024, rates 4 to 16: nine in ten within 15 %.
 double direct_time(const grim_bcr* h, const SpmmArgs& a) {
-  const bool few = a.ncols <= 64;
-  const double per_chunk = h->bh <= 4 ? (few ? 0.29e-3 : 0.33e-3) : (h->bh <= 8 ? (few ? 0.44e-3 : 0.5e-3) : (few ? 0.6e-3 : 1.0e-3));
-  return 4.0 + per_chunk * (double)h->rc_chunks * (double)((a.ncols + 127) / 128);
+  const Shape s = shape_for(h, a);
+  const int b = h->bh <= 4 ? 0 : (h->bh <= 8 ? 1 : 2);
+  const double tiles = (double)((a.ncols + 32 * s.nc - 1) / (32 * s.nc)) * s.nc;  // of 32 columns
+  const double serial = (double)h->rc_chunks / ((double)h->nbr * s.parts), chunks = (double)h->rc_chunks * tiles * 1e-3, bands = (double)h->nbr * tiles * 1e-3;
+  if (a.conv) {
+    static const double c[2][3][4] = {{{2.3, 0.47, 0.10, 1.0}, {2.6, 0.95, 0.14, 1.8}, {3.3, 1.9, 0.09, 4.4}},     // fp32
+                                      {{2.2, 0.59, 0.16, 1.0}, {3.1, 0.92, 0.30, 1.8}, {4.1, 1.9, 0.23, 4.4}}};   // bf16
+    const double* v = c[a.x_dtype == GRIM_BF16][b];
+    return v[0] + v[1] * serial + v[2] * chunks + v[3] * bands;
+  }
+  static const double c[2][3][4] = {{{1.8, 0.62, 0.06, 1.3}, {1.7, 0.86, 0.02, 2.8}, {2.5, 1.04, 0.02, 6.5}},      // N <= 64
+                                    {{1.95, 0.41, 0.06, 0.4}, {2.25, 0.66, 0.06, 1.3}, {3.0, 1.04, 0.08, 5.0}}};  // wider
+  const double* v = c[a.ncols > 64][b];
+  return v[0] + v[1] * serial + v[2] * chunks + v[3] * bands;
 }
 
-// Where the direct kernel is the faster of the CUDA-core kernels (measured on square matrices of 512 to 8192, pruning rate
-// 8, the three block shapes; times in us, slab kernel -> direct kernel).
+// Where the direct kernel is the faster of the CUDA-core kernels.
 bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
   if (!direct_path_supported(h, a)) return false;
-  const double flops = 2.0 * (double)h->nnz * (double)a.ncols;
   // Convolutions: the slab kernel's gather costs more than it saves at every size (512 channels, 28 x 28: one image
   // 86 -> 63, 32 images 1320 -> 1220; 64 channels, 112 x 112: 58 -> 26; 5 x 5 on 96 channels, 17 x 23: 416 -> 18).
   if (a.conv) return true;
   if (a.ncols <= kSkinnyMaxN) {
-    // Few columns leave most lanes idle, so the time goes with the number of chunks (about 2.5 us and 0.3 ns each).  Against
-    // the gathering kernel, which has more to set up: up to some 5000 chunks (1024^2, 8 x 32, N = 7: 3.4 against 5.2; 512^2:
-    // 3.0 against 5.2), and where that one needs two passes up to 17000 (2048^2, 16 x 64, N = 16: 6.7 against 7.6).
+    // Few columns leave most lanes idle and the chunks of a warp are walked one after the other; the gathering kernel has more to
+    // set up (about 4 us) but takes 32 columns of W at a time, and where it needs two passes some 11 us per million weights
+    // (1024^2, 8 x 32, N = 7: 3.4 against 5.2; 4032^2 at rate 16, 16 x 64, N = 14: 11.8 against 16.8; 640 x 5952, N = 16: 15.9
+    // against 8.6; 256 x 8128, N = 11: 37.7 against 17.5).
     // Handles that hold only the wide regime's layouts go on refusing what grim.h says they refuse: they only take these widths
     // from eight columns on, and where the tensor-core tile or the slab kernel's narrow tile is there for them.
     if ((h->flags & GRIM_PACK_WIDE_ONLY) && h->gemv_ok &&
         (a.ncols < 8 || !(h->dtype == GRIM_F32 ? h->bh >= 8 && ffma_path_supported(h, a) : tc_path_supported(h, a) && h->tc_mtiles >= 8)))
       return false;
-    if (a.x_dtype == GRIM_BF16 && a.ncols >= 8) return !h->d_chunks && h->rc_chunks <= 5000;
-    return h->rc_chunks <= (h->bh > 8 && a.ncols > 8 ? 17000 : 5000) && a.ncols >= 5;
+    if (a.ncols < 5 || (a.x_dtype == GRIM_BF16 && a.ncols >= 8 && h->d_chunks)) return false;
+    // (fp32, 16-row blocks, more than eight columns: whatever takes them otherwise needs longer)
+    const double other = h->dtype == GRIM_F32 && h->bh > 8 && a.ncols > 8 ? std::min(narrow_time(h, a.ncols), slab_time(h, a)) : 0.0;
+    return direct_time(h, a) <= std::max(5.0, 1.1 * other);
   }
-  // The slab kernel needs rows of X that TMA can fetch; its other loaders are slow (N = 1023: 1477 -> 1213, N = 131 in
-  // bf16: 328 -> 30), except that a slab row of 16-row bands is used often enough to pay for them in large products.
-  if (!slab_rows_by_tma(a)) return a.x_dtype == GRIM_BF16 || h->bh <= 8 || flops <= 1e9;
-  // Otherwise: whichever is estimated to be done first.  The direct kernel's time goes with the chunks and 128-column tiles
-  // (0.33, 0.5 and 1.0 ns each for 4, 8 and 16 rows, less for up to 64 columns), the slab kernel's with the stages it takes one after the other.
-  // (1024^2, N = 128: 6.4 against 11; 2048^2, 4 x 16, N = 256: 44 against 26; 8 x 32: 23 against 22; 4096 x 1024, N = 256:
-  // 26 against 21; 1024 x 4096: 22 against 33.)
-  return direct_time(h, a) <= slab_time(h, a);
+  // bf16: the slab kernel widens what it gathers, element by element, where TMA cannot fetch the rows (N = 131: 328 -> 30)
+  if (a.x_dtype == GRIM_BF16 && !slab_rows_by_tma(a)) return true;
+  // X stored column by column (the GRU's inputs where they are not turned around): a lane's loads do not coalesce, so wide ones are
+  // better gathered (GRU step of a batch of 64, 4 x 16: 184 against 155; 48: equal; 32: 84 against 150; 8 x 32: 99 against 172 at
+  // 64; a sequence of 400 steps 1320 against 1297)
+  if (a.x_sq != 1) return a.ncols <= (h->bh <= 4 ? 48 : 384) && (h->bh <= 8 || 2.0 * (double)h->nnz * (double)a.ncols <= 1e9);
+  // Otherwise: whichever is estimated to be done first.  The slab kernel's time goes with the stages it takes one after the other
+  // (slab against direct: 1024^2, N = 128: 11 - 6.4; 2048^2, 4 x 16, N = 256: 26 - 42; N = 131: 59 - 82; 4096^2, 8 x 32, N = 64: 36 -
+  // 32; 8192^2, 4 x 16, N = 32: 347 - 420; 1664 x 896, 16 x 64, N = 1000: 28 - 46).
+  // The estimate of the gathering loader is the less certain one.
+  return direct_time(h, a) <= slab_time(h, a) * (slab_rows_by_tma(a) ? 1.0 : 1.15);
 }
 
 grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
@@ -182,11 +213,8 @@ grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s
   if (a.tile_n > 32 && direct_choice(a.tile_n)) {
     nc = a.tile_n % 32; parts = a.tile_n / 256;
   } else {
-    auto warps = [&](int n) { return ((a.ncols + 32 * n - 1) / (32 * n)) * h->nbr; };
-    nc = a.ncols <= 32 && !a.conv ? 1 : 2;
-    if (a.ncols > 64 && warps(4) >= sms && 4 * ((a.ncols + 127) / 128) * 4 <= 5 * 2 * ((a.ncols + 63) / 64)) nc = 4;
-    parts = 1;
-    while (parts < (nc == 4 ? 8 : 16) && warps(nc) * parts * 2 <= (int64_t)sms * 16 && h->nbc >= 2 * parts) parts *= 2;
+    const Shape shape = shape_for(h, a);
+    nc = shape.nc; parts = shape.parts;
   }
   p.parts = parts;
   int xv = 1;

@@ -220,11 +220,12 @@ bool stream_path_supported(const grim_bcr* h, int64_t N);
 grim_status_t launch_narrow(const grim_bcr* h, const void* X, int x_dtype, int64_t ldx, int64_t N, void* Y, int y_dtype, int64_t ldy,
                             int parts, cudaStream_t s);
 bool narrow_path_supported(const grim_bcr* h, int64_t N);
-bool narrow_preferred(const grim_bcr* h, int64_t N);
+bool narrow_preferred(const grim_bcr* h, const SpmmArgs& a);
+double narrow_time(const grim_bcr* h, int64_t N);  // estimate in us (fp32, more than eight columns)
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA
-double direct_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us (plain products)
+double direct_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
 // bf16 handles: a copy of X with aligned rows for the tensor-core kernels, where the scratch for it is there
 size_t x_copy_size(const grim_bcr* h, int64_t ncols);
 size_t x_copy_area(const grim_bcr* h, int64_t max_ncols);  // what is reserved for copies of up to max_ncols columns

@@ -323,14 +323,23 @@ __global__ void __launch_bounds__(256) pad_rows_kernel(const T* __restrict__ X, 
 
 // Where this kernel is the best of those that take 2 <= N <= 16 (measured on square matrices of 512 to 8192 at rate 8 in the
 // three block shapes, both types, N = 2, 4, 7, 8, 16; times in us).
-bool narrow_preferred(const grim_bcr* h, int64_t N) {
+bool narrow_preferred(const grim_bcr* h, const SpmmArgs& a) {
+  const int64_t N = a.ncols;
   if (!narrow_path_supported(h, N)) return false;
   // up to four columns and eight rows to a band the streaming kernel's larger transfers win (8192^2, 8 x 32, N = 4: 17.5
   // against 21.5; bf16 19.8 against 21); with 16 rows its lanes walk mostly pruned rows (16 x 64: 29 against 19)
   if (N <= 4) return h->bh > 8;
-  // two passes over the weights for 16 x 16 accumulators: the CUDA-core kernels' tiles are better (8192^2, N = 16: 51 against 64)
-  if (h->dtype == GRIM_F32 && h->bh > 8 && N > 8) return false;
+  // The slab kernel's narrow tile, where it can fetch the rows and is estimated to be done first: against two passes over the
+  // weights for 16 x 16 accumulators (5696^2, N = 16: 28 against 46; 640 x 5952: 21 against 8.6), and for more than eight columns
+  // where many columns of W are kept in few rows each, because a gathered row of X costs the same whatever its column keeps
+  // (8 x 32: 5376^2, heavy-tailed, N = 12: 37 against 50; 4096^2, uniform, N = 16: 20 against 15)
+  if (h->dtype == GRIM_F32 && h->bh >= 8 && N > 8) return narrow_time(h, N) <= slab_time(h, a);
   return true;
+}
+
+double narrow_time(const grim_bcr* h, int64_t N) {
+  if (h->dtype == GRIM_F32 && h->bh > 8 && N > 8) return 4.0 + 11e-6 * (double)h->nnz + 9e-3 * (double)h->nbr;
+  return 1.0 + (N > 8 ? 1.05e-3 : 0.6e-3) * (double)h->nchunks;
 }
 
 bool narrow_path_supported(const grim_bcr* h, int64_t N) {
