@@ -320,25 +320,35 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
   a.stride = d->stride; a.pad = d->pad; a.OH = (int)OH; a.OW = (int)OW;
   const bool one = d->KH == 1 && d->KW == 1 && d->stride == 1 && d->pad == 0 && !(d->flags & kKernelFlags);
   const int64_t hw = d->H * d->W;
-  // 1 x 1 kernels on several images: a launch per image costs 6 us and more each, so all images go through one convolution -
-  // the gathering tensor-core kernel's where it can, the direct kernel's up to the image size from which a product per image
-  // is large enough (bf16: 32 images, 64 channels, 56 x 56: 187 -> 16 us; 512 channels, 7 x 7, 8 images: 25 -> 12;
-  // 28 x 28, 128 -> 512, 16 images: 118 -> 81 .. 122)
+  auto one_image = [&](int64_t n) {  // (1 x 1 kernels) image n as a plain product
+    const size_t in_esz = d->in_dtype == GRIM_BF16 ? 2 : 4, out_esz = d->out_dtype == GRIM_BF16 ? 2 : 4;
+    SpmmArgs m;
+    m.X = static_cast<const uint8_t*>(in) + (size_t)(n * d->C * hw) * in_esz;
+    m.Y = static_cast<uint8_t*>(out) + (size_t)(n * h->M * hw) * out_esz;
+    m.ncols = hw; m.x_sk = hw; m.x_sq = 1; m.y_sr = hw; m.y_sq = 1;
+    m.x_dtype = d->in_dtype; m.y_dtype = d->out_dtype;
+    m.bias = d->bias_dev; m.relu = a.relu;
+    return m;
+  };
+  // 1 x 1 kernels on several images: a launch per image costs some 6 us and more, so small images go through one convolution -
+  // the gathering tensor-core kernel's where it can (64 channels, 56 x 56, 32 images: 187 -> 16 us), else the direct kernel's where
+  // that is estimated to be done before as many products (512 channels, 7 x 7, 8 images: 25 -> 12; but 1024 -> 1024, 28 x 28, two
+  // images in bf16: 110 against 50).  A product on the tensor cores takes about 6 us and 0.75 per K tile.
   if (one && d->N > 1) {
     if (conv_tc_supported(h, a)) return launch_conv_tc(h, a, (cudaStream_t)stream);
-    if (direct_path_supported(h, a) && (hw <= 1024 || (h->dtype == GRIM_F32 && hw <= 4096 && (h->bh > 4 || d->N >= 16)))) return launch_direct(h, a, (cudaStream_t)stream);
+    if (direct_path_supported(h, a)) {
+      SpmmArgs m = one_image(0);
+      // (with a margin of 15 % for what is the better known: the tensor cores' time, the direct kernel's against the slab kernel's)
+      const bool tensor = tc_path_supported(h, m) && hw >= 128;
+      const double each = tensor ? 6.0 + 0.75 * (double)h->tc_ktiles : 1.0 + std::max(3.5, std::min(direct_time(h, m), slab_time(h, m)));
+      if (direct_time(h, a) <= each * (double)d->N * (tensor ? 0.85 : 1.15)) return launch_direct(h, a, (cudaStream_t)stream);
+    }
   }
   if (one) {
     // 1 x 1 kernels: the expanded input IS the input - per image a plain Cout x C times C x (H*W) product on the
     // tensors as they lie in memory (row stride H*W), no gather at all; one launch per image
-    const size_t in_esz = d->in_dtype == GRIM_BF16 ? 2 : 4, out_esz = d->out_dtype == GRIM_BF16 ? 2 : 4;
     for (int64_t n = 0; n < d->N; ++n) {
-      SpmmArgs m;
-      m.X = static_cast<const uint8_t*>(in) + (size_t)(n * d->C * hw) * in_esz;
-      m.Y = static_cast<uint8_t*>(out) + (size_t)(n * h->M * hw) * out_esz;
-      m.ncols = hw; m.x_sk = hw; m.x_sq = 1; m.y_sr = hw; m.y_sq = 1;
-      m.x_dtype = d->in_dtype; m.y_dtype = d->out_dtype;
-      m.bias = d->bias_dev; m.relu = a.relu;
+      const SpmmArgs m = one_image(n);
       grim_status_t st;
       if (tc2_path_supported(h, m) && hw >= 256 && h->tc_mtiles >= 2 &&
           2 * ((h->tc_mtiles + 1) / 2) * ((hw + 511) / 512) * 3 >= 2 * (int64_t)sm_count(h->device))
