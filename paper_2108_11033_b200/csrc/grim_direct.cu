@@ -185,7 +185,7 @@ bool direct_preferred(const grim_bcr* h, const SpmmArgs& a) {
       return false;
     if (a.ncols < 5 || (a.x_dtype == GRIM_BF16 && a.ncols >= 8 && h->d_chunks)) return false;
     // (fp32, 16-row blocks, more than eight columns: whatever takes them otherwise needs longer)
-    const double other = h->dtype == GRIM_F32 && h->bh > 8 && a.ncols > 8 ? std::min(narrow_time(h, a.ncols), slab_time(h, a)) : 0.0;
+    const double other = h->dtype == GRIM_F32 && h->bh > 8 && a.ncols > 8 ? std::min(narrow_time(h), slab_time(h, a)) : 0.0;
     return direct_time(h, a) <= std::max(5.0, 1.1 * other);
   }
   // bf16: the slab kernel widens what it gathers, element by element, where TMA cannot fetch the rows (N = 131: 328 -> 30)
@@ -208,7 +208,6 @@ grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s
   p.band_order = h->d_band_order; p.nbr = (int)h->nbr; p.M = (int)h->M; p.bh = h->bh;
   p.a = a;
   const int BHc = h->bh <= 4 ? 4 : (h->bh <= 8 ? 8 : 16);
-  const int sms = sm_count(h->device);
   int nc, parts;
   if (a.tile_n > 32 && direct_choice(a.tile_n)) {
     nc = a.tile_n % 32; parts = a.tile_n / 256;

@@ -221,7 +221,7 @@ grim_status_t launch_narrow(const grim_bcr* h, const void* X, int x_dtype, int64
                             int parts, cudaStream_t s);
 bool narrow_path_supported(const grim_bcr* h, int64_t N);
 bool narrow_preferred(const grim_bcr* h, const SpmmArgs& a);
-double narrow_time(const grim_bcr* h, int64_t N);  // estimate in us (fp32, more than eight columns)
+double narrow_time(const grim_bcr* h);  // estimate in us (fp32, nine to sixteen columns)
 grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA

@@ -333,13 +333,12 @@ bool narrow_preferred(const grim_bcr* h, const SpmmArgs& a) {
   // weights for 16 x 16 accumulators (5696^2, N = 16: 28 against 46; 640 x 5952: 21 against 8.6), and for more than eight columns
   // where many columns of W are kept in few rows each, because a gathered row of X costs the same whatever its column keeps
   // (8 x 32: 5376^2, heavy-tailed, N = 12: 37 against 50; 4096^2, uniform, N = 16: 20 against 15)
-  if (h->dtype == GRIM_F32 && h->bh >= 8 && N > 8) return narrow_time(h, N) <= slab_time(h, a);
+  if (h->dtype == GRIM_F32 && h->bh >= 8 && N > 8) return narrow_time(h) <= slab_time(h, a);
   return true;
 }
 
-double narrow_time(const grim_bcr* h, int64_t N) {
-  if (h->dtype == GRIM_F32 && h->bh > 8 && N > 8) return 4.0 + 11e-6 * (double)h->nnz + 9e-3 * (double)h->nbr;
-  return 1.0 + (N > 8 ? 1.05e-3 : 0.6e-3) * (double)h->nchunks;
+double narrow_time(const grim_bcr* h) {
+  return h->bh > 8 ? 4.0 + 11e-6 * (double)h->nnz + 9e-3 * (double)h->nbr : 1.0 + 1.05e-3 * (double)h->nchunks;
 }
 
 bool narrow_path_supported(const grim_bcr* h, int64_t N) {
