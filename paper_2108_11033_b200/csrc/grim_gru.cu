@@ -8,7 +8,10 @@
 // once, so that W_hh is read from HBM once per sequence instead of once per step.  Per step the blocks
 // multiply their bands with h_{t-1}, apply the gate non-linearities and exchange their slices of h_t.
 //
-// Two exchange schemes:
+// Exchange schemes:
+//   gru_cluster_reg_kernel, gru_stack_kernel
+//                         one cluster holds W_hh in registers; of a stack of two or three layers all run in one launch, a few
+//                         steps behind each other.  Used whenever the layers fit.
 //   gru_cluster_kernel    one thread-block cluster (up to 16 CTAs) holds all of W_hh; h_t is broadcast
 //                         with distributed-shared-memory stores and the step ends with the hardware
 //                         cluster barrier.  Used whenever the layer fits one cluster.
@@ -17,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <future>
 #include <new>
 #include <numeric>
 
@@ -37,7 +41,7 @@ struct ModeCfg {
 };
 }  // namespace
 
-namespace { struct GruParams; }
+namespace { struct GruParams; struct GruStack; }
 
 struct grim_gru {
   int L = 0;
@@ -47,7 +51,8 @@ struct grim_gru {
   std::vector<float*> d_bih, d_bhh;
   std::vector<uint32_t*> d_pos_of_band;     // schedule position of every band of W_hh
   std::vector<uint32_t*> d_pos_of_band_ih;  // ... of W_ih
-  std::vector<float*> d_img_val;      // per layer: register image of the register-resident kernel (may be empty)
+  std::vector<float*> d_img_val;      // register images of the register-resident kernel (may be empty): W_hh of every layer, then,
+                                      // where the layers run in one launch, W_ih of layers 1 ...
   std::vector<uint32_t*> d_img_col;
   std::vector<float*> d_gi_saved;  // grim_gru_seq_static parks d_gi here while it points the pass at the static array
   std::vector<float*> d_gi;  // per layer: hoisted pre-activations, T x 3H (layers overlap in time, so each has its own)
@@ -68,7 +73,9 @@ struct grim_gru {
   unsigned* d_sync = nullptr;  // [0..L): barrier counters, [L]: status word
   ModeCfg grid, cluster;       // launch shapes of the shared-memory kernels
   ModeCfg regc;                // launch shape of the register-resident cluster kernel
-  void (*reg_kern)(const GruParams) = nullptr;  // its compiled variant
+  void (*reg_kern)(const GruParams) = nullptr;    // its compiled variant
+  ModeCfg stack;                                  // launch shape of the same variant for all layers in one launch
+  void (*stack_kern)(const GruStack) = nullptr;
   int device = -1;
   cudaStream_t last_stream = nullptr;
   int dbg_skip_cta = -1;
@@ -90,7 +97,7 @@ struct GruParams {
   const uint32_t* pos_of_band;
   const float* b_hh;
   const float* gi;   // T x 3H, b_ih already added
-  const float* b_ih; // 3H or null: added to gi here (not used by the register-resident kernel)
+  const float* b_ih; // 3H or null: added to gi here
   const float* h0;   // H or null
   float* out;        // T x H
   float* outT;       // null, or the same values unit-major: outT[unit * ldT + t] (input of the next layer's projection)
@@ -102,10 +109,31 @@ struct GruParams {
   uint32_t max_chunks, max_cw, max_vals;
   int skip_cta;
   unsigned spin_limit;
-  // register image of the register-resident kernel: what every thread keeps for the whole sequence, laid out
+  // register image of the register-resident kernels: what every thread keeps for the whole sequence, laid out
   // so that the threads of a block read consecutive words ([cta][item][slot][row or column][thread])
   const float* img_val;
   const uint32_t* img_col;
+};
+
+// The stacked kernel: cluster c of a launch plays role[c], an even one the recurrence of layer c / 2, an odd one the
+// projection of layer (c + 1) / 2.
+constexpr int kMaxStack = 3;                    // layers in one launch
+constexpr unsigned kNotYet = 0xFFFFFFFFu;       // what buffers between clusters are filled with: a NaN that no arithmetic produces
+struct GruRole {
+  const float* img_val;
+  const uint32_t* img_col;
+  const float* bias;         // recurrence: b_hh, projection: b_ih
+  const float* in;           // recurrence: pre-activations, T x 3H; projection: outputs of the layer below, T x H
+  float* out;                // recurrence: T x H; projection: T x 3H
+  const float* h0;           // H or null
+  float* hT;                 // H or null
+  int waits;                 // another cluster writes `in` in the same launch: kNotYet where it has not yet
+};
+struct GruStack {
+  GruRole role[2 * kMaxStack - 1];
+  unsigned* status;
+  int H, bh, T, tpc, ks;
+  unsigned spin_limit;
 };
 
 __device__ __forceinline__ void gru_mbar_init(uint64_t* bar, unsigned count) {
@@ -131,6 +159,18 @@ __device__ __forceinline__ void gru_st_async_f32(uint32_t local, uint32_t bar_lo
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// Values that another thread block of the same launch polls for: the value itself says that it is there.
+__device__ __forceinline__ void st_shared_value(float* p, float v) { asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory"); }
+__device__ __forceinline__ float ld_shared_value(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_shared_values(const float* p) {  // each of the four on its own
+  float4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
@@ -570,6 +610,340 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
   cluster.sync();  // no CTA leaves while another may still address its shared memory
 }
 
+// The same for a stack of layers in one launch: a cluster per matrix, W_hh of every layer and W_ih of the upper ones.
+// Four more warps, which hold no weights (registers are dealt out again at the start), move what has to be moved through memory:
+// three bring the next steps' pre-activations (or, in a cluster that projects, inputs) into shared memory, loads a step ahead
+// of their use, one writes results.  They meet the others at the block barrier of every step and are otherwise off the chain.
+// Clusters of a stack wait for each other value by value: buffers between them start out as kNotYet, and who finds that in
+// place of a value asks again.  (Flags beside the values cost a fence per step: 2.3 us a step instead of 1.35.)  So a layer is a
+// few steps behind the one below it, where launches per layer and chunk of time were a chunk and a launch behind: two layers of
+// 1024, 200 steps 385 -> 298 us; three of 1024, 133 steps 332 -> 213; 20 steps of two layers 81 -> 50.
+// A cluster only ever waits for one with a lower number, which needs nothing from it: whatever order they start in, all end.
+constexpr int kHelperThreads = 128, kHelperRegs = 40, kAheadSlots = 4, kBringers = 96, kInFlight = 3;
+template <int THREADS>
+struct MainRegs {  // what the weight-holding warps of a block may have: its registers at launch without the helpers' share
+  static constexpr int wgs = THREADS / 128, at_launch = 65536 / (THREADS + kHelperThreads) / 8 * 8;
+  static constexpr int all = (at_launch * (wgs + 1) - kHelperRegs) / wgs / 8 * 8, value = all < 248 ? all : 248;
+};
+template <int BH, int NI, int S, int THREADS>
+__global__ void __launch_bounds__(THREADS + kHelperThreads, 1) gru_stack_kernel(const __grid_constant__ GruStack p) {
+  extern __shared__ __align__(16) float smem_f[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int rank = (int)cluster.block_rank();
+  const int CS = (int)cluster.num_blocks();
+  const GruRole& role = p.role[blockIdx.x / CS];
+  const bool projects = (blockIdx.x / CS) & 1;
+  const int nb = 3 * p.tpc;
+  const int U = p.tpc * p.bh;
+  const int H = p.H;
+  const int ks = p.ks;
+  const int nmain = (int)blockDim.x - kHelperThreads;  // a multiple of 128
+  float* hs = smem_f;                          // [2][H]: the state; of a projection: the inputs of two steps
+  float* partial = hs + 2 * H;                 // [2][nb][ks][BH]: steps alternate, so that a warp that is ahead overwrites nothing
+  const int part_len = nb * ks * BH;
+  float* ahead = partial + 2 * part_len;       // [kAheadSlots][3][U]: pre-activations of the steps to come
+  float* s_bias = ahead + kAheadSlots * 3 * U; // [3][U]: b_hh
+  float* done = s_bias + 3 * U;                // [2][U]: new states, on their way to memory
+  // The state exchange: the threads that own a hidden unit send its new value into the next-step buffer of every
+  // CTA of the cluster with asynchronous stores that count their bytes on the receiver's mbarrier; a warp starts a
+  // step when the H values of that step have been counted.  No cluster-wide barrier and no fence per step: values of a
+  // step leave a CTA only after all its warps have read the state before it (the block barrier below), and a buffer is
+  // written again only by CTAs that have received such values from everybody - so every CTA has to own units and send: one
+  // that does not could fall two steps behind and find the bytes of two states in one phase of its barrier.
+  uint64_t* hbar = reinterpret_cast<uint64_t*>(done + 2 * U + (U & 1));  // [2], 8-byte aligned (all counts are even)
+  volatile int* s_failed = reinterpret_cast<volatile int*>(hbar + 2);
+  if (tid == 0) {
+    *s_failed = 0;
+    gru_mbar_init(hbar, 1);
+    gru_mbar_init(hbar + 1, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  auto meet = [] { __syncthreads(); };  // all warps, once per step
+
+  if (tid >= nmain) {
+    // ------------------------------------------------------------------ helpers
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs));
+    const int ht = tid - nmain;
+    if (ht < kBringers) {
+      // The first kInFlight items per lane are asked for a step before they are put down, the others (large layers) at once.  Few
+      // instructions per step: the schedulers' slots are the multiply's (written with indexes recomputed this took 0.1 us of a step).
+      bool lost = false;
+      auto gave_up = [&](unsigned it) {
+        if (it != p.spin_limit && !((it & 63u) == 63u && *s_failed)) return false;
+        lost = true;
+        if (!*s_failed) {
+          *s_failed = 1;
+          atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
+        }
+        return true;
+      };
+      const bool waits = role.waits != 0;
+      auto absent = [&](float v) { return waits && !lost && __float_as_uint(v) == kNotYet; };
+      if (projects) {  // items: four neighbouring inputs
+        auto settle = [&](float4 v, const float* src) {
+          for (unsigned it = 0; absent(v.x) || absent(v.y) || absent(v.z) || absent(v.w); ++it) {
+            if (gave_up(it)) break;
+            v = ld_shared_values(src);
+          }
+          return v;
+        };
+        const int items = H / 4;
+        float4 w[kInFlight];
+        const float* src = role.in + 4 * ht;  // of the step that is asked for next
+        const bool live[kInFlight] = {ht < items, ht + kBringers < items, ht + 2 * kBringers < items};
+        auto ask = [&]() {
+#pragma unroll
+          for (int k = 0; k < kInFlight; ++k)
+            if (live[k]) w[k] = ld_shared_values(src + 4 * k * kBringers);
+          src += H;
+        };
+        auto put = [&](int t) {  // (src is a step ahead)
+          float4* dst = reinterpret_cast<float4*>(hs + (t & 1) * H) + ht;
+#pragma unroll
+          for (int k = 0; k < kInFlight; ++k)
+            if (live[k]) dst[k * kBringers] = settle(w[k], src - H + 4 * k * kBringers);
+#pragma unroll 1
+          for (int i = kInFlight * kBringers; i + ht < items; i += kBringers) dst[i] = settle(ld_shared_values(src - H + 4 * i), src - H + 4 * i);
+        };
+        ask();
+        put(0);
+        if (p.T > 1) ask();
+        __syncwarp();
+        cluster.sync();
+        for (int t = 1; t <= p.T; ++t) {
+          // the buffer of step t was last read before the barrier of step t - 2
+          if (t < p.T) put(t);
+          if (t + 1 < p.T) ask();
+          __syncwarp();
+          meet();
+        }
+      } else {  // items: the CTA's 3 x U pre-activations
+        auto settle = [&](float v, const float* src) {
+          for (unsigned it = 0; absent(v); ++it) {
+            if (gave_up(it)) break;
+            v = ld_shared_value(src);
+          }
+          return v;
+        };
+        auto from = [&](int i) {  // place in a row of `in`, or -1
+          const int g = i / U, unit = rank * U + i - g * U;
+          return i < 3 * U && unit < H ? g * H + unit : -1;
+        };
+        float w[kInFlight];
+        int at[kInFlight];
+#pragma unroll
+        for (int k = 0; k < kInFlight; ++k) at[k] = from(ht + k * kBringers);
+        const float* src = role.in;  // the row that is asked for next
+        const int64_t row = 3 * (int64_t)H;
+        float* dst = ahead + ht;
+        int slot = 0;
+        auto ask = [&]() {
+#pragma unroll
+          for (int k = 0; k < kInFlight; ++k)
+            if (at[k] >= 0) w[k] = ld_shared_value(src + at[k]);
+          src += row;
+        };
+        auto put = [&]() {  // (src is a row ahead)
+#pragma unroll
+          for (int k = 0; k < kInFlight; ++k)
+            if (at[k] >= 0) dst[k * kBringers] = settle(w[k], src - row + at[k]);
+#pragma unroll 1
+          for (int i = kInFlight * kBringers; i + ht < 3 * U; i += kBringers)
+            if (from(i + ht) >= 0) dst[i] = settle(ld_shared_value(src - row + from(i + ht)), src - row + from(i + ht));
+          slot = slot + 1 == kAheadSlots ? 0 : slot + 1;
+          dst = ahead + ht + slot * 3 * U;
+        };
+        ask();
+        put();
+        if (p.T > 1) ask();
+        __syncwarp();
+        cluster.sync();
+        for (int t = 1; t <= p.T; ++t) {
+          if (t < p.T) put();
+          if (t + 1 < p.T) ask();
+          __syncwarp();
+          meet();
+        }
+      }
+      meet();
+    } else {
+      // this lane's units: lane, lane + 32, ... of the CTA's (the last CTA may own fewer)
+      const int units = min(U, H - rank * U);
+      float* out = role.out + rank * U + lane;
+      auto write_state = [&](int t) {
+        const float* from = done + (t & 1) * U + lane;
+#pragma unroll 1
+        for (int i = 0; i + lane < units; i += 32) {
+          const float v = from[i];
+          st_shared_value(out + i, v);
+          if (t == p.T - 1 && role.hT) role.hT[rank * U + lane + i] = v;
+        }
+        out += H;
+      };
+      cluster.sync();
+      for (int t = 0; t < p.T; ++t) {
+        meet();
+        if (projects) {
+          const float* part_t = partial + (t & 1) * part_len;
+          for (int i = 0; i + lane < units; i += 32) {
+            const float* part = part_t + (i + lane) / p.bh * 3 * ks * BH + (i + lane) % p.bh;
+            float v[3];
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+              v[g] = __ldg(role.bias + g * H + rank * U + lane + i) + part[g * ks * BH];
+              for (int k = 1; k < ks; ++k) v[g] += part[(g * ks + k) * BH];
+            }
+#pragma unroll
+            for (int g = 0; g < 3; ++g) st_shared_value(out + g * H + i, v[g]);
+          }
+          out += 3 * H;
+        } else if (t > 0) {
+          write_state(t - 1);
+        }
+        __syncwarp();
+      }
+      meet();
+      if (!projects) write_state(p.T - 1);
+    }
+    __syncwarp();
+    cluster.sync();
+    return;
+  }
+
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(MainRegs<THREADS>::value));
+  // ---- one-time: this thread's share of the matrix (built on the host when the handle was created): coalesced loads
+  unsigned long long val[NI][S][BH / 2];  // pairs of neighbouring rows
+  uint32_t col[NI][(S + 1) / 2];          // columns of two slots
+  {
+    const float2* iv = reinterpret_cast<const float2*>(role.img_val) + (size_t)rank * NI * S * (BH / 2) * THREADS + tid;
+    const uint32_t* ic = role.img_col + (size_t)rank * NI * ((S + 1) / 2) * THREADS + tid;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+#pragma unroll
+      for (int s = 0; s < (S + 1) / 2; ++s) col[i][s] = __ldg(ic + (size_t)(i * ((S + 1) / 2) + s) * THREADS);
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int r = 0; r < BH / 2; ++r) {
+          const float2 v = __ldg(iv + (size_t)((i * S + s) * (BH / 2) + r) * THREADS);
+          val[i][s][r] = walk_pair(v.x, v.y);
+        }
+    }
+  }
+
+  // The gates of the CTA's U hidden units are worked out by several groups of warps at once, each of which sends the new
+  // values to its share of the cluster (sixteen stores one after the other by the same warp were 300 cycles of the step).
+  const int wg = (U + 31) / 32, groups = min(min((nmain >> 5) / wg, 4), CS), group = warp / wg;
+  const int gu = (warp - group * wg) * 32 + lane;
+  const int g_tri = gu / p.bh, g_r = gu % p.bh;
+  const int unit = rank * U + gu;
+  const bool gate_live = !projects && group < groups && gu < U && unit < H;  // (the last CTA may own fewer groups of units)
+  const int dst0 = CS * group / groups, dst1 = CS * (group + 1) / groups;
+  const bool keeps = group == groups - 1;  // leaves the new values for the helper that writes them to memory
+  float h_own = 0.f;  // the unit's state
+  if (gate_live) {
+    for (int g = 0; g < 3; ++g) s_bias[g * U + gu] = role.bias[g * H + unit];
+    h_own = role.h0 ? role.h0[unit] : 0.f;
+  }
+  if (!projects)
+    for (int i = tid; i < H; i += nmain) hs[i] = role.h0 ? role.h0[i] : 0.f;
+  cluster.sync();
+  const uint32_t hs_local = (uint32_t)__cvta_generic_to_shared(hs), bar_local = (uint32_t)__cvta_generic_to_shared(hbar);
+
+  bool lost = false;  // one of this warp's waits has run out (or another warp's, before it)
+  for (int t = 0; t < p.T; ++t) {
+    const int cur = t & 1, nxt = cur ^ 1;
+    const float* hcur = hs + cur * H;
+    float* part_t = partial + cur * part_len;
+    // this step's outputs arrive on the next buffer's barrier: announce the byte count (fast CTAs may already be
+    // sending, which drives the count negative; the pending arrival keeps the phase open until it is announced)
+    if (tid == 0 && !projects && t + 1 < p.T && !lost) gru_mbar_arrive_expect_tx(hbar + nxt, (unsigned)H * 4u);
+    float gi[3] = {0.f, 0.f, 0.f};  // read now, so that nothing waits for them later
+    if (gate_live) {
+      const float* at = ahead + (t & (kAheadSlots - 1)) * 3 * U + gu;
+      gi[0] = at[0] + s_bias[gu]; gi[1] = at[U] + s_bias[U + gu]; gi[2] = at[2 * U];
+    }
+    // RI items are multiplied and then reduced together (their exchanges overlap)
+    constexpr int RI = NI * BH == 16 || NI * BH == 32 ? NI : 1;
+#pragma unroll
+    for (int i0 = 0; i0 < NI; i0 += RI) {
+      float acc[RI * BH];
+#pragma unroll
+      for (int i = 0; i < RI; ++i) {
+        unsigned long long sum[BH / 2];
+#pragma unroll
+        for (int r = 0; r < BH / 2; ++r) sum[r] = 0ull;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          const uint32_t cw = col[i0 + i][s / 2];
+          const float xv = hcur[(s & 1) ? cw >> 16 : cw & 0xFFFFu];
+          const unsigned long long x2 = walk_pair(xv, xv);
+#pragma unroll
+          for (int r = 0; r < BH / 2; ++r) walk_ffma2(sum[r], val[i0 + i][s][r], x2);
+        }
+#pragma unroll
+        for (int r = 0; r < BH / 2; ++r) {
+          acc[i * BH + 2 * r] = __uint_as_float((unsigned)sum[r]);
+          acc[i * BH + 2 * r + 1] = __uint_as_float((unsigned)(sum[r] >> 32));
+        }
+      }
+      warp_reduce_rows<RI * BH>(acc, lane);
+      const int at = (warp * NI + i0) * BH + warp_row<RI * BH>(lane);
+      if (at < part_len) part_t[at] = acc[0];
+    }
+    meet();
+    if (projects) continue;
+    if (gate_live) {
+      float q[3];
+#pragma unroll
+      for (int g = 0; g < 3; ++g) {
+        const float* part = part_t + (g_tri * 3 + g) * ks * BH + g_r;
+        q[g] = g == 2 ? s_bias[2 * U + gu] + part[0] : part[0];
+        for (int k = 1; k < ks; ++k) q[g] += part[k * BH];
+      }
+      const float rg = __frcp_rn(1.f + expf(-(gi[0] + q[0]))), zg = __frcp_rn(1.f + expf(-(gi[1] + q[1])));
+      const float ng = tanh_both(gi[2] + rg * q[2]);
+      h_own = (1.f - zg) * ng + zg * h_own;
+      if (t + 1 < p.T && !lost) {
+        // one 4-byte store per destination (pooling four neighbours' values into 16-byte stores was slower: the
+        // shuffles lengthen the chain more than the fewer messages save)
+        const uint32_t dst_local = hs_local + (uint32_t)(nxt * H + unit) * 4u, bar_nxt = bar_local + (uint32_t)nxt * 8u;
+#pragma unroll 4
+        for (int dst = dst0; dst < dst1; ++dst) gru_st_async_f32(dst_local, bar_nxt, (uint32_t)dst, h_own);
+      }
+      if (keeps) done[cur * U + gu] = h_own;
+    }
+    if (t + 1 < p.T) {
+      // the next step's state: bounded wait on the local barrier (its (t / 2)-th use), one thread of every warp.  When it
+      // runs out the block goes through its remaining steps without waiting: the results are invalid and reported.  A warp that
+      // knows neither announces nor sends any more (a phase that is still open takes no second announcement, and bytes that
+      // nobody waits for would pile up on the others' barriers), so the others' waits run out too.  (The vote costs nothing:
+      // 396 -> 385 us for two layers of 1024, 200 steps.)
+      const unsigned parity = (unsigned)((t >> 1) & 1);
+      if (lane == 0) {
+        bool ok = false;
+        if (!*s_failed)
+          for (unsigned it = 0; it < p.spin_limit && !ok; ++it) {
+            ok = gru_mbar_try_wait(hbar + nxt, parity);
+            if (!ok && (it & 63u) == 63u && *s_failed) break;
+          }
+        if (__builtin_expect(!ok, 0)) {
+          lost = true;
+          if (!*s_failed) {
+            *s_failed = 1;
+            atomicExch(p.status, (unsigned)GRIM_ERR_TIMEOUT);
+          }
+        }
+      }
+      lost = __any_sync(0xffffffffu, lost);
+    }
+  }
+  meet();
+  cluster.sync();  // no CTA leaves while another may still address its shared memory
+}
+
 size_t smem_bytes(const grim_gru* g, const ModeCfg& m, int BH, bool cluster) {
   const int nb = 3 * m.tpc;
   size_t b = (size_t)nb * m.ks * BH * 4;
@@ -596,16 +970,23 @@ cudaError_t launch_grid(const grim_gru* g, const GruParams& p, cudaStream_t s) {
   return e;
 }
 
+// Once, when the handle is created (the kernel keeps them).
+template <typename Kern>
+cudaError_t cluster_attributes(Kern kern, const ModeCfg& m) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
+  if (e == cudaSuccess && m.ctas > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
 template <typename Kern>
 cudaError_t cluster_launch_config(Kern kern, const ModeCfg& m, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr,
-                                  cudaStream_t s, bool set_attributes) {
-  if (set_attributes) {  // once, when the handle is created (the kernel keeps them)
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.smem);
-    if (e == cudaSuccess && m.ctas > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+                                  cudaStream_t s, bool set_attributes, int clusters = 1) {
+  if (set_attributes) {
+    const cudaError_t e = cluster_attributes(kern, m);
     if (e != cudaSuccess) return e;
   }
   *cfg = cudaLaunchConfig_t{};
-  cfg->gridDim = dim3(m.ctas);
+  cfg->gridDim = dim3(m.ctas * clusters);
   cfg->blockDim = dim3(m.threads);
   cfg->dynamicSmemBytes = m.smem;
   cfg->stream = s;
@@ -618,22 +999,22 @@ cudaError_t cluster_launch_config(Kern kern, const ModeCfg& m, cudaLaunchConfig_
   return cudaSuccess;
 }
 
-// Can one cluster of this shape be resident?  (asked once, at creation)
+// How many clusters of this shape can be resident?  (asked once, at creation)
 template <typename Kern>
-bool cluster_fits(Kern kern, const ModeCfg& m) {
+int clusters_that_fit(Kern kern, const ModeCfg& m) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  if (cluster_launch_config(kern, m, &cfg, attr, nullptr, true) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (cluster_launch_config(kern, m, &cfg, attr, nullptr, true) != cudaSuccess) { cudaGetLastError(); return 0; }
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
-  return n >= 1;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
 }
 
-template <typename Kern>
-cudaError_t launch_cluster(Kern kern, const ModeCfg& m, const GruParams& p, cudaStream_t s) {
+template <typename Kern, typename Params>
+cudaError_t launch_cluster(Kern kern, const ModeCfg& m, const Params& p, cudaStream_t s, int clusters = 1) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  cudaError_t e = cluster_launch_config(kern, m, &cfg, attr, s, false);
+  cudaError_t e = cluster_launch_config(kern, m, &cfg, attr, s, false, clusters);
   if (e != cudaSuccess) return e;
   e = cudaLaunchKernelEx(&cfg, kern, p);
   count_launch();
@@ -642,41 +1023,46 @@ cudaError_t launch_cluster(Kern kern, const ModeCfg& m, const GruParams& p, cuda
 
 // The compiled variants of the register-resident kernel.
 using GruKernel = void (*)(const GruParams);
+using StackKernel = void (*)(const GruStack);
 struct RegVariant {
   int BH, ni, s, threads;
   GruKernel kern;
+  StackKernel stack;
 };
+#define GRIM_GRU_VARIANT(BH, NI, S, TH) {BH, NI, S, TH, gru_cluster_reg_kernel<BH, NI, S, TH>, gru_stack_kernel<BH, NI, S, TH>}
 const RegVariant kRegVariants[] = {
-    {8, 1, 2, 512, gru_cluster_reg_kernel<8, 1, 2, 512>},
-    {8, 1, 4, 768, gru_cluster_reg_kernel<8, 1, 4, 768>},
-    {8, 2, 6, 384, gru_cluster_reg_kernel<8, 2, 6, 384>},
-    {8, 3, 8, 256, gru_cluster_reg_kernel<8, 3, 8, 256>},
-    {4, 1, 2, 768, gru_cluster_reg_kernel<4, 1, 2, 768>},
-    {4, 1, 4, 768, gru_cluster_reg_kernel<4, 1, 4, 768>},
-    {4, 2, 4, 384, gru_cluster_reg_kernel<4, 2, 4, 384>},
-    {4, 4, 4, 384, gru_cluster_reg_kernel<4, 4, 4, 384>},
-    {4, 4, 6, 384, gru_cluster_reg_kernel<4, 4, 6, 384>},
-    {4, 4, 7, 384, gru_cluster_reg_kernel<4, 4, 7, 384>},
-    {4, 6, 8, 256, gru_cluster_reg_kernel<4, 6, 8, 256>},
-    {16, 1, 2, 512, gru_cluster_reg_kernel<16, 1, 2, 512>},
-    {16, 1, 4, 512, gru_cluster_reg_kernel<16, 1, 4, 512>},
-    {16, 1, 6, 384, gru_cluster_reg_kernel<16, 1, 6, 384>},
-    {16, 1, 8, 384, gru_cluster_reg_kernel<16, 1, 8, 384>}};
+    GRIM_GRU_VARIANT(8, 1, 2, 512),
+    GRIM_GRU_VARIANT(8, 1, 4, 768),
+    GRIM_GRU_VARIANT(8, 2, 6, 384),
+    GRIM_GRU_VARIANT(8, 3, 8, 256),
+    GRIM_GRU_VARIANT(4, 1, 2, 768),
+    GRIM_GRU_VARIANT(4, 1, 4, 768),
+    GRIM_GRU_VARIANT(4, 2, 4, 384),
+    GRIM_GRU_VARIANT(4, 4, 4, 384),
+    GRIM_GRU_VARIANT(4, 4, 6, 384),
+    GRIM_GRU_VARIANT(4, 4, 7, 384),
+    GRIM_GRU_VARIANT(4, 6, 8, 256),
+    GRIM_GRU_VARIANT(16, 1, 2, 512),
+    GRIM_GRU_VARIANT(16, 1, 4, 512),
+    GRIM_GRU_VARIANT(16, 1, 6, 384),
+    GRIM_GRU_VARIANT(16, 1, 8, 384)};
 GruKernel smem_cluster_kernel(int BH) {
   return BH == 4 ? gru_cluster_kernel<4> : (BH == 8 ? gru_cluster_kernel<8> : gru_cluster_kernel<16>);
 }
 
-// Largest number of kept columns in a band, over all bands of all layers.
-int max_band_columns(const grim_gru* g) {
-  uint32_t mx = 0;
-  for (const grim_bcr* wh : g->Whh)
-    for (int64_t pos = 0; pos < wh->nbr; ++pos) {
-      uint32_t n = 0;
-      for (uint32_t k = wh->h_gemv_band_ptr[(size_t)pos]; k < wh->h_gemv_band_ptr[(size_t)pos + 1]; ++k)
-        n += wh->h_chunks[k].ncols_kr & 0xFFFFu;
+// Largest number of kept columns in a band, over all bands of the matrices.
+int max_band_columns(const std::vector<const grim_bcr*>& mats) {
+  int mx = 0;
+  for (const grim_bcr* w : mats)
+    for (int64_t band = 0; band < w->nbr; ++band) {
+      int n = 0;
+      for (int64_t j = 0; j < w->nbc; ++j) {
+        const HostBlock& hb = w->blocks[(size_t)(band * w->nbc + j)];
+        n += hb.kr ? hb.kc : 0;
+      }
       mx = std::max(mx, n);
     }
-  return (int)mx;
+  return mx;
 }
 
 // How much of the chunk layout the busiest CTA would hold when CTA c owns groups [c*tpc, (c+1)*tpc).
@@ -734,8 +1120,21 @@ constexpr size_t kSmemLimit = 200 * 1024;
 }  // namespace
 
 namespace {
-// out[k * ld + t] = in[t * K + k]: the caller's T x K input, feature-major.
-__global__ void transpose_input_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t T, int64_t K, int64_t ld) {
+// out[k * ld + t] = in[t * K + k]: the caller's T x K input, feature-major.  Blocks past the input's (blockIdx.y >= kblocks) fill the
+// buffers between the clusters of a stacked launch with kNotYet.
+struct FillArgs {
+  uint4* at[2 * kMaxStack - 2];
+  int64_t n[2 * kMaxStack - 2];  // 16-byte pieces
+};
+__global__ void transpose_input_kernel(const float* __restrict__ in, float* __restrict__ out, int64_t T, int64_t K, int64_t ld, int kblocks,
+                                       const __grid_constant__ FillArgs fill) {
+  if ((int)blockIdx.y >= kblocks) {
+    const int64_t blocks = (int64_t)gridDim.x * (gridDim.y - kblocks), block = (int64_t)(blockIdx.y - kblocks) * gridDim.x + blockIdx.x;
+#pragma unroll
+    for (int b = 0; b < 2 * kMaxStack - 2; ++b)
+      for (int64_t i = block * 256 + threadIdx.y * 32 + threadIdx.x; i < fill.n[b]; i += blocks * 256) fill.at[b][i] = make_uint4(kNotYet, kNotYet, kNotYet, kNotYet);
+    return;
+  }
   __shared__ float tile[32][33];
   const int64_t t0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -864,52 +1263,69 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
         t.smem = smem_bytes(g, t, BHc, true);
         if (t.smem > kSmemLimit) continue;  // the cluster scheme is only used with weights on-chip
         g->cluster = t;
-        g->cluster.ok = cluster_fits(smem_cluster_kernel(BHc), g->cluster);
+        g->cluster.ok = clusters_that_fit(smem_cluster_kernel(BHc), g->cluster) >= 1;
         if (!g->cluster.ok) g->cluster = ModeCfg{};
       }
       // ---- register-resident cluster shape
-      const int max_cols = max_band_columns(g);
+      // The matrices that are kept in registers: W_hh, and W_ih of the upper layers where all layers run in one launch - if a
+      // variant holds both, and as many clusters run at once.  (More than three layers: layers l and l + 2 share a buffer.)
+      std::vector<const grim_bcr*> mats = g->Whh;
+      const size_t only_hh = mats.size();
+      bool stack = layers > 1 && layers <= kMaxStack;
+      for (int l = 1; l < layers; ++l) stack = stack && W_ih[l]->bh == bh;
+      if (stack) mats.insert(mats.end(), g->Wih.begin() + 1, g->Wih.end());
       const RegVariant* rv = nullptr;
-      for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
-        // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
-        const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc;
-        struct Candidate { double cost; const RegVariant* v; ModeCfg shape; };
-        std::vector<Candidate> cands;
-        for (const RegVariant& v : kRegVariants)
-          for (int ks = 1; ks <= 8; ks *= 2) {
-            const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
-            if (v.BH != BHc || 32 * v.s * ks < max_cols + ks - 1 || std::max(32 * warps, (tpc * bh + 31) / 32 * 32) > v.threads) continue;
-            // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
-            // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
-            const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
-            ModeCfg t;
-            t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
-            t.threads = std::max(32 * warps, std::max((tpc * bh + 31) / 32 * 32, 128));
-            t.smem = ((((size_t)2 * H + (size_t)2 * nb * ks * BHc) * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
-            if (t.smem <= kSmemLimit) cands.push_back({cost, &v, t});
-          }
-        // (asked in the order of their costs: the question costs more than all else here)
-        std::stable_sort(cands.begin(), cands.end(), [](const Candidate& x, const Candidate& y) { return x.cost < y.cost; });
-        for (const Candidate& c : cands)
-          if (cluster_fits(c.v->kern, c.shape)) {
-            rv = c.v; g->regc = c.shape; g->regc.ok = true; g->reg_kern = rv->kern;
-            break;
-          }
+      for (int attempt = stack ? 0 : 1; attempt < 2 && !g->regc.ok; ++attempt) {
+        if (attempt == 1) mats.resize(only_hh);
+        const int max_cols = max_band_columns(mats);
+        for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
+          // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
+          const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc, units = tpc * bh;
+          struct Candidate { double cost; const RegVariant* v; ModeCfg shape, stack; };
+          std::vector<Candidate> cands;
+          for (const RegVariant& v : kRegVariants)
+            for (int ks = 1; ks <= 8; ks *= 2) {
+              const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
+              if (v.BH != BHc || 32 * v.s * ks < max_cols + ks - 1 || std::max(32 * warps, (units + 31) / 32 * 32) > v.threads) continue;
+              // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
+              // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
+              const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
+              const size_t words = (size_t)2 * H + (size_t)2 * nb * ks * BHc;
+              ModeCfg t;
+              t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
+              t.threads = std::max(32 * warps, std::max((units + 31) / 32 * 32, 128));
+              t.smem = ((words * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
+              ModeCfg u = t;
+              u.threads = (t.threads + 127) / 128 * 128 + kHelperThreads;  // whole warpgroups
+              // + pre-activations ahead and biases, states to be written
+              u.smem = (((words + (size_t)(kAheadSlots + 1) * 3 * units + 2 * (size_t)units + 1) * 4 + 15) & ~size_t(15)) + 32;
+              if (std::max(t.smem, u.smem) <= kSmemLimit) cands.push_back({cost, &v, t, u});
+            }
+          // (asked in the order of their costs: the question costs more than all else here)
+          std::stable_sort(cands.begin(), cands.end(), [](const Candidate& x, const Candidate& y) { return x.cost < y.cost; });
+          for (const Candidate& c : cands)
+            // (where the blocks with helpers fit, those without do: asking is what takes the time)
+            if (attempt == 0 ? clusters_that_fit(c.v->stack, c.stack) >= 2 * layers - 1 && cluster_attributes(c.v->kern, c.shape) == cudaSuccess
+                             : clusters_that_fit(c.v->kern, c.shape) >= 1) {
+              rv = c.v; g->regc = c.shape; g->regc.ok = true; g->reg_kern = rv->kern;
+              if (attempt == 0) { g->stack = c.stack; g->stack.ok = true; g->stack_kern = rv->stack; }
+              break;
+            }
+        }
       }
       if (g->regc.ok) {
         // register image: for every thread of every CTA the columns it owns (global index + values at row positions); threads
         // are numbered with the variant's stride
         const int NI = rv->ni, S = rv->s, S2 = (S + 1) / 2, TH = rv->threads, ks = g->regc.ks, tpc = g->regc.tpc, cs = g->regc.ctas, nbb = 3 * tpc;
         const size_t nval = (size_t)cs * NI * S * BHc * TH, ncol = (size_t)cs * NI * S2 * TH;
-        std::vector<float> iv(nval);
-        std::vector<uint32_t> ic(ncol);
+        struct Image { std::vector<float> val; std::vector<uint32_t> col; };
         struct ColRec { uint32_t col, rowmask, kc; const float* v; };  // kept row a (of rowmask) has v[a * kc]
-        std::vector<ColRec> cols, dealt;
-        std::vector<size_t> before;  // columns dealt before each round
-        for (int l = 0; l < layers && st == GRIM_OK; ++l) {
-          const grim_bcr* wh = W_hh[l];
-          std::fill(iv.begin(), iv.end(), 0.f);
-          std::fill(ic.begin(), ic.end(), 0u);
+        auto image_of = [&](const grim_bcr* wh) {  // empty: does not fit
+          Image im{std::vector<float>(nval), std::vector<uint32_t>(ncol)};
+          std::vector<float>& iv = im.val;
+          std::vector<uint32_t>& ic = im.col;
+          std::vector<ColRec> cols, dealt;
+          std::vector<size_t> before;  // columns dealt before each round
           for (int rank = 0; rank < cs; ++rank)
             for (int lb = 0; lb < nbb; ++lb) {
               if (rank * tpc + lb / 3 >= ntri) continue;
@@ -952,7 +1368,7 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
                 for (size_t k = 0; k < dealt.size(); ++k) {
                   const ColRec& cr = dealt[k];
                   const int sl = (int)(k / 32), tid = warp * 32 + (int)(k % 32);
-                  if (sl >= S || tid >= TH) { st = GRIM_ERR_UNSUPPORTED; break; }
+                  if (sl >= S || tid >= TH) return Image{};
                   ic[((size_t)(rank * NI + i) * S2 + sl / 2) * TH + tid] |= cr.col << (16 * (sl & 1));
                   const float* v = cr.v;
                   for (uint32_t rm = cr.rowmask; rm; rm &= rm - 1, v += cr.kc) {
@@ -962,13 +1378,21 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
                 }
               }
             }
-          if (st != GRIM_OK) break;
+          return im;
+        };
+        // (a thread per matrix: most of the time that creating a model takes)
+        std::vector<std::future<Image>> images;
+        for (const grim_bcr* wh : mats) images.push_back(std::async(image_of, wh));
+        for (std::future<Image>& f : images) {
+          const Image im = f.get();
+          if (st == GRIM_OK && im.val.empty()) st = GRIM_ERR_UNSUPPORTED;
+          if (st != GRIM_OK) continue;
           float* dv = nullptr;
           uint32_t* dc = nullptr;
           cudaError_t e = cudaMalloc((void**)&dv, nval * 4);
           if (e == cudaSuccess) { g->d_img_val.push_back(dv); e = cudaMalloc((void**)&dc, ncol * 4); }
-          if (e == cudaSuccess) { g->d_img_col.push_back(dc); e = cudaMemcpy(dv, iv.data(), nval * 4, cudaMemcpyHostToDevice); }
-          if (e == cudaSuccess) e = cudaMemcpy(dc, ic.data(), ncol * 4, cudaMemcpyHostToDevice);
+          if (e == cudaSuccess) { g->d_img_col.push_back(dc); e = cudaMemcpy(dv, im.val.data(), nval * 4, cudaMemcpyHostToDevice); }
+          if (e == cudaSuccess) e = cudaMemcpy(dc, im.col.data(), ncol * 4, cudaMemcpyHostToDevice);
           if (e != cudaSuccess) st = e == cudaErrorMemoryAllocation ? GRIM_ERR_ALLOC : GRIM_ERR_CUDA;
         }
       }
@@ -998,13 +1422,15 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
   const int BHc = g->bh <= 4 ? 4 : (g->bh <= 8 ? 8 : 16);
   if (cudaMemsetAsync(g->d_sync, 0, (size_t)(L + 1) * 4, s0) != cudaSuccess) return GRIM_ERR_CUDA;
 
-  // Time is cut into chunks; layer l works on chunk k while layer l - 1 works on chunk k + 1 (each layer on its own
+  // All layers in one launch, unless they are to run one after the other (as the static variant does, whose layers share their scratch).
+  const bool stacked = use_reg && g->stack.ok && g->pipeline;
+  // Otherwise time is cut into chunks; layer l works on chunk k while layer l - 1 works on chunk k + 1 (each layer on its own
   // stream, ordered by events), so a stack of L layers takes about (1 + (L - 1) / chunks) single-layer times instead
   // of L.  The kernels with a global barrier (fall-back) and single-layer models run as one chunk on one stream.
   int chunks = 1;
   // With four or more layers, layers l and l + 2 share an inter-layer buffer, and layer l reads its chunk-entering
   // state from that buffer while layer l + 2 may already be writing it: such stacks run one layer after the other.
-  if (g->pipeline && L > 1 && L <= 3 && (use_reg || use_cluster))
+  if (!stacked && g->pipeline && L > 1 && L <= 3 && (use_reg || use_cluster))
     chunks = g->want_chunks > 0 ? (int)std::min<int64_t>(g->want_chunks, T)
                                 : (int)std::max<int64_t>(1, std::min<int64_t>(5, T / 25));
   const int64_t clen = ((T + chunks - 1) / chunks + 3) / 4 * 4;  // a multiple of 4: chunk starts stay 16-byte aligned
@@ -1037,6 +1463,23 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
     const grim_status_t st = launch_cuda_cores(wi, a, s);
     if (g->profile) profile_mark(g, 1, s);
     return st;
+  };
+  auto launch_stack = [&]() -> grim_status_t {
+    GruStack k = {};
+    k.status = g->d_sync + L; k.H = (int)H; k.bh = g->bh; k.T = (int)T; k.tpc = g->stack.tpc; k.ks = g->stack.ks; k.spin_limit = g->spin_limit;
+    for (int l = 0; l < L; ++l) {
+      float* seq_out = l == L - 1 ? y : g->d_seq[l & 1];
+      if (l > 0)
+        k.role[2 * l - 1] = {g->d_img_val[(size_t)(L + l - 1)], g->d_img_col[(size_t)(L + l - 1)], g->d_bih[(size_t)l], g->d_seq[(l - 1) & 1],
+                             g->d_gi[(size_t)l], nullptr, nullptr, 1};
+      k.role[2 * l] = {g->d_img_val[(size_t)l], g->d_img_col[(size_t)l], g->d_bhh[(size_t)l], g->d_gi[(size_t)l], seq_out,
+                       h0 ? h0 + (int64_t)l * H : nullptr, hT ? hT + (int64_t)l * H : nullptr, l > 0};
+    }
+    if (g->profile) profile_mark(g, 2, s0);
+    const cudaError_t e = launch_cluster(g->stack_kern, g->stack, k, s0, 2 * L - 1);
+    if (g->profile) profile_mark(g, 3, s0);
+    if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+    return GRIM_OK;
   };
   auto launch_recurrence = [&](int l, float* seq_out, int64_t t0, int64_t n, cudaStream_t s) -> grim_status_t {
     const grim_bcr* wh = g->Whh[(size_t)l];
@@ -1083,11 +1526,21 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
       const float* seq_in = l == 0 ? x : g->d_seq[(l - 1) & 1];
       float* seq_out = (l == L - 1) ? y : g->d_seq[l & 1];
       grim_status_t st = GRIM_OK;
+      if (stacked && l > 0) continue;
       if (l == 0) {
         if (c == 0) {  // the first layer's input is all there: one launch (after turning it feature-major)
           if (tin) {
             const int64_t K0 = g->Wih[0]->K;
-            transpose_input_kernel<<<dim3((unsigned)((T + 31) / 32), (unsigned)((K0 + 31) / 32)), dim3(32, 8), 0, s>>>(x, g->d_xT, T, K0, ldT);
+            const unsigned tb = (unsigned)((T + 31) / 32), kb = (unsigned)((K0 + 31) / 32);
+            FillArgs fill = {};
+            int64_t pieces = 0;
+            for (int b = 1; stacked && b < L; ++b) {  // (H is a multiple of 4)
+              fill.at[2 * b - 2] = reinterpret_cast<uint4*>(g->d_seq[(b - 1) & 1]); fill.n[2 * b - 2] = T * H / 4;
+              fill.at[2 * b - 1] = reinterpret_cast<uint4*>(g->d_gi[(size_t)b]); fill.n[2 * b - 1] = T * 3 * H / 4;
+              pieces += T * H;
+            }
+            const unsigned fb = (unsigned)std::min<int64_t>(((pieces + 511) / 512 + tb - 1) / tb, 512);  // two pieces per thread
+            transpose_input_kernel<<<dim3(tb, kb + fb), dim3(32, 8), 0, s>>>(x, g->d_xT, T, K0, ldT, (int)kb, fill);
             count_launch();
           }
           st = launch_projection(0, x, 0, T, s);
@@ -1101,7 +1554,7 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
         if (st == GRIM_OK && chunks > 1 && (cudaEventRecord(ready, ps) != cudaSuccess || cudaStreamWaitEvent(s, ready, 0) != cudaSuccess)) return GRIM_ERR_CUDA;
       }
       if (st != GRIM_OK) return st;
-      st = launch_recurrence(l, seq_out, t0, n, s);
+      st = stacked ? launch_stack() : launch_recurrence(l, seq_out, t0, n, s);
       if (st != GRIM_OK) return st;
       if (chunks > 1 && cudaEventRecord(g->ev_chunk[(size_t)l * g->max_chunks + c], s) != cudaSuccess) return GRIM_ERR_CUDA;
     }

@@ -977,6 +977,17 @@ def test_gru_unit_groups_for_fewer_blocks_than_the_largest_cluster(B, cfg):
         check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 207, 0))
 
 
+@pytest.mark.parametrize("cfg", [(9, 64, 2, 1, 8, 32, 4), (9, 64, 3, 2, 8, 32, 4), (12, 72, 2, 3, 4, 16, 3), (30, 1040, 2, 5, 8, 32, 10), (20, 1536, 3, 4, 16, 64, 30),
+                                 (17, 1200, 2, 9, 4, 16, 16), (8, 16, 3, 150, 16, 16, 2)])
+def test_gru_layers_in_one_launch(B, cfg):
+    """Sequences shorter than what is brought ahead, layers whose words per thread block are more than are in flight at once, a last
+    thread block with fewer units; three times on one handle (the buffers between the layers start anew)."""
+    in_f, H, L, T, bh, bw, rate = cfg
+    m = gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=441)
+    check_gru(B, m)
+    check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 442, 0))
+
+
 @pytest.mark.parametrize("cfg", [(37, 128, 2, 33, 4, 16), (20, 96, 1, 31, 16, 32), (64, 160, 3, 64, 16, 64), (9, 60, 2, 2, 5, 16), (500, 64, 2, 7, 8, 32)])
 def test_gru_batched_step_block_shapes(B, cfg):
     """Batches around a tile of 32 sequences, block heights, inputs wider and narrower than the state."""
