@@ -57,7 +57,7 @@ struct Stage {
 
 template <int BH, int NQ, typename VT>
 __host__ __device__ constexpr size_t narrow_smem() {
-  return (size_t)kNWarps * (Stage<BH, NQ, VT>::kDepth * Stage<BH, NQ, VT>::kBytes + BH * NQ * 4);
+  return (size_t)kNWarps * Stage<BH, NQ, VT>::kDepth * Stage<BH, NQ, VT>::kBytes;
 }
 
 __device__ __forceinline__ void nfma2(unsigned long long& acc, unsigned long long w2, unsigned long long x2) {
@@ -93,8 +93,10 @@ __device__ __noinline__ void kept_products(const NParams& p, int pos, int part, 
   }
 }
 
+// Blocks per SM: as many as registers allow.  In bf16 four, and their rings have to leave room for it (the sums take the place of
+// the rings): with three, products of some four thousand warps take a second round (4096^2, 8 x 32 at rate 8, N = 16: 10.3 -> 8.8 us).
 template <int BH, int NQ, typename VT>
-__global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 4 ? 1 : 2) bcr_narrow_kernel(const __grid_constant__ NParams p) {
+__global__ void __launch_bounds__(kNWarps * 32, sizeof(VT) == 2 ? 4 : (BH * NQ >= 128 ? 1 : 2)) bcr_narrow_kernel(const __grid_constant__ NParams p) {
   using S = Stage<BH, NQ, VT>;
   constexpr bool MMA = sizeof(VT) == 2;
   constexpr int D = S::kDepth;
@@ -107,7 +109,9 @@ __global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 
   const int q0 = blockIdx.y * NQ;
   const uint32_t ring = (uint32_t)__cvta_generic_to_shared(nsm) + (uint32_t)warp * (D * S::kBytes);
   const uint8_t* ring_p = nsm + (size_t)warp * (D * S::kBytes);
-  float* sums = reinterpret_cast<float*>(nsm + (size_t)kNWarps * D * S::kBytes);  // [warp][row][column]
+  constexpr int kSumsLd = D * S::kBytes / 4;  // a warp's sums, [row][column], take the place of its ring
+  static_assert(D * S::kBytes >= BH * NQ * 4, "sums fit the ring");
+  float* sums = reinterpret_cast<float*>(nsm);
 
   int c = 0, end = 0;  // next chunk of this warp to be fetched
   if (pos < p.nbr) {
@@ -238,7 +242,8 @@ __global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 
   }
   cp_wait<0>();
 
-  float* mine = sums + warp * (BH * NQ);
+  __syncwarp();
+  float* mine = sums + warp * kSumsLd;
   if constexpr (!MMA) {
     const int row = warp_row<BH>(lane);
 #pragma unroll
@@ -279,7 +284,7 @@ __global__ void __launch_bounds__(kNWarps * 32, BH * NQ >= 128 && sizeof(VT) == 
     const int64_t row = (int64_t)__ldg(p.band_order + at) * p.bh + r;
     if (row >= p.M) continue;
     float t = 0.f;
-    for (int s = 0; s < p.parts; ++s) t += sums[(b * p.parts + s) * (BH * NQ) + rq];
+    for (int s = 0; s < p.parts; ++s) t += sums[(b * p.parts + s) * kSumsLd + rq];
     if (p.y_dtype == GRIM_F32) static_cast<float*>(p.Y)[row * p.ldy + q] = t;
     else static_cast<__nv_bfloat16*>(p.Y)[row * p.ldy + q] = __float2bfloat16_rn(t);
   }
