@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(GATHER ? kGatherThreads : kThreads, 1) conv_tc
                                                                                        const __grid_constant__ CUtensorMap tm_w, const ConvParams p) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_smem(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);   // (even block) the tiles of a stage have landed, both blocks' bytes
   uint64_t* empty = full + kMaxStages;                  // the multiplies of a stage are done
   uint64_t* acc_full = empty + kMaxStages;              // [nacc] an accumulator is complete

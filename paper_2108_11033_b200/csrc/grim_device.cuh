@@ -46,6 +46,10 @@ namespace grim {
 namespace ptx {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// The first 1 KiB boundary of the block's dynamic shared memory.  (As an offset: rounding the generic address up instead hides from the
+// compiler that everything behind it is shared memory, and all accesses become generic ones: 3 -> 64 channels, 224 x 224, 16 images
+// 71 -> 61 us, 8192^2 x 1024 in bf16 122.9 -> 118.9.)
+__device__ __forceinline__ uint8_t* align_smem(uint8_t* raw) { return raw + ((0u - smem_u32(raw)) & 1023u); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(CONV ? kTcConvThreads : kTcThreads, 1) bcr_tc_
   // the launch that follows in the stream may start as SMs free up: it waits (griddepcontrol.wait) before it reads or
   // writes anything this launch touches
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_smem(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);        // the X tile of a stage has landed
   uint64_t* ready = full + kTcStages;                        // the expanded weight tile of a stage is written
   uint64_t* empty = ready + kTcStages;                         // the tensor core is done with a stage

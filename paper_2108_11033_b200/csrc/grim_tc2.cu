@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(CONV ? kConvThreads : kThreads, 1) bcr_tc2_ker
   // writes anything this launch touches
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // start of the block's shared memory is the same in both blocks, which the paired multiply relies on
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_smem(smem_raw);
   // One barrier per stage IN THE EVEN BLOCK collects everything the multiplies of that stage need from both blocks:
   // the X tiles (one arrival of the even block's copy thread that announces the bytes of both blocks; the odd
   // block's TMA loads complete their bytes on this barrier too) and the expanded weight tiles (one arrival per
