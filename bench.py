@@ -317,7 +317,7 @@ class SpmmWorkload:
             self.tuned = B.grim_bcr_tune(h, x, y, reps=-5 if self.rotating else 5)
         torch.cuda.synchronize()
         tile = self.tuned["tile_n"]
-        names = {1: "bcr_direct_kernel" if tile & 32 else "bcr_ffma_kernel", 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
+        names = {1: "bcr_split_kernel" if tile == 64 else ("bcr_direct_kernel" if tile & 32 else "bcr_ffma_kernel"), 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
                  3: "bcr_narrow_kernel" if tile >= 4 else ("bcr_skinny_kernel" if tile == 1 else "bcr_stream_kernel")}
         self.kernel = names.get(self.tuned["path"], self.kernel)
         self.peak_kind = "tensor" if self.tuned["path"] in (2, 5) else "alu"

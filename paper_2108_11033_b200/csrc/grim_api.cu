@@ -64,6 +64,7 @@ grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, a.tile_n == 4 ? 0 : a.tile_n / 8, s);
   }
   if (path == 1 && direct_choice(a.tile_n)) return launch_direct(h, a, s);
+  if (path == 1 && a.tile_n >= 64 && a.tile_n <= 72 && split_path_supported(h, a)) return launch_split(h, a, s);
   if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
   if (path == 0 && narrow_preferred(h, a))
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, 0, s);
@@ -186,6 +187,7 @@ cudaError_t launch_maxpool(const void* in, void* out, int64_t planes, int64_t OH
 
 namespace grim {
 grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
+  if (split_preferred(h, a)) return launch_split(h, a, s);
   if (direct_preferred(h, a)) return launch_direct(h, a, s);
   return ffma_path_supported(h, a) ? launch_ffma(h, a, s) : launch_spmm(h, a, s);
 }
@@ -217,7 +219,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
   float best_t = -1.f;
   grim_tune_t cand_best{};
   // candidates: (path, tile_n); a candidate that cannot take the request is skipped
-  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {3, 4}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
+  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {1, 64}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {3, 4}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
   for (const auto& cd : cand) {
     grim_tune_t c{};
     c.path = cd[0];
@@ -228,8 +230,10 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
     if (c.path == 1 && c.tile_n <= 4 && c.tile_n > (h->bh <= 4 ? 4 : (h->bh <= 8 ? 2 : 1))) continue;
     if (c.path == 1 && (c.tile_n == 8 || c.tile_n == 9) && (h->bh > (c.tile_n == 8 ? 8 : 4) || X->cols <= 128)) continue;
     // ... 17, 18, 20 = the narrow tile (at most 16 columns) with 1, 2, 4 bands per warp
-    if (c.path == 1 && c.tile_n >= 17 && c.tile_n != 32 && (X->cols > 16 || c.tile_n - 16 > (h->bh <= 8 ? 4 : 2))) continue;
+    if (c.path == 1 && c.tile_n >= 17 && c.tile_n < 32 && (X->cols > 16 || c.tile_n - 16 > (h->bh <= 8 ? 4 : 2))) continue;
     if (c.path == 1 && c.tile_n < 17 && X->cols <= 16) continue;
+    // ... 64 = fp32 on the tensor cores: where it is as exact as the others
+    if (c.path == 1 && c.tile_n == 64 && !split_precise(h, mat_args(X, Y))) continue;
     st = run_spmm(h, X, Y, &c, s);  // warm-up
     if (st == GRIM_ERR_UNSUPPORTED) { st = GRIM_OK; continue; }
     if (st != GRIM_OK) break;
@@ -340,7 +344,9 @@ extern "C" grim_status_t grim_bcr_conv2d(grim_bcr_t h, const grim_conv_desc_t* d
       SpmmArgs m = one_image(0);
       // (with a margin of 15 % for what is the better known: the tensor cores' time, the direct kernel's against the slab kernel's)
       const bool tensor = tc_path_supported(h, m) && hw >= 128;
-      const double each = tensor ? 6.0 + 0.75 * (double)h->tc_ktiles : 1.0 + std::max(3.5, std::min(direct_time(h, m), slab_time(h, m)));
+      const double fp32 = split_preferred(h, m) ? split_time(h, m) : std::min(direct_time(h, m), slab_time(h, m));
+      const double each = tensor ? 6.0 + 0.75 * (double)h->tc_ktiles : 1.0 + std::max(3.5, fp32);
+      if (split_preferred(h, a) && split_time(h, a) <= each * (double)d->N) return launch_split(h, a, (cudaStream_t)stream);
       if (direct_time(h, a) <= each * (double)d->N * (tensor ? 0.85 : 1.15)) return launch_direct(h, a, (cudaStream_t)stream);
     }
   }

@@ -667,6 +667,17 @@ ConvPlan plan_for(int nkt, int64_t npix, int64_t M, int sms, bool gather) {
 
 }  // namespace
 
+// Tensor map of an fp32 matrix with contiguous rows (16-byte aligned, a multiple of four values apart).
+bool matrix_map_f32(const void* X, int64_t cols, int64_t rows, int64_t ld, int box_cols, int box_rows, void* map) {
+  if (!encode_tiled_fn()) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
+  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, estr[2] = {1, 1};
+  return encode_tiled_fn()(static_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(X), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Channels per copy of input pixels for a convolution with `taps` kernel positions: as few K tiles as possible.
 ConvLayout conv_layout_shape(int64_t K, int taps) {
   ConvLayout best;

@@ -148,6 +148,8 @@ Shape shape_for(const grim_bcr* h, const SpmmArgs& a) {
 }
 }  // namespace
 
+int direct_parts(const grim_bcr* h, const SpmmArgs& a) { return shape_for(h, a).parts; }
+
 // What a warp does one after the other (its chunks), what all warps issue (chunks and bands times tiles).  Fitted to 400 products and
 // 340 convolutions of 100 .. 8192 rows, 200 .. 8192 columns of W, N of 2 to 1024, rates 4 to 16: nine in ten within 15 %.
 double direct_time(const grim_bcr* h, const SpmmArgs& a) {

@@ -778,6 +778,14 @@ double slab_time(const grim_bcr* h, const SpmmArgs& a) {
   return 5.0 + (double)pl.stages * stage;
 }
 
+double slab_parts(const grim_bcr* h, const SpmmArgs& a) {
+  SlabPlan pl;
+  if (!ffma_path_supported(h, a) || !plan_slab(h, a, pl)) return 1.0;
+  double sum = 0.0;
+  for (int i = 0; i < pl.nseg; ++i) sum += (double)pl.seg[i].n / pl.seg[i].split;
+  return (double)pl.tiles / sum;
+}
+
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a) {
   if (h->device < 0 || !h->d_rc_stage || !h->d_status) return false;
   if (h->nbc > kJlistCap || h->rc_max_blob == 0 || h->rc_max_blob > 0xFFFF * 16u) return false;

@@ -104,6 +104,10 @@ inline uint32_t td_offset(uint32_t row, uint32_t col) {
   return row * 128u + ((((col >> 3) ^ (row & 7u))) << 4) + (col & 7u) * 2u;
 }
 
+// The same for fp32 handles whose weights are split into two fp16 numbers (grim_split.cu): a record of n entries (a multiple of eight;
+// the first one is repeated) holds n words hi | lo << 16 of the value times its row's scale, then n 16-bit offsets.  Entries are dealt
+// so that the 32 lanes of a warp, each with eight neighbouring entries, store into different banks as far as they go.
+
 // ---------------------------------------------------------------------------------------------
 // Weights of the tensor-core convolution (bf16 handles whose K is a multiple of the kernel positions of a 3 x 3 or 5 x 5
 // convolution): expanded, rows in natural order, columns by (kernel position, input channel) instead of (input channel,
@@ -160,6 +164,11 @@ struct grim_bcr {
   void* d_arena = nullptr;  // the one allocation that holds every array below except the scratch
   grim::RcStage* d_rc_stage = nullptr;
   grim::RcHead* d_rc_head = nullptr;
+  float* d_row_scale = nullptr;  // fp32 handles whose weights can be split into two fp16 numbers: power of two by which row r's are scaled
+  int64_t sp_mtiles = 0, sp_ktiles = 0;  // ... and their records, one per tile
+  uint32_t sp_max_rec = 0;
+  grim::RcStage* d_sp_stage = nullptr;
+  uint8_t* d_sp_blob = nullptr;
   int64_t rc_chunks = 0;  // chunks of eight kept columns, summed over all blocks
   uint8_t* d_rc_blob = nullptr;
   // tensor-core layout
@@ -226,13 +235,15 @@ grim_status_t launch_ffma(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool ffma_path_supported(const grim_bcr* h, const SpmmArgs& a);
 bool slab_rows_by_tma(const SpmmArgs& a);  // X is a matrix whose rows the slab kernel can fetch with TMA
 double direct_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
+int direct_parts(const grim_bcr* h, const SpmmArgs& a);    // warps that share a row's sum
 // bf16 handles: a copy of X with aligned rows for the tensor-core kernels, where the scratch for it is there
 size_t x_copy_size(const grim_bcr* h, int64_t ncols);
 size_t x_copy_area(const grim_bcr* h, int64_t max_ncols);  // what is reserved for copies of up to max_ncols columns
 bool x_copy_possible(const grim_bcr* h, const SpmmArgs& a);
 grim_status_t launch_x_copy(const grim_bcr* h, SpmmArgs& a, cudaStream_t s);  // a.X and a.x_sk become the copy's
 double slab_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
-// the CUDA-core kernel for a request: direct, slab or, for operands neither takes, the shared-memory slab fall-back
+double slab_parts(const grim_bcr* h, const SpmmArgs& a);  // thread blocks that share a row's sum, on average
+// fp32: the kernel that splits operands, where preferred; else the CUDA-core kernel for a request: direct, slab or, for operands neither takes, the shared-memory slab fall-back
 grim_status_t launch_cuda_cores(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 // small and middle-sized products without a block-wide pipeline (also convolutions)
 grim_status_t launch_direct(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
@@ -249,6 +260,14 @@ grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
 bool conv_tc_supported(const grim_bcr* h, const SpmmArgs& a);
 ConvLayout conv_layout_shape(int64_t K, int taps);
 size_t conv_scratch_bytes(const grim_bcr* h, int64_t max_ncols);
+// fp32 operands split into two fp16 numbers each, on the tensor cores (also convolutions)
+bool matrix_map_f32(const void* X, int64_t cols, int64_t rows, int64_t ld, int box_cols, int box_rows, void* map);  // a CUtensorMap
+grim_status_t launch_split(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
+bool split_path_supported(const grim_bcr* h, const SpmmArgs& a);
+double split_time(const grim_bcr* h, const SpmmArgs& a);  // estimate in us
+bool split_precise(const grim_bcr* h, const SpmmArgs& a);    // as exact as the kernel that would run otherwise
+bool split_preferred(const grim_bcr* h, const SpmmArgs& a);  // ... and done earlier
+grim_status_t build_split_records(grim_bcr* h);
 void count_launch(int n = 1);
 // streaming multiprocessors of a device (read once per device through the runtime)
 int sm_count(int device);

@@ -1,0 +1,738 @@
+// fp32 products and convolutions on the tensor cores (tcgen05), every operand split into two fp16 numbers: large right-hand
+// sides of fp32 handles (Section 3.1: every layer is a GEMM; Sections 4.3 - 4.5: compact weights expanded only on chip,
+// the expanded input of a convolution never produced in memory).
+//
+// A value v is scaled by a power of two to y with |y| < 2^13 and written as y = hi + lo, hi = fp16(y), lo = fp16(y - hi): 22
+// to 24 bits of it.  A product is then lo * hi + hi * lo + hi * hi (what is left out is below 2^-22 of it), three multiplies
+// that the tensor core sums in fp32.  Its additions truncate, so a sum only runs over 64 values of k (16 at a time) there;
+// the sums of those chunks are added up in registers, rounded to nearest.  The scale of the activations is
+// chosen per output column and chunk (the largest value in 64 rows of X), so that columns and groups of rows of very
+// different size keep their bits; the weights' per row.  Columns for which that is not enough - infinities, NaN, values
+// outside 2^-97 .. 2^60, more than two of 64 that are more than 2^16 below the largest but not zero - are worked out again
+// with fp32 multiplies (row_walk), product by kept product.
+//
+// The multiply is transposed: 128 columns of X are the rows of the tensor core's tile, 128 rows of W its columns.  A thread
+// that owns a column of X then finds the column's largest value, splits it and adds it up without looking at its
+// neighbours; loads and stores of 32 neighbouring columns are whole lines; and the activations go from registers to tensor memory
+// (the A operand is read from there), so that shared memory, whose bandwidth bounds the bf16 kernels, holds weights only.
+//
+// Per thread block: one thread requests packed weights (bulk copies), another 64 x 128 values of X (TMA, two K tiles ahead), four
+// warps expand the weights (a list of pairs of fp16 numbers and their places, made when the matrix is packed) into two swizzled tiles
+// of a 64-wide K tile (hi and lo), two groups of four warps split activations, K tiles in turn, one thread issues the multiplies (12
+// per K tile), eight warps add up.  With few tiles the blocks of a cluster share one, each multiplying a part of K; the sums
+// meet over distributed shared memory.
+//
+// What bounds it: the instructions of the two converting groups, some 3700 cycles a K tile each, against 768 cycles of multiplies
+// (8192^2, rate 8, N = 1024: 513 us, 128 K tiles in four rounds; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions
+// read pixels one by one and take 1.65 us a K tile, matrices 1.0.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "grim_device.cuh"
+#include "grim_internal.h"
+#include "grim_rowwalk.cuh"
+
+namespace grim {
+namespace {
+
+using namespace ptx;
+
+constexpr int kTile = 128;                        // rows of W and columns of X per thread block
+constexpr int kK = 64;                            // K per stage, and per sum in tensor memory
+constexpr int kStages = 3;
+constexpr int kXBytes = kK * kTile * 4;            // a K tile of activations as TMA brings it
+constexpr int kHalfBytes = kTile * kK * 2;        // one expanded tile of 16-bit weights
+constexpr int kStageBytes = 2 * kHalfBytes;       // hi and lo
+constexpr int kMaxRec = 8;                        // ring of packed weights
+constexpr int kExpand0 = 4, kConvert0 = 8, kSum0 = 16, kWarps = 24;  // first warps of the roles; 0: copies, 1: tensor core
+constexpr int kThreads = 32 * kWarps;
+// Registers per thread of the roles.  The block is launched with 80 x 768; what the first two give back the others take.
+constexpr int kRegsMisc = 40, kRegsExpand = 56, kRegsConvert = 96, kRegsSum = 96;
+static_assert(kRegsMisc + kRegsExpand + 2 * kRegsConvert + 2 * kRegsSum <= 6 * 80, "more registers than the block is launched with");
+constexpr int kMaxParts = 8;                      // thread blocks that share a tile
+constexpr int kInvSlots = 8;
+// shared memory: barriers and tables, stages, packed weights.  After the multiplies the stages hold the exchange of the
+// sums ([part][row][column]), behind it columns that were worked out again, behind those the walk's weight buffers.
+constexpr int kBars = 0, kTmem = 512, kAbort = 516, kAnyBad = 520, kMeta = 1024;           // kMeta: [record] entries
+constexpr int kRow = kMeta + kMaxRec * 4, kScale = kRow + kTile * 4, kInv = kScale + kTile * 4;  // [128] rows, scales; [8][128] 1 / scale
+constexpr int kBad = kInv + kInvSlots * kTile * 4, kTaps = kBad + kTile * 4;               // [128] flags; [2][2][64] kernel positions
+constexpr int kHdr = (kTaps + 2 * 2 * kK * 8 + 1023) / 1024 * 1024;
+constexpr int kExchangeBytes = (kTile + kMaxParts) * kTile * 4, kPatchBytes = kTile * kTile * 4;
+constexpr int kTailBytes = kExchangeBytes + kPatchBytes + 8 * kWalkBufFloats * 4;
+
+struct SplitParams {
+  RowWalk w;
+  const RcStage* stage;
+  const uint8_t* blob;
+  const uint32_t* band_order;
+  const float* row_scale;
+  unsigned* status;
+  int nbr, M, K, nbc, nkt;
+  int mtiles, parts, kt_per;
+  int nrec, tma;
+  uint32_t rec_stride;
+  unsigned spin_limit;
+  SpmmArgs a;
+};
+
+// K-major tile with rows of 128 bytes in the 128-byte swizzle, groups of eight rows 1 KiB apart.
+__device__ __forceinline__ uint64_t tile_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// fp32 sums, fp16 x fp16, both operands K-major, 128 x 128
+constexpr uint32_t kIdesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bdesc, uint32_t accumulate) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
+               ::"r"(d), "r"(a_tmem), "l"(bdesc), "r"(kIdesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+      "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Two values as fp16 pairs: hi = fp16(y), lo = fp16(y - hi).
+__device__ __forceinline__ void split2(float y0, float y1, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(y0, y1);
+  const float2 back = __half22float2(h);
+  const __half2 l = __floats2half2_rn(y0 - back.x, y1 - back.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// Expands a record (grim_internal.h) into the hi tile at `tile` and the lo tile behind it, both cleared before; the 128 threads of
+// the group (wt) take eight entries at a time.
+__device__ __forceinline__ void expand_record(uint32_t rec, uint32_t n, uint32_t tile, int wt) {
+  for (uint32_t v = (uint32_t)wt; v < (n >> 3); v += 128u) {
+    const uint4 a = lds128(rec + v * 32u), b = lds128(rec + v * 32u + 16u), at = lds128(rec + n * 4u + v * 16u);
+    const uint32_t val[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}, off[4] = {at.x, at.y, at.z, at.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t to = tile + (i & 1 ? off[i >> 1] >> 16 : off[i >> 1] & 0xFFFFu);
+      sts16(to, val[i]);
+      sts16(to + kHalfBytes, val[i] >> 16);
+    }
+  }
+}
+
+// Writes the record of a tile: a thread block per tile, a warp per block of the matrix, a lane per kept weight.
+constexpr int kBuildThreads = 128;
+__global__ void __launch_bounds__(kBuildThreads) build_records_kernel(RowWalk w, const RcStage* __restrict__ stage, const uint32_t* __restrict__ band_order,
+                                                                      const float* __restrict__ row_scale, int nbr, int bh, uint8_t* __restrict__ out) {
+  __shared__ uint32_t first[kTile / 4 * (kK / 16)];   // entries before each block
+  __shared__ uint32_t size[32];                       // entries that fall into each bank
+  __shared__ uint16_t rank_of[kTile * kK];            // ... and how many of its bank came before an entry
+  const int kt = blockIdx.x, mt = blockIdx.y, nkt = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const RcStage se = stage[(int64_t)mt * nkt + kt];
+  if (se.bytes == 0) return;
+  const int NB = kTile / bh, J = kK / w.bw, blocks = NB * J;
+  auto head_of = [&](int i) {
+    const int pos = mt * NB + i / J, j = kt * J + i % J;
+    RcHead h{0u, 0u, {0u, 0u}};
+    if (pos < nbr && j < w.nbc) h = w.head[(int64_t)pos * w.nbc + j];
+    return h;
+  };
+  if (tid < 32) size[tid] = 0;
+  for (int i = tid; i < blocks; i += kBuildThreads) {
+    const RcHead h = head_of(i);
+    first[i] = (uint32_t)(__popc(rc_head_rows(h.rows_kc)) * rc_head_kc(h.rows_kc));
+  }
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t sum = 0;
+    for (int i = 0; i < blocks; ++i) { const uint32_t n = first[i]; first[i] = sum; sum += n; }
+  }
+  __syncthreads();
+  const uint32_t n = se.bytes / 6;  // a multiple of eight: the first entry is repeated
+  uint32_t total = 0;
+  // position of an entry that is number r of its bank's: number r of all banks come before, then those of the banks to the left
+  auto position = [&](uint32_t bank, uint32_t r) {
+    uint32_t p = 0;
+    for (uint32_t b = 0; b < 32; ++b) p += min(size[b], r) + (b < bank && size[b] > r ? 1u : 0u);
+    return p;
+  };
+  // entry number p of a run of 256 is stored by lane p % lanes as its (p / lanes)-th of eight
+  auto put = [&](uint32_t p, uint32_t val, uint32_t off) {
+    const uint32_t run = p & ~255u, i = p - run, lanes = min(256u, n - run) >> 3, at = run + 8u * (i % lanes) + i / lanes;
+    reinterpret_cast<uint32_t*>(out + (size_t)se.off16 * 16)[at] = val;
+    reinterpret_cast<uint16_t*>(out + (size_t)se.off16 * 16 + (size_t)n * 4)[at] = (uint16_t)off;
+  };
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1)
+      for (int b = 0; b < 32; ++b) total += size[b];
+    for (int i = warp; i < blocks; i += kBuildThreads / 32) {
+      const RcHead h = head_of(i);
+      const uint32_t rows = rc_head_rows(h.rows_kc);
+      const int kc = rc_head_kc(h.rows_kc), kr = __popc(rows), nch = (kc + kRcChunk - 1) / kRcChunk;
+      const uint8_t* rec = w.blob + (size_t)h.rec16 * 16;
+      const float* wv = reinterpret_cast<const float*>(rec + ((8 + nch * kRcChunk + 15) & ~15));
+      for (int e = lane; e < kr * kc; e += 32) {
+        const int a = e / kc, c = e - a * kc;
+        uint32_t m = rows;
+        for (int k = 0; k < a; ++k) m &= m - 1;
+        const int r = __ffs(m) - 1, row = (i / J) * bh + r, col = (i % J) * w.bw + rec[8 + c];
+        const uint32_t off = (uint32_t)row * 128u + (((uint32_t)(col >> 3) ^ (uint32_t)(row & 7)) << 4) + (uint32_t)(col & 7) * 2u;
+        const uint32_t bank = (off >> 2) & 31u, id = first[i] + (uint32_t)e;
+        if (pass == 0) {
+          rank_of[id] = (uint16_t)atomicAdd(&size[bank], 1u);
+        } else {
+          const float y = wv[((c / kRcChunk) * kr + a) * kRcChunk + c % kRcChunk] * row_scale[(int64_t)band_order[mt * NB + i / J] * bh + r];
+          const __half hi = __float2half_rn(y), lo = __float2half_rn(y - __half2float(hi));
+          const uint32_t val = (uint32_t)__half_as_ushort(hi) | ((uint32_t)__half_as_ushort(lo) << 16);
+          put(position(bank, rank_of[id]), val, off);
+          if (id == 0)
+            for (uint32_t p = total; p < n; ++p) put(p, val, off);
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Columns that the split cannot hold, product by kept product: rows of the tile's bands worker, worker + 8, ... for the flagged ones
+// among 32 columns, into patch[row][column].
+template <int BH, int CONV>
+__device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, int64_t q0, int j0, int j1, int worker, int lane, const int* bad,
+                                           float* patch, float* wbuf) {
+  for (int c0 = 0; c0 < kTile; c0 += 32) {
+    const bool mine = bad[c0 + lane] != 0;
+    if (!__any_sync(0xffffffffu, mine)) continue;
+    RowWalk w = p.w;
+    w.j0 = j0; w.stride = p.nbc; w.nbc = j1 - j0;
+    WalkCols<1, 1> wc;
+    walk_setup<1, 1, float, CONV>(p.a, q0 + c0, lane, wc);
+    for (int lb = worker; lb < kTile / BH; lb += 8) {
+      const int pos = tile * (kTile / BH) + lb;
+      if (pos >= p.nbr) break;
+      float acc[BH];
+      unsigned long long unused[1][1];
+#pragma unroll
+      for (int r = 0; r < BH; ++r) acc[r] = 0.f;
+      row_walk<BH, 1, 1, float, CONV, true, true>(w, p.a, pos, 0, 1, wc, wbuf, lane, acc, unused, [] {});
+#pragma unroll
+      for (int r = 0; r < BH; ++r)
+        if (mine) patch[(lb * BH + r) * kTile + c0 + lane] = acc[r];
+      __syncwarp();
+    }
+  }
+}
+
+template <int N>
+__device__ __forceinline__ void more_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void fewer_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
+template <int BH, int CONV>
+__global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ SplitParams p) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  extern __shared__ uint8_t smem_raw[];
+  // (the offset of the 1 KiB boundary is the same in all blocks of a cluster)
+  uint8_t* smem = align_smem(smem_raw);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBars);  // both operands of a K tile are in place
+  uint64_t* empty = full + kStages;                            // its multiplies are done
+  uint64_t* sum_full = empty + kStages;                        // [2] a chunk's sums are complete
+  uint64_t* sum_empty = sum_full + 2;                          // [2] ... and have been read
+  uint64_t* rec_full = sum_empty + 2;
+  uint64_t* rec_empty = rec_full + kMaxRec;
+  uint64_t* x_full = rec_empty + kMaxRec;                      // [2] activations have landed
+  uint64_t* x_empty = x_full + 2;                              // [2] ... and are in registers
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kAbort);
+  int* s_any = reinterpret_cast<int*>(smem + kAnyBad);
+  uint32_t* s_meta = reinterpret_cast<uint32_t*>(smem + kMeta);
+  int* s_row = reinterpret_cast<int*>(smem + kRow);
+  float* s_scale = reinterpret_cast<float*>(smem + kScale);
+  float* s_inv = reinterpret_cast<float*>(smem + kInv);
+  int* s_bad = reinterpret_cast<int*>(smem + kBad);
+  uint8_t* stages = smem + kHdr;
+  uint8_t* xs = stages + kStages * kStageBytes;
+  uint8_t* recs = xs + (p.tma ? 2 * kXBytes : 0);
+
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const SpmmArgs& a = p.a;
+  const int parts = p.parts, part = parts > 1 ? (int)cluster_ctarank() : 0;
+  const int t = (int)blockIdx.x / parts, mt = t % p.mtiles;
+  const int64_t q0 = (int64_t)(t / p.mtiles) * kTile;
+  const int kt0 = part * p.kt_per, n = min(p.kt_per, p.nkt - kt0);  // this block's K tiles
+  const int J = kK / p.w.bw;
+  constexpr int NB = kTile / BH;
+
+  if (tid == 0) {
+    for (int s = 0; s < kStages; ++s) { mbar_init(full + s, 8); mbar_init(empty + s, 1); }
+    for (int s = 0; s < 2; ++s) { mbar_init(sum_full + s, 1); mbar_init(sum_empty + s, 8); mbar_init(x_full + s, 1); mbar_init(x_empty + s, 4); }
+    for (int s = 0; s < kMaxRec; ++s) { mbar_init(rec_full + s, 1); mbar_init(rec_empty + s, 4); }
+    *s_abort = 0;
+    *s_any = 0;
+    fence_mbar_init();
+  }
+  if (tid < kTile) {
+    const int pos = mt * NB + tid / BH;
+    int row = -1;
+    if (pos < p.nbr) row = (int)p.band_order[pos] * BH + (tid & (BH - 1));
+    if (row >= p.M) row = -1;
+    s_row[tid] = row;
+    s_scale[tid] = row >= 0 ? __frcp_rn(__ldg(p.row_scale + row)) : 1.f;  // (the inverse of a power of two is exact)
+    s_bad[tid] = 0;
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(smem + kTmem)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kTmem);
+  const uint32_t tmem_a = tmem + 256;  // columns 0 .. 255: two chunks' sums; then 64 per stage: 32 of hi, 32 of lo
+
+  // Every role goes through the same block barriers at its own end (registers are dealt by role, so the ends are not shared).
+  // After the first all multiplies are done and the stages are free.
+  auto end_of_loop = [&](bool failed, int fail_site) {
+    if (__any_sync(0xffffffffu, failed)) {
+      *s_abort = 1;
+      if (fail_site) atomicOr(p.status, (unsigned)GRIM_ERR_TIMEOUT | (1u << (8 + fail_site)));
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (*s_abort) let_copies_land();
+  };
+  auto rest = [&]() {  // of the barriers, for the roles that have nothing to do between them
+    if (*s_any && !*s_abort) { __syncthreads(); __syncthreads(); }
+    if (parts > 1) { cluster_sync_all(); cluster_sync_all(); }
+    __syncthreads();
+  };
+  float* exchange = reinterpret_cast<float*>(stages);
+  float* patch = reinterpret_cast<float*>(stages + kExchangeBytes);
+  bool failed = false;
+  int fail_site = 0;
+  if (warp < kExpand0) {
+    fewer_registers<kRegsMisc>();
+    if (warp == 0 && elect_one()) {
+      // ---------------------------------------------------------------- packed weights
+      const RcStage* stage = p.stage + (int64_t)mt * p.nkt + kt0;
+      RcStage next = stage[0];
+      int rs = 0;
+      unsigned par = 1;
+      for (int it = 0; it < n; ++it) {
+        const RcStage se = next;
+        if (it + 1 < n) next = stage[it + 1];
+        if (!mbar_wait(rec_empty + rs, par, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 1; break; }
+        s_meta[rs] = se.bytes / 6;
+        mbar_arrive_expect_tx(rec_full + rs, se.bytes);
+        if (se.bytes) bulk_load(recs + (size_t)rs * p.rec_stride, p.blob + (size_t)se.off16 * 16, se.bytes, rec_full + rs);
+        if (++rs == p.nrec) { rs = 0; par ^= 1u; }
+      }
+    } else if (warp == 1 && elect_one()) {
+      // ---------------------------------------------------------------- tensor core
+      int s = 0;
+      unsigned par = 0;
+      for (int it = 0; it < n; ++it) {
+        const int buf = it & 1;
+        if (!mbar_wait_tight(full + s, par, p.spin_limit << 2, s_abort)) { failed = true, fail_site = 2; break; }
+        if (!mbar_wait_tight(sum_empty + buf, (unsigned)((it >> 1) + 1) & 1u, p.spin_limit << 2, s_abort)) { failed = true, fail_site = 3; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem + (uint32_t)buf * kTile, xa = tmem_a + (uint32_t)s * 64u;
+        const uint64_t hi = tile_desc(smem_u32(stages + s * kStageBytes)), lo = hi + (kHalfBytes >> 4);
+        // the small products first; 16 values of k: eight columns of tensor memory, 32 bytes of a tile's rows
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 32u + 8u * k, hi + 2u * k, k > 0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 8u * k, lo + 2u * k, 1u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 8u * k, hi + 2u * k, 1u);
+        commit(empty + s);
+        commit(sum_full + buf);
+        if (++s == kStages) { s = 0; par ^= 1u; }
+      }
+    } else if (warp == 3 && p.tma && elect_one()) {
+      // ---------------------------------------------------------------- activations, two K tiles ahead
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      for (int it = 0; it < n; ++it) {
+        const int g = it & 1;
+        if (!mbar_wait(x_empty + g, (unsigned)((it >> 1) + 1) & 1u, p.spin_limit, s_abort, 20)) { failed = true, fail_site = 8; break; }
+        mbar_arrive_expect_tx(x_full + g, kXBytes);
+        tma_load_2d(xs + g * kXBytes, &tm_x, (int)q0, (kt0 + it) * kK, x_full + g);
+      }
+    }
+    __syncwarp();
+    end_of_loop(failed, fail_site);
+    rest();
+    if (warp == 2) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    }
+  } else if (warp < kConvert0) {
+    // ------------------------------------------------------------------ weights
+    fewer_registers<kRegsExpand>();
+    const int gw = warp & 3;
+    int rs = 0;
+    unsigned rpar = 0, par = 1;  // (a fresh barrier counts as emptied one round before)
+    int s = 0;
+    for (int it = 0; it < n; ++it, s = s + 1 == kStages ? 0 : s + 1, par ^= s == 0 ? 1u : 0u) {
+      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 32))) failed = true, fail_site = 4, *s_abort = 1;
+      uint8_t* tile = stages + s * kStageBytes;
+      if (!failed) {
+#pragma unroll
+        for (int i = 0; i < kStageBytes / 16 / 128; ++i) sts128(smem_u32(tile) + (uint32_t)(gw * 32 + lane + i * 128) * 16u, 0u, 0u, 0u, 0u);
+        if (!__all_sync(0xffffffffu, mbar_wait(rec_full + rs, rpar, p.spin_limit, s_abort, 32))) failed = true, fail_site = 5, *s_abort = 1;
+      }
+      named_barrier(1, 128);  // (also for a warp that has given up: the others may be waiting here)
+      if (failed) continue;
+      expand_record(smem_u32(recs + (size_t)rs * p.rec_stride), s_meta[rs], smem_u32(tile), gw * 32 + lane);
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(full + s);
+        mbar_arrive(rec_empty + rs);
+      }
+      if (++rs == p.nrec) { rs = 0; rpar ^= 1u; }
+    }
+    end_of_loop(failed, fail_site);
+    rest();
+  } else if (warp < kSum0) {
+    // ------------------------------------------------------------------ activations
+    more_registers<kRegsConvert>();
+    const int grp = (warp - kConvert0) >> 2, quarter = warp & 3, col = quarter * 32 + lane;
+    const uint32_t lanes = (uint32_t)(quarter * 32) << 16;
+    WalkCols<1, 1> wc;
+    walk_setup<1, 1, float, CONV>(a, q0 + quarter * 32, lane, wc);
+    const bool valid = q0 + col < a.ncols;
+    const float* X = static_cast<const float*>(wc.ptr[0]);
+    int2* taps = reinterpret_cast<int2*>(smem + kTaps) + grp * 2 * kK;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // what earlier launches in the stream wrote is complete
+    int s = grp;
+    unsigned par = 1;
+    auto advance = [&]() {
+      s += 2;
+      if (s >= kStages) { s -= kStages; par ^= 1u; }
+    };
+    for (int it = grp; it < n; it += 2, advance()) {
+      const int k0 = (kt0 + it) * kK;
+      float x[kK];
+      if (!CONV && p.tma) {
+        if (!failed && !__all_sync(0xffffffffu, mbar_wait(x_full + grp, (unsigned)(it >> 1) & 1u, p.spin_limit, s_abort, 32))) failed = true, fail_site = 9, *s_abort = 1;
+        const float* src = reinterpret_cast<const float*>(xs + grp * kXBytes) + col;  // (zeros past the last row and column)
+#pragma unroll
+        for (int k = 0; k < kK; ++k) x[k] = src[k * kTile];
+      } else if (CONV) {
+        // k -> offset in the input and kernel position (none that is inside, past the last k)
+        int2* tp = taps + ((it >> 1) & 1) * kK;
+        const int i = quarter * 32 + lane;
+        if (i < kK) {
+          const int k = k0 + i, khw = a.KH * a.KW, c = k / khw, rest = k - c * khw, kh = rest / a.KW, kw = rest - kh * a.KW;
+          tp[i] = k < p.K ? make_int2((c * a.H + kh) * a.W + kw, (int)((1u << kh) | (1u << (16 + kw)))) : make_int2(0, -1);
+        }
+        if (grp) named_barrier(3, 128); else named_barrier(2, 128);
+#pragma unroll
+        for (int k = 0; k < kK; ++k) {
+          const int2 tk = tp[k];
+          x[k] = 0.f;
+          if ((wc.valid[0] & (unsigned)tk.y) == (unsigned)tk.y) x[k] = __ldg(X + tk.x);
+        }
+      } else {
+        const float* xk = X + (int64_t)k0 * a.x_sk;
+        if (k0 + kK <= p.K) {
+#pragma unroll
+          for (int k = 0; k < kK; ++k, xk += a.x_sk) x[k] = __ldg(xk);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kK; ++k, xk += a.x_sk) x[k] = k0 + k < p.K ? __ldg(xk) : 0.f;
+        }
+      }
+      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 32))) failed = true, fail_site = 6, *s_abort = 1;
+      if (failed) continue;  // (as above)
+      // the largest magnitude (a NaN stays one), and the smallest but zero (2 * bits - 1: zero becomes the largest number)
+      float largest = 0.f;
+      uint32_t least = ~0u;
+#pragma unroll
+      for (int k = 0; k < kK; k += 2) {
+        asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(largest) : "f"(x[k]), "f"(x[k + 1]));
+        const uint32_t b0 = __float_as_uint(x[k]), b1 = __float_as_uint(x[k + 1]);
+        least = min(min(least, b0 + b0 - 1u), b1 + b1 - 1u);
+      }
+      const uint32_t big = __float_as_uint(largest);
+      if (!CONV && p.tma) {  // (all of x has been looked at)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(x_empty + grp);
+      }
+      const uint32_t e = big >> 23;  // scale 2^(12 - exponent): values below 2^13
+      const bool none = big == 0u;
+      bool bad = !none && (e < 30u || e > 187u);
+      if (!bad && !none && (least + 1u) >> 24 < e - 16u) {
+        int small = 0;
+        const float below = __uint_as_float((e - 16u) << 23);
+#pragma unroll
+        for (int k = 0; k < kK; ++k) small += x[k] != 0.f && fabsf(x[k]) < below;
+        bad = small > 2;
+      }
+      if (bad && valid) { s_bad[col] = 1; *s_any = 1; }
+      const bool plain = none || bad;
+      const float scale = plain ? (bad ? 0.f : 1.f) : __uint_as_float((266u - e) << 23);
+      s_inv[(it & (kInvSlots - 1)) * kTile + col] = plain ? 1.f : __uint_as_float((e - 12u) << 23);
+      const uint32_t to = tmem_a + lanes + (uint32_t)s * 64u;
+      uint32_t hi[kK / 2], lo[kK / 2];
+#pragma unroll
+      for (int i = 0; i < kK / 2; ++i) split2(x[2 * i] * scale, x[2 * i + 1] * scale, hi[i], lo[i]);
+      tmem_st32(to, hi);
+      tmem_st32(to + 32u, lo);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + s);
+    }
+    end_of_loop(failed, fail_site);
+    if (*s_any && !*s_abort) {
+      __syncthreads();  // the sums lie in `patch`
+      float* wbuf = reinterpret_cast<float*>(stages + kExchangeBytes + kPatchBytes) + (warp - kConvert0) * kWalkBufFloats;
+      exact_columns<BH, CONV>(p, mt, q0, kt0 * J, min(p.nbc, (kt0 + n) * J), warp - kConvert0, lane, s_bad, patch, wbuf);
+      __syncthreads();
+    }
+    if (parts > 1) { cluster_sync_all(); cluster_sync_all(); }
+    __syncthreads();
+  } else {
+    // ------------------------------------------------------------------ sums of the chunks
+    more_registers<kRegsSum>();
+    const int quarter = warp & 3, half = (warp - kSum0) >> 2, col = quarter * 32 + lane;
+    const uint32_t from = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64);
+    unsigned long long acc[32];  // a column of X, 64 rows of the tile, in pairs
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0ull;
+    for (int it = 0; it < n; ++it) {
+      const int buf = it & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(sum_full + buf, (unsigned)(it >> 1) & 1u, p.spin_limit << 2, s_abort, 32))) { failed = true, fail_site = 7; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const float inv = s_inv[(it & (kInvSlots - 1)) * kTile + col];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t v[16];
+        tmem_ld16(from + (uint32_t)(buf * kTile + c * 16), v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) walk_ffma2(acc[8 * c + i], walk_pair(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), walk_pair(inv, inv));
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sum_empty + buf);
+    }
+    end_of_loop(failed, fail_site);
+    const int64_t q = q0 + col;
+    // (through shared memory, so that what follows is loops and no more registers)
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      patch[(half * 64 + 2 * i) * kTile + col] = __uint_as_float((unsigned)acc[i]);
+      patch[(half * 64 + 2 * i + 1) * kTile + col] = __uint_as_float((unsigned)(acc[i] >> 32));
+    }
+    if (*s_any && !*s_abort) {
+      __syncthreads();  // flagged columns are worked out again by the warps that read the activations
+      __syncthreads();
+    }
+    const bool again = s_bad[col] != 0, writes = q < a.ncols && !*s_abort;
+    auto value = [&](int r) { return patch[r * kTile + col] * (again ? 1.f : s_scale[r]); };
+    int64_t at_q = q * a.y_sq, row_stride = a.y_sr;
+    if (CONV) {
+      row_stride = (int64_t)a.OH * a.OW;
+      const int64_t img = q / row_stride;
+      at_q = img * p.M * row_stride + (q - img * row_stride);
+    }
+    float* out = static_cast<float*>(a.Y) + at_q;
+    auto store = [&](int row, float v) {  // (row is the same in all lanes)
+      if (a.relu) v = fmaxf(v, 0.f);
+      if (writes) out[(int64_t)row * row_stride] = v;
+    };
+    if (parts == 1) {
+#pragma unroll 4
+      for (int r = half * 64; r < half * 64 + 64; ++r) {
+        const int row = s_row[r];
+        if (row >= 0) store(row, value(r) + (a.bias ? __ldg(a.bias + row) : 0.f));
+      }
+    } else {
+      // Every block of the cluster owns some of the tile's rows: each sends its sums of them to their owner, who adds them up.
+      const int nr = (kTile + parts - 1) / parts;
+      cluster_sync_all();
+      const uint32_t mine = smem_u32(exchange) + ((uint32_t)part * (uint32_t)nr * kTile + (uint32_t)col) * 4u;
+      for (int r = half * 64; r < half * 64 + 64;) {
+        const int owner = r / nr, first = owner * nr, end = min(first + nr, half * 64 + 64);
+        uint32_t to;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(mine + (uint32_t)(r - first) * (kTile * 4)), "r"(owner));
+#pragma unroll 4
+        for (; r < end; ++r, to += kTile * 4) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to), "f"(value(r)) : "memory");
+      }
+      __syncwarp();
+      cluster_sync_all();
+#pragma unroll 2
+      for (int r = half; r < min(nr, kTile - part * nr); r += 2) {
+        const int row = s_row[part * nr + r];
+        if (row < 0) continue;
+        // what the additions round off is summed on the side: otherwise a third of the whole error
+        float sum = 0.f, off = 0.f;
+        auto add = [&](float v) {
+          const float t = sum + v, w = t - sum;
+          off += (sum - (t - w)) + (v - w);
+          sum = t;
+        };
+        for (int s = 0; s < parts; ++s) add(exchange[(s * nr + r) * kTile + col]);
+        if (a.bias) add(__ldg(a.bias + row));
+        store(row, isfinite(off) ? sum + off : sum);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+uint32_t rec_stride_of(const grim_bcr* h) { return (h->sp_max_rec + 127u) & ~127u; }
+size_t smem_need(const grim_bcr* h, int nrec, bool tma) {
+  return 1024 + kHdr + std::max<size_t>((size_t)kStages * kStageBytes + (tma ? 2 * kXBytes : 0) + (size_t)nrec * rec_stride_of(h), kTailBytes);
+}
+int rec_slots(const grim_bcr* h, bool tma) {
+  for (int n = kMaxRec; n >= 2; --n)
+    if (smem_need(h, n, tma) <= 227 * 1024) return n;
+  return 0;
+}
+
+template <int BH>
+cudaError_t launch_rows(const CUtensorMap& tm, const SplitParams& p, unsigned grid, size_t smem, cudaStream_t s) {
+  auto kern = p.a.conv ? bcr_split_kernel<BH, 1> : bcr_split_kernel<BH, 0>;
+  const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)p.parts;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.parts > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, tm, p);
+}
+
+}  // namespace
+
+// Fills h->d_sp_blob, whose records h->d_sp_stage names, from the row-chunk layout.
+grim_status_t build_split_records(grim_bcr* h) {
+  RowWalk w;
+  w.head = h->d_rc_head; w.blob = h->d_rc_blob; w.nbc = (int)h->nbc; w.bw = h->bw;
+  build_records_kernel<<<dim3((unsigned)h->sp_ktiles, (unsigned)h->sp_mtiles), kBuildThreads>>>(w, h->d_sp_stage, h->d_band_order, h->d_row_scale, (int)h->nbr,
+                                                                                               h->bh, h->d_sp_blob);
+  return cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(nullptr) == cudaSuccess ? GRIM_OK : GRIM_ERR_CUDA;
+}
+
+bool split_path_supported(const grim_bcr* h, const SpmmArgs& a) {
+  if (h->device < 0 || h->dtype != GRIM_F32 || !h->d_sp_blob || !h->d_rc_head || !h->d_status || !rec_slots(h, false)) return false;
+  if (a.x_dtype != GRIM_F32 || a.y_dtype != GRIM_F32 || a.ncols <= 0) return false;
+  const int64_t tiles = (h->M + kTile) / kTile * ((a.ncols + kTile - 1) / kTile);
+  if (a.ncols > (int64_t(1) << 31) - 512 || tiles > (int64_t(1) << 27)) return false;
+  if (!a.conv && a.x_sk * 4 >= (int64_t(1) << 32)) return false;
+  if (a.conv && (a.KH > 16 || a.KW > 16 || (int64_t)a.C * a.H * a.W >= (int64_t(1) << 31))) return false;
+  return true;
+}
+
+namespace {
+// Thread blocks per tile: as many as run at once with K tiles for all of them (clusters of n that run at once on 148 SMs).
+struct Plan { int parts, kt_per; double rounds; };
+Plan plan_for(const grim_bcr* h, const SpmmArgs& a) {
+  static const int at_once[kMaxParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+  const int64_t tiles = h->sp_mtiles * ((a.ncols + kTile - 1) / kTile);
+  const int nkt = (int)h->sp_ktiles, sms = sm_count(h->device);
+  Plan pl{1, nkt, (double)((tiles + sms - 1) / sms)};
+  for (int n = 2; n <= kMaxParts; ++n) {
+    const int per = (nkt + n - 1) / n;
+    if (tiles * 148 <= (int64_t)at_once[n] * sms && per >= 2 && per < pl.kt_per && (n - 1) * per < nkt) pl = {n, per, 1.0};
+  }
+  return pl;
+}
+// rows that TMA can fetch come through shared memory, others (and a convolution's pixels) are read by the threads that split them
+bool rows_by_tma(const grim_bcr* h, const SpmmArgs& a) {
+  return !a.conv && a.x_sq == 1 && a.x_sk % 4 == 0 && reinterpret_cast<uintptr_t>(a.X) % 16 == 0 && rec_slots(h, true) >= 3;
+}
+}  // namespace
+
+// Estimate in us, fitted to 90 products and 100 convolutions of 256 .. 8192 rows and columns of W and N of 17 .. 105,000, rates 4 to 16:
+// nine in ten within 15 %.
+double split_time(const grim_bcr* h, const SpmmArgs& a) {
+  const Plan pl = plan_for(h, a);
+  if (a.conv) return 5.0 + pl.rounds * (pl.kt_per * 1.65 + 6.0) + (pl.parts > 1 ? 2.0 : 0.0);
+  return 6.0 + pl.rounds * (pl.kt_per * (rows_by_tma(h, a) ? 1.0 : 1.3) + 4.0) + (pl.parts > 1 ? 1.0 : 0.0);
+}
+
+// Errors, as a fraction of the result's norm.  Here: what the split and the tensor core's truncated sums leave, 1.1 .. 1.2e-7, and the
+// sums of chunks on top, so that 64 K tiles in a row come to 1.7e-7 and 128 to 2.1e-7.  fp32 kernels: 1.7e-8 (convolutions, whose results
+// ReLU thins out: 1.3e-8) times the square root of the products that one thread adds up; where several share a row, less by the root of
+// their number, but the sum of their sums comes on top.  Measured against fp64 over the same products as the estimate above: where this says
+// yes the error is 0.33 to 1.01 times that of the kernel whose place is taken, 0.6 on average (8192^2, N = 1024: 2.14e-7 against
+// 5.08e-7; 512 -> 512 channels, 28 x 28, one image: 1.26e-7 against 1.30e-7).
+bool split_precise(const grim_bcr* h, const SpmmArgs& a) {
+  if (!split_path_supported(h, a)) return false;
+  const double direct = direct_path_supported(h, a) ? direct_time(h, a) : 1e30, slab = a.conv ? 1e30 : slab_time(h, a);
+  const double keep = (double)h->nnz / (double)h->M, per = plan_for(h, a).kt_per;
+  const double parts = slab < direct ? slab_parts(h, a) : direct_parts(h, a), one = a.conv ? 1.3e-8 : 1.7e-8;
+  const double there = one * one * keep / parts + (parts > 1.0 ? 4.8e-16 * parts : 0.0);
+  const double here = a.conv ? 1.21e-14 * (1.0 + per / 60.0) : 1.44e-14 * (1.0 + per / 50.0);
+  return here <= there;
+}
+
+// Measured against the kernel that ran before (us): 8192^2, 8 x 32, N = 1024: 667 -> 513; 2240 x 2008, 16 x 64, N = 769: 280 -> 50;
+// 2880^2, 4 x 16, N = 17: 106 -> 21; 918 x 6592, N = 82: equal; 512 -> 512 channels, 28 x 28, one image: 62 -> 38; 384 -> 1250 inputs
+// kept to 314, 2500 pixels: 72 -> 31.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 19, and so on.
+bool split_preferred(const grim_bcr* h, const SpmmArgs& a) {
+  if (a.ncols <= kSkinnyMaxN || a.tile_n != 0 || (!a.conv && a.x_sq != 1) || !split_path_supported(h, a)) return false;
+  const double direct = direct_path_supported(h, a) ? direct_time(h, a) : 1e30, slab = a.conv ? 1e30 : slab_time(h, a);
+  return split_time(h, a) <= 0.92 * std::min(direct, slab) && split_precise(h, a);
+}
+
+grim_status_t launch_split(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s) {
+  if (!split_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
+  SplitParams p;
+  p.w.head = h->d_rc_head; p.w.blob = h->d_rc_blob; p.w.nbc = (int)h->nbc; p.w.bw = h->bw;
+  p.stage = h->d_sp_stage; p.blob = h->d_sp_blob; p.band_order = h->d_band_order; p.row_scale = h->d_row_scale; p.status = h->d_status;
+  p.nbr = (int)h->nbr; p.M = (int)h->M; p.K = (int)h->K; p.nbc = (int)h->nbc;
+  p.nkt = (int)h->sp_ktiles;
+  p.mtiles = (int)h->sp_mtiles;
+  CUtensorMap tm = {};
+  p.tma = rows_by_tma(h, a) && matrix_map_f32(a.X, a.ncols, h->K, a.x_sk, kTile, kK, &tm);
+  p.nrec = rec_slots(h, p.tma);
+  p.rec_stride = rec_stride_of(h);
+  p.spin_limit = 1u << 20;
+  p.a = a;
+  const int64_t tiles = (int64_t)p.mtiles * ((a.ncols + kTile - 1) / kTile);
+  const Plan pl = plan_for(h, a);
+  p.parts = pl.parts;
+  p.kt_per = pl.kt_per;
+  const int asked = a.tile_n - 64;  // test / tuning override
+  if (asked > 0 && asked <= kMaxParts && (asked - 1) * ((p.nkt + asked - 1) / asked) < p.nkt) {
+    p.parts = asked;
+    p.kt_per = (p.nkt + p.parts - 1) / p.parts;
+  }
+  const size_t smem = smem_need(h, p.nrec, p.tma);
+  const unsigned grid = (unsigned)(tiles * p.parts);
+  const cudaError_t e = h->bh == 4 ? launch_rows<4>(tm, p, grid, smem, s) : (h->bh == 8 ? launch_rows<8>(tm, p, grid, smem, s) : launch_rows<16>(tm, p, grid, smem, s));
+  count_launch();
+  if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
+  return GRIM_OK;
+}
+
+}  // namespace grim

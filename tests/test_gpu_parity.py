@@ -239,6 +239,73 @@ def test_direct_kernel_convolution(B, geom, bf16):
     check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=bf16, kernel_flags=B.GRIM_CONV_DIRECT)
 
 
+@pytest.mark.parametrize("parts", [1, 2, 3, 8])
+@pytest.mark.parametrize("case", [(128, 512, 128, 8, 32), (130, 577, 129, 8, 16), (259, 1090, 30, 16, 64), (600, 600, 260, 4, 16), (33, 900, 17, 4, 64), (300, 530, 1, 16, 16)])
+def test_split_operands(B, case, parts):
+    """Operands as pairs of fp16 numbers: rows, columns and K just past the tiles of 128, 128 and 64, every block height, up to eight
+    thread blocks to a tile (the last with less of K); rows and bands that keep nothing."""
+    M, K, N, bh, bw = case
+    W = gen.dense_weight(M, K, seed=411)
+    mask = gen.bcr_mask(M, K, bh, bw, compression=5, dist="zipf", seed=412, empty_frac=0.15)
+    mask[:2 * bh] = 0
+    X = gen.normal_f32((K, N), 1.0, 413, 0)
+    X[::3] = np.maximum(X[::3], 0.0)
+    check_spmm(B, W, mask, X, bh, bw, flags=parts & 1, path=1, tile_n=64 + parts)
+
+
+@pytest.mark.parametrize("parts", [1, 3])
+@pytest.mark.parametrize("bh,bw", [(4, 16), (8, 32), (16, 64)])
+def test_split_operands_of_any_range(B, bh, bw, parts):
+    """Columns of X that two fp16 numbers cannot hold - rows of very different size, an infinity, a NaN, numbers near the ends of
+    fp32's range - are as good as the others, and nothing of them reaches a row that does not keep them or another column."""
+    M, K, N = 300, 700, 140
+    W = gen.dense_weight(M, K, seed=421)
+    W[np.abs(W) < 1e-3] = 0.01
+    mask = gen.bcr_mask(M, K, bh, bw, compression=4, dist="uniform", seed=422, empty_frac=0.2)
+    X = gen.normal_f32((K, N), 1.0, 423, 0)
+    used = np.flatnonzero(mask.any(axis=0))
+    X[:, 3] *= 10.0 ** (np.arange(K) % 13 - 6)
+    X[:, 40] *= np.float32(1e-36)
+    X[:, 41] *= np.float32(1e35)
+    X[:, 42] = 0.0
+    X[:, 43] *= np.where(np.arange(K) % 16 == 0, 1.0, 1e-7).astype(np.float32)
+    X[used[5], 128], X[used[40], 129], X[used[-1], 139] = np.inf, np.nan, -np.inf
+    h = B.grim_bcr_pack(W, mask, bh, bw, B.GRIM_F32, 0)
+    try:
+        Y = torch.full((M, N), 7.0, device="cuda")
+        B.grim_bcr_spmm_ex(h, to_dev(X), Y, path=1, tile_n=64 + parts)
+        got = Y.cpu().numpy()
+        assert B.grim_bcr_status(h) == B.GRIM_OK
+    finally:
+        B.grim_bcr_destroy(h)
+    fin = np.isfinite(X)
+    X0, Wm = np.where(fin, X, 0.0).astype(np.float64), (W * mask).astype(np.float64)
+    want = Wm @ X0
+    for k, q in zip(*np.nonzero(~fin)):
+        want[mask[:, k] != 0, q] += W[mask[:, k] != 0, k].astype(np.float64) * X[k, q]
+    ok = np.isfinite(want)
+    assert not ok.all() and np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
+    # per element, against what the row itself keeps: fp32 sums lose about eps32 * sqrt(sum of squared products), times the square
+    # root of the number of additions (below 700); the 64-fold covers both and the split's 2^-22 of every product
+    scale = np.sqrt((Wm ** 2) @ (X0 ** 2))
+    assert np.all(np.abs(got[ok] - want[ok]) <= 64 * 2.0 ** -24 * scale[ok] + 1e-44)
+
+
+@pytest.mark.parametrize("geom", [(1, 200, 130, 25, 27, 3, 1, 1), (2, 133, 260, 31, 33, 5, 2, 2), (3, 400, 72, 61, 63, 3, 2, 0),
+                                  (3, 16, 264, 48, 61, 16, 3, 5), (2, 700, 500, 30, 29, 1, 1, 0), (5, 400, 520, 13, 15, 3, 1, 1)])
+def test_split_operands_convolution(B, geom):
+    """Convolutions that the kernel above is preferred for: pixels and rows just past its tiles, tiles that meet two images, strides,
+    kernels of 1 to 16; one thread block to a tile and several."""
+    nb, cin, cout, hh, ww, ksize, stride, pad = geom
+    K = cin * ksize * ksize
+    mask = gen.bcr_mask(cout, K, 8, 32, compression=3, dist="uniform", seed=431, empty_frac=0.1)
+    x = np.maximum(gen.normal_f32((nb, cin, hh, ww), 1.0, 432, 0), 0.0)
+    L = dict(W=gen.dense_weight(cout, K, seed=433), mask=mask, bias=gen.normal_f32((cout,), 0.05, 434, 0), bh=8, bw=32)
+    y = check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=False)
+    direct = check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=False, kernel_flags=B.GRIM_CONV_DIRECT)
+    assert not np.array_equal(y, direct)  # (another kernel)
+
+
 @pytest.mark.parametrize("out_bf16", [False, True])
 @pytest.mark.parametrize("geom", [
     (1, 64, 64, 16, 16, 3, 1, 1), (2, 30, 72, 9, 13, 3, 1, 1), (2, 17, 48, 12, 10, 5, 2, 2), (1, 130, 300, 15, 17, 3, 2, 1),
@@ -711,6 +778,7 @@ def check_conv(B, L, batch_x, *, ksize, stride, pad, bf16, relu=True, out_bf16=F
         scale = np.linalg.norm(Wm, axis=1)[None, :, None, None] * conv_col_norms(x, ksize, stride, pad)
         assert_close(got, want, scale, bf16_in=bf16, out_bf16=out_bf16,
                      bias_abs=np.abs(bias.astype(np.float64))[None, :, None, None], what="conv")
+        return got
     finally:
         B.grim_bcr_destroy(h)
 
