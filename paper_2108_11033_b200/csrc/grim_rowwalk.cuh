@@ -12,6 +12,8 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "grim_device.cuh"
 #include "grim_internal.h"
 
@@ -21,7 +23,9 @@ struct RowWalk {
   const RcHead* head;   // [schedule position][block column]
   const uint8_t* blob;
   int nbc, bw;
-  int j0 = 0, stride = 0;  // RANGE walks: the first block column, and the block columns of a band (nbc then counts those walked)
+};
+struct RowRange : RowWalk {  // only nbc block columns from j0 on, of `stride` that a band has
+  int j0, stride;
 };
 
 constexpr int kWalkChunkFloats = 8 * 16 + 8;               // a chunk's weights (at most 16 rows x 8 columns) and a row of slack
@@ -81,13 +85,20 @@ __device__ __forceinline__ void walk_setup(const SpmmArgs& a, int64_t q0, int la
 //
 // One chunk is in flight ahead of the one that is multiplied.  (Two were measured: no gain, the copies between register
 // sets cost what the latency gave - these kernels issue instructions most of the time.)
-// RANGE: only block columns w.j0 .. w.j0 + w.nbc - 1.
-template <int BH, int NC, int XV, typename XT, int CONV, bool SKIP, bool RANGE = false, typename BeforeX>
-__device__ __forceinline__ void row_walk(const RowWalk& w, const SpmmArgs& a, int pos, int part, int parts, const WalkCols<NC, XV>& wc,
+template <int BH, int NC, int XV, typename XT, int CONV, bool SKIP, typename Walk, typename BeforeX>
+__device__ __forceinline__ void row_walk(const Walk& w, const SpmmArgs& a, int pos, int part, int parts, const WalkCols<NC, XV>& wc,
                                          float* wbuf, int lane, float (&acc1)[NC == 1 ? BH : 1],
                                          unsigned long long (&acc2)[NC == 1 ? 1 : BH][NC == 1 ? 1 : NC / 2], BeforeX before_x) {
   constexpr int NP = NC == 1 ? 1 : NC / 2;
-  const uint4* heads = reinterpret_cast<const uint4*>(w.head) + (RANGE ? (int64_t)pos * w.stride + w.j0 : (int64_t)pos * w.nbc);
+  constexpr bool RANGE = std::is_same<Walk, RowRange>::value;
+  int j0 = 0;
+  const uint4* heads = reinterpret_cast<const uint4*>(w.head);
+  if constexpr (RANGE) {
+    j0 = w.j0;
+    heads += (int64_t)pos * w.stride + j0;
+  } else {
+    heads += (int64_t)pos * w.nbc;
+  }
   // a batch of up to 32 blocks: lane l holds the head of block column part + parts * (32 * batch + l)
   int jb = -1;
   unsigned todo = 0;  // lanes of the batch whose block has not been walked yet
@@ -119,7 +130,7 @@ __device__ __forceinline__ void row_walk(const RowWalk& w, const SpmmArgs& a, in
     kc = rc_head_kc(d);
     kr = __popc(rm);
     ch = 0;
-    k0 = ((RANGE ? w.j0 : 0) + part + parts * (jb * 32 + src)) * w.bw;
+    k0 = (j0 + part + parts * (jb * 32 + src)) * w.bw;
     return true;
   };
 

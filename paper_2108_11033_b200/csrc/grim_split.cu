@@ -217,7 +217,8 @@ __device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, in
   for (int c0 = 0; c0 < kTile; c0 += 32) {
     const bool mine = bad[c0 + lane] != 0;
     if (!__any_sync(0xffffffffu, mine)) continue;
-    RowWalk w = p.w;
+    RowRange w;
+    w.head = p.w.head; w.blob = p.w.blob; w.bw = p.w.bw;
     w.j0 = j0; w.stride = p.nbc; w.nbc = j1 - j0;
     WalkCols<1, 1> wc;
     walk_setup<1, 1, float, CONV>(p.a, q0 + c0, lane, wc);
@@ -228,7 +229,7 @@ __device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, in
       unsigned long long unused[1][1];
 #pragma unroll
       for (int r = 0; r < BH; ++r) acc[r] = 0.f;
-      row_walk<BH, 1, 1, float, CONV, true, true>(w, p.a, pos, 0, 1, wc, wbuf, lane, acc, unused, [] {});
+      row_walk<BH, 1, 1, float, CONV, true>(w, p.a, pos, 0, 1, wc, wbuf, lane, acc, unused, [] {});
 #pragma unroll
       for (int r = 0; r < BH; ++r)
         if (mine) patch[(lb * BH + r) * kTile + c0 + lane] = acc[r];
@@ -698,7 +699,10 @@ bool split_precise(const grim_bcr* h, const SpmmArgs& a) {
 // Measured against the kernel that ran before (us): 8192^2, 8 x 32, N = 1024: 667 -> 513; 2240 x 2008, 16 x 64, N = 769: 280 -> 50;
 // 2880^2, 4 x 16, N = 17: 106 -> 21; 918 x 6592, N = 82: equal; 512 -> 512 channels, 28 x 28, one image: 62 -> 38; 384 -> 1250 inputs
 // kept to 314, 2500 pixels: 72 -> 31.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 19, and so on.
+// (Below ten million products the direct kernel is done before this one has filled its pipeline, some 12 us: no estimates for the
+// smallest calls, 256^2, N = 64, whose 3.6 us are the host's: 3.65 -> 3.63.)
 bool split_preferred(const grim_bcr* h, const SpmmArgs& a) {
+  if (h->nnz * a.ncols < 10000000) return false;
   if (a.ncols <= kSkinnyMaxN || a.tile_n != 0 || (!a.conv && a.x_sq != 1) || !split_path_supported(h, a)) return false;
   const double direct = direct_path_supported(h, a) ? direct_time(h, a) : 1e30, slab = a.conv ? 1e30 : slab_time(h, a);
   return split_time(h, a) <= 0.92 * std::min(direct, slab) && split_precise(h, a);
