@@ -23,7 +23,7 @@
 // meet over distributed shared memory.
 //
 // What bounds it: the instructions of the two converting groups, some 3700 cycles a K tile each, against 768 cycles of multiplies
-// (8192^2, rate 8, N = 1024: 513 us, 128 K tiles in four rounds; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions
+// (8192^2, rate 8, N = 1024: 490 us, 128 K tiles in three rounds and a half; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions
 // read pixels one by one and take 1.65 us a K tile, matrices 1.0.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -74,6 +74,7 @@ struct SplitParams {
   int nrec, tma;
   uint32_t rec_stride;
   unsigned spin_limit;
+  int tile0;  // first tile of this launch
   SpmmArgs a;
 };
 
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const SpmmArgs& a = p.a;
   const int parts = p.parts, part = parts > 1 ? (int)cluster_ctarank() : 0;
-  const int t = (int)blockIdx.x / parts, mt = t % p.mtiles;
+  const int t = p.tile0 + (int)blockIdx.x / parts, mt = t % p.mtiles;
   const int64_t q0 = (int64_t)(t / p.mtiles) * kTile;
   const int kt0 = part * p.kt_per, n = min(p.kt_per, p.nkt - kt0);  // this block's K tiles
   const int J = kK / p.w.bw;
@@ -653,17 +654,20 @@ bool split_path_supported(const grim_bcr* h, const SpmmArgs& a) {
 }
 
 namespace {
-// Thread blocks per tile: as many as run at once with K tiles for all of them (clusters of n that run at once on 148 SMs).
-struct Plan { int parts, kt_per; double rounds; };
+// Whole rounds of tiles, a thread block each, and the tiles of the last round, which would leave SMs idle: as many blocks of a
+// cluster to each as run at once with K tiles for all of them (clusters of n that run at once on 148 SMs).  8192^2, N = 1024: 512
+// tiles are three rounds and 68 pairs, 490 us, where four rounds took 517.
+struct Plan { int64_t whole, tail; int parts, kt_per; };
 Plan plan_for(const grim_bcr* h, const SpmmArgs& a) {
   static const int at_once[kMaxParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
   const int64_t tiles = h->sp_mtiles * ((a.ncols + kTile - 1) / kTile);
   const int nkt = (int)h->sp_ktiles, sms = sm_count(h->device);
-  Plan pl{1, nkt, (double)((tiles + sms - 1) / sms)};
+  Plan pl{tiles - tiles % sms, tiles % sms, 1, nkt};
   for (int n = 2; n <= kMaxParts; ++n) {
     const int per = (nkt + n - 1) / n;
-    if (tiles * 148 <= (int64_t)at_once[n] * sms && per >= 2 && per < pl.kt_per && (n - 1) * per < nkt) pl = {n, per, 1.0};
+    if (pl.tail * 148 <= (int64_t)at_once[n] * sms && per >= 2 && per < pl.kt_per && (n - 1) * per < nkt) pl.parts = n, pl.kt_per = per;
   }
+  if (pl.whole && nkt - pl.kt_per < 6) pl = {tiles, 0, 1, nkt};  // (a second launch costs a few us)
   return pl;
 }
 // rows that TMA can fetch come through shared memory, others (and a convolution's pixels) are read by the threads that split them
@@ -676,8 +680,11 @@ bool rows_by_tma(const grim_bcr* h, const SpmmArgs& a) {
 // nine in ten within 15 %.
 double split_time(const grim_bcr* h, const SpmmArgs& a) {
   const Plan pl = plan_for(h, a);
-  if (a.conv) return 5.0 + pl.rounds * (pl.kt_per * 1.65 + 6.0) + (pl.parts > 1 ? 2.0 : 0.0);
-  return 6.0 + pl.rounds * (pl.kt_per * (rows_by_tma(h, a) ? 1.0 : 1.3) + 4.0) + (pl.parts > 1 ? 1.0 : 0.0);
+  const int sms = sm_count(h->device);
+  const double kt = a.conv ? 1.65 : (rows_by_tma(h, a) ? 1.0 : 1.3), ends = a.conv ? 6.0 : 4.0;
+  double t = (a.conv ? 5.0 : 6.0) + (double)((pl.whole + sms - 1) / sms) * ((double)h->sp_ktiles * kt + ends);
+  if (pl.tail) t += pl.kt_per * kt + ends + (pl.parts > 1 ? (a.conv ? 2.0 : 1.0) : 0.0) + (pl.whole && pl.parts > 1 ? 3.0 : 0.0);
+  return t;
 }
 
 // Errors, as a fraction of the result's norm.  Here: what the split and the tensor core's truncated sums leave, 1.1 .. 1.2e-7, and the
@@ -689,14 +696,15 @@ double split_time(const grim_bcr* h, const SpmmArgs& a) {
 bool split_precise(const grim_bcr* h, const SpmmArgs& a) {
   if (!split_path_supported(h, a)) return false;
   const double direct = direct_path_supported(h, a) ? direct_time(h, a) : 1e30, slab = a.conv ? 1e30 : slab_time(h, a);
-  const double keep = (double)h->nnz / (double)h->M, per = plan_for(h, a).kt_per;
+  const Plan pl = plan_for(h, a);
+  const double keep = (double)h->nnz / (double)h->M, per = pl.whole ? (double)h->sp_ktiles : (double)pl.kt_per;
   const double parts = slab < direct ? slab_parts(h, a) : direct_parts(h, a), one = a.conv ? 1.3e-8 : 1.7e-8;
   const double there = one * one * keep / parts + (parts > 1.0 ? 4.8e-16 * parts : 0.0);
   const double here = a.conv ? 1.21e-14 * (1.0 + per / 60.0) : 1.44e-14 * (1.0 + per / 50.0);
   return here <= there;
 }
 
-// Measured against the kernel that ran before (us): 8192^2, 8 x 32, N = 1024: 667 -> 513; 2240 x 2008, 16 x 64, N = 769: 280 -> 50;
+// Measured against the kernel that ran before (us): 8192^2, 8 x 32, N = 1024: 667 -> 490; 2240 x 2008, 16 x 64, N = 769: 280 -> 50;
 // 2880^2, 4 x 16, N = 17: 106 -> 21; 918 x 6592, N = 82: equal; 512 -> 512 channels, 28 x 28, one image: 62 -> 38; 384 -> 1250 inputs
 // kept to 314, 2500 pixels: 72 -> 31.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 19, and so on.
 // (Below ten million products the direct kernel is done before this one has filled its pipeline, some 12 us: no estimates for the
@@ -722,19 +730,23 @@ grim_status_t launch_split(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s)
   p.rec_stride = rec_stride_of(h);
   p.spin_limit = 1u << 20;
   p.a = a;
-  const int64_t tiles = (int64_t)p.mtiles * ((a.ncols + kTile - 1) / kTile);
-  const Plan pl = plan_for(h, a);
-  p.parts = pl.parts;
-  p.kt_per = pl.kt_per;
+  Plan pl = plan_for(h, a);
   const int asked = a.tile_n - 64;  // test / tuning override
-  if (asked > 0 && asked <= kMaxParts && (asked - 1) * ((p.nkt + asked - 1) / asked) < p.nkt) {
-    p.parts = asked;
-    p.kt_per = (p.nkt + p.parts - 1) / p.parts;
-  }
+  if (asked > 0 && asked <= kMaxParts && (asked - 1) * ((p.nkt + asked - 1) / asked) < p.nkt)
+    pl = {0, pl.whole + pl.tail, asked, (p.nkt + asked - 1) / asked};
+  if (pl.parts == 1) pl = {0, pl.whole + pl.tail, 1, p.nkt};
   const size_t smem = smem_need(h, p.nrec, p.tma);
-  const unsigned grid = (unsigned)(tiles * p.parts);
-  const cudaError_t e = h->bh == 4 ? launch_rows<4>(tm, p, grid, smem, s) : (h->bh == 8 ? launch_rows<8>(tm, p, grid, smem, s) : launch_rows<16>(tm, p, grid, smem, s));
-  count_launch();
+  auto launch = [&](int64_t first, int64_t tiles, int parts, int kt_per) {
+    p.tile0 = (int)first;
+    p.parts = parts;
+    p.kt_per = kt_per;
+    const unsigned grid = (unsigned)(tiles * parts);
+    count_launch();
+    return h->bh == 4 ? launch_rows<4>(tm, p, grid, smem, s) : (h->bh == 8 ? launch_rows<8>(tm, p, grid, smem, s) : launch_rows<16>(tm, p, grid, smem, s));
+  };
+  cudaError_t e = cudaSuccess;
+  if (pl.whole) e = launch(0, pl.whole, 1, p.nkt);
+  if (pl.tail && e == cudaSuccess) e = launch(pl.whole, pl.tail, pl.parts, pl.kt_per);
   if (e != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_CUDA; }
   return GRIM_OK;
 }

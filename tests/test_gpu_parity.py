@@ -253,6 +253,15 @@ def test_split_operands(B, case, parts):
     check_spmm(B, W, mask, X, bh, bw, flags=parts & 1, path=1, tile_n=64 + parts)
 
 
+@pytest.mark.parametrize("M,K,N", [(1300, 1000, 1810), (390, 1100, 4900), (2600, 520, 1800)])
+def test_split_operands_last_round(B, M, K, N):
+    """More tiles than SMs: whole rounds in one launch, the tiles of the last one shared by clusters in another (165 tiles: 17 by eight
+    blocks; 156: 8; 315: 19, of a K that is cut into fewer parts than that)."""
+    W = gen.dense_weight(M, K, seed=441)
+    mask = gen.bcr_mask(M, K, 8, 32, compression=6, dist="uniform", seed=442)
+    check_spmm(B, W, mask, gen.normal_f32((K, N), 1.0, 443, 0), 8, 32, path=1, tile_n=64)
+
+
 @pytest.mark.parametrize("parts", [1, 3])
 @pytest.mark.parametrize("bh,bw", [(4, 16), (8, 32), (16, 64)])
 def test_split_operands_of_any_range(B, bh, bw, parts):
