@@ -463,6 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
       }
       if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 32))) failed = true, fail_site = 6, *s_abort = 1;
       if (failed) continue;  // (as above)
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");  // (another thread's multiplies have read what is overwritten below)
       // the largest magnitude (a NaN stays one), and the smallest but zero (2 * bits - 1: zero becomes the largest number)
       float largest = 0.f;
       uint32_t least = ~0u;
