@@ -104,8 +104,9 @@ typedef struct {
                       16-byte aligned), 32 + 1, 2 or 4 = with that many columns per lane, then plus 256 x the
                       number of warps that share a row band (1, 2, 4, 8, 16);
                       or 64 = the tensor-core kernel for fp32 handles with block heights 4, 8, 16 and widths 16, 32, 64
-                      (every operand is split into two fp16 numbers, products are summed in fp32, and columns of X
-                      whose range that cannot hold are worked out in fp32), 64 + 1 - 8 = with that many thread blocks
+                      (every operand is split into three bf16 numbers that hold all of it, products are summed in
+                      fp32; columns of X with infinities, NaN or magnitudes below 2^-108 or from 2^61 on are worked out
+                      in fp32), 64 + 1 - 8 = with that many thread blocks
                       that share a tile's K (where it cannot take the request, this means nothing);
                       path 3: 1 = values staged in registers, 2 = values streamed through shared memory by bulk
                       asynchronous copies (persistent thread blocks), 0 = the streaming variant when it fits,

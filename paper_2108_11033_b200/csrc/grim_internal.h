@@ -104,9 +104,12 @@ inline uint32_t td_offset(uint32_t row, uint32_t col) {
   return row * 128u + ((((col >> 3) ^ (row & 7u))) << 4) + (col & 7u) * 2u;
 }
 
-// The same for fp32 handles whose weights are split into two fp16 numbers (grim_split.cu): a record of n entries (a multiple of eight;
-// the first one is repeated) holds n words hi | lo << 16 of the value times its row's scale, then n 16-bit offsets.  Entries are dealt
-// so that the 32 lanes of a warp, each with eight neighbouring entries, store into different banks as far as they go.
+// The same for fp32 handles whose weights are split into three bf16 numbers (grim_split.cu): a record of n entries (a multiple of eight;
+// the first one is repeated) holds n values, then n 16-bit offsets.  Entries are dealt
+// so that the 32 lanes of a warp, each with eight neighbouring entries, store into different banks as far as they go.  Magnitudes that
+// are split, as bits: zero, and from 2^-108 (24 bits of it are there in bf16, whose last step is 2^-133) to below 2^61 of the activations
+// and 2^41 of the weights (no sum of the parts' products leaves fp32's range).
+constexpr uint32_t kSplitLeast = (127u - 108u) << 23, kSplitBeyondX = (127u + 61u) << 23, kSplitBeyondW = (127u + 41u) << 23;
 
 // ---------------------------------------------------------------------------------------------
 // Weights of the tensor-core convolution (bf16 handles whose K is a multiple of the kernel positions of a 3 x 3 or 5 x 5
@@ -164,8 +167,7 @@ struct grim_bcr {
   void* d_arena = nullptr;  // the one allocation that holds every array below except the scratch
   grim::RcStage* d_rc_stage = nullptr;
   grim::RcHead* d_rc_head = nullptr;
-  float* d_row_scale = nullptr;  // fp32 handles whose weights can be split into two fp16 numbers: power of two by which row r's are scaled
-  int64_t sp_mtiles = 0, sp_ktiles = 0;  // ... and their records, one per tile
+  int64_t sp_mtiles = 0, sp_ktiles = 0;  // fp32 handles whose weights can be split into three bf16 numbers: their records, one per tile
   uint32_t sp_max_rec = 0;
   grim::RcStage* d_sp_stage = nullptr;
   uint8_t* d_sp_blob = nullptr;
@@ -260,7 +262,7 @@ grim_status_t launch_conv_tc(const grim_bcr* h, const SpmmArgs& a, cudaStream_t 
 bool conv_tc_supported(const grim_bcr* h, const SpmmArgs& a);
 ConvLayout conv_layout_shape(int64_t K, int taps);
 size_t conv_scratch_bytes(const grim_bcr* h, int64_t max_ncols);
-// fp32 operands split into two fp16 numbers each, on the tensor cores (also convolutions)
+// fp32 operands split into three bf16 numbers each, on the tensor cores (also convolutions)
 bool matrix_map_f32(const void* X, int64_t cols, int64_t rows, int64_t ld, int box_cols, int box_rows, void* map);  // a CUtensorMap
 grim_status_t launch_split(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s);
 bool split_path_supported(const grim_bcr* h, const SpmmArgs& a);

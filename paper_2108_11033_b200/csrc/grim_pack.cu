@@ -93,10 +93,10 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
     std::vector<uint8_t> col_used((size_t)K, 0);
     std::vector<int64_t> row_nnz((size_t)M, 0);
     uint64_t nnz = 0;
-    // what the kernel that splits fp32 operands takes, and what it has to know about a row's weights: their largest and smallest magnitude
-    const bool split_shape = vdt == GRIM_F32 && (bh == 4 || bh == 8 || bh == 16) && (bw == 16 || bw == 32 || bw == 64) &&
-                             !(flags & (GRIM_PACK_NARROW_ONLY | GRIM_PACK_HOST_ONLY));
-    std::vector<uint32_t> row_big(split_shape ? (size_t)M : 0, 0u), row_least(split_shape ? (size_t)M : 0, ~0u);
+    // what the kernel that splits fp32 operands takes: these shapes, and weights whose magnitudes it can split
+    bool split = vdt == GRIM_F32 && (bh == 4 || bh == 8 || bh == 16) && (bw == 16 || bw == 32 || bw == 64) &&
+                 !(flags & (GRIM_PACK_NARROW_ONLY | GRIM_PACK_HOST_ONLY));
+    uint32_t largest = 0u, least = ~0u;
     for (int64_t i = 0; i < nbr; ++i) {
       const int hb = (int)std::min<int64_t>(bh, M - i * bh);
       for (int64_t j = 0; j < nbc; ++j) {
@@ -132,18 +132,13 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
                 h->vals.push_back(vdt == GRIM_BF16 ? round_bf16(wr[c]) : wr[c]);
                 col_used[(size_t)(j * bw + c)] = 1;
               }
-            if (split_shape) {
-              const float* v = h->vals.data() + h->vals.size() - b.kc;
-              uint32_t big = row_big[(size_t)(i * bh + r)], least = row_least[(size_t)(i * bh + r)];
-              for (int c = 0; c < b.kc; ++c) {
+            if (split)
+              for (const float *v = h->vals.data() + h->vals.size() - b.kc, *end = v + b.kc; v < end; ++v) {
                 uint32_t u;
-                std::memcpy(&u, v + c, 4);
-                big = std::max(big, u & 0x7FFFFFFFu);
+                std::memcpy(&u, v, 4);
+                largest = std::max(largest, u & 0x7FFFFFFFu);
                 least = std::min(least, (u & 0x7FFFFFFFu) - 1u);  // (zero becomes the largest)
               }
-              row_big[(size_t)(i * bh + r)] = big;
-              row_least[(size_t)(i * bh + r)] = least;
-            }
           }
           nnz += (uint64_t)b.kr * b.kc;
         }
@@ -406,43 +401,11 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
                           nbr * 4;
     }
 
-    // ---- scales of the rows for the tensor-core kernel that splits fp32 operands (grim_split.cu): the largest weight of a row
-    // becomes at least 2^12 and less than 2^13.  No scales, and with them no such kernel, where a row holds what that leaves too few
-    // bits of: more than a few weights that are not zero and more than 2^16 below its largest, or a largest one of unusual size.
-    std::vector<float> row_scale;
-    if (split_shape) {
-      // (a row whose smallest weight but zero is large enough, which is nearly all of them, need not be counted)
-      std::vector<uint32_t> small((size_t)M, 0u);
-      bool count = false;
-      auto below = [&](size_t r) { return row_big[r] >> 23 > 16 ? ((row_big[r] >> 23) - 16) << 23 : 0u; };
-      for (size_t r = 0; r < (size_t)M; ++r) count = count || row_least[r] + 1u < below(r);
-      for (int64_t i = 0; count && i < nbr; ++i)
-        for (int64_t j = 0; j < nbc; ++j) {
-          const HostBlock& b = h->blocks[(size_t)(i * nbc + j)];
-          const float* v = h->vals.data() + b.val_off;
-          for (uint32_t rm = b.kc ? b.rowmask : 0u; rm; rm &= rm - 1, v += b.kc) {
-            const size_t r = (size_t)(i * bh + __builtin_ctz(rm));
-            for (int c = 0; c < b.kc; ++c) {
-              uint32_t u;
-              std::memcpy(&u, v + c, 4);
-              small[r] += (u & 0x7FFFFFFFu) - 1u < below(r) - 1u;
-            }
-          }
-        }
-      row_scale.assign((size_t)M, 1.f);
-      for (int64_t r = 0; r < M; ++r) {
-        const uint32_t e = row_big[(size_t)r] >> 23;
-        if (row_big[(size_t)r] == 0) continue;
-        if (e < 87 || e > 167 || (int64_t)small[(size_t)r] > 2 + row_nnz[(size_t)r] / 64) { row_scale.clear(); break; }
-        const uint32_t u = (266u - e) << 23;
-        std::memcpy(&row_scale[(size_t)r], &u, 4);
-      }
-    }
-
-    // its records, one per 128 x 64 tile: their places here, their contents on the device once the row-chunk layout is there
+    split = split && largest < kSplitBeyondW && least >= kSplitLeast - 1u;
+    // ---- records for that kernel, one per 128 x 64 tile: their places here, their contents on the device once the row-chunk layout is there
     std::vector<RcStage> sp_stage;
     uint64_t sp_bytes = 0;
-    if (!row_scale.empty()) {
+    if (split) {
       const int S = kTcRows / bh, J = kTcK / bw;
       h->sp_mtiles = (nbr + S - 1) / S;
       h->sp_ktiles = (nbc + J - 1) / J;
@@ -459,7 +422,7 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
         h->sp_max_rec = std::max(h->sp_max_rec, n * 6);
         sp_bytes += (uint64_t)n * 6;
       }
-      if (sp_bytes / 16 >= (uint64_t(1) << 32) || h->sp_mtiles > 65535) row_scale.clear();
+      if (sp_bytes / 16 >= (uint64_t(1) << 32) || h->sp_mtiles > 65535) split = false;
     }
 
     // ---- tensor-core tiling (bf16 handles whose block shape tiles 128 x 64 evenly)
@@ -582,8 +545,7 @@ extern "C" grim_status_t grim_bcr_pack(const float* W, int64_t ldw, const uint8_
         ar.add(&h->d_rc_stage, rc_stage.data(), rc_stage.size() * sizeof(RcStage));
         ar.add(&h->d_rc_head, rc_head.data(), rc_head.size() * sizeof(RcHead));
         ar.add(&h->d_rc_blob, rc_blob.data(), rc_blob.size());
-        if (!row_scale.empty()) {
-          ar.add(&h->d_row_scale, row_scale.data(), row_scale.size() * 4);
+        if (split) {
           ar.add(&h->d_sp_stage, sp_stage.data(), sp_stage.size() * sizeof(RcStage));
           ar.add(&h->d_sp_blob, nullptr, 0, (size_t)sp_bytes);
         }

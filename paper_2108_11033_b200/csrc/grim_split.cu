@@ -1,32 +1,35 @@
-// fp32 products and convolutions on the tensor cores (tcgen05), every operand split into two fp16 numbers: large right-hand
+// fp32 products and convolutions on the tensor cores (tcgen05), every operand split into three bf16 numbers: large right-hand
 // sides of fp32 handles (Section 3.1: every layer is a GEMM; Sections 4.3 - 4.5: compact weights expanded only on chip,
 // the expanded input of a convolution never produced in memory).
 //
-// A value v is scaled by a power of two to y with |y| < 2^13 and written as y = hi + lo, hi = fp16(y), lo = fp16(y - hi): 22
-// to 24 bits of it.  A product is then lo * hi + hi * lo + hi * hi (what is left out is below 2^-22 of it), three multiplies
-// that the tensor core sums in fp32.  Its additions truncate, so a sum only runs over 64 values of k (16 at a time) there;
-// the sums of those chunks are added up in registers, rounded to nearest.  The scale of the activations is
-// chosen per output column and chunk (the largest value in 64 rows of X), so that columns and groups of rows of very
-// different size keep their bits; the weights' per row.  Columns for which that is not enough - infinities, NaN, values
-// outside 2^-97 .. 2^60, more than two of 64 that are more than 2^16 below the largest but not zero - are worked out again
-// with fp32 multiplies (row_walk), product by kept product.
+// A value v is written as b1 + b2 + b3, b1 = bf16(v), b2 = bf16(v - b1), b3 = v - b1 - b2: three times eight bits, so that the sum is v
+// itself, all 24 bits of it, whatever its neighbours are (bf16 has fp32's exponents; nothing is scaled).  A product is the sum of the six
+// products of parts that are not below its own last bit (b1 b1, b1 b2, b2 b1, b2 b2, b1 b3, b3 b1; what is left out is below 2^-25 of it),
+// the small ones first, which the tensor core sums in fp32.  Its additions truncate, so a sum only runs over 64 values of k (16 at a
+// time) there; the sums of those chunks are added up in registers, rounded to nearest.  (Measured: products and sums down to 2^-149 are
+// kept as fp32 multiplies keep them.)  Columns of X with infinities, NaN or numbers so small or large that parts or sums of products leave
+// the range (kSplitLeast and the following) are worked out again with fp32 multiplies (row_walk), product by kept product; handles with such
+// weights have no layout for this kernel.
+// (Two fp16 numbers and a scale per column and 64 values of k need half the multiplies, but lose what is much smaller than its
+// neighbours in k: a row of a pruned matrix that does not keep the large ones then consists of what was lost.)
 //
 // The multiply is transposed: 128 columns of X are the rows of the tensor core's tile, 128 rows of W its columns.  A thread
-// that owns a column of X then finds the column's largest value, splits it and adds it up without looking at its
+// that owns a column of X then splits it and adds it up without looking at its
 // neighbours; loads and stores of 32 neighbouring columns are whole lines; and the activations go from registers to tensor memory
 // (the A operand is read from there), so that shared memory, whose bandwidth bounds the bf16 kernels, holds weights only.
 //
 // Per thread block: one thread requests packed weights (bulk copies), another 64 x 128 values of X (TMA, two K tiles ahead), four
-// warps expand the weights (a list of pairs of fp16 numbers and their places, made when the matrix is packed) into two swizzled tiles
-// of a 64-wide K tile (hi and lo), two groups of four warps split activations, K tiles in turn, one thread issues the multiplies (12
+// warps expand the weights (a list of them and their places, made when the matrix is packed) into three swizzled tiles
+// of a 64-wide K tile, two groups of four warps split activations, K tiles in turn, one thread issues the multiplies (24
 // per K tile), eight warps add up.  With few tiles the blocks of a cluster share one, each multiplying a part of K; the sums
 // meet over distributed shared memory.
 //
-// What bounds it: the instructions of the two converting groups, some 3700 cycles a K tile each, against 768 cycles of multiplies
-// (8192^2, rate 8, N = 1024: 490 us, 128 K tiles in three rounds and a half; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions
-// read pixels one by one and take 1.65 us a K tile, matrices 1.0.
+// What bounds it: the chains of the expanding and the converting warps, some 2200 cycles a K tile (two stages, so that a K tile's operands
+// are written while the tile before it is multiplied) against 1536 of multiplies (8192^2, rate 8, N = 1024: 524 us, 128 K tiles in three
+// rounds and a half; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions read pixels one by one and take 1.55 us a K tile,
+// matrices 1.15.
 #include <cuda.h>
-#include <cuda_fp16.h>
+#include <cuda_bf16.h>
 
 #include <algorithm>
 
@@ -41,23 +44,23 @@ using namespace ptx;
 
 constexpr int kTile = 128;                        // rows of W and columns of X per thread block
 constexpr int kK = 64;                            // K per stage, and per sum in tensor memory
-constexpr int kStages = 3;
+constexpr int kStages = 2;                        // a converting group's own each
+constexpr int kParts = 3;                         // bf16 numbers to a value
 constexpr int kXBytes = kK * kTile * 4;            // a K tile of activations as TMA brings it
-constexpr int kHalfBytes = kTile * kK * 2;        // one expanded tile of 16-bit weights
-constexpr int kStageBytes = 2 * kHalfBytes;       // hi and lo
+constexpr int kPartBytes = kTile * kK * 2;        // one expanded tile of 16-bit weights
+constexpr int kStageBytes = kParts * kPartBytes;
+constexpr int kPartCols = kK / 2, kStageCols = kParts * kPartCols;  // columns of tensor memory that a part, a stage of activations takes
 constexpr int kMaxRec = 8;                        // ring of packed weights
 constexpr int kExpand0 = 4, kConvert0 = 8, kSum0 = 16, kWarps = 24;  // first warps of the roles; 0: copies, 1: tensor core
 constexpr int kThreads = 32 * kWarps;
 // Registers per thread of the roles.  The block is launched with 80 x 768; what the first two give back the others take.
-constexpr int kRegsMisc = 40, kRegsExpand = 56, kRegsConvert = 96, kRegsSum = 96;
+constexpr int kRegsMisc = 40, kRegsExpand = 56, kRegsConvert = 104, kRegsSum = 88;
 static_assert(kRegsMisc + kRegsExpand + 2 * kRegsConvert + 2 * kRegsSum <= 6 * 80, "more registers than the block is launched with");
 constexpr int kMaxParts = 8;                      // thread blocks that share a tile
-constexpr int kInvSlots = 8;
 // shared memory: barriers and tables, stages, packed weights.  After the multiplies the stages hold the exchange of the
 // sums ([part][row][column]), behind it columns that were worked out again, behind those the walk's weight buffers.
 constexpr int kBars = 0, kTmem = 512, kAbort = 516, kAnyBad = 520, kMeta = 1024;           // kMeta: [record] entries
-constexpr int kRow = kMeta + kMaxRec * 4, kScale = kRow + kTile * 4, kInv = kScale + kTile * 4;  // [128] rows, scales; [8][128] 1 / scale
-constexpr int kBad = kInv + kInvSlots * kTile * 4, kTaps = kBad + kTile * 4;               // [128] flags; [2][2][64] kernel positions
+constexpr int kRow = kMeta + kMaxRec * 4, kBad = kRow + kTile * 4, kTaps = kBad + kTile * 4;  // [128] rows; [128] flags; [2][2][64] kernel positions
 constexpr int kHdr = (kTaps + 2 * 2 * kK * 8 + 1023) / 1024 * 1024;
 constexpr int kExchangeBytes = (kTile + kMaxParts) * kTile * 4, kPatchBytes = kTile * kTile * 4;
 constexpr int kTailBytes = kExchangeBytes + kPatchBytes + 8 * kWalkBufFloats * 4;
@@ -67,7 +70,6 @@ struct SplitParams {
   const RcStage* stage;
   const uint8_t* blob;
   const uint32_t* band_order;
-  const float* row_scale;
   unsigned* status;
   int nbr, M, K, nbc, nkt;
   int mtiles, parts, kt_per;
@@ -82,8 +84,8 @@ struct SplitParams {
 __device__ __forceinline__ uint64_t tile_desc(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
-// fp32 sums, fp16 x fp16, both operands K-major, 128 x 128
-constexpr uint32_t kIdesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+// fp32 sums, bf16 x bf16, both operands K-major, 128 x 128
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bdesc, uint32_t accumulate) {
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
@@ -92,14 +94,11 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bde
 __device__ __forceinline__ void commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
-      "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -112,34 +111,49 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Two values as fp16 pairs: hi = fp16(y), lo = fp16(y - hi).
-__device__ __forceinline__ void split2(float y0, float y1, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(y0, y1);
-  const float2 back = __half22float2(h);
-  const __half2 l = __floats2half2_rn(y0 - back.x, y1 - back.y);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
+// The next part of two values: their bf16 numbers, which leave them.  PAIR: both subtractions in one instruction, which wants
+// neighbouring registers (the convolution's loop has none to spare for that).
+template <bool PAIR>
+__device__ __forceinline__ uint32_t take_part(unsigned long long& x) {
+  const float x0 = __uint_as_float((uint32_t)x), x1 = __uint_as_float((uint32_t)(x >> 32));
+  const __nv_bfloat162 b = __floats2bfloat162_rn(x0, x1);
+  const uint32_t u = *reinterpret_cast<const uint32_t*>(&b);
+  const float b0 = __uint_as_float(u << 16), b1 = __uint_as_float(u & 0xFFFF0000u);
+  if (PAIR) walk_ffma2(x, walk_pair(b0, b1), walk_pair(-1.f, -1.f));
+  else x = walk_pair(x0 - b0, x1 - b1);
+  return u;
 }
 
-// Expands a record (grim_internal.h) into the hi tile at `tile` and the lo tile behind it, both cleared before; the 128 threads of
-// the group (wt) take eight entries at a time.
-__device__ __forceinline__ void expand_record(uint32_t rec, uint32_t n, uint32_t tile, int wt) {
-  for (uint32_t v = (uint32_t)wt; v < (n >> 3); v += 128u) {
+// Entries v of a record (grim_internal.h), eight of them: their parts and places.
+struct Entries {
+  uint32_t part[kParts][4], off[4];
+  __device__ __forceinline__ void load(uint32_t rec, uint32_t n, uint32_t v) {
     const uint4 a = lds128(rec + v * 32u), b = lds128(rec + v * 32u + 16u), at = lds128(rec + n * 4u + v * 16u);
-    const uint32_t val[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}, off[4] = {at.x, at.y, at.z, at.w};
+    unsigned long long w[4] = {(unsigned long long)a.y << 32 | a.x, (unsigned long long)a.w << 32 | a.z,
+                               (unsigned long long)b.y << 32 | b.x, (unsigned long long)b.w << 32 | b.z};
+    off[0] = at.x; off[1] = at.y; off[2] = at.z; off[3] = at.w;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t to = tile + (i & 1 ? off[i >> 1] >> 16 : off[i >> 1] & 0xFFFFu);
-      sts16(to, val[i]);
-      sts16(to + kHalfBytes, val[i] >> 16);
+    for (int l = 0; l < kParts; ++l)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) part[l][i] = take_part<true>(w[i]);
+  }
+  __device__ __forceinline__ void store(uint32_t tile) const {  // into the three tiles there
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t to0 = tile + (off[i] & 0xFFFFu), to1 = tile + (off[i] >> 16);
+#pragma unroll
+      for (int l = 0; l < kParts; ++l) {
+        sts16(to0 + l * kPartBytes, part[l][i]);
+        sts16(to1 + l * kPartBytes, part[l][i] >> 16);
+      }
     }
   }
-}
+};
 
 // Writes the record of a tile: a thread block per tile, a warp per block of the matrix, a lane per kept weight.
 constexpr int kBuildThreads = 128;
-__global__ void __launch_bounds__(kBuildThreads) build_records_kernel(RowWalk w, const RcStage* __restrict__ stage, const uint32_t* __restrict__ band_order,
-                                                                      const float* __restrict__ row_scale, int nbr, int bh, uint8_t* __restrict__ out) {
+__global__ void __launch_bounds__(kBuildThreads) build_records_kernel(RowWalk w, const RcStage* __restrict__ stage,
+                                                                      int nbr, int bh, uint8_t* __restrict__ out) {
   __shared__ uint32_t first[kTile / 4 * (kK / 16)];   // entries before each block
   __shared__ uint32_t size[32];                       // entries that fall into each bank
   __shared__ uint16_t rank_of[kTile * kK];            // ... and how many of its bank came before an entry
@@ -197,9 +211,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_records_kernel(RowWalk w,
         if (pass == 0) {
           rank_of[id] = (uint16_t)atomicAdd(&size[bank], 1u);
         } else {
-          const float y = wv[((c / kRcChunk) * kr + a) * kRcChunk + c % kRcChunk] * row_scale[(int64_t)band_order[mt * NB + i / J] * bh + r];
-          const __half hi = __float2half_rn(y), lo = __float2half_rn(y - __half2float(hi));
-          const uint32_t val = (uint32_t)__half_as_ushort(hi) | ((uint32_t)__half_as_ushort(lo) << 16);
+          const uint32_t val = __float_as_uint(wv[((c / kRcChunk) * kr + a) * kRcChunk + c % kRcChunk]);
           put(position(bank, rank_of[id]), val, off);
           if (id == 0)
             for (uint32_t p = total; p < n; ++p) put(p, val, off);
@@ -262,8 +274,6 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
   int* s_any = reinterpret_cast<int*>(smem + kAnyBad);
   uint32_t* s_meta = reinterpret_cast<uint32_t*>(smem + kMeta);
   int* s_row = reinterpret_cast<int*>(smem + kRow);
-  float* s_scale = reinterpret_cast<float*>(smem + kScale);
-  float* s_inv = reinterpret_cast<float*>(smem + kInv);
   int* s_bad = reinterpret_cast<int*>(smem + kBad);
   uint8_t* stages = smem + kHdr;
   uint8_t* xs = stages + kStages * kStageBytes;
@@ -293,7 +303,6 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
     if (pos < p.nbr) row = (int)p.band_order[pos] * BH + (tid & (BH - 1));
     if (row >= p.M) row = -1;
     s_row[tid] = row;
-    s_scale[tid] = row >= 0 ? __frcp_rn(__ldg(p.row_scale + row)) : 1.f;  // (the inverse of a power of two is exact)
     s_bad[tid] = 0;
   }
   if (warp == 2) {
@@ -304,7 +313,7 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kTmem);
-  const uint32_t tmem_a = tmem + 256;  // columns 0 .. 255: two chunks' sums; then 64 per stage: 32 of hi, 32 of lo
+  const uint32_t tmem_a = tmem + 256;  // columns 0 .. 255: two chunks' sums; then 96 per stage
 
   // Every role goes through the same block barriers at its own end (registers are dealt by role, so the ends are not shared).
   // After the first all multiplies are done and the stages are free.
@@ -353,15 +362,19 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
         if (!mbar_wait_tight(full + s, par, p.spin_limit << 2, s_abort)) { failed = true, fail_site = 2; break; }
         if (!mbar_wait_tight(sum_empty + buf, (unsigned)((it >> 1) + 1) & 1u, p.spin_limit << 2, s_abort)) { failed = true, fail_site = 3; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + (uint32_t)buf * kTile, xa = tmem_a + (uint32_t)s * 64u;
-        const uint64_t hi = tile_desc(smem_u32(stages + s * kStageBytes)), lo = hi + (kHalfBytes >> 4);
+        const uint32_t d = tmem + (uint32_t)buf * kTile, xa = tmem_a + (uint32_t)s * kStageCols;
+        const uint64_t w = tile_desc(smem_u32(stages + s * kStageBytes));
         // the small products first; 16 values of k: eight columns of tensor memory, 32 bytes of a tile's rows
+        auto products = [&](int of_x, int of_w, bool first) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 32u + 8u * k, hi + 2u * k, k > 0);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 8u * k, lo + 2u * k, 1u);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) mma_ts(d, xa + 8u * k, hi + 2u * k, 1u);
+          for (int k = 0; k < 4; ++k) mma_ts(d, xa + of_x * kPartCols + 8u * k, w + of_w * (kPartBytes >> 4) + 2u * k, !(first && k == 0));
+        };
+        products(2, 0, true);
+        products(0, 2, false);
+        products(1, 1, false);
+        products(1, 0, false);
+        products(0, 1, false);
+        products(0, 0, false);
         commit(empty + s);
         commit(sum_full + buf);
         if (++s == kStages) { s = 0; par ^= 1u; }
@@ -391,16 +404,24 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
     unsigned rpar = 0, par = 1;  // (a fresh barrier counts as emptied one round before)
     int s = 0;
     for (int it = 0; it < n; ++it, s = s + 1 == kStages ? 0 : s + 1, par ^= s == 0 ? 1u : 0u) {
-      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 32))) failed = true, fail_site = 4, *s_abort = 1;
-      uint8_t* tile = stages + s * kStageBytes;
+      // (a thread's first entries, mostly all that it has, are split before the stage is free)
+      if (!failed && !__all_sync(0xffffffffu, mbar_wait(rec_full + rs, rpar, p.spin_limit, s_abort, 32))) failed = true, fail_site = 5, *s_abort = 1;
+      const uint32_t rec = smem_u32(recs + (size_t)rs * p.rec_stride), tile = smem_u32(stages + s * kStageBytes), wt = (uint32_t)(gw * 32 + lane);
+      const uint32_t n = failed ? 0u : s_meta[rs];
+      Entries e;
+      if (wt < (n >> 3)) e.load(rec, n, wt);
+      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 0))) failed = true, fail_site = 4, *s_abort = 1;
       if (!failed) {
 #pragma unroll
-        for (int i = 0; i < kStageBytes / 16 / 128; ++i) sts128(smem_u32(tile) + (uint32_t)(gw * 32 + lane + i * 128) * 16u, 0u, 0u, 0u, 0u);
-        if (!__all_sync(0xffffffffu, mbar_wait(rec_full + rs, rpar, p.spin_limit, s_abort, 32))) failed = true, fail_site = 5, *s_abort = 1;
+        for (int i = 0; i < kStageBytes / 16 / 128; ++i) sts128(tile + (wt + i * 128) * 16u, 0u, 0u, 0u, 0u);
       }
       named_barrier(1, 128);  // (also for a warp that has given up: the others may be waiting here)
       if (failed) continue;
-      expand_record(smem_u32(recs + (size_t)rs * p.rec_stride), s_meta[rs], smem_u32(tile), gw * 32 + lane);
+      if (wt < (n >> 3)) e.store(tile);
+      for (uint32_t v = wt + 128u; v < (n >> 3); v += 128u) {
+        e.load(rec, n, v);
+        e.store(tile);
+      }
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) {
@@ -422,15 +443,11 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
     const float* X = static_cast<const float*>(wc.ptr[0]);
     int2* taps = reinterpret_cast<int2*>(smem + kTaps) + grp * 2 * kK;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // what earlier launches in the stream wrote is complete
-    int s = grp;
+    const int s = grp;  // (two groups, two stages)
     unsigned par = 1;
-    auto advance = [&]() {
-      s += 2;
-      if (s >= kStages) { s -= kStages; par ^= 1u; }
-    };
-    for (int it = grp; it < n; it += 2, advance()) {
+    for (int it = grp; it < n; it += 2, par ^= 1u) {
       const int k0 = (kt0 + it) * kK;
-      float x[kK];
+      union { float x[kK]; unsigned long long x2[kK / 2]; };
       if (!CONV && p.tma) {
         if (!failed && !__all_sync(0xffffffffu, mbar_wait(x_full + grp, (unsigned)(it >> 1) & 1u, p.spin_limit, s_abort, 32))) failed = true, fail_site = 9, *s_abort = 1;
         const float* src = reinterpret_cast<const float*>(xs + grp * kXBytes) + col;  // (zeros past the last row and column)
@@ -461,43 +478,36 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
           for (int k = 0; k < kK; ++k, xk += a.x_sk) x[k] = k0 + k < p.K ? __ldg(xk) : 0.f;
         }
       }
-      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 32))) failed = true, fail_site = 6, *s_abort = 1;
+      if (!failed && !__all_sync(0xffffffffu, mbar_wait(empty + s, par, p.spin_limit, s_abort, 0))) failed = true, fail_site = 6, *s_abort = 1;
       if (failed) continue;  // (as above)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");  // (another thread's multiplies have read what is overwritten below)
-      // the largest magnitude (a NaN stays one), and the smallest but zero (2 * bits - 1: zero becomes the largest number)
-      float largest = 0.f;
-      uint32_t least = ~0u;
+      // the largest and the smallest magnitude but zero among the first parts, in pairs of 16 bits: less one and with the sign bit
+      // set a zero becomes the smallest number without a sign and the largest with one
+      uint32_t largest = 0u, least = 0x7FFF7FFFu;
+      const uint32_t to = tmem_a + lanes + (uint32_t)s * kStageCols;
 #pragma unroll
-      for (int k = 0; k < kK; k += 2) {
-        asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(largest) : "f"(x[k]), "f"(x[k + 1]));
-        const uint32_t b0 = __float_as_uint(x[k]), b1 = __float_as_uint(x[k + 1]);
-        least = min(min(least, b0 + b0 - 1u), b1 + b1 - 1u);
-      }
-      const uint32_t big = __float_as_uint(largest);
-      if (!CONV && p.tma) {  // (all of x has been looked at)
-        __syncwarp();
-        if (lane == 0) mbar_arrive(x_empty + grp);
-      }
-      const uint32_t e = big >> 23;  // scale 2^(12 - exponent): values below 2^13
-      const bool none = big == 0u;
-      bool bad = !none && (e < 30u || e > 187u);
-      if (!bad && !none && (least + 1u) >> 24 < e - 16u) {
-        int small = 0;
-        const float below = __uint_as_float((e - 16u) << 23);
+      for (int l = 0; l < kParts; ++l)
 #pragma unroll
-        for (int k = 0; k < kK; ++k) small += x[k] != 0.f && fabsf(x[k]) < below;
-        bad = small > 2;
-      }
+        for (int h = 0; h < kPartCols; h += 16) {
+          uint32_t part[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            part[i] = take_part<!CONV>(x2[h + i]);
+            if (l == 0) {
+              const uint32_t b = (part[i] | 0x80008000u) - 0x00010001u;
+              largest = __vmaxu2(largest, b);
+              least = __vmins2(least, b);
+            }
+          }
+          tmem_st16(to + l * kPartCols + h, part);
+          if (!CONV && p.tma && l == 0 && h) {  // (all of x is in registers)
+            __syncwarp();
+            if (lane == 0) mbar_arrive(x_empty + grp);
+          }
+        }
+      const int low = min((int)(int16_t)(least & 0xFFFFu), (int)(int16_t)(least >> 16));
+      const bool bad = max(largest & 0xFFFFu, largest >> 16) >= 0x7FFFu + (kSplitBeyondX >> 16) || low < -0x8001 + (int)(kSplitLeast >> 16);
       if (bad && valid) { s_bad[col] = 1; *s_any = 1; }
-      const bool plain = none || bad;
-      const float scale = plain ? (bad ? 0.f : 1.f) : __uint_as_float((266u - e) << 23);
-      s_inv[(it & (kInvSlots - 1)) * kTile + col] = plain ? 1.f : __uint_as_float((e - 12u) << 23);
-      const uint32_t to = tmem_a + lanes + (uint32_t)s * 64u;
-      uint32_t hi[kK / 2], lo[kK / 2];
-#pragma unroll
-      for (int i = 0; i < kK / 2; ++i) split2(x[2 * i] * scale, x[2 * i + 1] * scale, hi[i], lo[i]);
-      tmem_st32(to, hi);
-      tmem_st32(to + 32u, lo);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -524,13 +534,13 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
       const int buf = it & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(sum_full + buf, (unsigned)(it >> 1) & 1u, p.spin_limit << 2, s_abort, 32))) { failed = true, fail_site = 7; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const float inv = s_inv[(it & (kInvSlots - 1)) * kTile + col];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         uint32_t v[16];
         tmem_ld16(from + (uint32_t)(buf * kTile + c * 16), v);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) walk_ffma2(acc[8 * c + i], walk_pair(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), walk_pair(inv, inv));
+        for (int i = 0; i < 8; ++i)
+          asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[8 * c + i]) : "l"(walk_pair(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]))));
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -548,8 +558,8 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
       __syncthreads();  // flagged columns are worked out again by the warps that read the activations
       __syncthreads();
     }
-    const bool again = s_bad[col] != 0, writes = q < a.ncols && !*s_abort;
-    auto value = [&](int r) { return patch[r * kTile + col] * (again ? 1.f : s_scale[r]); };
+    const bool writes = q < a.ncols && !*s_abort;
+    auto value = [&](int r) { return patch[r * kTile + col]; };
     int64_t at_q = q * a.y_sq, row_stride = a.y_sr;
     if (CONV) {
       row_stride = (int64_t)a.OH * a.OW;
@@ -639,8 +649,7 @@ cudaError_t launch_rows(const CUtensorMap& tm, const SplitParams& p, unsigned gr
 grim_status_t build_split_records(grim_bcr* h) {
   RowWalk w;
   w.head = h->d_rc_head; w.blob = h->d_rc_blob; w.nbc = (int)h->nbc; w.bw = h->bw;
-  build_records_kernel<<<dim3((unsigned)h->sp_ktiles, (unsigned)h->sp_mtiles), kBuildThreads>>>(w, h->d_sp_stage, h->d_band_order, h->d_row_scale, (int)h->nbr,
-                                                                                               h->bh, h->d_sp_blob);
+  build_records_kernel<<<dim3((unsigned)h->sp_ktiles, (unsigned)h->sp_mtiles), kBuildThreads>>>(w, h->d_sp_stage, (int)h->nbr, h->bh, h->d_sp_blob);
   return cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(nullptr) == cudaSuccess ? GRIM_OK : GRIM_ERR_CUDA;
 }
 
@@ -657,7 +666,7 @@ bool split_path_supported(const grim_bcr* h, const SpmmArgs& a) {
 namespace {
 // Whole rounds of tiles, a thread block each, and the tiles of the last round, which would leave SMs idle: as many blocks of a
 // cluster to each as run at once with K tiles for all of them (clusters of n that run at once on 148 SMs).  8192^2, N = 1024: 512
-// tiles are three rounds and 68 pairs, 490 us, where four rounds took 517.
+// tiles are three rounds and 68 pairs, 5 % less than four rounds.
 struct Plan { int64_t whole, tail; int parts, kt_per; };
 Plan plan_for(const grim_bcr* h, const SpmmArgs& a) {
   static const int at_once[kMaxParts + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
@@ -677,37 +686,42 @@ bool rows_by_tma(const grim_bcr* h, const SpmmArgs& a) {
 }
 }  // namespace
 
-// Estimate in us, fitted to 90 products and 100 convolutions of 256 .. 8192 rows and columns of W and N of 17 .. 105,000, rates 4 to 16:
-// nine in ten within 15 %.
+// Estimate in us, fitted to 119 products and 81 convolutions of 17 .. 8192 rows and 64 .. 12,800 columns of W and N of 17 .. 105,000, rates
+// 4 to 16: nine in ten within 15 %.
 double split_time(const grim_bcr* h, const SpmmArgs& a) {
   const Plan pl = plan_for(h, a);
   const int sms = sm_count(h->device);
-  const double kt = a.conv ? 1.65 : (rows_by_tma(h, a) ? 1.0 : 1.3), ends = a.conv ? 6.0 : 4.0;
-  double t = (a.conv ? 5.0 : 6.0) + (double)((pl.whole + sms - 1) / sms) * ((double)h->sp_ktiles * kt + ends);
+  const double kt = a.conv ? 1.55 : (rows_by_tma(h, a) ? 1.15 : 1.2), ends = a.conv ? 8.0 : 6.0;
+  double t = (a.conv ? 3.0 : 5.0) + (double)((pl.whole + sms - 1) / sms) * ((double)h->sp_ktiles * kt + ends);
   if (pl.tail) t += pl.kt_per * kt + ends + (pl.parts > 1 ? (a.conv ? 2.0 : 1.0) : 0.0) + (pl.whole && pl.parts > 1 ? 3.0 : 0.0);
   return t;
 }
 
-// Errors, as a fraction of the result's norm.  Here: what the split and the tensor core's truncated sums leave, 1.1 .. 1.2e-7, and the
-// sums of chunks on top, so that 64 K tiles in a row come to 1.7e-7 and 128 to 2.1e-7.  fp32 kernels: 1.7e-8 (convolutions, whose results
-// ReLU thins out: 1.3e-8) times the square root of the products that one thread adds up; where several share a row, less by the root of
-// their number, but the sum of their sums comes on top.  Measured against fp64 over the same products as the estimate above: where this says
-// yes the error is 0.33 to 1.01 times that of the kernel whose place is taken, 0.6 on average (8192^2, N = 1024: 2.14e-7 against
-// 5.08e-7; 512 -> 512 channels, 28 x 28, one image: 1.26e-7 against 1.30e-7).
+// Errors, squared, as fractions of the result's norm, fitted (with 10 % on this kernel's side) to fp64 comparisons of the products and
+// convolutions above: weights and activations of both signs, and all of one sign, where roundings of fp32 sums average out over
+// the threads that share a row's sum and the tensor core's truncations do not.  Here: truncations and the sums of chunks.  fp32 kernels: the
+// square root of the products that one thread adds up (convolutions, half of whose inputs ReLU has made zero: of fewer), and
+// the sum of the threads' sums.  Where this says yes the error is 0.24 to 0.97 times that of the kernel whose place is taken, 0.6 on average
+// (8192^2, N = 1024: 1.9e-7 against 5.1e-7; 512 -> 512 channels, 28 x 28, one image: 0.85e-7 against 1.26e-7), with one sign 0.25 to 1.11 times (1.4e-7
+// against 3.8e-7; 0.58e-7 against 0.67e-7), or below the rounding of a single result, 2^-24.
+// Up to 16 columns other kernels run, which spread a row over 32 lanes: no comparison, no yes.
 bool split_precise(const grim_bcr* h, const SpmmArgs& a) {
-  if (!split_path_supported(h, a)) return false;
+  if (a.ncols <= kSkinnyMaxN || !split_path_supported(h, a)) return false;
   const double direct = direct_path_supported(h, a) ? direct_time(h, a) : 1e30, slab = a.conv ? 1e30 : slab_time(h, a);
   const Plan pl = plan_for(h, a);
   const double keep = (double)h->nnz / (double)h->M, per = pl.whole ? (double)h->sp_ktiles : (double)pl.kt_per;
-  const double parts = slab < direct ? slab_parts(h, a) : direct_parts(h, a), one = a.conv ? 1.3e-8 : 1.7e-8;
-  const double there = one * one * keep / parts + (parts > 1.0 ? 4.8e-16 * parts : 0.0);
-  const double here = a.conv ? 1.21e-14 * (1.0 + per / 60.0) : 1.44e-14 * (1.0 + per / 50.0);
-  return here <= there;
+  const double threads = slab < direct ? slab_parts(h, a) : direct_parts(h, a), more = threads > 1.0 ? threads : 0.0;
+  const double share = per / (pl.whole ? 1.0 : (double)pl.parts);
+  const double here = a.conv ? 3.4e-15 + 2.5e-16 * per : 4.9e-15 + 2.1e-16 * per;
+  const double there = (a.conv ? 1.69e-16 : 2.89e-16) * keep / threads + 4.8e-16 * more;
+  const double here1 = a.conv ? 2.8e-15 + 1.3e-16 * share : 3.4e-15 + 1.2e-16 * share;
+  const double there1 = a.conv ? 1.0e-15 + 0.9e-16 * keep / (threads * threads) + 2e-16 * more : 1.4e-15 + 2.2e-16 * keep / (threads * threads) + 2e-16 * more;
+  return here <= there && here1 <= std::max(there1, 3.55e-15);
 }
 
-// Measured against the kernel that ran before (us): 8192^2, 8 x 32, N = 1024: 667 -> 490; 2240 x 2008, 16 x 64, N = 769: 280 -> 50;
-// 2880^2, 4 x 16, N = 17: 106 -> 21; 918 x 6592, N = 82: equal; 512 -> 512 channels, 28 x 28, one image: 62 -> 38; 384 -> 1250 inputs
-// kept to 314, 2500 pixels: 72 -> 31.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 19, and so on.
+// Measured against the kernel that runs otherwise (us): 8192^2, 8 x 32, N = 1024: 665 -> 524; 4096^2, 4 x 16, N = 512: 312 -> 91; 2880^2,
+// 4 x 16, N = 17: 66 -> 24; 4096 x 512, rate 4, N = 512: 34 -> 20; 4096^2, 16 x 64, N = 1024: equal; 512 -> 512 channels, 28 x 28, one
+// image: 62 -> 39.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 20, and so on.
 // (Below ten million products the direct kernel is done before this one has filled its pipeline, some 12 us: no estimates for the
 // smallest calls, 256^2, N = 64, whose 3.6 us are the host's: 3.65 -> 3.63.)
 bool split_preferred(const grim_bcr* h, const SpmmArgs& a) {
@@ -721,7 +735,7 @@ grim_status_t launch_split(const grim_bcr* h, const SpmmArgs& a, cudaStream_t s)
   if (!split_path_supported(h, a)) return GRIM_ERR_UNSUPPORTED;
   SplitParams p;
   p.w.head = h->d_rc_head; p.w.blob = h->d_rc_blob; p.w.nbc = (int)h->nbc; p.w.bw = h->bw;
-  p.stage = h->d_sp_stage; p.blob = h->d_sp_blob; p.band_order = h->d_band_order; p.row_scale = h->d_row_scale; p.status = h->d_status;
+  p.stage = h->d_sp_stage; p.blob = h->d_sp_blob; p.band_order = h->d_band_order; p.status = h->d_status;
   p.nbr = (int)h->nbr; p.M = (int)h->M; p.K = (int)h->K; p.nbc = (int)h->nbc;
   p.nkt = (int)h->sp_ktiles;
   p.mtiles = (int)h->sp_mtiles;

@@ -239,11 +239,27 @@ def test_direct_kernel_convolution(B, geom, bf16):
     check_conv(B, L, x, ksize=ksize, stride=stride, pad=pad, bf16=bf16, kernel_flags=B.GRIM_CONV_DIRECT)
 
 
+def split_and_direct(B, W, mask, X, bh, bw, parts, flags=0):
+    """Results of the kernel that splits operands and of the direct kernel, which have to be two kernels."""
+    h = B.grim_bcr_pack(W, mask, bh, bw, B.GRIM_F32, flags)
+    try:
+        out = []
+        for tile_n in (64 + parts, 32):
+            Y = torch.full((W.shape[0], X.shape[1]), 7.0, device="cuda")
+            B.grim_bcr_spmm_ex(h, to_dev(X), Y, path=1, tile_n=tile_n)
+            out.append(Y.cpu().numpy())
+        assert B.grim_bcr_status(h) == B.GRIM_OK
+    finally:
+        B.grim_bcr_destroy(h)
+    assert not np.array_equal(out[0], out[1], equal_nan=True)
+    return out
+
+
 @pytest.mark.parametrize("parts", [1, 2, 3, 8])
-@pytest.mark.parametrize("case", [(128, 512, 128, 8, 32), (130, 577, 129, 8, 16), (259, 1090, 30, 16, 64), (600, 600, 260, 4, 16), (33, 900, 17, 4, 64), (300, 530, 1, 16, 16)])
+@pytest.mark.parametrize("case", [(128, 512, 128, 8, 32), (130, 1000, 129, 8, 16), (259, 1500, 30, 16, 64), (600, 1000, 260, 4, 16), (33, 1500, 17, 4, 64), (300, 990, 1, 16, 16)])
 def test_split_operands(B, case, parts):
-    """Operands as pairs of fp16 numbers: rows, columns and K just past the tiles of 128, 128 and 64, every block height, up to eight
-    thread blocks to a tile (the last with less of K); rows and bands that keep nothing."""
+    """Operands as three bf16 numbers each: rows, columns and K just past the tiles of 128, 128 and 64, every block height, up to eight
+    thread blocks to a tile (the last with less of K; eight share 8, 16 and 24 K tiles); rows and bands that keep nothing."""
     M, K, N, bh, bw = case
     W = gen.dense_weight(M, K, seed=411)
     mask = gen.bcr_mask(M, K, bh, bw, compression=5, dist="zipf", seed=412, empty_frac=0.15)
@@ -251,6 +267,7 @@ def test_split_operands(B, case, parts):
     X = gen.normal_f32((K, N), 1.0, 413, 0)
     X[::3] = np.maximum(X[::3], 0.0)
     check_spmm(B, W, mask, X, bh, bw, flags=parts & 1, path=1, tile_n=64 + parts)
+    split_and_direct(B, W, mask, X, bh, bw, parts, parts & 1)
 
 
 @pytest.mark.parametrize("M,K,N", [(1300, 1000, 1810), (390, 1100, 4900), (2600, 520, 1800)])
@@ -259,14 +276,24 @@ def test_split_operands_last_round(B, M, K, N):
     blocks; 156: 8; 315: 19, of a K that is cut into fewer parts than that)."""
     W = gen.dense_weight(M, K, seed=441)
     mask = gen.bcr_mask(M, K, 8, 32, compression=6, dist="uniform", seed=442)
-    check_spmm(B, W, mask, gen.normal_f32((K, N), 1.0, 443, 0), 8, 32, path=1, tile_n=64)
+    X = gen.normal_f32((K, N), 1.0, 443, 0)
+    check_spmm(B, W, mask, X, 8, 32, path=1, tile_n=64)
+    split_and_direct(B, W, mask, X, 8, 32, 0)
+
+
+# Per element, against what the row itself keeps: fp32 sums lose about eps32 * sqrt(sum of squared products), times the square
+# root of the number of additions (below 700); the 64-fold covers both and what the split leaves out (2^-25 of every product).
+def assert_elements(got, Wm, X):
+    Wm, X = Wm.astype(np.float64), X.astype(np.float64)
+    scale = np.sqrt((Wm ** 2) @ (X ** 2))
+    assert np.all(np.abs(got - Wm @ X) <= 64 * 2.0 ** -24 * scale + 1e-44)
 
 
 @pytest.mark.parametrize("parts", [1, 3])
 @pytest.mark.parametrize("bh,bw", [(4, 16), (8, 32), (16, 64)])
 def test_split_operands_of_any_range(B, bh, bw, parts):
-    """Columns of X that two fp16 numbers cannot hold - rows of very different size, an infinity, a NaN, numbers near the ends of
-    fp32's range - are as good as the others, and nothing of them reaches a row that does not keep them or another column."""
+    """Rows of very different size; and columns of X that are not split - an infinity, a NaN, numbers near the ends of fp32's range -
+    are as good as the others, and nothing of them reaches a row that does not keep them or another column."""
     M, K, N = 300, 700, 140
     W = gen.dense_weight(M, K, seed=421)
     W[np.abs(W) < 1e-3] = 0.01
@@ -278,15 +305,10 @@ def test_split_operands_of_any_range(B, bh, bw, parts):
     X[:, 41] *= np.float32(1e35)
     X[:, 42] = 0.0
     X[:, 43] *= np.where(np.arange(K) % 16 == 0, 1.0, 1e-7).astype(np.float32)
+    X[:, 44] *= np.float32(2.0 ** -107)  # some below what is split, most above
+    X[:, 45] *= np.float32(2.0 ** 61)
     X[used[5], 128], X[used[40], 129], X[used[-1], 139] = np.inf, np.nan, -np.inf
-    h = B.grim_bcr_pack(W, mask, bh, bw, B.GRIM_F32, 0)
-    try:
-        Y = torch.full((M, N), 7.0, device="cuda")
-        B.grim_bcr_spmm_ex(h, to_dev(X), Y, path=1, tile_n=64 + parts)
-        got = Y.cpu().numpy()
-        assert B.grim_bcr_status(h) == B.GRIM_OK
-    finally:
-        B.grim_bcr_destroy(h)
+    got, _ = split_and_direct(B, W, mask, X, bh, bw, parts)
     fin = np.isfinite(X)
     X0, Wm = np.where(fin, X, 0.0).astype(np.float64), (W * mask).astype(np.float64)
     want = Wm @ X0
@@ -294,10 +316,37 @@ def test_split_operands_of_any_range(B, bh, bw, parts):
         want[mask[:, k] != 0, q] += W[mask[:, k] != 0, k].astype(np.float64) * X[k, q]
     ok = np.isfinite(want)
     assert not ok.all() and np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
-    # per element, against what the row itself keeps: fp32 sums lose about eps32 * sqrt(sum of squared products), times the square
-    # root of the number of additions (below 700); the 64-fold covers both and the split's 2^-22 of every product
-    scale = np.sqrt((Wm ** 2) @ (X0 ** 2))
-    assert np.all(np.abs(got[ok] - want[ok]) <= 64 * 2.0 ** -24 * scale[ok] + 1e-44)
+    assert_elements(np.where(ok, got, Wm @ X0), Wm, X0)
+
+
+@pytest.mark.parametrize("parts", [1, 3])
+@pytest.mark.parametrize("large", ["activations", "weights"])
+@pytest.mark.parametrize("few", [1, 2, 24])
+@pytest.mark.parametrize("power", [17, 20, 24, 28, 36, 40, 60])
+def test_split_operands_elements_beside_large_ones(B, power, few, large, parts):
+    """In every 64 of k one activation that is 2^power times the others, in every row weights that are; one, two or many others.  A row
+    that keeps none of the large activations, a column that is zero at the large weights, consists of the others alone: its
+    elements are as exact as any."""
+    M, K, N, bh, bw = 320, 512, 136, 8, 32
+    W = gen.dense_weight(M, K, seed=451)
+    W[np.abs(W) < 1e-3] = 0.01
+    mask = gen.bcr_mask(M, K, bh, bw, compression=5, dist="uniform", seed=452)
+    rng = np.random.default_rng(453)
+    keep = rng.random((K // 64, 64, N)).argsort(axis=1).reshape(K, N) < few
+    X = np.where(keep, gen.normal_f32((K, N), 1.0, 454, 0), np.float32(0))
+    at = np.arange(K // 64) * 64 + 1 + 7 * np.arange(K // 64)
+    if large == "activations":
+        X[at] = np.float32(1.3 * 2.0 ** power)
+        small = (mask[:, at] == 0).all(axis=1)  # rows
+        assert 5 < small.sum() < M - 5
+    else:
+        others = np.setdiff1d(np.arange(K), at[:few]) if few <= 2 else at
+        W[:, others] *= np.float32(2.0 ** (power - 30))
+        W[:, np.setdiff1d(np.arange(K), others)] *= np.float32(2.0 ** -30)
+        X[at[:few]] = 1.0
+        X[others, : N // 2] = 0.0
+    got, _ = split_and_direct(B, W, mask, X, bh, bw, parts)
+    assert_elements(got, W * mask, X)
 
 
 @pytest.mark.parametrize("geom", [(1, 200, 130, 25, 27, 3, 1, 1), (2, 133, 260, 31, 33, 5, 2, 2), (3, 400, 72, 61, 63, 3, 2, 0),
