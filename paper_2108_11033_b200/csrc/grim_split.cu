@@ -59,8 +59,9 @@ static_assert(kRegsMisc + kRegsExpand + 2 * kRegsConvert + 2 * kRegsSum <= 6 * 8
 constexpr int kMaxParts = 8;                      // thread blocks that share a tile
 // shared memory: barriers and tables, stages, packed weights.  After the multiplies the stages hold the exchange of the
 // sums ([part][row][column]), behind it columns that were worked out again, behind those the walk's weight buffers.
-constexpr int kBars = 0, kTmem = 512, kAbort = 516, kAnyBad = 520, kMeta = 1024;           // kMeta: [record] entries
-constexpr int kRow = kMeta + kMaxRec * 4, kBad = kRow + kTile * 4, kTaps = kBad + kTile * 4;  // [128] rows; [128] flags; [2][2][64] kernel positions
+constexpr int kBars = 0, kTmem = 512, kAbort = 516, kAnyFlag = 520, kMeta = 1024;           // kMeta: [record] entries
+constexpr int kFlagTiles = 256;                   // K tiles of a block whose flagged columns are told apart
+constexpr int kRow = kMeta + kMaxRec * 4, kFlags = kRow + kTile * 4, kTaps = kFlags + kFlagTiles * kTile / 8;  // [128] rows; [K tile][128] flags; [2][2][64] kernel positions
 constexpr int kHdr = (kTaps + 2 * 2 * kK * 8 + 1023) / 1024 * 1024;
 constexpr int kExchangeBytes = (kTile + kMaxParts) * kTile * 4, kPatchBytes = kTile * kTile * 4;
 constexpr int kTailBytes = kExchangeBytes + kPatchBytes + 8 * kWalkBufFloats * 4;
@@ -222,17 +223,23 @@ __global__ void __launch_bounds__(kBuildThreads) build_records_kernel(RowWalk w,
   }
 }
 
-// Columns that the split cannot hold, product by kept product: rows of the tile's bands worker, worker + 8, ... for the flagged ones
-// among 32 columns, into patch[row][column].
+// What the split cannot hold, product by kept product: flagged columns of a K tile (bits of flags[K tile][column]), where the parts have
+// been left out, rows of the tile's bands worker, worker + 8, ..., are added to patch[row][column].  A block of more than
+// kFlagTiles K tiles has one set of flags, and its flagged columns are worked out again over all of its K.  (One row of X of 8192 x 1024
+// that is not finite: 8192^2, 8 x 32: 0.74 ms beside 0.54; worked out over the whole of K: 5.7 ms.)
 template <int BH, int CONV>
-__device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, int64_t q0, int j0, int j1, int worker, int lane, const int* bad,
+__device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, int64_t q0, int kt0, int n, int worker, int lane, const uint32_t* flags,
                                            float* patch, float* wbuf) {
-  for (int c0 = 0; c0 < kTile; c0 += 32) {
-    const bool mine = bad[c0 + lane] != 0;
-    if (!__any_sync(0xffffffffu, mine)) continue;
+  const bool apart = n <= kFlagTiles;
+  const int J = kK / p.w.bw;
+  for (int i = 0; i < (apart ? n : 1) * (kTile / 32); ++i) {
+    const int it = i / (kTile / 32), c0 = i % (kTile / 32) * 32;
+    const uint32_t flagged = flags[i];
+    if (!flagged) continue;
+    const bool mine = (flagged >> lane) & 1u;
     RowRange w;
     w.head = p.w.head; w.blob = p.w.blob; w.bw = p.w.bw;
-    w.j0 = j0; w.stride = p.nbc; w.nbc = j1 - j0;
+    w.j0 = (kt0 + it) * J; w.stride = p.nbc; w.nbc = min((apart ? 1 : n) * J, p.nbc - w.j0);
     WalkCols<1, 1> wc;
     walk_setup<1, 1, float, CONV>(p.a, q0 + c0, lane, wc);
     for (int lb = worker; lb < kTile / BH; lb += 8) {
@@ -244,8 +251,10 @@ __device__ __forceinline__ void exact_columns(const SplitParams& p, int tile, in
       for (int r = 0; r < BH; ++r) acc[r] = 0.f;
       row_walk<BH, 1, 1, float, CONV, true>(w, p.a, pos, 0, 1, wc, wbuf, lane, acc, unused, [] {});
 #pragma unroll
-      for (int r = 0; r < BH; ++r)
-        if (mine) patch[(lb * BH + r) * kTile + c0 + lane] = acc[r];
+      for (int r = 0; r < BH; ++r) {
+        float* at = patch + (lb * BH + r) * kTile + c0 + lane;
+        if (mine) *at = apart ? *at + acc[r] : acc[r];
+      }
       __syncwarp();
     }
   }
@@ -271,10 +280,10 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
   uint64_t* x_full = rec_empty + kMaxRec;                      // [2] activations have landed
   uint64_t* x_empty = x_full + 2;                              // [2] ... and are in registers
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kAbort);
-  int* s_any = reinterpret_cast<int*>(smem + kAnyBad);
+  int* s_any = reinterpret_cast<int*>(smem + kAnyFlag);
   uint32_t* s_meta = reinterpret_cast<uint32_t*>(smem + kMeta);
   int* s_row = reinterpret_cast<int*>(smem + kRow);
-  int* s_bad = reinterpret_cast<int*>(smem + kBad);
+  uint32_t* s_flags = reinterpret_cast<uint32_t*>(smem + kFlags);
   uint8_t* stages = smem + kHdr;
   uint8_t* xs = stages + kStages * kStageBytes;
   uint8_t* recs = xs + (p.tma ? 2 * kXBytes : 0);
@@ -286,7 +295,6 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
   const int t = p.tile0 + (int)blockIdx.x / parts, mt = t % p.mtiles;
   const int64_t q0 = (int64_t)(t / p.mtiles) * kTile;
   const int kt0 = part * p.kt_per, n = min(p.kt_per, p.nkt - kt0);  // this block's K tiles
-  const int J = kK / p.w.bw;
   constexpr int NB = kTile / BH;
 
   if (tid == 0) {
@@ -303,8 +311,8 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
     if (pos < p.nbr) row = (int)p.band_order[pos] * BH + (tid & (BH - 1));
     if (row >= p.M) row = -1;
     s_row[tid] = row;
-    s_bad[tid] = 0;
   }
+  for (int i = tid; i < kFlagTiles * kTile / 32; i += kThreads) s_flags[i] = 0u;
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(smem + kTmem)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -507,7 +515,22 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
         }
       const int low = min((int)(int16_t)(least & 0xFFFFu), (int)(int16_t)(least >> 16));
       const bool bad = max(largest & 0xFFFFu, largest >> 16) >= 0x7FFFu + (kSplitBeyondX >> 16) || low < -0x8001 + (int)(kSplitLeast >> 16);
-      if (bad && valid) { s_bad[col] = 1; *s_any = 1; }
+      const uint32_t flagged = __ballot_sync(0xffffffffu, bad && valid);
+      if (flagged) {  // their parts are left out
+        if (lane == 0) {
+          atomicOr(s_flags + (n <= kFlagTiles ? it : 0) * (kTile / 32) + quarter, flagged);
+          *s_any = 1;
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+#pragma unroll 1
+        for (int c = 0; c < kStageCols; c += 16) {
+          uint32_t part[16];
+          tmem_ld16(to + c, part);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) part[i] = bad ? 0u : part[i];
+          tmem_st16(to + c, part);
+        }
+      }
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -517,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) bcr_split_kernel(const __grid_con
     if (*s_any && !*s_abort) {
       __syncthreads();  // the sums lie in `patch`
       float* wbuf = reinterpret_cast<float*>(stages + kExchangeBytes + kPatchBytes) + (warp - kConvert0) * kWalkBufFloats;
-      exact_columns<BH, CONV>(p, mt, q0, kt0 * J, min(p.nbc, (kt0 + n) * J), warp - kConvert0, lane, s_bad, patch, wbuf);
+      exact_columns<BH, CONV>(p, mt, q0, kt0, n, warp - kConvert0, lane, s_flags, patch, wbuf);
       __syncthreads();
     }
     if (parts > 1) { cluster_sync_all(); cluster_sync_all(); }
