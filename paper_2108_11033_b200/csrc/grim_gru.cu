@@ -51,8 +51,8 @@ struct grim_gru {
   std::vector<float*> d_bih, d_bhh;
   std::vector<uint32_t*> d_pos_of_band;     // schedule position of every band of W_hh
   std::vector<uint32_t*> d_pos_of_band_ih;  // ... of W_ih
-  std::vector<float*> d_img_val;      // register images of the register-resident kernel (may be empty): W_hh of every layer, then,
-                                      // where the layers run in one launch, W_ih of layers 1 ...
+  std::vector<float*> d_img_val;      // register images of the register-resident kernels (may be empty): W_hh of every layer, and where
+                                      // the layers run in one launch W_hh from number stack_hh on, W_ih of layer l at stack_ih + l
   std::vector<uint32_t*> d_img_col;
   std::vector<float*> d_gi_saved;  // grim_gru_seq_static parks d_gi here while it points the pass at the static array
   std::vector<float*> d_gi;  // per layer: hoisted pre-activations, T x 3H (layers overlap in time, so each has its own)
@@ -74,6 +74,7 @@ struct grim_gru {
   ModeCfg grid, cluster;       // launch shapes of the shared-memory kernels
   ModeCfg regc;                // launch shape of the register-resident cluster kernel
   void (*reg_kern)(const GruParams) = nullptr;    // its compiled variant
+  int stack_hh = 0, stack_ih = 0;
   ModeCfg stack;                                  // launch shape of the same variant for all layers in one launch
   void (*stack_kern)(const GruStack) = nullptr;
   int device = -1;
@@ -1266,62 +1267,68 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
         g->cluster.ok = clusters_that_fit(smem_cluster_kernel(BHc), g->cluster) >= 1;
         if (!g->cluster.ok) g->cluster = ModeCfg{};
       }
-      // ---- register-resident cluster shape
-      // The matrices that are kept in registers: W_hh, and W_ih of the upper layers where all layers run in one launch - if a
-      // variant holds both, and as many clusters run at once.  (More than three layers: layers l and l + 2 share a buffer.)
-      std::vector<const grim_bcr*> mats = g->Whh;
-      const size_t only_hh = mats.size();
+      // ---- register-resident cluster shapes: for W_hh, and where all layers run in one launch for W_hh and the upper layers' W_ih
+      struct Candidate { double cost; const RegVariant* v; ModeCfg shape, stack; };
+      // variants that hold bands of max_cols columns on clusters of cs blocks, in the order of their costs (asking whether one fits costs
+      // more than all else here)
+      auto candidates = [&](int max_cols, int cs, bool stack) {
+        std::vector<Candidate> cands;
+        // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
+        const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc, units = tpc * bh;
+        for (const RegVariant& v : kRegVariants)
+          for (int ks = 1; ks <= 8; ks *= 2) {
+            const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
+            if (v.BH != BHc || 32 * v.s * ks < max_cols + ks - 1 || std::max(32 * warps, (units + 31) / 32 * 32) > v.threads) continue;
+            // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
+            // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
+            const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
+            const size_t words = (size_t)2 * H + (size_t)2 * nb * ks * BHc;
+            ModeCfg t;
+            t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
+            t.threads = std::max(32 * warps, std::max((units + 31) / 32 * 32, 128));
+            t.smem = ((words * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
+            ModeCfg u = t;
+            u.threads = (t.threads + 127) / 128 * 128 + kHelperThreads;  // whole warpgroups
+            // + pre-activations ahead and biases, states to be written
+            u.smem = (((words + (size_t)(kAheadSlots + 1) * 3 * units + 2 * (size_t)units + 1) * 4 + 15) & ~size_t(15)) + 32;
+            if ((stack ? u.smem : t.smem) <= kSmemLimit) cands.push_back({cost, &v, t, u});
+          }
+        std::stable_sort(cands.begin(), cands.end(), [](const Candidate& x, const Candidate& y) { return x.cost < y.cost; });
+        return cands;
+      };
+      // One launch for all layers: if a variant holds all matrices, as many clusters run at once, and its steps are not much longer than
+      // W_hh's own variant would make them (costs; steps against those of layers chunk by chunk, us: 752 and 632: 1.69 and 2.29; 384 and
+      // 285: 1.68 and 1.75; 354 and 230: 2.14 and 2.06; 648 and 188: 2.40 and 1.58).  More than three layers: layers l and l + 2 share a buffer.
+      constexpr double kLongerSteps = 1.4;
       bool stack = layers > 1 && layers <= kMaxStack;
       for (int l = 1; l < layers; ++l) stack = stack && W_ih[l]->bh == bh;
-      if (stack) mats.insert(mats.end(), g->Wih.begin() + 1, g->Wih.end());
-      const RegVariant* rv = nullptr;
-      for (int attempt = stack ? 0 : 1; attempt < 2 && !g->regc.ok; ++attempt) {
-        if (attempt == 1) mats.resize(only_hh);
-        const int max_cols = max_band_columns(mats);
-        for (int cs = 16; cs >= 1 && !g->regc.ok && H <= 65536; cs >>= 1) {
-          // (only CTAs that own units: the exchange's flow control rests on every CTA sending in every step)
-          const int tpc = (ntri + cs - 1) / cs, live = (ntri + tpc - 1) / tpc, nb = 3 * tpc, units = tpc * bh;
-          struct Candidate { double cost; const RegVariant* v; ModeCfg shape, stack; };
-          std::vector<Candidate> cands;
-          for (const RegVariant& v : kRegVariants)
-            for (int ks = 1; ks <= 8; ks *= 2) {
-              const int items = nb * ks, warps = (items + v.ni - 1) / v.ni;
-              if (v.BH != BHc || 32 * v.s * ks < max_cols + ks - 1 || std::max(32 * warps, (units + 31) / 32 * 32) > v.threads) continue;
-              // issue of a scheduler's share, then the items that a warp works off one after the other (1024 units, 8 x 32:
-              // 12 warps x 2 items 327 us for 200 steps, 8 x 3 items 325, 16 x 3 half items 361)
-              const double cost = (double)items * (v.s * (3 + BHc / 2) + 4 * BHc + 10) / 4 + v.ni * 20;
-              const size_t words = (size_t)2 * H + (size_t)2 * nb * ks * BHc;
-              ModeCfg t;
-              t.ctas = live; t.ks = ks; t.tpc = tpc; t.resident = 1;
-              t.threads = std::max(32 * warps, std::max((units + 31) / 32 * 32, 128));
-              t.smem = ((words * 4 + 15) & ~size_t(15)) + 32;  // + the two state barriers and a flag
-              ModeCfg u = t;
-              u.threads = (t.threads + 127) / 128 * 128 + kHelperThreads;  // whole warpgroups
-              // + pre-activations ahead and biases, states to be written
-              u.smem = (((words + (size_t)(kAheadSlots + 1) * 3 * units + 2 * (size_t)units + 1) * 4 + 15) & ~size_t(15)) + 32;
-              if (std::max(t.smem, u.smem) <= kSmemLimit) cands.push_back({cost, &v, t, u});
-            }
-          // (asked in the order of their costs: the question costs more than all else here)
-          std::stable_sort(cands.begin(), cands.end(), [](const Candidate& x, const Candidate& y) { return x.cost < y.cost; });
-          for (const Candidate& c : cands)
-            // (where the blocks with helpers fit, those without do: asking is what takes the time)
-            if (attempt == 0 ? clusters_that_fit(c.v->stack, c.stack) >= 2 * layers - 1 && cluster_attributes(c.v->kern, c.shape) == cudaSuccess
-                             : clusters_that_fit(c.v->kern, c.shape) >= 1) {
-              rv = c.v; g->regc = c.shape; g->regc.ok = true; g->reg_kern = rv->kern;
-              if (attempt == 0) { g->stack = c.stack; g->stack.ok = true; g->stack_kern = rv->stack; }
-              break;
-            }
-        }
+      const std::vector<const grim_bcr*> upper(g->Wih.begin() + 1, g->Wih.end());
+      const int cols_hh = max_band_columns(g->Whh), cols_all = stack ? std::max(cols_hh, max_band_columns(upper)) : 0;
+      Candidate hh{}, all{};
+      for (int cs = 16; cs >= 1 && !hh.v && H <= 65536; cs >>= 1) {
+        const std::vector<Candidate> own = candidates(cols_hh, cs, false);
+        if (stack && !own.empty())
+          for (const Candidate& c : candidates(cols_all, cs, true)) {
+            if (c.cost > kLongerSteps * own[0].cost) break;
+            if (clusters_that_fit(c.v->stack, c.stack) >= 2 * layers - 1) { all = c; break; }
+          }
+        for (const Candidate& c : own)
+          // (where the blocks with helpers fit, those without do)
+          if (c.v == all.v && c.shape.ks == all.shape.ks ? cluster_attributes(c.v->kern, c.shape) == cudaSuccess : clusters_that_fit(c.v->kern, c.shape) >= 1) {
+            hh = c;
+            break;
+          }
+        if (!hh.v) all = Candidate{};
       }
-      if (g->regc.ok) {
-        // register image: for every thread of every CTA the columns it owns (global index + values at row positions); threads
+      if (hh.v) {
+        g->regc = hh.shape; g->regc.ok = true; g->reg_kern = hh.v->kern;
+        // register images: for every thread of every CTA the columns it owns (global index + values at row positions); threads
         // are numbered with the variant's stride
-        const int NI = rv->ni, S = rv->s, S2 = (S + 1) / 2, TH = rv->threads, ks = g->regc.ks, tpc = g->regc.tpc, cs = g->regc.ctas, nbb = 3 * tpc;
-        const size_t nval = (size_t)cs * NI * S * BHc * TH, ncol = (size_t)cs * NI * S2 * TH;
         struct Image { std::vector<float> val; std::vector<uint32_t> col; };
         struct ColRec { uint32_t col, rowmask, kc; const float* v; };  // kept row a (of rowmask) has v[a * kc]
-        auto image_of = [&](const grim_bcr* wh) {  // empty: does not fit
-          Image im{std::vector<float>(nval), std::vector<uint32_t>(ncol)};
+        auto image_of = [&](const grim_bcr* wh, const Candidate& c) {  // empty: does not fit
+          const int NI = c.v->ni, S = c.v->s, S2 = (S + 1) / 2, TH = c.v->threads, ks = c.shape.ks, tpc = c.shape.tpc, cs = c.shape.ctas, nbb = 3 * tpc;
+          Image im{std::vector<float>((size_t)cs * NI * S * BHc * TH), std::vector<uint32_t>((size_t)cs * NI * S2 * TH)};
           std::vector<float>& iv = im.val;
           std::vector<uint32_t>& ic = im.col;
           std::vector<ColRec> cols, dealt;
@@ -1380,19 +1387,29 @@ extern "C" grim_status_t grim_gru_create(int layers, const grim_bcr_t* W_ih, con
             }
           return im;
         };
-        // (a thread per matrix: most of the time that creating a model takes)
+        // (a thread per image: most of the time that creating a model takes)
         std::vector<std::future<Image>> images;
-        for (const grim_bcr* wh : mats) images.push_back(std::async(image_of, wh));
+        for (const grim_bcr* w : g->Whh) images.push_back(std::async(image_of, w, hh));
+        if (all.v) {
+          g->stack = all.stack; g->stack.ok = true; g->stack_kern = all.v->stack;
+          g->stack_hh = 0;
+          if (all.v != hh.v || all.shape.ks != hh.shape.ks) {  // (of another variant)
+            g->stack_hh = (int)images.size();
+            for (const grim_bcr* w : g->Whh) images.push_back(std::async(image_of, w, all));
+          }
+          g->stack_ih = (int)images.size() - 1;  // (none for layer 0)
+          for (const grim_bcr* w : upper) images.push_back(std::async(image_of, w, all));
+        }
         for (std::future<Image>& f : images) {
           const Image im = f.get();
           if (st == GRIM_OK && im.val.empty()) st = GRIM_ERR_UNSUPPORTED;
           if (st != GRIM_OK) continue;
           float* dv = nullptr;
           uint32_t* dc = nullptr;
-          cudaError_t e = cudaMalloc((void**)&dv, nval * 4);
-          if (e == cudaSuccess) { g->d_img_val.push_back(dv); e = cudaMalloc((void**)&dc, ncol * 4); }
-          if (e == cudaSuccess) { g->d_img_col.push_back(dc); e = cudaMemcpy(dv, im.val.data(), nval * 4, cudaMemcpyHostToDevice); }
-          if (e == cudaSuccess) e = cudaMemcpy(dc, im.col.data(), ncol * 4, cudaMemcpyHostToDevice);
+          cudaError_t e = cudaMalloc((void**)&dv, im.val.size() * 4);
+          if (e == cudaSuccess) { g->d_img_val.push_back(dv); e = cudaMalloc((void**)&dc, im.col.size() * 4); }
+          if (e == cudaSuccess) { g->d_img_col.push_back(dc); e = cudaMemcpy(dv, im.val.data(), im.val.size() * 4, cudaMemcpyHostToDevice); }
+          if (e == cudaSuccess) e = cudaMemcpy(dc, im.col.data(), im.col.size() * 4, cudaMemcpyHostToDevice);
           if (e != cudaSuccess) st = e == cudaErrorMemoryAllocation ? GRIM_ERR_ALLOC : GRIM_ERR_CUDA;
         }
       }
@@ -1470,9 +1487,9 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
     for (int l = 0; l < L; ++l) {
       float* seq_out = l == L - 1 ? y : g->d_seq[l & 1];
       if (l > 0)
-        k.role[2 * l - 1] = {g->d_img_val[(size_t)(L + l - 1)], g->d_img_col[(size_t)(L + l - 1)], g->d_bih[(size_t)l], g->d_seq[(l - 1) & 1],
+        k.role[2 * l - 1] = {g->d_img_val[(size_t)(g->stack_ih + l)], g->d_img_col[(size_t)(g->stack_ih + l)], g->d_bih[(size_t)l], g->d_seq[(l - 1) & 1],
                              g->d_gi[(size_t)l], nullptr, nullptr, 1};
-      k.role[2 * l] = {g->d_img_val[(size_t)l], g->d_img_col[(size_t)l], g->d_bhh[(size_t)l], g->d_gi[(size_t)l], seq_out,
+      k.role[2 * l] = {g->d_img_val[(size_t)(g->stack_hh + l)], g->d_img_col[(size_t)(g->stack_hh + l)], g->d_bhh[(size_t)l], g->d_gi[(size_t)l], seq_out,
                        h0 ? h0 + (int64_t)l * H : nullptr, hT ? hT + (int64_t)l * H : nullptr, l > 0};
     }
     if (g->profile) profile_mark(g, 2, s0);

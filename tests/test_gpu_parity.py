@@ -1016,6 +1016,7 @@ def build_gru(B, m, max_T):
 
 
 def check_gru(B, m, h0=None, grid_kernel=False):
+    """Two passes on one handle against the oracle; returns the launches of the second."""
     T, H, L = m["T"], m["hidden"], len(m["layers"])
     g, handles = build_gru(B, m, T)
     try:
@@ -1025,11 +1026,14 @@ def check_gru(B, m, h0=None, grid_kernel=False):
         y = torch.full((T, H), float("nan"), device="cuda")
         hT = torch.full((L, H), float("nan"), device="cuda")
         for _ in range(2):  # the handle is reusable
+            n0 = B.grim_launch_count()
             B.grim_gru_seq(g, x, y, h0=to_dev(h0) if h0 is not None else None, hT=hT)
             assert B.grim_gru_status(g) == B.GRIM_OK
+            launches = B.grim_launch_count() - n0
         want_y, want_h = orc.gru_seq(m["layers"], m["x"], h0=h0)
         assert rel_fro(y.cpu().numpy(), want_y) <= F32_TOL, rel_fro(y.cpu().numpy(), want_y)
         assert rel_fro(hT.cpu().numpy(), want_h) <= F32_TOL
+        return launches
     finally:
         B.grim_gru_destroy(g)
         for h in handles:
@@ -1105,15 +1109,36 @@ def test_gru_unit_groups_for_fewer_blocks_than_the_largest_cluster(B, cfg):
         check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 207, 0))
 
 
-@pytest.mark.parametrize("cfg", [(9, 64, 2, 1, 8, 32, 4), (9, 64, 3, 2, 8, 32, 4), (12, 72, 2, 3, 4, 16, 3), (30, 1040, 2, 5, 8, 32, 10), (20, 1536, 3, 4, 16, 64, 30),
-                                 (17, 1200, 2, 9, 4, 16, 16), (8, 16, 3, 150, 16, 16, 2)])
+@pytest.mark.parametrize("cfg", [(9, 64, 2, 1, 8, 32, 4), (9, 64, 3, 2, 8, 32, 4), (12, 72, 2, 3, 4, 16, 3), (30, 1000, 2, 5, 8, 32, 10), (20, 1280, 3, 4, 16, 64, 30),
+                                 (17, 1000, 2, 9, 4, 16, 16), (8, 16, 3, 150, 16, 16, 2)])
 def test_gru_layers_in_one_launch(B, cfg):
-    """Sequences shorter than what is brought ahead, layers whose words per thread block are more than are in flight at once, a last
-    thread block with fewer units; three times on one handle (the buffers between the layers start anew)."""
+    """Sequences shorter than what is brought ahead, more inputs to a projection than are in flight at once (1280), a last thread block
+    with fewer units (1000); twice on each handle (the buffers between the layers start anew).  A transposing launch, the first layer's
+    projection, the layers."""
     in_f, H, L, T, bh, bw, rate = cfg
     m = gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=441)
-    check_gru(B, m)
-    check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 442, 0))
+    assert check_gru(B, m) == 3
+    assert check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 442, 0)) == 3
+
+
+@pytest.mark.parametrize("cfg", [(30, 1040, 2, 5, 8, 32, 10), (20, 1536, 3, 4, 16, 64, 30), (17, 1200, 2, 9, 4, 16, 16)])
+def test_gru_layers_beyond_the_registers(B, cfg):
+    """Layers that no variant of the register-resident kernels holds: one after the other over the whole grid."""
+    in_f, H, L, T, bh, bw, rate = cfg
+    m = gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=441)
+    assert check_gru(B, m) == 1 + 2 * L
+    assert check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 442, 0)) == 1 + 2 * L
+
+
+@pytest.mark.parametrize("cfg", [(40, 256, 2, 60, 8, 32, 8, 2), (20, 512, 3, 53, 8, 32, 10, 4), (20, 512, 2, 60, 8, 32, 16, 2)])
+def test_gru_input_weights_denser_than_the_recurrent_ones(B, cfg):
+    """The upper layers' W_ih would need a variant whose steps are much longer than W_hh's: the layers run chunk by chunk."""
+    in_f, H, L, T, bh, bw, rate, rate_ih = cfg
+    m = gen.gru_model(in_f, H, L, T, bh=bh, bw=bw, compression=rate, seed=461)
+    for l, lay in enumerate(m["layers"][1:]):
+        lay["mask_ih"] = gen.bcr_mask(3 * H, H, bh, bw, compression=rate_ih, seed=462 + l)
+    pieces = 2
+    assert check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 463, 0)) == 2 + (2 * L - 1) * pieces
 
 
 @pytest.mark.parametrize("cfg", [(37, 128, 2, 33, 4, 16), (20, 96, 1, 31, 16, 32), (64, 160, 3, 64, 16, 64), (9, 60, 2, 2, 5, 16), (500, 64, 2, 7, 8, 32)])
