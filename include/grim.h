@@ -318,11 +318,12 @@ grim_status_t grim_gru_destroy(grim_gru_t g);
 grim_status_t grim_gru_step(grim_gru_t g, const float* x_dev, int64_t B, float* h_dev, float* y_dev, grim_stream_t stream);
 
 /* Layer pipelining of grim_gru_seq (execution detail, Section 4.2's concern with keeping all units busy; the paper
- * has no multi-layer schedule).  Two or three layers whose matrices fit the registers run in one launch, each layer a
- * few steps behind the one below it.  Otherwise the sequence is cut into `chunks` pieces in time and layer l works on
+ * has no multi-layer schedule).  The sequence is cut into `chunks` pieces in time (at most 8) and layer l works on
  * piece k while layer l - 1 works on piece k + 1, each layer on an internal stream ordered by events; the caller's stream
- * continues after the last layer.  Stacks of more than three layers are not pipelined.  chunks = 0 lets the library
- * choose, 1 runs the layers one after the other on the caller's stream, at most 8.  Results do not depend on it. */
+ * continues after the last layer.  Stacks of more than three layers are not pipelined.  chunks = 1 runs the layers one
+ * after the other on the caller's stream, 0 lets the library choose: two or three layers whose matrices fit the
+ * registers run in one launch, each layer a few steps behind the one below it.  Results are the same up to the order
+ * in which fp32 sums are rounded. */
 grim_status_t grim_gru_set_pipeline(grim_gru_t g, int chunks);
 
 /* grim_gru_seq without any device allocation behind it.  (The paper has no counterpart: this entry

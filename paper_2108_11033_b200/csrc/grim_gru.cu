@@ -1439,8 +1439,9 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
   const int BHc = g->bh <= 4 ? 4 : (g->bh <= 8 ? 8 : 16);
   if (cudaMemsetAsync(g->d_sync, 0, (size_t)(L + 1) * 4, s0) != cudaSuccess) return GRIM_ERR_CUDA;
 
-  // All layers in one launch, unless they are to run one after the other (as the static variant does, whose layers share their scratch).
-  const bool stacked = use_reg && g->stack.ok && g->pipeline;
+  // All layers in one launch, unless they are to run in a given number of pieces or one after the other (as the static variant does,
+  // whose layers share their scratch).
+  const bool stacked = use_reg && g->stack.ok && g->pipeline && g->want_chunks == 0;
   // Otherwise time is cut into chunks; layer l works on chunk k while layer l - 1 works on chunk k + 1 (each layer on its own
   // stream, ordered by events), so a stack of L layers takes about (1 + (L - 1) / chunks) single-layer times instead
   // of L.  The kernels with a global barrier (fall-back) and single-layer models run as one chunk on one stream.

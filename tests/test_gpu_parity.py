@@ -1169,7 +1169,9 @@ def test_config2_gru_full(B, grid_kernel):
 @pytest.mark.parametrize("chunks", [1, 2, 5, 8])
 def test_gru_layer_pipelining_gives_the_same_result(B, chunks):
     """Three layers cut into `chunks` pieces in time and run as a wavefront on internal streams: same outputs and
-    final states as the oracle, with and without an initial state, on a sequence length that does not divide."""
+    final states as the oracle, with and without an initial state, on a sequence length that does not divide.  A transposing
+    launch, the first layer's projection, and per piece a recurrent launch per layer and a projection per upper one
+    (pieces are multiples of four steps: eight of 53 are seven)."""
     m = gen.gru_model(30, 128, 3, 53, bh=8, bw=32, compression=4, seed=95)
     T, H, L = m["T"], m["hidden"], 3
     g, handles = build_gru(B, m, T)
@@ -1179,7 +1181,9 @@ def test_gru_layer_pipelining_gives_the_same_result(B, chunks):
         for init in (None, h0):
             y = torch.full((T, H), float("nan"), device="cuda")
             hT = torch.full((L, H), float("nan"), device="cuda")
+            n0 = B.grim_launch_count()
             B.grim_gru_seq(g, to_dev(m["x"]), y, h0=to_dev(init) if init is not None else None, hT=hT)
+            assert B.grim_launch_count() - n0 == 2 + 5 * min(chunks, 7)
             assert B.grim_gru_status(g) == B.GRIM_OK
             want_y, want_h = orc.gru_seq(m["layers"], m["x"], h0=init)
             assert rel_fro(y.cpu().numpy(), want_y) <= F32_TOL
