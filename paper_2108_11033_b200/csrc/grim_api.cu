@@ -28,6 +28,8 @@ SpmmArgs mat_args(const grim_mat_t* X, const grim_mat_t* Y) {
   return a;
 }
 
+constexpr int kSplitTile = 64;  // (tile_n under path 1) the split kernel
+
 // Slot of the tune cache for a request: right-hand sides whose widths fall into the same power-of-two bucket share
 // an answer (tile choices change with the order of magnitude of N, not with N).
 grim_tune_t* tuned_slot(grim_bcr_t h, const grim_mat_t* X, const grim_mat_t* Y) {
@@ -64,7 +66,7 @@ grim_status_t run_choice(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, a.tile_n == 4 ? 0 : a.tile_n / 8, s);
   }
   if (path == 1 && direct_choice(a.tile_n)) return launch_direct(h, a, s);
-  if (path == 1 && a.tile_n >= 64 && a.tile_n <= 72 && split_path_supported(h, a)) return launch_split(h, a, s);
+  if (path == 1 && a.tile_n >= kSplitTile && a.tile_n <= kSplitTile + 8 && split_path_supported(h, a)) return launch_split(h, a, s);
   if (path == 0 && X->cols > 1 && X->cols <= kSkinnyMaxN && direct_preferred(h, a)) return launch_direct(h, a, s);
   if (path == 0 && narrow_preferred(h, a))
     return launch_narrow(h, X->ptr, X->dtype, X->ld, X->cols, Y->ptr, Y->dtype, Y->ld, 0, s);
@@ -109,9 +111,10 @@ grim_status_t run_spmm(grim_bcr_t h, const grim_mat_t* X, grim_mat_t* Y, const g
   if (st != GRIM_OK) return st;
   if (tune) return run_choice(h, X, Y, tune, s);
   // no explicit choice: an earlier grim_bcr_tune for this kind of request decides, unless its kernel cannot take these operands
-  // (it was found with others, whose alignment or strides may differ)
+  // (it was found with others, whose alignment or strides may differ) or is the split kernel, which is as exact as the others at
+  // some widths of a slot and not at all of them
   const grim_tune_t* t = tuned_slot(h, X, Y);
-  if (t->path != 0) {
+  if (t->path != 0 && !(t->path == 1 && t->tile_n == kSplitTile && !split_precise(h, mat_args(X, Y)))) {
     st = run_choice(h, X, Y, t, s);
     if (st != GRIM_ERR_UNSUPPORTED) return st;
   }
@@ -219,7 +222,7 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
   float best_t = -1.f;
   grim_tune_t cand_best{};
   // candidates: (path, tile_n); a candidate that cannot take the request is skipped
-  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {1, 64}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {3, 4}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
+  const int cand[][2] = {{1, 32}, {1, 1}, {1, 2}, {1, 4}, {1, 8}, {1, 9}, {1, 17}, {1, 18}, {1, 20}, {1, kSplitTile}, {2, 0}, {5, 0}, {3, 1}, {3, 2}, {3, 4}, {4, 16}, {4, 32}, {4, 64}, {4, 128}};
   for (const auto& cd : cand) {
     grim_tune_t c{};
     c.path = cd[0];
@@ -232,8 +235,8 @@ extern "C" grim_status_t grim_bcr_tune(grim_bcr_t h, const grim_mat_t* X, grim_m
     // ... 17, 18, 20 = the narrow tile (at most 16 columns) with 1, 2, 4 bands per warp
     if (c.path == 1 && c.tile_n >= 17 && c.tile_n < 32 && (X->cols > 16 || c.tile_n - 16 > (h->bh <= 8 ? 4 : 2))) continue;
     if (c.path == 1 && c.tile_n < 17 && X->cols <= 16) continue;
-    // ... 64 = fp32 on the tensor cores: where it is as exact as the others
-    if (c.path == 1 && c.tile_n == 64 && !split_precise(h, mat_args(X, Y))) continue;
+    // ... fp32 on the tensor cores: where it is as exact as the others
+    if (c.path == 1 && c.tile_n == kSplitTile && !split_precise(h, mat_args(X, Y))) continue;
     st = run_spmm(h, X, Y, &c, s);  // warm-up
     if (st == GRIM_ERR_UNSUPPORTED) { st = GRIM_OK; continue; }
     if (st != GRIM_OK) break;

@@ -351,6 +351,40 @@ def test_split_operands_elements_beside_large_ones(B, power, few, large, parts):
     assert_elements(got, W * mask, X)
 
 
+@pytest.mark.parametrize("M,K,rate,N", [(1024, 1024, 8, 640), (2048, 512, 16, 640), (2048, 512, 16, 768)])
+def test_tuned_split_operands_only_where_as_exact(B, M, K, rate, N):
+    """The tile search at 1024 columns finds the kernel above; at widths of the same power of two where that is less exact than what runs
+    otherwise, the search's answer is not taken."""
+    W = gen.dense_weight(M, K, seed=471)
+    mask = gen.bcr_mask(M, K, 4, 16, compression=rate, dist="uniform", seed=472)
+    X = to_dev(gen.normal_f32((K, 1024), 1.0, 473, 0))
+    tuned, plain = (B.grim_bcr_pack(W, mask, 4, 16, B.GRIM_F32, 1) for _ in range(2))
+    try:
+        t = B.grim_bcr_tune(tuned, X, torch.empty(M, 1024, device="cuda"), reps=20)
+        if (t["path"], t["tile_n"]) != (1, 64):  # (it takes 20 us here and the next one 27)
+            pytest.skip("another kernel was faster")
+        out = []
+        for h in (tuned, plain):
+            out.append(torch.empty(M, N, device="cuda"))
+            B.grim_bcr_spmm(h, X[:, :N].contiguous(), out[-1])
+        assert torch.equal(*out)
+    finally:
+        B.grim_bcr_destroy(tuned)
+        B.grim_bcr_destroy(plain)
+
+
+def test_tile_search_at_sixteen_columns_leaves_split_operands_out(B):
+    """There the kernels that run otherwise spread a row over 32 lanes and are more exact."""
+    M = K = 8192
+    h = B.grim_bcr_pack(gen.dense_weight(M, K, seed=474), gen.bcr_mask(M, K, 8, 32, compression=4, dist="uniform", seed=475), 8, 32, B.GRIM_F32, 1)
+    try:
+        X = to_dev(gen.normal_f32((K, 16), 1.0, 476, 0))
+        t = B.grim_bcr_tune(h, X, torch.empty(M, 16, device="cuda"), reps=-3)
+        assert (t["path"], t["tile_n"]) != (1, 64)
+    finally:
+        B.grim_bcr_destroy(h)
+
+
 @pytest.mark.parametrize("geom", [(1, 200, 130, 25, 27, 3, 1, 1), (2, 133, 260, 31, 33, 5, 2, 2), (3, 400, 72, 61, 63, 3, 2, 0),
                                   (3, 16, 264, 48, 61, 16, 3, 5), (2, 700, 500, 30, 29, 1, 1, 0), (5, 400, 520, 13, 15, 3, 1, 1)])
 def test_split_operands_convolution(B, geom):
