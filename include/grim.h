@@ -356,7 +356,8 @@ grim_status_t grim_gru_seq_static(grim_gru_t g, const float* x_dev, int64_t T, c
 /* Test hook for the bounded waits of the recurrent kernel (no counterpart in the paper): thread
  * block `skip_cta` stays away from the per-step barrier (-1 = normal operation) and a waiting
  * block gives up after `spin_limit` polls (0 = default).  With a block missing, every wait runs
- * out, the kernel returns, and grim_gru_status reports GRIM_ERR_TIMEOUT; nothing waits forever. */
+ * out, the kernel returns, and grim_gru_status reports GRIM_ERR_TIMEOUT; nothing waits forever.
+ * skip_cta = -2, for models whose layers run in one launch: what the upper layers wait for is withheld instead. */
 grim_status_t grim_gru_debug_barrier(grim_gru_t g, int skip_cta, unsigned spin_limit);
 
 /* Per-kernel timing of the GRU path (measurement aid, Section 6 reports per-kernel times): when

@@ -80,6 +80,7 @@ struct grim_gru {
   int device = -1;
   cudaStream_t last_stream = nullptr;
   int dbg_skip_cta = -1;
+  float* d_never = nullptr;  // (test hook) pre-activations that never arrive
   unsigned spin_limit = 1u << 22;
   bool force_grid = false;
   bool profile = false;
@@ -119,6 +120,7 @@ struct GruParams {
 // The stacked kernel: cluster c of a launch plays role[c], an even one the recurrence of layer c / 2, an odd one the
 // projection of layer (c + 1) / 2.
 constexpr int kMaxStack = 3;                    // layers in one launch
+constexpr int kWithhold = -2;                   // (grim_gru_debug_barrier)
 constexpr unsigned kNotYet = 0xFFFFFFFFu;       // what buffers between clusters are filled with: a NaN that no arithmetic produces
 struct GruRole {
   const float* img_val;
@@ -608,6 +610,7 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
       lost = __any_sync(0xffffffffu, lost);
     }
   }
+  if (*s_failed) ptx::let_copies_land();
   cluster.sync();  // no CTA leaves while another may still address its shared memory
 }
 
@@ -942,6 +945,7 @@ __global__ void __launch_bounds__(THREADS + kHelperThreads, 1) gru_stack_kernel(
     }
   }
   meet();
+  if (*s_failed) ptx::let_copies_land();
   cluster.sync();  // no CTA leaves while another may still address its shared memory
 }
 
@@ -1100,6 +1104,7 @@ void destroy(grim_gru* g) {
   for (uint32_t* p : g->d_pos_of_band_ih) cudaFree(p);
   for (float* p : g->d_img_val) cudaFree(p);
   for (uint32_t* p : g->d_img_col) cudaFree(p);
+  cudaFree(g->d_never);
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
   for (float* p : g->d_gi) cudaFree(p);
   for (cudaStream_t st : g->lstream) cudaStreamDestroy(st);
@@ -1490,8 +1495,8 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
       if (l > 0)
         k.role[2 * l - 1] = {g->d_img_val[(size_t)(g->stack_ih + l)], g->d_img_col[(size_t)(g->stack_ih + l)], g->d_bih[(size_t)l], g->d_seq[(l - 1) & 1],
                              g->d_gi[(size_t)l], nullptr, nullptr, 1};
-      k.role[2 * l] = {g->d_img_val[(size_t)(g->stack_hh + l)], g->d_img_col[(size_t)(g->stack_hh + l)], g->d_bhh[(size_t)l], g->d_gi[(size_t)l], seq_out,
-                       h0 ? h0 + (int64_t)l * H : nullptr, hT ? hT + (int64_t)l * H : nullptr, l > 0};
+      k.role[2 * l] = {g->d_img_val[(size_t)(g->stack_hh + l)], g->d_img_col[(size_t)(g->stack_hh + l)], g->d_bhh[(size_t)l],
+                       l > 0 && g->dbg_skip_cta == kWithhold ? g->d_never : g->d_gi[(size_t)l], seq_out, h0 ? h0 + (int64_t)l * H : nullptr, hT ? hT + (int64_t)l * H : nullptr, l > 0};
     }
     if (g->profile) profile_mark(g, 2, s0);
     const cudaError_t e = launch_cluster(g->stack_kern, g->stack, k, s0, 2 * L - 1);
@@ -1597,9 +1602,20 @@ extern "C" grim_status_t grim_gru_status(grim_gru_t g) {
 // Test hook: selects the cooperative-grid kernel (the one with spin waits) whenever skip_cta >= 0 or a
 // poll limit is given, makes thread block `skip_cta` stay away from its barrier and sets the number of
 // polls after which a waiting block gives up.  The waits then run out and the status word reports it;
-// no thread block ever waits without a bound.
+// no thread block ever waits without a bound.  skip_cta = kWithhold leaves the choice of kernel; where the layers run in one
+// launch, the upper layers' pre-activations never arrive.
 extern "C" grim_status_t grim_gru_debug_barrier(grim_gru_t g, int skip_cta, unsigned spin_limit) {
   if (!g) return GRIM_ERR_INVALID_ARG;
+  if (skip_cta == kWithhold) {
+    if (!g->stack.ok) return GRIM_ERR_UNSUPPORTED;
+    const size_t bytes = (size_t)g->max_T * 3 * g->H * 4;
+    if (!g->d_never && cudaMalloc((void**)&g->d_never, bytes) != cudaSuccess) { cudaGetLastError(); return GRIM_ERR_ALLOC; }
+    if (cudaMemset(g->d_never, 0xFF, bytes) != cudaSuccess) return GRIM_ERR_CUDA;  // kNotYet
+    g->dbg_skip_cta = skip_cta;
+    g->spin_limit = spin_limit ? spin_limit : (1u << 22);
+    g->force_grid = false;
+    return GRIM_OK;
+  }
   if ((skip_cta >= 0 || spin_limit) && !g->grid.ok) return GRIM_ERR_UNSUPPORTED;
   g->dbg_skip_cta = skip_cta;
   g->spin_limit = spin_limit ? spin_limit : (1u << 22);

@@ -1276,3 +1276,24 @@ def test_gru_bounded_wait_reports_timeout(B):
     B.grim_gru_destroy(g)
     for h in handles:
         B.grim_bcr_destroy(h)
+
+
+@pytest.mark.parametrize("L,T", [(2, 1), (2, 7), (3, 12)])
+def test_gru_bounded_waits_between_layers_report_timeout(B, L, T):
+    """What the upper layers of a single launch wait for never comes: their waits run out, the launch ends and the status word says
+    so; afterwards the handle works normally."""
+    m = gen.gru_model(20, 256, L, T, bh=8, bw=32, compression=4, seed=83)
+    g, handles = build_gru(B, m, T)
+    x = to_dev(m["x"])
+    y = torch.zeros(T, 256, device="cuda")
+    B.grim_gru_debug_barrier(g, -2, 2000)
+    B.grim_gru_seq(g, x, y)
+    assert B.grim_gru_status(g) == B.GRIM_ERR_TIMEOUT
+    B.grim_gru_debug_barrier(g, -1, 0)
+    B.grim_gru_seq(g, x, y)
+    assert B.grim_gru_status(g) == B.GRIM_OK
+    want_y, _ = orc.gru_seq(m["layers"], m["x"])
+    assert rel_fro(y.cpu().numpy(), want_y) <= F32_TOL
+    B.grim_gru_destroy(g)
+    for h in handles:
+        B.grim_bcr_destroy(h)
