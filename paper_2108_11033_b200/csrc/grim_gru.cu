@@ -1446,7 +1446,9 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
 
   // All layers in one launch, unless they are to run in a given number of pieces or one after the other (as the static variant does,
   // whose layers share their scratch).
-  const bool stacked = use_reg && g->stack.ok && g->pipeline && g->want_chunks == 0;
+  // (The transposing launch then has up to kFillRows rows of blocks more than the input has: a grid has 65535.)
+  constexpr int64_t kFillRows = 512;
+  const bool stacked = use_reg && g->stack.ok && g->pipeline && g->want_chunks == 0 && (g->Wih[0]->K + 31) / 32 <= 65535 - kFillRows;
   // Otherwise time is cut into chunks; layer l works on chunk k while layer l - 1 works on chunk k + 1 (each layer on its own
   // stream, ordered by events), so a stack of L layers takes about (1 + (L - 1) / chunks) single-layer times instead
   // of L.  The kernels with a global barrier (fall-back) and single-layer models run as one chunk on one stream.
@@ -1562,7 +1564,7 @@ extern "C" grim_status_t grim_gru_seq(grim_gru_t g, const float* x, int64_t T, c
               fill.at[2 * b - 1] = reinterpret_cast<uint4*>(g->d_gi[(size_t)b]); fill.n[2 * b - 1] = T * 3 * H / 4;
               pieces += T * H;
             }
-            const unsigned fb = (unsigned)std::min<int64_t>(((pieces + 511) / 512 + tb - 1) / tb, 512);  // two pieces per thread
+            const unsigned fb = (unsigned)std::min<int64_t>(((pieces + 511) / 512 + tb - 1) / tb, kFillRows);  // two pieces per thread
             transpose_input_kernel<<<dim3(tb, kb + fb), dim3(32, 8), 0, s>>>(x, g->d_xT, T, K0, ldT, (int)kb, fill);
             count_launch();
           }

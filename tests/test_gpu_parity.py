@@ -1155,6 +1155,30 @@ def test_gru_layers_in_one_launch(B, cfg):
     assert check_gru(B, m, h0=gen.normal_f32((L, H), 0.5, 442, 0)) == 3
 
 
+def test_gru_as_many_inputs_as_a_grid_has_rows(B):
+    """2,097,120 inputs: the transposing launch has no rows of blocks left for filling the buffers between the layers."""
+    in_f, H = 65535 * 32, 16
+    m = gen.gru_model(64, H, 2, 3, bh=16, bw=64, compression=2, seed=481)
+    lay, x = m["layers"][0], m["x"]
+    at = np.concatenate([np.arange(32), np.arange(in_f - 32, in_f)])  # where the 64 inputs lie
+    def wide(a):
+        out = np.zeros((a.shape[0], in_f), a.dtype)
+        out[:, at] = a
+        return out
+    big = dict(m, x=wide(x), layers=[dict(lay, W_ih=wide(lay["W_ih"]), mask_ih=wide(np.ones_like(lay["mask_ih"])))] + m["layers"][1:])
+    g, handles = build_gru(B, big, 3)
+    try:
+        y = torch.full((3, H), float("nan"), device="cuda")
+        B.grim_gru_seq(g, to_dev(big["x"]), y)
+        assert B.grim_gru_status(g) == B.GRIM_OK
+        want_y, _ = orc.gru_seq([dict(lay, mask_ih=np.ones_like(lay["mask_ih"]))] + m["layers"][1:], x)
+        assert rel_fro(y.cpu().numpy(), want_y) <= F32_TOL
+    finally:
+        B.grim_gru_destroy(g)
+        for h in handles:
+            B.grim_bcr_destroy(h)
+
+
 @pytest.mark.parametrize("cfg", [(30, 1040, 2, 5, 8, 32, 10), (20, 1536, 3, 4, 16, 64, 30), (17, 1200, 2, 9, 4, 16, 16)])
 def test_gru_layers_beyond_the_registers(B, cfg):
     """Layers that no variant of the register-resident kernels holds: one after the other over the whole grid."""
