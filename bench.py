@@ -220,7 +220,7 @@ class GruWorkload:
             self.notional_bytes += self.T * (ih.value_bytes + ih.index_bytes_gemv + 3 * self.H * 4 + 2 * self.H * 4)
         self.h2d = self.x_host.numel() * 4
         self.d2h = self.y_host.numel() * 4
-        self.kernel = "gru_cluster_reg_kernel"
+        self.kernel = "gru_stack_kernel"
         self.peak_kind = "alu"
         self.force_bound = "hbm"  # far from any throughput roof: a chain of T dependent steps (latency-bound)
 
@@ -317,12 +317,13 @@ class SpmmWorkload:
             self.tuned = B.grim_bcr_tune(h, x, y, reps=-5 if self.rotating else 5)
         torch.cuda.synchronize()
         tile = self.tuned["tile_n"]
-        names = {1: "bcr_split_kernel" if tile == 64 else ("bcr_direct_kernel" if tile & 32 else "bcr_ffma_kernel"), 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
+        split = self.tuned["path"] == 1 and tile == 64
+        names = {1: "bcr_split_kernel" if split else ("bcr_direct_kernel" if tile & 32 else "bcr_ffma_kernel"), 2: "bcr_tc_kernel", 4: "bcr_spmm_kernel", 5: "bcr_tc2_kernel",
                  3: "bcr_narrow_kernel" if tile >= 4 else ("bcr_skinny_kernel" if tile == 1 else "bcr_stream_kernel")}
         self.kernel = names.get(self.tuned["path"], self.kernel)
-        self.peak_kind = "tensor" if self.tuned["path"] in (2, 5) else "alu"
-        if self.peak_kind == "tensor":
-            self.kernel_bytes = float(i.value_bytes + i.index_bytes_tc + i.k_used * self.N * esz + self.M * self.N * 4)
+        self.peak_kind = "split" if split else ("tensor" if self.tuned["path"] in (2, 5) else "alu")
+        if self.peak_kind != "alu":  # (the split kernel's records: two index bytes per value)
+            self.kernel_bytes = float(i.value_bytes + (2 * i.nnz if split else i.index_bytes_tc) + i.k_used * self.N * esz + self.M * self.N * 4)
 
     def step(self):
         h, x, y = self.sets[self._i % len(self.sets)]
@@ -448,13 +449,13 @@ class ConvWorkload:
         self.y_host = torch.empty(self.batch, 512, 28, 28, dtype=tdt).pin_memory()
         i = B.grim_bcr_info(self.h)
         esz = 2 if self.bf16 else 4
-        idx = i.index_bytes_tc if self.bf16 else i.index_bytes_spmm
+        idx = i.index_bytes_tc if self.bf16 else 2 * i.nnz
         self.kernel_bytes = float(i.value_bytes + idx + self.x.numel() * esz + self.y.numel() * esz)
         self.min_bytes = float(i.value_bytes + min_index_bytes(i) + self.x.numel() * esz + self.y.numel() * esz)
         self.h2d = self.x_host.numel() * esz
         self.d2h = self.y_host.numel() * esz
-        self.kernel = "conv_tc_kernel (implicit im2col)" if self.bf16 else "bcr_direct_kernel (implicit im2col)"
-        self.peak_kind = "tensor" if self.bf16 else "alu"
+        self.kernel = "conv_tc_kernel (implicit im2col)" if self.bf16 else "bcr_split_kernel (implicit im2col)"
+        self.peak_kind = "tensor" if self.bf16 else "split"
         self._ev = (torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
         self.sets = [(self.h, self.x, self.y)]
         for _ in range(rotation_sets(self.kernel_bytes) - 1):
@@ -871,14 +872,17 @@ class Bench:
 
     def roofline(self, wl, k_ms):
         """Binding bound of the dominant kernel: the slower of (algorithmic bytes at the measured HBM bandwidth) and
-        (effective flops 2*nnz*N at the peak of the unit that does the arithmetic: the measured fp32 FMA rate, or the
-        measured dense bf16 tensor rate for the tcgen05 kernel)."""
+        (effective flops 2*nnz*N at the peak of the unit that does the arithmetic: the measured fp32 FMA rate, the
+        measured dense bf16 tensor rate for the tcgen05 kernels, or for the one that splits fp32 operands that rate over
+        the six bf16 products of every dense tile)."""
         peaks = self.peaks
-        flop_peak = peaks["bf16_tflops_burst"] if wl.peak_kind == "tensor" else self.ffma_tflops
+        split = wl.peak_kind == "split"
+        flop_peak = (peaks["bf16_tflops_burst"] * wl.nnz / wl.dense_elems / 6 if split else
+                     peaks["bf16_tflops_burst"] if wl.peak_kind == "tensor" else self.ffma_tflops)
         t_hbm = wl.kernel_bytes / (peaks["hbm_gbs"] * 1e9)
         t_min = getattr(wl, "min_bytes", wl.kernel_bytes) / (peaks["hbm_gbs"] * 1e9)
         t_flop = wl.flops / (flop_peak * 1e12)
-        bound = getattr(wl, "force_bound", None) or ("hbm" if t_hbm >= t_flop else wl.peak_kind)
+        bound = getattr(wl, "force_bound", None) or ("hbm" if t_hbm >= t_flop else "tensor" if split else wl.peak_kind)
         t = k_ms * 1e-3
         if bound == "hbm":
             achieved = wl.kernel_bytes / t / 1e9
@@ -890,7 +894,8 @@ class Bench:
             achieved = wl.flops / t / 1e12
             roof = dict(bound=bound, achieved=achieved, peak=flop_peak, unit="TFLOP/s", frac=achieved / flop_peak, traffic=None,
                         kernel=wl.kernel, kernel_ms=k_ms,
-                        peak_source=("measured dense bf16 (burst)" if bound == "tensor" else
+                        peak_source=("measured dense bf16 (burst), six products of every dense tile" if split else
+                                     "measured dense bf16 (burst)" if bound == "tensor" else
                                      f"measured fp32 FMA micro-kernel at run time (derived from unit counts at the maximum "
                                      f"clock: {self.ffma_derived:.1f})"))
         roof["traffic"] = profile_traffic(wl.name)
