@@ -24,10 +24,11 @@
 // per K tile), eight warps add up.  With few tiles the blocks of a cluster share one, each multiplying a part of K; the sums
 // meet over distributed shared memory.
 //
-// What bounds it: the chains of the expanding and the converting warps, some 2200 cycles a K tile (two stages, so that a K tile's operands
-// are written while the tile before it is multiplied) against 1536 of multiplies (8192^2, rate 8, N = 1024: 524 us, 128 K tiles in three
-// rounds and a half; the slab kernel, bound by its fp32 multiplies, 665).  Convolutions read pixels one by one and take 1.55 us a K tile,
-// matrices 1.15.
+// What bounds it: some 2200 cycles a K tile, 1536 of them the multiplies' at their nominal rate (two stages, so that a K tile's operands
+// are written while the tile before it is multiplied): 8192^2, rate 8, N = 1024, 128 K tiles in three rounds and a half, 524 us, where six
+// dense bf16 products at the rate that a library's product reaches take 503.  In loops of seconds the card is at its power limit: 593,
+// and 597 at that product's sustained rate.  (The slab kernel, bound by its fp32 multiplies: 665.)  Convolutions read pixels one by one and
+// take 1.55 us a K tile, matrices 1.15.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -742,7 +743,7 @@ bool split_precise(const grim_bcr* h, const SpmmArgs& a) {
   return here <= there && here1 <= std::max(there1, 3.55e-15);
 }
 
-// Measured against the kernel that runs otherwise (us): 8192^2, 8 x 32, N = 1024: 665 -> 524; 4096^2, 4 x 16, N = 512: 312 -> 91; 2880^2,
+// Measured against the kernel that runs otherwise (us): 8192^2, 8 x 32, N = 1024: 665 -> 524 (593 at the power limit); 4096^2, 4 x 16, N = 512: 312 -> 91; 2880^2,
 // 4 x 16, N = 17: 66 -> 24; 4096 x 512, rate 4, N = 512: 34 -> 20; 4096^2, 16 x 64, N = 1024: equal; 512 -> 512 channels, 28 x 28, one
 // image: 62 -> 39.  Small matrices, few columns: 1533 x 2050, N = 131: 10.7 against 20, and so on.
 // (Below ten million products the direct kernel is done before this one has filled its pipeline, some 12 us: no estimates for the
