@@ -610,7 +610,6 @@ __global__ void __launch_bounds__(THREADS, 1) gru_cluster_reg_kernel(const GruPa
       lost = __any_sync(0xffffffffu, lost);
     }
   }
-  if (*s_failed) ptx::let_copies_land();
   cluster.sync();  // no CTA leaves while another may still address its shared memory
 }
 
